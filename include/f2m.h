@@ -137,13 +137,14 @@ typedef struct {
 #define F2M_FLAG_FINISHER_HOST 16u
 #define F2M_FLAG_FINISHER_GPU 32u
 
-/* f2m_params.flags: run the full pricing scan (pricing = 1) with the
- * tensor-core filter (per 128 x 128 tile pair, quantised coordinates and radii
- * in a frame fitted to the pair; the test |D|^2 < (R_u + R_v)^2 as one exact
- * small-integer fp16 matrix product with an fp32 accumulator; candidates then
- * decided by the fp32 filter and exactly) instead of the default fp32 filter on
- * the CUDA cores.  The same pairs either way; at n = 100k the default is faster
- * (0.96 against 1.3 ms per scan on a GB300). */
+/* f2m_params.flags: run the full pricing scan (pricing = 1) with the filter on
+ * the 5th-generation tensor cores (tcgen05.mma, accumulators in tensor memory)
+ * instead of the default, the same exact small-integer test as mma.sync
+ * products whose results stay in registers (per tile pair, quantised
+ * coordinates and radii in a frame fitted to the pair; |D|^2 < (R_u + R_v)^2;
+ * candidates then decided by an fp32 filter and exactly).  The same pairs
+ * either way; at n = 100k the default is faster (0.39 against 1.3 ms per scan
+ * on a GB300). */
 #define F2M_FLAG_PRICING_TENSOR 64u
 
 typedef struct {
@@ -570,9 +571,11 @@ int64_t f2m_kernel_launches(void);
 /* Checks, on the current device, the tensor-core arithmetic that the full
  * pricing scan's filter relies on (fp16 operands, fp32 accumulator, results
  * that must be exact integers): `rounds` products of 128 x 128 pairs of
- * operand rows drawn from `seed` within the ranges the filter produces, each
- * accumulator value compared with the exact integer product.  *checked: the
- * values compared; *mismatches: those that differ.  Runs on the legacy default
+ * operand rows drawn from `seed` within the ranges the filter produces, for
+ * each of the two scans' instructions (F2M_FLAG_PRICING_TENSOR's tcgen05.mma,
+ * the default's mma.sync), each accumulator value compared with the exact
+ * integer product.  *checked: the values compared per instruction;
+ * *mismatches: those that differ.  Runs on the legacy default
  * stream and synchronizes it.  A diagnostic with no counterpart in the paper.
  * Returns F2M_OK, F2M_ERR_INVALID_ARG (NULL output, rounds < 0), F2M_ERR_CUDA
  * or F2M_ERR_TIMEOUT (an mbarrier wait gave up). */

@@ -340,8 +340,8 @@ extern "C" void f2m_destroy(f2m_ctx* c) {
   dfree(c->d_trace_b2); dfree(c->d_trace_ch); dfree(c->d_pts); dfree(c->d_pairs);
   dfree(c->d_pts4); dfree(c->d_pstat); dfree(c->d_mranges); dfree(c->d_mtblk); dfree(c->d_mbox);
   dfree(c->d_mlmax); dfree(c->d_mframes); dfree(c->d_mcand); dfree(c->d_mncand);
-  dfree(c->d_lam_ref); dfree(c->d_raised); dfree(c->d_pts_raised); dfree(c->d_nraised);
-  dfree(c->d_ranges); dfree(c->d_boxes); dfree(c->d_smax);
+  dfree(c->d_lam_ref); dfree(c->d_raised); dfree(c->d_pts_raised);
+  dfree(c->d_boxes); dfree(c->d_smax); dfree(c->d_pctl); dfree(c->d_pseg); dfree(c->d_plist);
   dfree(c->d_count); dfree(c->d_tile); dfree(c->d_deg); dfree(c->d_tmp_rp); dfree(c->d_new_rp);
   dfree(c->d_block_sums); dfree(c->d_tmp_col); dfree(c->d_out_a); dfree(c->d_out_b);
   dfree(c->d_check); dfree(c->d_scalar); dfree(c->d_bad); dfree(c->d_b); dfree(c->d_b_int);
@@ -480,8 +480,6 @@ f2m_status f2m::create_internal(const int32_t* xy, int32_t n, const int32_t* row
       c->ec_alt_cap = c->ec_cap;
       e = dalloc(&c->d_ec_alt, c->ec_alt_cap);
       if (e == cudaSuccess) e = dalloc(&c->d_pts, n);
-      if (e == cudaSuccess) e = dalloc(&c->d_count, 1);
-      if (e == cudaSuccess) e = dalloc(&c->d_tile, 1);
       if (e == cudaSuccess) e = dalloc(&c->d_pairs, c->pairs_cap);
       if (e == cudaSuccess) e = dalloc(&c->d_deg, n + 1);
       if (e == cudaSuccess) e = dalloc(&c->d_tmp_rp, n + 1);
@@ -492,7 +490,6 @@ f2m_status f2m::create_internal(const int32_t* xy, int32_t n, const int32_t* row
         e = dalloc(&c->d_lam_ref, n);
         if (e == cudaSuccess) e = dalloc(&c->d_raised, n);
         if (e == cudaSuccess) e = dalloc(&c->d_pts_raised, n);
-        if (e == cudaSuccess) e = dalloc(&c->d_nraised, 1);
       }
     }
     if (e == cudaSuccess) e = dalloc(&c->d_lam[0], n);
@@ -752,21 +749,6 @@ extern "C" f2m_status f2m_gdp(f2m_ctx* c, int64_t max_sweeps, int64_t* sweeps, i
   return s;
 }
 
-// pricing scan into d_pairs (grown until every pair fits); count in c->npairs
-// Tile pairs of the pair triangle of every segment selected for this scan.
-static void build_tiles(const f2m_ctx* c, std::vector<int4>& tiles) {
-  tiles.clear();
-  const int32_t nseg = (int32_t)c->seg_off.size() - 1;
-  for (int32_t s = 0; s < nseg; ++s) {
-    if (!c->seg_scan.empty() && !c->seg_scan[s]) continue;
-    const int32_t a = c->seg_off[s], b = c->seg_off[s + 1];
-    for (int32_t i0 = a; i0 < b; i0 += kPricingTile)
-      for (int32_t j0 = i0; j0 < b; j0 += kPricingJ)  // half-height tiles: a shorter last wave
-        tiles.push_back(make_int4(i0, i0 + kPricingTile < b ? i0 + kPricingTile : b, j0,
-                                  j0 + kPricingJ < b ? j0 + kPricingJ : b));
-  }
-}
-
 // the tensor-core scan's tile pairs: per scanned segment, i-blocks of
 // kMmaTileI positions from its start, each against j-blocks of kMmaTileJ from
 // the i-block's start (every pair u < v of the segment in exactly one)
@@ -793,23 +775,140 @@ static void build_mma_tiles(const f2m_ctx* c, std::vector<int4>& tiles, std::vec
   }
 }
 
-// pricing scan into d_pairs (grown until every pair fits); count in c->npairs,
-// per-segment counts in c->seg_pairs
-f2m_status f2m::price_internal(f2m_ctx* c, double* ms, const int32_t* lam_override) {
-  if (!c->d_pts) {
-    CK(c, dalloc(&c->d_pts, c->n));
-    CK(c, dalloc(&c->d_count, 1));
-    CK(c, dalloc(&c->d_tile, 1));
-  }
+// the buffers of a pricing scan, and the segments' positions and blocks
+static f2m_status price_setup(f2m_ctx* c) {
+  const int32_t nseg = (int32_t)c->seg_off.size() - 1;
   if (!c->d_pairs) {
     c->pairs_cap = c->p.pricing_cap;
     CK(c, dalloc(&c->d_pairs, c->pairs_cap));
   }
+  if (c->d_pseg) return F2M_OK;
+  std::vector<int32_t> h(c->seg_off.begin(), c->seg_off.end());
+  int32_t nb = 0;
+  for (int32_t s = 0; s <= nseg; ++s) {
+    h.push_back(nb);
+    if (s < nseg) nb += (c->seg_off[s + 1] - c->seg_off[s] + kPriceBlock - 1) / kPriceBlock;
+  }
+  c->price_blocks = nb;
+  if (!c->d_pts) CK(c, dalloc(&c->d_pts, c->n));
+  CK(c, dalloc(&c->d_boxes, 2LL * nb));  // of the points, and of some rows gathered
+  CK(c, dalloc(&c->d_smax, 2LL * nb));
+  CK(c, dalloc(&c->d_pctl, 1));
+  int32_t* d = nullptr;
+  CK(c, dalloc(&d, 3LL * (nseg + 1) + (nseg + 3) / 4));  // and a byte per segment: scanned
+  c->d_pseg = d;
+  CK(c, cudaMemcpyAsync(d, h.data(), sizeof(int32_t) * h.size(), cudaMemcpyHostToDevice, c->st));
+  CK(c, cudaStreamSynchronize(c->st));
+  return F2M_OK;
+}
+
+// room for `need` pairs, or block pairs, found past the capacity of the last try
+static f2m_status price_grow(f2m_ctx* c, const PriceCtl& h, bool* again) {
+  *again = false;
+  if ((int64_t)h.count > c->pairs_cap) {
+    dfree(c->d_pairs);
+    c->pairs_cap = (int64_t)h.count + ((int64_t)h.count >> 2) + 1024;
+    CK(c, dalloc(&c->d_pairs, c->pairs_cap));
+    *again = true;
+  }
+  if ((int64_t)h.listed > c->plist_cap) {
+    dfree(c->d_plist);
+    c->plist_cap = std::min<int64_t>((int64_t)h.listed + ((int64_t)h.listed >> 3) + 1024, INT_MAX);
+    CK(c, dalloc(&c->d_plist, c->plist_cap));
+    *again = true;
+  }
+  return F2M_OK;
+}
+
+// The scan on the tensor cores (F2M_FLAG_PRICING_TENSOR).
+static f2m_status price_mma(f2m_ctx* c, const int32_t* lam, int32_t fb, double* ms) {
+  // the tile-pair list depends only on the segments scanned: it stays on the
+  // device from one scan to the next while they are the same
+  if (!c->d_pts4) {
+    CK(c, dalloc(&c->d_count, 1));
+    CK(c, dalloc(&c->d_tile, 1));
+    CK(c, dalloc(&c->d_pts4, c->n));
+    CK(c, dalloc(&c->d_pstat, 1));
+    CK(c, dalloc(&c->d_mncand, 1));
+    c->mcand_cap = std::max<int64_t>(4LL * c->n, 1 << 20);
+    CK(c, dalloc(&c->d_mcand, c->mcand_cap));
+  }
+  if (!(c->tiles_valid && c->tiles_seg_scan == c->seg_scan)) {
+    std::vector<int4> tiles, tblk;
+    std::vector<int2> ranges;
+    build_mma_tiles(c, tiles, tblk, ranges);
+    if ((int64_t)ranges.size() > c->mblocks_cap) {
+      dfree(c->d_mranges);
+      dfree(c->d_mbox);
+      dfree(c->d_mlmax);
+      c->mblocks_cap = (int64_t)ranges.size() + 64;
+      CK(c, dalloc(&c->d_mranges, c->mblocks_cap));
+      CK(c, dalloc(&c->d_mbox, c->mblocks_cap));
+      CK(c, dalloc(&c->d_mlmax, c->mblocks_cap));
+    }
+    if ((int64_t)tiles.size() > c->mtiles_cap) {
+      dfree(c->d_tiles);
+      dfree(c->d_mtblk);
+      dfree(c->d_mframes);
+      c->mtiles_cap = (int64_t)tiles.size() + 64;
+      CK(c, dalloc(&c->d_tiles, c->mtiles_cap));
+      CK(c, dalloc(&c->d_mtblk, c->mtiles_cap));
+      CK(c, dalloc(&c->d_mframes, c->mtiles_cap));
+    }
+    if (!tiles.empty()) {
+      CK(c, cudaMemcpyAsync(c->d_mranges, ranges.data(), sizeof(int2) * ranges.size(), cudaMemcpyHostToDevice, c->st));
+      CK(c, cudaMemcpyAsync(c->d_mtblk, tblk.data(), sizeof(int4) * tblk.size(), cudaMemcpyHostToDevice, c->st));
+      CK(c, cudaMemcpyAsync(c->d_tiles, tiles.data(), sizeof(int4) * tiles.size(), cudaMemcpyHostToDevice, c->st));
+    }
+    c->mblocks = (int64_t)ranges.size();
+    c->ntiles = (int64_t)tiles.size();
+    c->tiles_valid = true;
+    c->tiles_seg_scan = c->seg_scan;
+  }
+  CK(c, cudaEventRecord(c->ev0, c->st));
+  CK(c, launch_pricing_mma_prep(c->d_xy, lam, c->plan.perm, c->n, c->d_pts4, c->st));
+  for (bool first = true;; first = false) {
+    if (!first) CK(c, cudaEventRecord(c->ev0, c->st));
+    CK(c, launch_pricing_mma_scan(c->d_pts4, c->d_xy, lam, c->d_rp, c->d_ec, fb, c->d_tiles, c->d_mtblk,
+                                  (int32_t)c->ntiles, c->d_mranges, (int32_t)c->mblocks, c->d_mbox, c->d_mlmax,
+                                  c->d_mframes, c->d_mcand, c->mcand_cap, c->d_mncand, c->d_pairs,
+                                  c->pairs_cap, c->d_count, c->d_tile, c->d_pstat, c->num_sms, c->st));
+    CK(c, cudaEventRecord(c->ev1, c->st));
+    unsigned long long cnt = 0, ncand = 0;
+    int32_t pstat = 0;
+    CK(c, cudaMemcpyAsync(&cnt, c->d_count, sizeof(cnt), cudaMemcpyDeviceToHost, c->st));
+    CK(c, cudaMemcpyAsync(&pstat, c->d_pstat, sizeof(pstat), cudaMemcpyDeviceToHost, c->st));
+    CK(c, cudaMemcpyAsync(&ncand, c->d_mncand, sizeof(ncand), cudaMemcpyDeviceToHost, c->st));
+    CK(c, cudaStreamSynchronize(c->st));
+    if (ms) *ms += elapsed_ms(c);
+    if (pstat) return fail(c, F2M_ERR_TIMEOUT, "pricing scan: a tensor-core wait ran past its budget");
+    if ((int64_t)ncand > c->mcand_cap) {  // the candidate list overflowed: grow it, scan again
+      dfree(c->d_mcand);
+      c->mcand_cap = (int64_t)ncand + ((int64_t)ncand >> 2) + 1024;
+      CK(c, dalloc(&c->d_mcand, c->mcand_cap));
+      continue;
+    }
+    c->npairs = (int64_t)cnt;
+    bool again = false;
+    PriceCtl h{};
+    h.count = cnt;
+    const f2m_status s = price_grow(c, h, &again);
+    if (s != F2M_OK || !again) return s;
+  }
+}
+
+// pricing scan into d_pairs (grown until every pair fits); count in c->npairs,
+// per-segment counts in c->seg_pairs
+f2m_status f2m::price_internal(f2m_ctx* c, double* ms, const int32_t* lam_override) {
+  f2m_status s = price_setup(c);
+  if (s != F2M_OK) return s;
   int32_t fb = 0;
   const int32_t* lam = cur_lambda(c, &fb);
   if (lam_override) lam = lam_override;
   const int32_t nseg = (int32_t)c->seg_off.size() - 1;
   const bool plain = !lam_override && !cut_count(c);  // a scan of lambda itself, F2M terms only
+  const bool culled = c->p.pricing == 2;
+  const bool mma = !culled && (c->p.flags & F2M_FLAG_PRICING_TENSOR);
   // The scan that certifies the finisher's lambda.  A complete scan at lambda
   // lam_ref left z >= 0 on every pair outside the CSR (the pairs it found were
   // merged); the finisher is the only change of lambda since, and returns
@@ -817,41 +916,8 @@ f2m_status f2m::price_internal(f2m_ctx* c, double* ms, const int32_t* lam_overri
   // ref_fb) - delta_u - delta_v can be negative only if delta_u > 0 or
   // delta_v > 0: only the rows of the nodes whose lambda rose are scanned,
   // against all points, for the same pairs as a full scan.
-  if (plain && nseg == 1 && c->p.pricing == 1 && !(c->p.flags & F2M_FLAG_PRICING_TENSOR) && c->d_lam_ref &&
-      c->ref_version == c->fin_src_version && c->lam_version == c->fin_dst_version && fb > c->ref_fb) {
-    CK(c, cudaEventRecord(c->ev0, c->st));
-    CK(c, launch_pricing_prep(c->d_xy, lam, nullptr, c->n, fb, c->d_pts, c->st));
-    CK(c, launch_pricing_raised(lam, c->d_lam_ref, c->n, fb - c->ref_fb, c->d_pts, c->d_raised, c->d_pts_raised,
-                                c->d_nraised, c->st));
-    unsigned int nu = 0;
-    CK(c, cudaMemcpyAsync(&nu, c->d_nraised, sizeof(nu), cudaMemcpyDeviceToHost, c->st));
-    CK(c, cudaStreamSynchronize(c->st));
-    const int64_t ntiles_r = (int64_t)((nu + kPricingTile - 1) / kPricingTile) * ((c->n + kPricingJ - 1) / kPricingJ);
-    for (bool first = true;; first = false) {
-      if (!first) CK(c, cudaEventRecord(c->ev0, c->st));
-      CK(c, launch_pricing_scan(c->d_pts, c->d_xy, lam, c->d_rp, c->d_ec, c->n, fb, nullptr, (int32_t)ntiles_r,
-                                c->d_pairs, c->pairs_cap, c->d_count, c->d_tile, c->num_sms, c->st,
-                                c->d_pts_raised, c->d_raised, (int32_t)nu));
-      CK(c, cudaEventRecord(c->ev1, c->st));
-      unsigned long long cnt = 0;
-      CK(c, cudaMemcpyAsync(&cnt, c->d_count, sizeof(cnt), cudaMemcpyDeviceToHost, c->st));
-      CK(c, cudaStreamSynchronize(c->st));
-      if (ms) *ms += elapsed_ms(c);
-      c->npairs = (int64_t)cnt;
-      if ((int64_t)cnt <= c->pairs_cap) break;
-      dfree(c->d_pairs);
-      c->pairs_cap = (int64_t)cnt + ((int64_t)cnt >> 2) + 1024;
-      CK(c, dalloc(&c->d_pairs, c->pairs_cap));
-    }
-    c->seg_pairs.assign(1, c->npairs);
-    c->last_scan_rows = (int64_t)nu;
-    c->last_scan_pairs = (int64_t)nu * c->n;
-    // a complete result for this lambda: it is the next reference
-    CK(c, cudaMemcpyAsync(c->d_lam_ref, lam, sizeof(int32_t) * c->n, cudaMemcpyDeviceToDevice, c->st));
-    c->ref_fb = fb;
-    c->ref_version = c->lam_version;
-    return F2M_OK;
-  }
+  const bool rows = plain && nseg == 1 && c->p.pricing == 1 && !mma && c->d_lam_ref &&
+                    c->ref_version == c->fin_src_version && c->lam_version == c->fin_dst_version && fb > c->ref_fb;
   c->last_scan_rows = -1;
   c->last_scan_pairs = 0;
   for (int32_t sg = 0; sg < nseg; ++sg)
@@ -859,161 +925,98 @@ f2m_status f2m::price_internal(f2m_ctx* c, double* ms, const int32_t* lam_overri
       const int64_t m = c->seg_off[sg + 1] - c->seg_off[sg];
       c->last_scan_pairs += m * (m - 1) / 2;
     }
-  // full scan: with the fp32 filter (caller order), or on the tensor cores
-  // (renumbered order); culled scan: fp32 filter in the renumbered (Morton)
-  // order, so that a tile is a compact patch with a small bounding box
-  const bool culled = c->p.pricing == 2;
-  const bool mma = !culled && (c->p.flags & F2M_FLAG_PRICING_TENSOR);
-  const int kind = mma ? 1 : 0;
-  // the full scan's tile-pair list depends only on the segments scanned: it
-  // stays on the device from one scan to the next while they are the same
-  std::vector<int4> tiles;
-  const bool reuse = !culled && c->tiles_valid && c->tiles_kind == kind && c->tiles_seg_scan == c->seg_scan &&
-                     c->tiles_seg_off == c->seg_off;
-  if (mma && !c->d_pts4) {
-    CK(c, dalloc(&c->d_pts4, c->n));
-    CK(c, dalloc(&c->d_pstat, 1));
-    CK(c, dalloc(&c->d_mncand, 1));
-    c->mcand_cap = std::max<int64_t>(4LL * c->n, 1 << 20);
-    CK(c, dalloc(&c->d_mcand, c->mcand_cap));
-  }
-  if (!reuse) {
-    if (mma) {
-      std::vector<int4> tblk;
-      std::vector<int2> ranges;
-      build_mma_tiles(c, tiles, tblk, ranges);
-      if ((int64_t)ranges.size() > c->mblocks_cap) {
-        dfree(c->d_mranges);
-        dfree(c->d_mbox);
-        dfree(c->d_mlmax);
-        c->mblocks_cap = (int64_t)ranges.size() + 64;
-        CK(c, dalloc(&c->d_mranges, c->mblocks_cap));
-        CK(c, dalloc(&c->d_mbox, c->mblocks_cap));
-        CK(c, dalloc(&c->d_mlmax, c->mblocks_cap));
+  if (mma) {
+    s = price_mma(c, lam, fb, ms);
+    if (s != F2M_OK) return s;
+  } else {
+    int32_t* seg = c->d_pseg;
+    uint8_t* d_scan = reinterpret_cast<uint8_t*>(seg + 3 * (nseg + 1));
+    // tile pairs of the full scan: large tiles where they fill the GPU several times over
+    long long ntiles = 0;
+    bool large = false;
+    if (!rows && !culled) {
+      std::vector<int32_t> tile(nseg + 1);
+      auto count_tiles = [&](int64_t ti, int64_t tj) {
+        int64_t t = 0;
+        for (int32_t sg = 0; sg < nseg; ++sg) {
+          tile[sg] = (int32_t)t;
+          if (!c->seg_scan.empty() && !c->seg_scan[sg]) continue;
+          const int64_t m = c->seg_off[sg + 1] - c->seg_off[sg], I = (m + ti - 1) / ti, J = (m + tj - 1) / tj;
+          t += I * J - ti / tj * (I * (I - 1) / 2);
+        }
+        return t;
+      };
+      ntiles = count_tiles(kPriceLargeI, kPriceLargeJ);
+      large = price_large_tiles(ntiles, c->num_sms);
+      if (!large) ntiles = count_tiles(kPriceBlock, kPriceBlock);
+      if (ntiles >= INT_MAX) return fail(c, F2M_ERR_INVALID_ARG, "too many pricing tile pairs");
+      tile[nseg] = (int32_t)ntiles;
+      if (tile != c->price_tile) {
+        CK(c, cudaMemcpyAsync(seg + 2 * (nseg + 1), tile.data(), sizeof(int32_t) * (nseg + 1),
+                              cudaMemcpyHostToDevice, c->st));
+        c->price_tile = tile;  // a pageable copy has left the host array when the call returns
       }
-      if ((int64_t)tblk.size() > c->mtiles_cap) {
-        dfree(c->d_mtblk);
-        dfree(c->d_mframes);
-        c->mtiles_cap = (int64_t)tblk.size() + 64;
-        CK(c, dalloc(&c->d_mtblk, c->mtiles_cap));
-        CK(c, dalloc(&c->d_mframes, c->mtiles_cap));
+    }
+    if (culled) {
+      if (!c->d_plist) {
+        c->plist_cap = 64LL * c->price_blocks + 4096;
+        CK(c, dalloc(&c->d_plist, c->plist_cap));
       }
-      if (!ranges.empty())
-        CK(c, cudaMemcpyAsync(c->d_mranges, ranges.data(), sizeof(int2) * ranges.size(), cudaMemcpyHostToDevice,
-                              c->st));
-      if (!tblk.empty())
-        CK(c, cudaMemcpyAsync(c->d_mtblk, tblk.data(), sizeof(int4) * tblk.size(), cudaMemcpyHostToDevice, c->st));
-      c->mblocks = (int64_t)ranges.size();
-    } else {
-      build_tiles(c, tiles);
+      if (!c->seg_scan.empty())
+        CK(c, cudaMemcpyAsync(d_scan, c->seg_scan.data(), nseg, cudaMemcpyHostToDevice, c->st));
+    }
+    PriceScan sc{};
+    sc.xy = c->d_xy;
+    sc.lam = lam;
+    sc.rp = c->d_rp;
+    sc.ec = c->d_ec;
+    sc.pts = sc.pts_i = c->d_pts;
+    sc.box = sc.box_i = c->d_boxes;
+    sc.smax = sc.smax_i = c->d_smax;
+    sc.seg_off = seg;
+    sc.seg_blk = seg + (nseg + 1);
+    sc.seg_tile = seg + 2 * (nseg + 1);
+    sc.ctl = c->d_pctl;
+    sc.nseg = nseg;
+    sc.n = c->n;
+    sc.fb = fb;
+    PriceCtl h{};
+    for (bool again = true; again;) {
+      sc.pairs = c->d_pairs;
+      sc.cap = c->pairs_cap;
+      sc.list = c->d_plist;
+      sc.list_cap = (int32_t)std::min<int64_t>(c->plist_cap, INT_MAX);
+      CK(c, cudaEventRecord(c->ev0, c->st));
+      CK(c, launch_pricing_prep(sc, c->plan.perm, c->price_blocks, c->d_pts, c->d_boxes, c->d_smax, c->st));
+      if (rows) {
+        PriceScan sr = sc;
+        sr.pts_i = c->d_pts_raised;
+        sr.box_i = c->d_boxes + c->price_blocks;
+        sr.smax_i = c->d_smax + c->price_blocks;
+        sr.inU = c->d_raised;
+        CK(c, launch_pricing_raised(c->d_lam_ref, fb - c->ref_fb, sc, c->d_raised, c->d_pts_raised,
+                                    c->d_boxes + c->price_blocks, c->d_smax + c->price_blocks, c->st));
+        CK(c, launch_pricing_rows(sr, c->num_sms, c->st));
+      } else if (culled) {
+        CK(c, launch_pricing_cull(sc, c->seg_scan.empty() ? nullptr : d_scan, c->price_blocks, c->d_plist, c->st));
+        CK(c, launch_pricing_list(sc, c->num_sms, c->st));
+      } else {
+        CK(c, launch_pricing_full(sc, large, ntiles, c->num_sms, c->st));
+      }
+      CK(c, cudaEventRecord(c->ev1, c->st));
+      CK(c, cudaMemcpyAsync(&h, c->d_pctl, sizeof(h), cudaMemcpyDeviceToHost, c->st));
+      CK(c, cudaStreamSynchronize(c->st));
+      if (ms) *ms += elapsed_ms(c);
+      s = price_grow(c, h, &again);
+      if (s != F2M_OK) return s;
+    }
+    c->npairs = (int64_t)h.count;
+    if (rows) {
+      c->last_scan_rows = (int64_t)h.rows;
+      c->last_scan_pairs = (int64_t)h.rows * c->n;
     }
   }
-  CK(c, cudaEventRecord(c->ev0, c->st));
-  if (mma)
-    CK(c, launch_pricing_mma_prep(c->d_xy, lam, c->plan.perm, c->n, c->d_pts4, c->st));
-  else
-    CK(c, launch_pricing_prep(c->d_xy, lam, culled ? c->plan.perm : nullptr, c->n, fb, c->d_pts, c->st));
-  if (culled && !tiles.empty()) {
-    // A pair (u, v) can have z < 0 only if its distance is below s_u + s_v
-    // (the filter's radii, see pricing.cu), so a tile pair whose bounding
-    // boxes are at least max s + max s apart holds none: it is skipped.
-    // the point ranges of the tiles: per segment, steps of kPricingTile from its start
-    std::vector<int2> ranges;
-    std::vector<int32_t> base(nseg + 1, 0);
-    for (int32_t sg = 0; sg < nseg; ++sg) {
-      base[sg] = (int32_t)ranges.size();
-      for (int32_t i0 = c->seg_off[sg]; i0 < c->seg_off[sg + 1]; i0 += kPricingTile)
-        ranges.push_back(make_int2(i0, std::min(i0 + kPricingTile, c->seg_off[sg + 1])));
-    }
-    auto range_id = [&](int32_t i0) {
-      const int32_t sg = (int32_t)(std::upper_bound(c->seg_off.begin(), c->seg_off.end(), i0) - c->seg_off.begin()) - 1;
-      return base[sg] + (i0 - c->seg_off[sg]) / kPricingTile;
-    };
-    std::vector<int32_t> rid_of(tiles.size()), cid_of(tiles.size());
-    for (size_t k = 0; k < tiles.size(); ++k) {
-      rid_of[k] = range_id(tiles[k].x);
-      cid_of[k] = range_id(tiles[k].z);
-    }
-    if ((int64_t)ranges.size() > c->ranges_cap) {
-      dfree(c->d_ranges);
-      dfree(c->d_boxes);
-      dfree(c->d_smax);
-      c->ranges_cap = (int64_t)ranges.size() + 64;
-      CK(c, dalloc(&c->d_ranges, c->ranges_cap));
-      CK(c, dalloc(&c->d_boxes, c->ranges_cap));
-      CK(c, dalloc(&c->d_smax, c->ranges_cap));
-    }
-    CK(c, cudaMemcpyAsync(c->d_ranges, ranges.data(), sizeof(int2) * ranges.size(), cudaMemcpyHostToDevice, c->st));
-    CK(c, launch_pricing_boxes(c->d_pts, c->d_ranges, (int32_t)ranges.size(), c->d_boxes, c->d_smax, c->st));
-    std::vector<float4> box(ranges.size());
-    std::vector<float> smax(ranges.size());
-    CK(c, cudaMemcpyAsync(box.data(), c->d_boxes, sizeof(float4) * box.size(), cudaMemcpyDeviceToHost, c->st));
-    CK(c, cudaMemcpyAsync(smax.data(), c->d_smax, sizeof(float) * smax.size(), cudaMemcpyDeviceToHost, c->st));
-    CK(c, cudaStreamSynchronize(c->st));
-    std::vector<int4> kept;
-    kept.reserve(tiles.size());
-    for (size_t k = 0; k < tiles.size(); ++k) {
-      const float4 a = box[rid_of[k]], b = box[cid_of[k]];
-      const double gx = std::max(0.0, std::max((double)a.x - b.z, (double)b.x - a.z));
-      const double gy = std::max(0.0, std::max((double)a.y - b.w, (double)b.y - a.w));
-      const double r = (double)smax[rid_of[k]] + (double)smax[cid_of[k]];
-      if (gx * gx + gy * gy < r * r * (1.0 + 1e-9) + 1.0) kept.push_back(tiles[k]);
-    }
-    tiles.swap(kept);
-  }
-  if (!reuse) {
-    if ((int64_t)tiles.size() > c->tiles_cap) {
-      dfree(c->d_tiles);
-      c->tiles_cap = (int64_t)tiles.size() + 64;
-      CK(c, dalloc(&c->d_tiles, c->tiles_cap));
-    }
-    if (!tiles.empty())
-      CK(c, cudaMemcpyAsync(c->d_tiles, tiles.data(), sizeof(int4) * tiles.size(), cudaMemcpyHostToDevice, c->st));
-    c->tiles_valid = !culled;
-    c->tiles_kind = kind;
-    c->tiles_seg_scan = c->seg_scan;
-    c->tiles_seg_off = c->seg_off;
-    c->ntiles = (int64_t)tiles.size();
-  }
-  const int64_t ntiles = c->ntiles;
-  bool first = true;
-  for (;;) {
-    if (!first) CK(c, cudaEventRecord(c->ev0, c->st));
-    first = false;
-    if (mma)
-      CK(c, launch_pricing_mma_scan(c->d_pts4, c->d_xy, lam, c->d_rp, c->d_ec, fb, c->d_tiles, c->d_mtblk,
-                                    (int32_t)ntiles, c->d_mranges, (int32_t)c->mblocks, c->d_mbox, c->d_mlmax,
-                                    c->d_mframes, c->d_mcand, c->mcand_cap, c->d_mncand, c->d_pairs,
-                                    c->pairs_cap, c->d_count, c->d_tile, c->d_pstat, c->num_sms, c->st));
-    else
-      CK(c, launch_pricing_scan(c->d_pts, c->d_xy, lam, c->d_rp, c->d_ec, c->n, fb, c->d_tiles,
-                                (int32_t)ntiles, c->d_pairs, c->pairs_cap, c->d_count, c->d_tile,
-                                c->num_sms, c->st));
-    CK(c, cudaEventRecord(c->ev1, c->st));
-    unsigned long long cnt = 0;
-    int32_t pstat = 0;
-    unsigned long long ncand = 0;
-    CK(c, cudaMemcpyAsync(&cnt, c->d_count, sizeof(cnt), cudaMemcpyDeviceToHost, c->st));
-    if (mma) {
-      CK(c, cudaMemcpyAsync(&pstat, c->d_pstat, sizeof(pstat), cudaMemcpyDeviceToHost, c->st));
-      CK(c, cudaMemcpyAsync(&ncand, c->d_mncand, sizeof(ncand), cudaMemcpyDeviceToHost, c->st));
-    }
-    CK(c, cudaStreamSynchronize(c->st));
-    if (ms) *ms += elapsed_ms(c);
-    if (pstat) return fail(c, F2M_ERR_TIMEOUT, "pricing scan: a tensor-core wait ran past its budget");
-    if (mma && (int64_t)ncand > c->mcand_cap) {  // the candidate list overflowed: grow it, scan again
-      dfree(c->d_mcand);
-      c->mcand_cap = (int64_t)ncand + ((int64_t)ncand >> 2) + 1024;
-      CK(c, dalloc(&c->d_mcand, c->mcand_cap));
-      continue;
-    }
-    c->npairs = (int64_t)cnt;
-    if ((int64_t)cnt <= c->pairs_cap) break;
-    dfree(c->d_pairs);
-    c->pairs_cap = (int64_t)cnt + ((int64_t)cnt >> 2) + 1024;
-    CK(c, dalloc(&c->d_pairs, c->pairs_cap));
-  }
-  if (plain && c->d_lam_ref) {  // the reference of a later certifying scan
+  if (plain && c->d_lam_ref) {  // a complete result for this lambda: the reference of a later certifying scan
     CK(c, cudaMemcpyAsync(c->d_lam_ref, lam, sizeof(int32_t) * c->n, cudaMemcpyDeviceToDevice, c->st));
     c->ref_fb = fb;
     c->ref_version = c->lam_version;
@@ -1026,9 +1029,9 @@ f2m_status f2m::price_internal(f2m_ctx* c, double* ms, const int32_t* lam_overri
     CK(c, cudaMemcpyAsync(h.data(), c->d_pairs, sizeof(int2) * c->npairs, cudaMemcpyDeviceToHost, c->st));
     CK(c, cudaStreamSynchronize(c->st));
     for (const int2& q : h) {
-      const int32_t s = (int32_t)(std::upper_bound(c->seg_off.begin(), c->seg_off.end(), q.x) -
-                                  c->seg_off.begin()) - 1;
-      c->seg_pairs[s] += 1;
+      const int32_t sg = (int32_t)(std::upper_bound(c->seg_off.begin(), c->seg_off.end(), q.x) -
+                                   c->seg_off.begin()) - 1;
+      c->seg_pairs[sg] += 1;
     }
   }
   return F2M_OK;

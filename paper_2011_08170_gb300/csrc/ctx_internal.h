@@ -23,17 +23,21 @@ struct f2m_ctx {
   std::vector<int64_t> seg_pairs;       // pairs per segment found by the last scan
   int32_t* d_seg_off = nullptr;         // device copy of seg_off (batches)
   uint8_t* d_fin_include = nullptr;     // per segment: the finisher may change it (NULL = all)
-  int4* d_tiles = nullptr;              // pricing tile-pair list
-  int64_t tiles_cap = 0;
+  int4* d_tiles = nullptr;              // tensor-core scan: tile-pair list
   int64_t ntiles = 0;                   // tile pairs in d_tiles
-  int tiles_kind = 0;                   // the list's form: 0 fp32 scan, 1 tensor-core scan
-  bool tiles_valid = false;             // d_tiles holds the full scan's list for:
+  bool tiles_valid = false;             // d_tiles holds the list for:
   std::vector<uint8_t> tiles_seg_scan;  //   these scanned segments
-  std::vector<int32_t> tiles_seg_off;   //   of these segments
-  int2* d_ranges = nullptr;             // culled pricing: point ranges of the tiles,
-  float4* d_boxes = nullptr;            // their bounding boxes
-  float* d_smax = nullptr;              // and largest filter radii
-  int64_t ranges_cap = 0;
+  // pricing scan: the points' blocks (bounding boxes, largest filter radii; a
+  // second set for some rows gathered), its counters, the segments' positions,
+  // blocks, tile pairs and scan flags, the culled scan's block pairs
+  float4* d_boxes = nullptr;
+  float* d_smax = nullptr;
+  f2m::PriceCtl* d_pctl = nullptr;
+  int32_t* d_pseg = nullptr;
+  int32_t price_blocks = 0;
+  std::vector<int32_t> price_tile;      // the segments' first tile pairs held in d_pseg
+  int2* d_plist = nullptr;
+  int64_t plist_cap = 0;
 
   int32_t n = 0;
   int64_t nnz = 0;
@@ -87,7 +91,6 @@ struct f2m_ctx {
   int32_t* d_lam_ref = nullptr; // [n] caller order
   uint8_t* d_raised = nullptr;  // [n] nodes whose lambda rose
   float4* d_pts_raised = nullptr;  // [n] their points
-  unsigned int* d_nraised = nullptr;
   int64_t last_scan_rows = -1;  // rows of the last scan if it was a certifying one, else -1
   int64_t last_scan_pairs = 0;  // pairs the last scan evaluated
   int2* d_pairs = nullptr;

@@ -8,13 +8,14 @@ namespace f2m {
 
 // Edge cost c(u,v): the nearest integer to sqrt(d2), d2 = dx^2 + dy^2 (TSPLIB
 // EUC_2D, the input convention of Section 5.1).  Integer-exact: s is the floor
-// of sqrt(4*d2) (a double square root as first guess, then corrected in
-// integers), and nint(sqrt(d2)) = floor((s + 1) / 2).  No tie exists: an
-// integer d2 never equals (r + 1/2)^2.
+// of sqrt(4*d2) (an fp32 square root as first guess, within 1 of it, then
+// corrected in integers; fp64 arithmetic is many times slower here), and
+// nint(sqrt(d2)) = floor((s + 1) / 2).  No tie exists: an integer d2 never
+// equals (r + 1/2)^2.
 __device__ __forceinline__ int32_t exact_cost(int32_t dx, int32_t dy) {
-  long long d2 = (long long)dx * dx + (long long)dy * dy;
-  long long q = 4 * d2;  // < 2^43, exact in double
-  long long s = (long long)sqrt((double)q);
+  const long long d2 = (long long)dx * dx + (long long)dy * dy;
+  const long long q = 4 * d2;  // < 2^43, its root below 2^22
+  long long s = (long long)__fsqrt_rn((float)q);
   while (s * s > q) --s;
   while ((s + 1) * (s + 1) <= q) ++s;
   return (int32_t)((s + 1) >> 1);

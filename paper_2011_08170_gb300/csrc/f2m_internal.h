@@ -106,29 +106,54 @@ cudaError_t launch_extract(const int32_t* rp, const int2* ec, const int32_t* bde
                            cudaStream_t st);
 // lam_out = lam_in >> 1 (F+1 bits -> F bits, floor)
 cudaError_t launch_halve(const int32_t* lam_in, int32_t* lam_out, int32_t n, cudaStream_t st);
-// all-pairs pricing scan: pairs (u < v) outside the CSR with z < 0
-// Tile pairs {i0, i1, j0, j1}: test i in [i0, i1) against j in [j0, j1), j > i.
-constexpr int kPricingTile = 1024;  // i-points of a pricing tile pair (and the most j-points)
-constexpr int kPricingJ = 512;      // j-points of a tile pair in the lists built for a scan
-// pts[v] = {x, y, s, node perm[v]} (perm NULL: node v), s the filter radius of the node
-cudaError_t launch_pricing_prep(const int2* xy, const int32_t* lam, const int32_t* perm, int32_t n, int32_t fb,
-                                float4* pts, cudaStream_t st);
-// bounding box {min x, min y, max x, max y} and largest s of each point range
-cudaError_t launch_pricing_boxes(const float4* pts, const int2* ranges, int32_t nranges, float4* box, float* smax,
-                                 cudaStream_t st);
-// the scan over the tile pairs (positions in pts); count and pairs (nodes, u < v)
-// tiles NULL: i-tiles of the ni points pts_i against j-tiles of all n points
-// (inU flags the nodes of pts_i; ntiles = its tile count), else the list's
-// tile pairs over pts (pts_i NULL)
-cudaError_t launch_pricing_scan(const float4* pts, const int2* xy, const int32_t* lam, const int32_t* rp,
-                                const int2* ec, int32_t n, int32_t fb, const int4* tiles, int32_t ntiles,
-                                int2* pairs, int64_t cap, unsigned long long* count, unsigned int* tile_counter,
-                                int num_sms, cudaStream_t st, const float4* pts_i = nullptr,
-                                const uint8_t* inU = nullptr, int32_t ni = 0);
-// nodes whose lambda rose above lam_ref << shift: flags, their points, their count
-cudaError_t launch_pricing_raised(const int32_t* lam, const int32_t* lam_ref, int32_t n, int32_t shift,
-                                  const float4* pts, uint8_t* inU, float4* pts_u, unsigned int* count,
-                                  cudaStream_t st);
+// all-pairs pricing scan (pricing.cu): pairs (u < v) outside the CSR with z < 0,
+// over the points in the renumbered order, in blocks of kPriceBlock positions
+constexpr int kPriceBlock = 128;   // positions of a block: the small tile, i and j
+constexpr int kPriceLargeI = 512;  // the large tile
+constexpr int kPriceLargeJ = 512;
+struct PriceCtl {
+  unsigned long long count;  // pairs found (past the capacity too)
+  unsigned int next;         // tile pairs handed out
+  unsigned int listed;       // block pairs of the culled scan's list (past its capacity too)
+  unsigned int rows;         // i-points of a scan of some rows
+};
+struct PriceScan {
+  const int2* xy;             // by node
+  const int32_t* lam;         // by node, units 2^-fb
+  const int32_t* rp;          // the candidate CSR
+  const int2* ec;
+  const float4* pts;          // by position: {x, y, s (the filter radius), node}
+  const float4* box;          // per block of pts: {min x, min y, max x, max y}
+  const float* smax;          // and its largest s
+  const float4* pts_i;        // the i-points: pts, or some rows gathered
+  const float4* box_i;
+  const float* smax_i;
+  const uint8_t* inU;         // by node: gathered into pts_i (NULL: the i-points are all points)
+  const int32_t* seg_off;     // [nseg + 1] positions of the segments
+  const int32_t* seg_blk;     // [nseg + 1] their first blocks
+  const int32_t* seg_tile;    // [nseg + 1] their first tile pairs (full scan)
+  const int2* list;           // block pairs (culled scan)
+  int2* pairs;                // the result
+  PriceCtl* ctl;
+  long long cap;              // of pairs
+  int32_t list_cap;
+  int32_t nseg, n, fb;
+};
+// points, blocks and cleared counters of a scan of lambda sc.lam
+cudaError_t launch_pricing_prep(const PriceScan& sc, const int32_t* perm, int32_t nblocks, float4* pts, float4* box,
+                                float* smax, cudaStream_t st);
+// all pairs of the segments' tile pairs, in large tiles or small
+bool price_large_tiles(long long large_tiles, int num_sms);
+cudaError_t launch_pricing_full(const PriceScan& sc, bool large, long long ntiles, int num_sms, cudaStream_t st);
+// the block pairs that can hold a pair with z < 0, then the scan of them
+cudaError_t launch_pricing_cull(const PriceScan& sc, const uint8_t* seg_scan, int32_t nblocks, int2* list,
+                                cudaStream_t st);
+cudaError_t launch_pricing_list(const PriceScan& sc, int num_sms, cudaStream_t st);
+// nodes whose lambda rose above lam_ref << shift: flags, their points and
+// blocks, their count in sc.ctl->rows; then their scan against all points
+cudaError_t launch_pricing_raised(const int32_t* lam_ref, int32_t shift, const PriceScan& sc, uint8_t* inU,
+                                  float4* pts_u, float4* box_u, float* smax_u, cudaStream_t st);
+cudaError_t launch_pricing_rows(const PriceScan& sc, int num_sms, cudaStream_t st);
 // the same scan on the tensor cores (pricing.cu): pts4[v] = {x, y, lambda, node
 // perm[v]}; tiles {i0, i1, j0, j1} of at most kMmaTileI x kMmaTileJ positions
 cudaError_t launch_pricing_mma_check(long long rounds, unsigned long long seed, unsigned long long* checked,

@@ -4,30 +4,63 @@
 // miss optimal edges (Section 5.3); this scan finds every such edge so the
 // final duals are feasible for the complete graph.
 //
-// N-body tiling: the host lists tile pairs (blocks of the pair triangle of
-// each segment, i.e. instance: up to kPricingTile i-points by up to
-// kPricingTile j-points; the scan's lists use kPricingJ j-points, so the last
-// wave of tile pairs is short), handed out by an atomic counter; a CTA keeps
-// the j-points in shared memory and each thread P i-points in registers, two
-// at a time in packed fp32x2 registers (Blackwell's two-lane FADD2 / FFMA2:
-// one issue slot for two pairs).
+// N-body tiling over the points in the renumbered (Morton) order, where a run
+// of points is a compact patch: i-tiles of 128 W points (128 per warp) by
+// j-tiles of J points, handed out by an atomic counter.  Three forms of the same
+// kernel: all tile pairs of the pair triangle of every scanned segment
+// (instance); the tile pairs of a list (culled scan: blocks whose boxes are
+// close enough); a gathered set of i-points against all points (rows).
 //
-// Filter.  r_v = max(lambda_v 2^-fb + 1/4, 0), s_v = (r_v + 2)(1 + 2^-17) in
-// fp32, a_v = x_v - s_v, c_v = x_v + s_v.  Per pair, with t = s_u + s_v:
+// A pair passes three tests, each deciding only what the previous lets through.
+//
+// 1. Integer filter, 128 pairs an instruction.  Coordinates and radii are
+// integers in a frame fitted to the tile pair (corner (bx, by) of its bounding
+// box, q = 2^b the smallest with every X = floor((x - bx) / q) - 1024 in
+// [-1024, 1023], Y likewise, and every radius R_v = ceil(s_v / q + 0.7075)
+// at most 1023, s_v test 2's radius).  The pair passes when
+//   e = |D|^2 - t^2 < 0,  D = (X_v - X_u, Y_v - Y_u),  t = R_u + R_v.
+// No false negatives: z < 0 gives d < T + 1/2, T = (lambda_u + lambda_v) 2^-fb,
+// and T + 1/2 < s_u + s_v.  The true difference vector is q D plus a rest
+// shorter than sqrt(2) q, so |D| < (s_u + s_v) / q + sqrt(2) <= t (0.7075 >
+// sqrt(2) / 2, and s has two length units to spare for the fp32 rounding).
+// Expanded, e = A_u + A_v - 2 (X_u X_v + Y_u Y_v + R_u R_v), A = X^2 + Y^2 - R^2,
+// is the product of the fp16 rows
+//   i-point: [A_hi, A_lo, 2048, 1, X, Y, R, 0]      (A = 2048 A_hi + A_lo)
+//   j-point: [2048, 1, A_hi, A_lo, -2X, -2Y, -2R, 0]
+// Every entry is an integer of at most 11 bits (exact in fp16), every product
+// at most 2^22 in magnitude and every partial sum below 2^24, so the fp32
+// accumulator holds e exactly whatever the order of the additions
+// (f2m_pricing_mma_check compares the hardware with integers).  One mma.sync
+// m16n8k8 gives 16 x 8 pairs, its results already in registers: a warp holds
+// the rows of its 128 i-points (16 registers a lane) and passes over the
+// j-tile in steps of 8 points; the sign bits of a lane's 32 pairs of a step are
+// OR-ed.  A row past the tile's points has A = 2^21: e > 0 with every point.
+//
+// 2. fp32 filter of one pair.  r_v = max(lambda_v 2^-fb + 1/4, 0), s_v = (r_v +
+// 2)(1 + 2^-17) in fp32, a_v = x_v - s_v, c_v = x_v + s_v, t = s_u + s_v:
 //   u = a_v - c_u = dx - t,  w = c_v - a_u = dx + t,  dy = y_v - y_u,
-//   e' = dy^2 + (u w - 1) = d^2 - t^2 - 1      (3 FADD2 + 2 FFMA2 per 2 pairs)
-// and the pair passes when e' < 0.  The sign bits are OR-ed over a thread's
-// pairs with 4 j-points; a warp appends the groups with a set bit to its list
-// in shared memory (ballot, no atomics) and, after every 64 j-points, its
-// lanes re-evaluate the listed pairs and decide the passing ones exactly, so
-// the hot loop holds no call and no block-wide barrier.  No false negatives: z < 0 implies c < T = (lambda_u + lambda_v)
-// 2^-fb, hence d < c + 1/2 < T + 1/2 <= R = r_u + r_v, and t >= (R + 4)(1 +
-// 2^-17.3) after the roundings of r (2^-23 relative) and s, so d^2 - t^2 <=
-// -(4 + 2^-17.3 t)(t + d).  The fp32 errors are at most 0.5 (t + d) (a, c and
-// u, w: 2^-24 of |x| + s < 2^20 + s each) plus 2^-20.9 t (t + d) (the products
-// and the sum), so e' stays negative.  Pairs that pass are decided exactly in
-// integers (exact cost, int64 z), then checked against the CSR row by binary
-// search, then appended.
+//   e' = dy^2 + (u w - 1) = d^2 - t^2 - 1.
+// z < 0 implies c < T, hence d < c + 1/2 < T + 1/2 <= R = r_u + r_v, and t >=
+// (R + 4)(1 + 2^-17.3) after the roundings of r (2^-23 relative) and s, so d^2 -
+// t^2 <= -(4 + 2^-17.3 t)(t + d).  The fp32 errors are at most 0.5 (t + d) (a, c
+// and u, w: 2^-24 of |x| + s < 2^20 + s each) plus 2^-20.9 t (t + d) (the
+// products and the sum), so e' stays negative.
+//
+// 3. Exactly, in integers (exact cost, int64 z), then against the CSR row by
+// binary search, then appended.
+//
+// A step with a set sign bit is computed again with every pair's own sign; the
+// warp appends those pairs to a list in shared memory (ballot, no atomics) and
+// runs test 2 on 32 of them at a time, and test 3 on 32 that passed test 2, so
+// that its dependent loads keep all lanes busy and the hot loop holds neither.
+//
+// Bound: the tensor pipe, 8.2 cycles per m16n8k8 and SM quarter (16 pairs a
+// cycle; a microbenchmark), with the sign ORs beside it on the ALU pipe.  Full
+// scan of 100,000 uniform points: 0.39 ms, the pipe 68 % busy, against 0.92 ms
+// for the same test in packed fp32 (3 FADD2, 2 FFMA2 per 2 pairs, an FFMA2
+// taking 2.7 cycles: 4.7 pairs a cycle at best); HADD2 / HFMA2 run at the
+// packed fp32 rate and gained nothing.  200,000 clustered points: 2.03 to 1.45
+// ms; 1,000 points: 0.11 to 0.05 ms a scan.
 #include <cuda_fp16.h>
 
 #include <climits>
@@ -39,86 +72,137 @@
 
 namespace f2m {
 
-// A CTA takes kPricingTile i-points (P per thread, as P / 2 packed pairs) and
-// kPricingTile j-points.  P = 8 (128 threads) when there are many tile pairs,
-// P = 4 (256 threads: twice the threads on one tile pair) when there are few.
-constexpr int kPriceTile = kPricingTile;
-constexpr int kPriceJMax = kPricingJ;  // j-points of a tile pair: the scan's lists never hold more
+// The segments (instances) of a scan on the device: segment k holds positions
+// [off[k], off[k + 1]), cut into blocks of kPriceBlock positions numbered from
+// blk[k] on, and tile pairs numbered from tile[k] on (none if it isn't scanned).
+__device__ __forceinline__ int price_segment(const int32_t* __restrict__ first, int nseg, int x) {
+  int lo = 0, hi = nseg - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (first[mid] <= x) lo = mid; else hi = mid - 1;
+  }
+  return lo;
+}
 
-// pts[v] = {x, y, s, node} of node perm[v] (perm NULL: node v); the node id is
-// carried in the last component's bits
-__global__ void pricing_prep_kernel(const int2* __restrict__ xy, const int32_t* __restrict__ lam,
-                                    const int32_t* __restrict__ perm, int32_t n, int32_t fb,
-                                    float4* __restrict__ pts) {
+struct PriceBox {
+  float x0, y0, x1, y1, sm;
+};
+
+__device__ __forceinline__ void box_reduce(PriceBox& b) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    b.x0 = fminf(b.x0, __shfl_xor_sync(0xffffffffu, b.x0, o));
+    b.y0 = fminf(b.y0, __shfl_xor_sync(0xffffffffu, b.y0, o));
+    b.x1 = fmaxf(b.x1, __shfl_xor_sync(0xffffffffu, b.x1, o));
+    b.y1 = fmaxf(b.y1, __shfl_xor_sync(0xffffffffu, b.y1, o));
+    b.sm = fmaxf(b.sm, __shfl_xor_sync(0xffffffffu, b.sm, o));
+  }
+}
+
+__device__ __forceinline__ void box_add(PriceBox& b, const float4& v) {
+  b.x0 = fminf(b.x0, v.x);
+  b.y0 = fminf(b.y0, v.y);
+  b.x1 = fmaxf(b.x1, v.x);
+  b.y1 = fmaxf(b.y1, v.y);
+  b.sm = fmaxf(b.sm, v.z);
+}
+
+// One warp per block: pts[v] = {x, y, s, node} of node perm[v] (the node id in
+// the last component's bits), the block's bounding box and its largest s.  The
+// first thread clears the scan's counters.
+__global__ void __launch_bounds__(256)
+pricing_prep_kernel(const int2* __restrict__ xy, const int32_t* __restrict__ lam,
+                    const int32_t* __restrict__ perm, const int32_t* __restrict__ seg_off,
+                    const int32_t* __restrict__ seg_blk, int32_t nseg, int32_t nblocks, int32_t fb,
+                    float4* __restrict__ pts, float4* __restrict__ box, float* __restrict__ smax,
+                    PriceCtl* ctl) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) *ctl = PriceCtl{};
+  const int b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (b >= nblocks) return;
+  const int sg = price_segment(seg_blk, nseg, b);
+  const int v0 = seg_off[sg] + (b - seg_blk[sg]) * kPriceBlock, v1 = min(v0 + kPriceBlock, seg_off[sg + 1]);
   const float scale = ldexpf(1.0f, -fb);
   const float grow = 1.0f + ldexpf(1.0f, -17);
-  for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < n;
-       v += (long long)gridDim.x * blockDim.x) {
-    const int u = perm ? perm[v] : (int)v;
-    const int2 p = xy[u];
-    const float r = fmaxf((float)lam[u] * scale + 0.25f, 0.0f);
-    pts[v] = make_float4((float)p.x, (float)p.y, (r + 2.0f) * grow, __int_as_float(u));
-  }
-}
-
-// bounding box and largest s of each listed point range: {min x, min y, max x, max y}, s
-__global__ void pricing_boxes_kernel(const float4* __restrict__ pts, const int2* __restrict__ ranges,
-                                     float4* __restrict__ box, float* __restrict__ smax) {
-  const int2 rg = ranges[blockIdx.x];
-  float x0 = 3e38f, y0 = 3e38f, x1 = -3e38f, y1 = -3e38f, sm = 0.f;
-  for (int i = rg.x + threadIdx.x; i < rg.y; i += blockDim.x) {
-    const float4 q = pts[i];
-    x0 = fminf(x0, q.x);
-    y0 = fminf(y0, q.y);
-    x1 = fmaxf(x1, q.x);
-    y1 = fmaxf(y1, q.y);
-    sm = fmaxf(sm, q.z);
-  }
-  for (int o = 16; o > 0; o >>= 1) {
-    x0 = fminf(x0, __shfl_xor_sync(0xffffffffu, x0, o));
-    y0 = fminf(y0, __shfl_xor_sync(0xffffffffu, y0, o));
-    x1 = fmaxf(x1, __shfl_xor_sync(0xffffffffu, x1, o));
-    y1 = fmaxf(y1, __shfl_xor_sync(0xffffffffu, y1, o));
-    sm = fmaxf(sm, __shfl_xor_sync(0xffffffffu, sm, o));
-  }
-  __shared__ float4 sb[32];
-  __shared__ float ss[32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (lane == 0) {
-    sb[warp] = make_float4(x0, y0, x1, y1);
-    ss[warp] = sm;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    float4 b = sb[0];
-    float m = ss[0];
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) {
-      b.x = fminf(b.x, sb[w].x);
-      b.y = fminf(b.y, sb[w].y);
-      b.z = fmaxf(b.z, sb[w].z);
-      b.w = fmaxf(b.w, sb[w].w);
-      m = fmaxf(m, ss[w]);
+  PriceBox bx{3e38f, 3e38f, -3e38f, -3e38f, 0.f};
+#pragma unroll
+  for (int k = 0; k < kPriceBlock / 32; ++k) {
+    const int v = v0 + k * 32 + lane;
+    if (v < v1) {
+      const int u = perm[v];
+      const int2 p = xy[u];
+      const float r = fmaxf((float)lam[u] * scale + 0.25f, 0.0f);
+      const float4 q = make_float4((float)p.x, (float)p.y, (r + 2.0f) * grow, __int_as_float(u));
+      pts[v] = q;
+      box_add(bx, q);
     }
-    box[blockIdx.x] = b;
-    smax[blockIdx.x] = m;
+  }
+  box_reduce(bx);
+  if (lane == 0) {
+    box[b] = make_float4(bx.x0, bx.y0, bx.x1, bx.y1);
+    smax[b] = bx.sm;
   }
 }
 
-// exact decision for a pair that passed the filter: positions ii < jj in the
-// point array (each unordered pair once), nodes i and j
-// (inU non-NULL: the i-points are the nodes flagged in inU, the j-points all
-// nodes; a pair of two flagged nodes is taken from the row of the smaller)
-__device__ __noinline__ void pricing_confirm(int ii, int jj, int i, int j, int32_t n, const int2* __restrict__ xy,
-                                             const int32_t* __restrict__ lam,
-                                             const int32_t* __restrict__ rp,
-                                             const int2* __restrict__ ec, int32_t fb, int2* pairs,
-                                             long long cap, unsigned long long* count,
-                                             const uint8_t* __restrict__ inU = nullptr) {
-  if (inU) {
-    if (jj >= n || j == i || (inU[j] && j < i)) return;
-  } else if (jj <= ii || jj >= n) {
-    return;  // each unordered pair once; tail of the last tile
+// Bounding boxes and largest s of the blocks of the *count points pts
+__global__ void __launch_bounds__(256)
+pricing_boxes_kernel(const float4* __restrict__ pts, const PriceCtl* ctl, float4* __restrict__ box,
+                     float* __restrict__ smax) {
+  const int m = (int)ctl->rows, lane = threadIdx.x & 31;
+  for (int b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); b * kPriceBlock < m;
+       b += gridDim.x * (blockDim.x >> 5)) {
+    PriceBox bx{3e38f, 3e38f, -3e38f, -3e38f, 0.f};
+#pragma unroll
+    for (int k = 0; k < kPriceBlock / 32; ++k) {
+      const int v = b * kPriceBlock + k * 32 + lane;
+      if (v < m) box_add(bx, pts[v]);
+    }
+    box_reduce(bx);
+    if (lane == 0) {
+      box[b] = make_float4(bx.x0, bx.y0, bx.x1, bx.y1);
+      smax[b] = bx.sm;
+    }
   }
+}
+
+// The culled scan's list: the block pairs (bi <= bj of one segment) that can
+// hold a pair with z < 0.  Such a pair's distance is below s_u + s_v, so boxes
+// farther apart than the largest radii together hold none.  One CTA per
+// i-block; ctl->listed counts on past cap (the caller grows the list).
+__global__ void __launch_bounds__(256)
+pricing_cull_kernel(const float4* __restrict__ box, const float* __restrict__ smax,
+                    const int32_t* __restrict__ seg_blk, const uint8_t* __restrict__ seg_scan, int32_t nseg,
+                    int2* __restrict__ list, int32_t cap, PriceCtl* ctl) {
+  const int bi = blockIdx.x, lane = threadIdx.x & 31;
+  const int sg = price_segment(seg_blk, nseg, bi);
+  if (seg_scan && !seg_scan[sg]) return;
+  const int end = seg_blk[sg + 1];
+  const float4 a = box[bi];
+  const float sa = smax[bi];
+  for (int b0 = bi; b0 < end; b0 += blockDim.x) {
+    const int bj = b0 + threadIdx.x;
+    bool keep = false;
+    if (bj < end) {
+      const float4 b = box[bj];
+      // integers below 2^20: the gaps are exact, the squares and r carry 2^-24 each
+      const float gx = fmaxf(0.f, fmaxf(a.x - b.z, b.x - a.z));
+      const float gy = fmaxf(0.f, fmaxf(a.y - b.w, b.y - a.w));
+      const float r = sa + smax[bj];
+      keep = gx * gx + gy * gy < r * r * 1.00001f + 1.0f;
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, keep);
+    if (!m) continue;
+    unsigned base = 0;
+    if (lane == 0) base = atomicAdd(&ctl->listed, (unsigned)__popc(m));
+    base = __shfl_sync(0xffffffffu, base, 0) + __popc(m & ((1u << lane) - 1u));
+    if (keep && base < (unsigned)cap) list[base] = make_int2(bi, bj);
+  }
+}
+
+// exact decision for a pair of nodes that passed the filters
+__device__ __noinline__ void pricing_confirm(int i, int j, const int2* __restrict__ xy,
+                                             const int32_t* __restrict__ lam, const int32_t* __restrict__ rp,
+                                             const int2* __restrict__ ec, int32_t fb, int2* pairs,
+                                             long long cap, unsigned long long* count) {
   if (j < i) {
     const int t = i;
     i = j;
@@ -147,226 +231,344 @@ __device__ __forceinline__ float pricing_filter(float aj, float cj, float yj, fl
   return __fmaf_rn(dy, dy, __fmaf_rn(u, w, -1.0f));
 }
 
-// j-points per sign test, and per chunk after which a warp decides its hits;
-// a warp's list holds one chunk (one entry per lane and group at most)
-constexpr int kPriceGroup = 4;
-constexpr int kPriceChunk = 64;
-constexpr int kWarpHits = (kPriceChunk / kPriceGroup) * 32;
-static_assert(kPriceJMax % kPriceChunk == 0 && kPriceChunk % kPriceGroup == 0, "chunking");
+constexpr int kPriceStep = 8;  // j-points of a step (the mma's columns)
+constexpr int kWarpI = 128;    // i-points of a warp: 8 row blocks of 16
 
-// Decide exactly every passing pair of the groups in a warp's hit list (each
-// entry: first j of the group << 8 | thread); all lanes of the warp take part.
-template <int P>
-__device__ __forceinline__ void pricing_hits(const int* hits, int nh, int lane, int4 tl, const float4* s_ac,
-                                          const float2* s_y, const float4* __restrict__ pts,
-                                          const float4* __restrict__ pts_i, const uint8_t* __restrict__ inU,
-                                          const int2* __restrict__ xy, const int32_t* __restrict__ lam,
-                                          const int32_t* __restrict__ rp, const int2* __restrict__ ec,
-                                          int32_t n, int32_t fb, int2* pairs, long long cap,
-                                          unsigned long long* count) {
-  constexpr int kPriceThreads = kPriceTile / P;
-  for (int h = lane; h < nh * P; h += 32) {
-    const int ent = hits[h / P], p = h % P;
-    const int t = ent & 0xFF, g = ent >> 8;
-    const int ii = tl.x + p * kPriceThreads + t;
-    if (ii >= tl.y) continue;
-    const float4 vi = pts_i[ii];
-    const float nai = -(vi.x - vi.z), nci = -(vi.x + vi.z), nyi = -vi.y;
-    for (int kk = 0; kk < kPriceGroup; ++kk) {
-      const int jj = tl.z + g + kk;
-      if (jj >= tl.w) break;
-      const float4 ac = s_ac[g + kk];
-      if (pricing_filter(ac.x, ac.z, s_y[g + kk].x, nai, nci, nyi) < 0.0f)
-        pricing_confirm(ii, jj, __float_as_int(vi.w), __float_as_int(pts[jj].w), min(n, tl.w), xy, lam, rp,
-                        ec, fb, pairs, cap, count, inU);
-    }
+// A warp's pairs on their way through tests 2 and 3 (shared memory): at most 31
+// wait for either between calls, and 32 more join at a time.
+struct PriceLists {
+  int2 passed1[64];  // positions of i and j
+  int2 passed2[64];  // nodes
+  int n1, n2;
+};
+
+__device__ __noinline__ void pricing_test3(PriceLists& L, int m, const PriceScan& sc) {
+  const int lane = threadIdx.x & 31, n2 = L.n2;
+  int2 rest = make_int2(0, 0);
+  if (lane < n2 - m) rest = L.passed2[lane + m];
+  if (lane < m) {
+    const int2 q = L.passed2[lane];
+    pricing_confirm(q.x, q.y, sc.xy, sc.lam, sc.rp, sc.ec, sc.fb, sc.pairs, sc.cap, &sc.ctl->count);
+  }
+  __syncwarp();
+  if (lane < n2 - m) L.passed2[lane] = rest;
+  if (lane == 0) L.n2 = n2 - m;
+  __syncwarp();
+}
+
+__device__ __noinline__ void pricing_test2(PriceLists& L, int m, const PriceScan& sc) {
+  const int lane = threadIdx.x & 31, n1 = L.n1, n2 = L.n2;
+  int2 rest = make_int2(0, 0);
+  if (lane < n1 - m) rest = L.passed1[lane + m];
+  bool pass = false;
+  int i = 0, j = 0;
+  if (lane < m) {
+    const int2 q = L.passed1[lane];
+    const float4 vi = sc.pts_i[q.x], vj = sc.pts[q.y];
+    i = __float_as_int(vi.w);
+    j = __float_as_int(vj.w);
+    // where the i-points are the nodes flagged in inU, a pair of two such
+    // nodes is taken from the row of the smaller
+    pass = !(sc.inU && (j == i || (sc.inU[j] && j < i))) &&
+           pricing_filter(vj.x - vj.z, vj.x + vj.z, vj.y, -(vi.x - vi.z), -(vi.x + vi.z), -vi.y) < 0.0f;
+  }
+  const unsigned b = __ballot_sync(0xffffffffu, pass);
+  if (pass) L.passed2[n2 + __popc(b & ((1u << lane) - 1u))] = make_int2(i, j);
+  if (lane < n1 - m) L.passed1[lane] = rest;
+  if (lane == 0) {
+    L.n1 = n1 - m;
+    L.n2 = n2 + __popc(b);
+  }
+  __syncwarp();
+  if (n2 + __popc(b) >= 32) pricing_test3(L, 32, sc);
+}
+
+// The pairs of one step that passed test 1: bit 4 m + q of a lane's mask is the
+// mma's value q of row block m; rows from position ib on, columns from jb on.
+__device__ __noinline__ void pricing_found(PriceLists& L, unsigned mask, int ib, int jb, int i1, int j1,
+                                           const PriceScan& sc) {
+  const int lane = threadIdx.x & 31;
+  while (__any_sync(0xffffffffu, mask != 0)) {
+    const int b = __ffs(mask) - 1;
+    const int ii = ib + 16 * (b >> 2) + 8 * ((b >> 1) & 1) + (lane >> 2), jj = jb + 2 * (lane & 3) + (b & 1);
+    // each unordered pair once, from its smaller position
+    const bool mine = mask != 0 && ii < i1 && jj < j1 && (sc.inU || jj > ii);
+    mask &= mask - 1;
+    const unsigned v = __ballot_sync(0xffffffffu, mine);
+    const int n1 = L.n1;
+    if (mine) L.passed1[n1 + __popc(v & ((1u << lane) - 1u))] = make_int2(ii, jj);
+    __syncwarp();
+    if (lane == 0) L.n1 = n1 + __popc(v);
+    __syncwarp();
+    if (n1 + __popc(v) >= 32) pricing_test2(L, 32, sc);
   }
 }
 
-template <int P>
-__global__ void __launch_bounds__(kPricingTile / P, P == 8 ? 7 : 4)
-pricing_kernel(const float4* __restrict__ pts, const int2* __restrict__ xy,
-               const int32_t* __restrict__ lam, const int32_t* __restrict__ rp,
-               const int2* __restrict__ ec, int32_t n, int32_t fb, const int4* __restrict__ tiles,
-               int32_t ntiles, int2* pairs, long long cap, unsigned long long* count,
-               unsigned int* tile_counter, const float4* __restrict__ pts_i, const uint8_t* __restrict__ inU,
-               int32_t ni, int32_t nj_tiles) {
-  constexpr int kPriceThreads = kPriceTile / P;
-  constexpr int Q = P / 2;
-  static_assert(kPriceThreads <= 256 && kPriceTile <= (1 << 23), "hit entry packing");
-  __shared__ float4 s_ac[kPriceJMax];                       // {a, a, c, c} of the j-points
-  __shared__ float2 s_y[kPriceJMax];                        // {y, y}
-  __shared__ int s_hit[(kPriceThreads / 32) * kWarpHits];  // one list per warp
+__device__ __forceinline__ unsigned pack_half(int lo, int hi) {
+  const __half2 h = __halves2half2(__int2half_rn(lo), __int2half_rn(hi));
+  return *reinterpret_cast<const unsigned*>(&h);
+}
+
+// a point's operand row: A's word k is its entries 2k and 2k + 1 as a row of
+// the i-points, B's as a row of the j-points
+struct PriceRow {
+  int X, Y, R, A;
+  __device__ __forceinline__ uint4 row_i() const {
+    return make_uint4(pack_half(A >> 11, A & 2047), pack_half(2048, 1), pack_half(X, Y), pack_half(R, 0));
+  }
+  __device__ __forceinline__ uint4 row_j() const {
+    return make_uint4(pack_half(2048, 1), pack_half(A >> 11, A & 2047), pack_half(-2 * X, -2 * Y),
+                      pack_half(-2 * R, 0));
+  }
+};
+__device__ __forceinline__ PriceRow price_row_far() { return PriceRow{0, 0, 0, 1 << 21}; }
+
+__device__ __forceinline__ void price_mma(float (&c)[4], unsigned a0, unsigned a1, unsigned b) {
+  asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%7,%7,%7,%7};"
+               : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3])
+               : "r"(a0), "r"(a1), "r"(b), "f"(0.0f));
+}
+
+enum PriceForm { kPriceFull, kPriceList, kPriceRows };
+
+// W warps of 128 i-points each, J j-points per tile pair.
+template <int FORM, int W, int J, int MINB>
+__global__ void __launch_bounds__(W * 32, MINB)
+pricing_kernel(const __grid_constant__ PriceScan sc) {
+  constexpr int T = W * 32, I = W * kWarpI;
+  static_assert(I % kPriceBlock == 0 && J % kPriceBlock == 0 && I % J == 0, "tiles are whole blocks");
+  static_assert(I / kPriceBlock + J / kPriceBlock <= 32, "one lane per block of the tile pair");
+  __shared__ uint4 s_i[I];                       // operand rows of the i-points
+  __shared__ unsigned s_j[J * 4];                // of the j-points: word k of point 32 a + 8 s + g at 128 a + 16 g + 4 k + s
+  __shared__ PriceLists s_lists[W];
   __shared__ int s_tp;
-  const float2 minus_one = make_float2(-1.0f, -1.0f);
-  const int lane = threadIdx.x & 31;
-  int* hits = s_hit + (threadIdx.x >> 5) * kWarpHits;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  PriceLists& lists = s_lists[warp];
+  if (lane == 0) lists.n1 = lists.n2 = 0;
+  const int rows = FORM == kPriceRows ? (int)sc.ctl->rows : 0;
+  const int nj_tiles = (sc.n + J - 1) / J;
+  const long long ntiles = FORM == kPriceFull  ? sc.seg_tile[sc.nseg]
+                           : FORM == kPriceList ? min((int)sc.ctl->listed, sc.list_cap)
+                                                : (long long)((rows + I - 1) / I) * nj_tiles;
   for (;;) {
     __syncthreads();
-    if (threadIdx.x == 0) s_tp = (int)atomicAdd(tile_counter, 1u);
+    if (threadIdx.x == 0) s_tp = (int)atomicAdd(&sc.ctl->next, 1u);
     __syncthreads();
     const int tp = s_tp;
     if (tp >= ntiles) break;
-    // i in [x, y), j in [z, w); no list: i-tiles of the ni i-points by j-tiles of all points
-    int4 tl;
-    if (tiles) {
-      tl = tiles[tp];
+    // the tile pair: i in [i0, i1), j in [j0, j1), and its blocks
+    int i0, i1, j0, j1, bi0, bj0;
+    if constexpr (FORM == kPriceFull) {
+      const int sg = price_segment(sc.seg_tile, sc.nseg, tp);
+      const int a = sc.seg_off[sg], n = sc.seg_off[sg + 1] - a, NJ = (n + J - 1) / J;
+      const int x = tp - sc.seg_tile[sg];
+      // i-tile it starts at tile pair it NJ - (I / J) it (it - 1) / 2 of the segment
+      int lo = 0, hi = (n + I - 1) / I - 1;
+      while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (mid * NJ - (I / J) * (mid * (mid - 1) / 2) <= x) lo = mid; else hi = mid - 1;
+      }
+      const int jt = lo * (I / J) + x - (lo * NJ - (I / J) * (lo * (lo - 1) / 2));
+      i0 = a + lo * I;
+      j0 = a + jt * J;
+      i1 = min(i0 + I, a + n);
+      j1 = min(j0 + J, a + n);
+      bi0 = sc.seg_blk[sg] + lo * (I / kPriceBlock);
+      bj0 = sc.seg_blk[sg] + jt * (J / kPriceBlock);
+    } else if constexpr (FORM == kPriceList) {
+      static_assert(FORM != kPriceList || (I == kPriceBlock && J == kPriceBlock), "the list holds block pairs");
+      const int2 bb = sc.list[tp];
+      const int sg = price_segment(sc.seg_blk, sc.nseg, bb.x);
+      const int a = sc.seg_off[sg], end = sc.seg_off[sg + 1], b0 = sc.seg_blk[sg];
+      i0 = a + (bb.x - b0) * kPriceBlock;
+      j0 = a + (bb.y - b0) * kPriceBlock;
+      i1 = min(i0 + I, end);
+      j1 = min(j0 + J, end);
+      bi0 = bb.x;
+      bj0 = bb.y;
     } else {
       const int it = tp / nj_tiles, jt = tp % nj_tiles;
-      tl = make_int4(it * kPriceTile, min((it + 1) * kPriceTile, ni), jt * kPriceJMax, min((jt + 1) * kPriceJMax, n));
+      i0 = it * I;
+      j0 = jt * J;
+      i1 = min(i0 + I, rows);
+      j1 = min(j0 + J, sc.n);
+      bi0 = it * (I / kPriceBlock);
+      bj0 = jt * (J / kPriceBlock);
     }
-
-    // i-points p = 2q + h at tl.x + p * kPriceThreads + tid, negated; a point
-    // past the range gets 1e18 (its e' stays above 1e36, finite)
-    float2 na[Q], nc[Q], ny[Q];
-#pragma unroll
-    for (int q = 0; q < Q; ++q) {
-      float a[2], c[2], y[2];
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int i = tl.x + (2 * q + h) * kPriceThreads + threadIdx.x;
-        if (i < tl.y) {
-          const float4 v = pts_i[i];
-          a[h] = v.x - v.z;
-          c[h] = v.x + v.z;
-          y[h] = v.y;
-        } else {
-          a[h] = 1e18f;
-          c[h] = 1e18f;
-          y[h] = 1e18f;
-        }
+    // the frame, from the boxes of the tile pair's blocks (one lane a block)
+    PriceBox bx{3e38f, 3e38f, -3e38f, -3e38f, 0.f};
+    {
+      const int nbi = (i1 - i0 + kPriceBlock - 1) / kPriceBlock, nbj = (j1 - j0 + kPriceBlock - 1) / kPriceBlock;
+      if (lane < nbi + nbj) {
+        const bool ib = lane < nbi;
+        const float4 q = ib ? sc.box_i[bi0 + lane] : sc.box[bj0 + lane - nbi];
+        bx = PriceBox{q.x, q.y, q.z, q.w, ib ? sc.smax_i[bi0 + lane] : sc.smax[bj0 + lane - nbi]};
       }
-      na[q] = make_float2(-a[0], -a[1]);
-      nc[q] = make_float2(-c[0], -c[1]);
-      ny[q] = make_float2(-y[0], -y[1]);
+      box_reduce(bx);
     }
-    // the tile's j-points, rounded up to whole chunks (at most kPriceTile)
-    const int kend = min(kPriceJMax, (tl.w - tl.z + kPriceChunk - 1) / kPriceChunk * kPriceChunk);
-    for (int k = threadIdx.x; k < kend; k += kPriceThreads) {
-      const int j = tl.z + k;
-      if (j < tl.w) {
-        const float4 v = pts[j];
-        const float a = v.x - v.z, c = v.x + v.z;
-        s_ac[k] = make_float4(a, a, c, c);
-        s_y[k] = make_float2(v.y, v.y);
-      } else {
-        s_ac[k] = make_float4(-1e18f, -1e18f, -1e18f, -1e18f);
-        s_y[k] = make_float2(-1e18f, -1e18f);
-      }
+    // q = 2^b: range / q < 2048 and s / q <= 1021 (then R <= 1023)
+    const float need = fmaxf(fmaxf(bx.x1 - bx.x0, bx.y1 - bx.y0) * (1.0f / 2048.0f), bx.sm * (1.0f / 1021.0f));
+    const int b = need < 1.0f ? 0 : ilogbf(need) + 1;
+    const float iq = ldexpf(1.0f, -b);
+    auto row_of = [&](const float4& v) {
+      PriceRow r;
+      r.X = (int)floorf((v.x - bx.x0) * iq) - 1024;
+      r.Y = (int)floorf((v.y - bx.y0) * iq) - 1024;
+      r.R = (int)ceilf(v.z * iq + 0.7075f);
+      r.A = r.X * r.X + r.Y * r.Y - r.R * r.R;
+      return r;
+    };
+#pragma unroll
+    for (int k = 0; k < I / T; ++k) {
+      const int i = k * T + threadIdx.x;
+      s_i[i] = (i0 + i < i1 ? row_of(sc.pts_i[i0 + i]) : price_row_far()).row_i();
+    }
+    // the tile's j-points, rounded up to four steps
+    const int kend = (j1 - j0 + 31) / 32 * 32;
+    for (int k = threadIdx.x; k < kend; k += T) {
+      const uint4 w = (j0 + k < j1 ? row_of(sc.pts[j0 + k]) : price_row_far()).row_j();
+      unsigned* d = s_j + (k & ~31) * 4 + 16 * (k & 7) + ((k >> 3) & 3);
+      d[0] = w.x;
+      d[4] = w.y;
+      d[8] = w.z;
+      d[12] = w.w;
     }
     __syncthreads();
-    for (int k0 = 0; k0 < kend; k0 += kPriceChunk) {
-      int nh = 0;  // entries in this warp's list (the same in every lane)
-#pragma unroll 2
-      for (int g = k0; g < k0 + kPriceChunk; g += kPriceGroup) {
-        unsigned int sign = 0u;
+    // the warp's rows: lane 4 g + k holds word k of rows 16 m + g and 16 m + g + 8
+    unsigned a[kWarpI / 16][2];
+    const unsigned* wi = reinterpret_cast<const unsigned*>(s_i + warp * kWarpI);
 #pragma unroll
-        for (int kk = 0; kk < kPriceGroup; ++kk) {
-          const float4 ac = s_ac[g + kk];
-          const float2 yj = s_y[g + kk];
-          const float2 aj = make_float2(ac.x, ac.y), cj = make_float2(ac.z, ac.w);
+    for (int m = 0; m < kWarpI / 16; ++m) {
+      a[m][0] = wi[64 * m + lane];
+      a[m][1] = wi[64 * m + 32 + lane];
+    }
+    for (int k0 = 0; k0 < kend; k0 += 32) {
+      const uint4 bj = *reinterpret_cast<const uint4*>(s_j + k0 * 4 + 4 * lane);
+      const unsigned bs[4] = {bj.x, bj.y, bj.z, bj.w};
 #pragma unroll
-          for (int q = 0; q < Q; ++q) {
-            const float2 u = __fadd2_rn(aj, nc[q]);
-            const float2 w = __fadd2_rn(cj, na[q]);
-            const float2 dy = __fadd2_rn(yj, ny[q]);
-            const float2 e = __ffma2_rn(dy, dy, __ffma2_rn(u, w, minus_one));
-            sign |= __float_as_uint(e.x) | __float_as_uint(e.y);
+      for (int st = 0; st < 4; ++st) {
+        unsigned sign = 0u;
+#pragma unroll
+        for (int m = 0; m < kWarpI / 16; ++m) {
+          float c[4];
+          price_mma(c, a[m][0], a[m][1], bs[st]);
+          sign |= __float_as_uint(c[0]) | __float_as_uint(c[1]);
+          sign |= __float_as_uint(c[2]) | __float_as_uint(c[3]);
+        }
+        if (__any_sync(0xffffffffu, (int)sign < 0)) {  // rare
+          unsigned mask = 0u;
+#pragma unroll
+          for (int m = 0; m < kWarpI / 16; ++m) {
+            float c[4];
+            price_mma(c, a[m][0], a[m][1], bs[st]);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) mask |= (__float_as_uint(c[q]) >> 31) << (4 * m + q);
           }
+          pricing_found(lists, mask, i0 + warp * kWarpI, j0 + k0 + st * kPriceStep, i1, j1, sc);
         }
-        const unsigned int m = __ballot_sync(0xffffffffu, (int)sign < 0);
-        if (m) {  // rare: append the lanes' groups to the warp's list
-          if ((int)sign < 0) hits[nh + __popc(m & ((1u << lane) - 1u))] = (g << 8) | (int)threadIdx.x;
-          nh += __popc(m);
-        }
-      }
-      if (nh) {  // the same branch in every lane of the warp
-        __syncwarp();
-        pricing_hits<P>(hits, nh, lane, tl, s_ac, s_y, pts, pts_i, inU, xy, lam, rp, ec, n, fb, pairs, cap, count);
-        __syncwarp();  // the list is free for the next chunk
       }
     }
   }
+  __syncwarp();
+  pricing_test2(lists, lists.n1, sc);
+  pricing_test3(lists, lists.n2, sc);
 }
 
 // the nodes whose lambda (units 2^-fb) exceeds the reference (units 2^-fb_ref,
-// fb >= fb_ref) scaled to fb: flagged in inU, their points appended to pts_u
-// (order unspecified), their number in *count
+// fb >= fb_ref) scaled to fb: flagged in inU (by node), their points appended
+// to pts_u, a warp's together (so that pts_u keeps most of the order of pts)
 __global__ void pricing_raised_kernel(const int32_t* __restrict__ lam, const int32_t* __restrict__ lam_ref,
                                       int32_t n, int32_t shift, const float4* __restrict__ pts,
-                                      uint8_t* __restrict__ inU, float4* __restrict__ pts_u,
-                                      unsigned int* count) {
-  for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < n;
-       v += (long long)gridDim.x * blockDim.x) {
-    const bool up = (long long)lam[v] > ((long long)lam_ref[v] << shift);
-    inU[v] = up ? 1 : 0;
-    if (up) pts_u[atomicAdd(count, 1u)] = pts[v];
+                                      uint8_t* __restrict__ inU, float4* __restrict__ pts_u, PriceCtl* ctl) {
+  const int lane = threadIdx.x & 31;
+  for (long long v0 = blockIdx.x * (long long)blockDim.x + (threadIdx.x & ~31); v0 < n;
+       v0 += (long long)gridDim.x * blockDim.x) {
+    const long long v = v0 + lane;
+    bool up = false;
+    float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (v < n) {
+      q = pts[v];
+      const int u = __float_as_int(q.w);
+      up = (long long)lam[u] > ((long long)lam_ref[u] << shift);
+      inU[u] = up ? 1 : 0;
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, up);
+    unsigned base = 0;
+    if (lane == 0 && m) base = atomicAdd(&ctl->rows, (unsigned)__popc(m));
+    base = __shfl_sync(0xffffffffu, base, 0);
+    if (up) pts_u[base + __popc(m & ((1u << lane) - 1u))] = q;
   }
 }
 
-cudaError_t launch_pricing_raised(const int32_t* lam, const int32_t* lam_ref, int32_t n, int32_t shift,
-                                  const float4* pts, uint8_t* inU, float4* pts_u, unsigned int* count,
-                                  cudaStream_t st) {
-  cudaError_t e = cudaMemsetAsync(count, 0, sizeof(unsigned int), st);
-  if (e != cudaSuccess) return e;
-  int blocks = (int)((n + 255) / 256);
-  if (blocks > 4096) blocks = 4096;
-  if (blocks < 1) blocks = 1;
-  pricing_raised_kernel<<<blocks, 256, 0, st>>>(lam, lam_ref, n, shift, pts, inU, pts_u, count);
+cudaError_t launch_pricing_raised(const int32_t* lam_ref, int32_t shift, const PriceScan& sc, uint8_t* inU,
+                                  float4* pts_u, float4* box_u, float* smax_u, cudaStream_t st) {
+  pricing_raised_kernel<<<(sc.n + 255) / 256, 256, 0, st>>>(sc.lam, lam_ref, sc.n, shift, sc.pts, inU, pts_u,
+                                                            sc.ctl);
+  count_launch();
+  const int nb = (sc.n + kPriceBlock - 1) / kPriceBlock;
+  pricing_boxes_kernel<<<(nb + 7) / 8, 256, 0, st>>>(pts_u, sc.ctl, box_u, smax_u);
   count_launch();
   return cudaGetLastError();
 }
 
-cudaError_t launch_pricing_prep(const int2* xy, const int32_t* lam, const int32_t* perm, int32_t n, int32_t fb,
-                                float4* pts, cudaStream_t st) {
-  const int threads = 256;
-  int blocks = (int)((n + threads - 1) / threads);
-  if (blocks > 4096) blocks = 4096;
-  pricing_prep_kernel<<<blocks, threads, 0, st>>>(xy, lam, perm, n, fb, pts);
+cudaError_t launch_pricing_prep(const PriceScan& sc, const int32_t* perm, int32_t nblocks, float4* pts, float4* box,
+                                float* smax, cudaStream_t st) {
+  pricing_prep_kernel<<<(nblocks + 7) / 8, 256, 0, st>>>(sc.xy, sc.lam, perm, sc.seg_off, sc.seg_blk, sc.nseg,
+                                                         nblocks, sc.fb, pts, box, smax, sc.ctl);
   count_launch();
   return cudaGetLastError();
 }
 
-cudaError_t launch_pricing_boxes(const float4* pts, const int2* ranges, int32_t nranges, float4* box, float* smax,
-                                 cudaStream_t st) {
-  if (nranges <= 0) return cudaSuccess;
-  pricing_boxes_kernel<<<nranges, 256, 0, st>>>(pts, ranges, box, smax);
+cudaError_t launch_pricing_cull(const PriceScan& sc, const uint8_t* seg_scan, int32_t nblocks, int2* list,
+                                cudaStream_t st) {
+  pricing_cull_kernel<<<nblocks, 256, 0, st>>>(sc.box, sc.smax, sc.seg_blk, seg_scan, sc.nseg, list, sc.list_cap,
+                                               sc.ctl);
   count_launch();
   return cudaGetLastError();
 }
 
-cudaError_t launch_pricing_scan(const float4* pts, const int2* xy, const int32_t* lam, const int32_t* rp,
-                                const int2* ec, int32_t n, int32_t fb, const int4* tiles, int32_t ntiles,
-                                int2* pairs, int64_t cap, unsigned long long* count, unsigned int* tile_counter,
-                                int num_sms, cudaStream_t st, const float4* pts_i, const uint8_t* inU, int32_t ni) {
-  if (!pts_i) pts_i = pts;
-  const int32_t nj_tiles = (n + kPriceJMax - 1) / kPriceJMax;
-  cudaError_t err = cudaMemsetAsync(count, 0, sizeof(unsigned long long), st);
-  if (err == cudaSuccess) err = cudaMemsetAsync(tile_counter, 0, sizeof(unsigned int), st);
-  if (err != cudaSuccess) return err;
-  if (ntiles == 0) return cudaSuccess;
-  // P = 8 when the tile pairs fill the GPU several times over
+// CTAs of a persistent launch
+static cudaError_t price_grid(const void* kern, int threads, int num_sms, long long ntiles, int* grid) {
   int per_sm = 0;
-  err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pricing_kernel<8>, kPriceTile / 8, 0);
-  if (err != cudaSuccess) return err;
-  if (per_sm < 1) per_sm = 1;
-  if ((long long)ntiles >= 4LL * num_sms * per_sm) {
-    const long long grid = (long long)num_sms * per_sm;
-    pricing_kernel<8><<<(int)grid, kPriceTile / 8, 0, st>>>(pts, xy, lam, rp, ec, n, fb, tiles, ntiles, pairs,
-                                                           cap, count, tile_counter, pts_i, inU, ni, nj_tiles);
-  } else {
-    err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, pricing_kernel<4>, kPriceTile / 4, 0);
-    if (err != cudaSuccess) return err;
-    if (per_sm < 1) per_sm = 1;
-    long long grid = (long long)num_sms * per_sm;
-    if (grid > ntiles) grid = ntiles;
-    pricing_kernel<4><<<(int)grid, kPriceTile / 4, 0, st>>>(pts, xy, lam, rp, ec, n, fb, tiles, ntiles, pairs,
-                                                           cap, count, tile_counter, pts_i, inU, ni, nj_tiles);
-  }
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, 0);
+  if (e != cudaSuccess) return e;
+  const long long g = (long long)num_sms * (per_sm < 1 ? 1 : per_sm);
+  *grid = (int)(g < ntiles ? g : (ntiles < 1 ? 1 : ntiles));
+  return cudaSuccess;
+}
+
+template <int FORM, int W, int J, int MINB>
+static cudaError_t price_launch(const PriceScan& sc, int num_sms, long long ntiles, cudaStream_t st) {
+  int grid = 0;
+  cudaError_t e = price_grid((const void*)pricing_kernel<FORM, W, J, MINB>, W * 32, num_sms, ntiles, &grid);
+  if (e != cudaSuccess) return e;
+  pricing_kernel<FORM, W, J, MINB><<<grid, W * 32, 0, st>>>(sc);
   count_launch();
   return cudaGetLastError();
 }
 
+// Large tiles (fewer prologues a pair) when they fill the GPU five times over
+// (6 CTAs per SM), else single-warp tiles (16 times as many).
+bool price_large_tiles(long long large_tiles, int num_sms) { return large_tiles >= 32LL * num_sms; }
+
+cudaError_t launch_pricing_full(const PriceScan& sc, bool large, long long ntiles, int num_sms, cudaStream_t st) {
+  if (ntiles <= 0) return cudaSuccess;
+  return large ? price_launch<kPriceFull, 4, kPriceLargeJ, 6>(sc, num_sms, ntiles, st)
+               : price_launch<kPriceFull, 1, kPriceBlock, 20>(sc, num_sms, ntiles, st);
+}
+
+cudaError_t launch_pricing_list(const PriceScan& sc, int num_sms, cudaStream_t st) {
+  return price_launch<kPriceList, 1, kPriceBlock, 20>(sc, num_sms, 1LL << 30, st);
+}
+
+cudaError_t launch_pricing_rows(const PriceScan& sc, int num_sms, cudaStream_t st) {
+  // the number of rows is on the device: sized for a fifth of the nodes
+  const long long large = (long long)((sc.n / 5 + kPriceLargeI - 1) / kPriceLargeI) *
+                          ((sc.n + kPriceLargeJ - 1) / kPriceLargeJ);
+  return price_large_tiles(large, num_sms)
+             ? price_launch<kPriceRows, 4, kPriceLargeJ, 6>(sc, num_sms, 1LL << 30, st)
+             : price_launch<kPriceRows, 1, kPriceBlock, 20>(sc, num_sms, 1LL << 30, st);
+}
 
 // ---- The scan on the tensor cores ------------------------------------------------
 //
@@ -983,9 +1185,55 @@ __global__ void __launch_bounds__(kMmaI, 1) pricing_mma_check_kernel(long long r
   if (warp == 0) tc::tmem_dealloc(tacc, kMmaJ);
 }
 
+// The same check of the default scan's mma.sync, over its ranges (coordinates in
+// [-1024, 1023]): a warp's 32 rows against 128 columns a round, entry k of the
+// rows {0 i-point, 1 j-point} drawn where both the operands and the integer
+// product can reach it.
+__device__ __forceinline__ int price_check_entry(unsigned long long base, int row, int side, int k) {
+  const unsigned long long key = base + (unsigned long long)side * 4096 + (unsigned long long)row * 8;
+  const bool far = (mma_check_hash(key + 7) & 15u) == 0u;
+  const int at = side ? k ^ 2 : k;  // j-rows hold {2048, 1} before A
+  if (k < 4 && at >= 2) return at == 2 ? 2048 : 1;
+  if (at == 0) return far ? 1024 : mma_check_draw(key, -512, 1023);
+  if (at == 1) return far ? 0 : mma_check_draw(key + 1, 0, 2047);
+  if (k == 7 || far) return 0;
+  const int v = k == 6 ? mma_check_draw(key + 4, 1, 1023) : mma_check_draw(key + k - 2, -1024, 1023);
+  return side ? -2 * v : v;
+}
+
+__global__ void __launch_bounds__(128) pricing_price_mma_check_kernel(long long rounds, unsigned long long seed,
+                                                                      unsigned long long* mismatches) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+  unsigned long long bad = 0;
+  for (long long r = 0; r < rounds; ++r) {
+    const unsigned long long base = (seed * 0x100000001B3ull + (unsigned long long)r) << 13;
+    for (int m = 0; m < 2; ++m) {
+      const int r0 = warp * 32 + m * 16 + g;
+      const unsigned a0 = pack_half(price_check_entry(base, r0, 0, 2 * t), price_check_entry(base, r0, 0, 2 * t + 1));
+      const unsigned a1 =
+          pack_half(price_check_entry(base, r0 + 8, 0, 2 * t), price_check_entry(base, r0 + 8, 0, 2 * t + 1));
+      for (int c0 = 0; c0 < 128; c0 += kPriceStep) {
+        const unsigned b = pack_half(price_check_entry(base, c0 + g, 1, 2 * t), price_check_entry(base, c0 + g, 1, 2 * t + 1));
+        float c[4];
+        price_mma(c, a0, a1, b);
+        for (int q = 0; q < 4; ++q) {
+          const int row = r0 + 8 * (q >> 1), col = c0 + 2 * t + (q & 1);
+          long long e = 0;
+          for (int k = 0; k < 8; ++k)
+            e += (long long)price_check_entry(base, row, 0, k) * price_check_entry(base, col, 1, k);
+          bad += (long long)c[q] != e || c[q] != (float)e;
+        }
+      }
+    }
+  }
+  atomicAdd(mismatches, bad);
+}
+
 cudaError_t launch_pricing_mma_check(long long rounds, unsigned long long seed, unsigned long long* checked,
                                      unsigned long long* mismatches, int32_t* status, cudaStream_t st) {
   pricing_mma_check_kernel<<<1, kMmaI, 0, st>>>(rounds, seed, checked, mismatches, status);
+  count_launch();
+  pricing_price_mma_check_kernel<<<1, 128, 0, st>>>(rounds, seed, mismatches);
   count_launch();
   return cudaGetLastError();
 }
