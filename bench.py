@@ -1,5 +1,5 @@
 """Benchmark: milliseconds to a certified F2M optimum, with the roofline of the
-dominant kernel (the pricing scan's FP32 rate or the GDP sweep's GB/s).
+dominant kernel (the pricing scan's tensor rate or the GDP sweep's GB/s).
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--workload c1|c2|c3|c4|c5]
     python bench.py --impl reference ...     # the CPU oracle on the same workload
@@ -57,8 +57,8 @@ def batch_specs(w, rank=0):
 METRIC = "ms to certified F2M optimum"
 GDP_BYTES_PER_ENTRY = 8   # {col, cost} streamed per directed entry
 GDP_BYTES_PER_NODE = 12   # row_ptr + lambda read + lambda write
-PRICING_OPS_PER_PAIR = 5  # FP32 lane operations of the kernel's packed filter: 3 adds (u, w, dy), 2 FMAs
-PRICING_SLOTS_PER_PAIR = 7  # algorithmic issue slots per pair: dx, dy, dx*dx, fma dy, r_u + r_v, square, compare
+PRICING_FLOPS_PER_PAIR = 16  # the filter's inner product: 8 multiply-adds (mma.sync m16n8k8)
+PRICING_PAIRS_PER_CYCLE = 64  # per SM: 128 pairs an mma.sync, one per 8 cycles and SM quarter (microbenchmark)
 
 
 def workload_name(w):
@@ -505,11 +505,11 @@ def single_line(args, wname, w, rank, world, local, dist, f2m, torch, nested=Fal
     pr_pairs = inf0.get("pricing_pairs") or inf0["pricing_rounds"] * n * (n - 1) / 2
     sm_mhz = clk.get("sm_mhz") or peaks.get("sm_max_mhz", 2070.0)
     num_sms = torch.cuda.get_device_properties(local).multi_processor_count
-    alu_peak = num_sms * 128 * sm_mhz * 1e6 / 1e12  # Tops/s at the sampled clock
-    pr_tops = pr_pairs * PRICING_SLOTS_PER_PAIR / (ms_pr * 1e-3) / 1e12 if ms_pr > 0 else 0.0
-    pr_tops_pipe = pr_pairs * PRICING_OPS_PER_PAIR / (ms_pr * 1e-3) / 1e12 if ms_pr > 0 else 0.0
+    pr_rate = pr_pairs / (ms_pr * 1e-3) if ms_pr > 0 else 0.0  # pairs/s
+    pr_tflops = pr_rate * PRICING_FLOPS_PER_PAIR / 1e12
+    pr_frac_pipe = pr_rate / (num_sms * PRICING_PAIRS_PER_CYCLE * sm_mhz * 1e6)
     traffic = load_traffic(wname)
-    gdp_kernel = "gdp_classes_kernel" if args.update == "classes" else "gdp_tiled2_kernel"
+    gdp_kernel = "gdp_classes_kernel" if args.update == "classes" else "gdp_ring_reg_kernel"
     if ms_gdp >= ms_pr:
         roofline = {"kernel": gdp_kernel, "bound": "hbm", "achieved": gdp_gbs,
                     "peak": peaks["hbm_gbs"], "unit": "GB/s", "frac": gdp_gbs / peaks["hbm_gbs"],
@@ -517,28 +517,27 @@ def single_line(args, wname, w, rank, world, local, dist, f2m, torch, nested=Fal
                     "note": "algorithmic bytes of the sweep over its time; the working set is shared-memory "
                             "and L2 resident, so this is an effective rate (DRAM sees the CSR once per phase)"}
     else:
-        roofline = {"kernel": "pricing_kernel", "bound": "alu", "achieved": pr_tops, "peak": alu_peak,
-                    "unit": "Tops/s", "frac": pr_tops / alu_peak,
+        roofline = {"kernel": "pricing_kernel", "bound": "tensor", "achieved": pr_tflops, "peak": peaks["bf16_tflops"],
+                    "unit": "TFLOP/s", "frac": pr_tflops / peaks["bf16_tflops"],
                     "traffic": traffic.get("pricing_kernel"),
-                    "work": f"{PRICING_SLOTS_PER_PAIR} issue slots per pair (2 FADD for dx, dy; FMUL, FFMA, "
-                            f"FADD r_u + r_v, FMUL square, FSETP) x n(n-1)/2 pairs per scan",
-                    "frac_pipe": pr_tops_pipe / alu_peak,
-                    "frac_pipe_work": f"{PRICING_OPS_PER_PAIR} FP32 lane operations per pair that the kernel's "
-                                      f"packed filter issues (3 adds, 2 FMAs)"}
+                    "work": f"{PRICING_FLOPS_PER_PAIR} flops per pair (8 multiply-adds of the exact integer "
+                            f"filter) x the pairs the scans evaluated",
+                    "frac_pipe": pr_frac_pipe,
+                    "frac_pipe_work": f"pairs against the issue rate of mma.sync m16n8k8, {PRICING_PAIRS_PER_CYCLE} "
+                                      f"pairs a cycle and SM"}
     roofline["peak_source"] = "MEASURED_PEAKS.json" if not peaks.get("_fallback") else "fallback"
-    roofline["peak_note"] = f"{num_sms} SMs x 128 FP32 lanes x the SM clock sampled in the timed region" \
+    roofline["peak_note"] = "bf16_tflops of MEASURED_PEAKS.json" \
         if roofline["kernel"] == "pricing_kernel" else "hbm_gbs of MEASURED_PEAKS.json"
     if args.pricing == 2 and roofline["kernel"] == "pricing_kernel":
         roofline["effective"] = True
         roofline["note"] = ("culled scan: the rate counts all n(n-1)/2 pairs per scan, but tile pairs that "
                             "cannot hold z < 0 are not evaluated, so it is an effective rate and can exceed "
-                            "the lane peak")
+                            "the peak")
     roofline["gdp_sweep_gbs"] = gdp_gbs
     roofline["gdp_sweep_frac_of_hbm"] = gdp_gbs / peaks["hbm_gbs"]
     roofline["gdp_working_set_mb"] = (GDP_BYTES_PER_ENTRY * nnz0 + GDP_BYTES_PER_NODE * n) / 1e6
-    roofline["pricing_tops"] = pr_tops
-    roofline["pricing_frac_of_alu"] = pr_tops / alu_peak
-    roofline["pricing_frac_pipe"] = pr_tops_pipe / alu_peak
+    roofline["pricing_tflops"] = pr_tflops
+    roofline["pricing_frac_pipe"] = pr_frac_pipe
 
     host_ms = {"flush_enqueue": statistics.median(h[0] for h in host),
                "f2m_solve": statistics.median(h[1] for h in host),
@@ -692,16 +691,14 @@ def run_batch(args, w, rank, world, local):
     pairs = float(sum(int(i.pricing_rounds) * n * (n - 1) / 2 for i, n in zip(infos, ns)))
     sm_mhz = clk.get("sm_mhz") or peaks.get("sm_max_mhz", 2070.0)
     num_sms = torch.cuda.get_device_properties(local).multi_processor_count
-    alu_peak = num_sms * 128 * sm_mhz * 1e6 / 1e12
-    pr_tops = pairs * PRICING_SLOTS_PER_PAIR / (ms_pr * 1e-3) / 1e12 if ms_pr > 0 else 0.0
-    pr_tops_pipe = pairs * PRICING_OPS_PER_PAIR / (ms_pr * 1e-3) / 1e12 if ms_pr > 0 else 0.0
+    pr_rate = pairs / (ms_pr * 1e-3) if ms_pr > 0 else 0.0
     roofline = {"kernel": "gdp_batch_kernel", "bound": "hbm", "achieved": gdp_gbs,
                 "peak": peaks["hbm_gbs"], "unit": "GB/s", "frac": gdp_gbs / peaks["hbm_gbs"],
                 "traffic": load_traffic(args.workload).get("gdp_batch_kernel"),
                 "peak_source": "MEASURED_PEAKS.json" if not peaks.get("_fallback") else "fallback",
                 "gdp_working_set_mb": float(np.sum(GDP_BYTES_PER_ENTRY * nnzs + GDP_BYTES_PER_NODE * ns)) / 1e6,
-                "pricing_tops": pr_tops, "pricing_frac_of_alu": pr_tops / alu_peak,
-                "pricing_frac_pipe": pr_tops_pipe / alu_peak}
+                "pricing_tflops": pr_rate * PRICING_FLOPS_PER_PAIR / 1e12,
+                "pricing_frac_pipe": pr_rate / (num_sms * PRICING_PAIRS_PER_CYCLE * sm_mhz * 1e6)}
     line = {"metric": METRIC + " (all instances of the batch)", "value": ms, "unit": "ms",
             "n_gpus": world, "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms,
             "higher_is_better": False, "scaling": "weak", "vs_baseline": None, "dtype": "int32",

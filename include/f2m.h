@@ -84,7 +84,8 @@ typedef struct {
   int32_t finisher;             /* 1 = exact finisher when rule (7) gives an infeasible x (default) */
   uint32_t flags;               /* F2M_FLAG_* bits; default 0 */
   int32_t gdp_lanes;            /* lanes per node in the tiled GDP kernel: 1 (one thread per node); 0 = auto */
-  int32_t gdp_ctas_per_sm;      /* tiled GDP CTAs per SM: 1 (x1024 threads), 2 (x512); 0 = auto */
+  int32_t gdp_ctas_per_sm;      /* tiled GDP CTAs per SM: 1 (x1024 threads), 2 (x512, one sweep
+                                   per exchange); 0 = auto */
   int32_t batch_shape;          /* batched GDP kernel shape (threads, copy stages, CTAs per SM):
                                    -1 = picked by the autotuner (default), 0..4 = a fixed one */
   int32_t batch_graph;          /* 1 = replay each batched GDP phase from a captured CUDA graph
@@ -92,16 +93,17 @@ typedef struct {
 } f2m_params;
 
 /* f2m_params.flags: run GDP with the streaming kernel (CSR read from global
- * memory every sweep, caller node order) instead of the default shared-memory
- * tiled kernel (nodes renumbered along a Morton curve, each CTA's rows, own
- * lambda and halo held in shared memory).  Both give identical results. */
+ * memory every sweep, caller node order) instead of the default tiled kernel
+ * (nodes renumbered along a Morton curve, each CTA's rows and own lambda on
+ * chip for the whole phase, with rings of neighbouring nodes around them, so
+ * that tiles exchange lambda once per few sweeps).  Both give identical
+ * results. */
 #define F2M_FLAG_STREAMING_GDP 1u
 
-/* f2m_params.flags: run the shared-memory tiled GDP kernel with one sweep per
- * device-wide barrier instead of the default two (the default keeps each
- * CTA's halo rows and a second halo ring, computes the halo rows' sweep
- * redundantly, and meets the other CTAs once per two sweeps).  Identical
- * results either way. */
+/* f2m_params.flags: run the tiled GDP kernel with one sweep per exchange between
+ * tiles instead of the default two to four (the default keeps the rows of the
+ * inner rings and computes their sweeps redundantly).  Identical results either
+ * way. */
 #define F2M_FLAG_ONE_SWEEP_GDP 2u
 
 /* f2m_params.flags: class-by-class GDP sweeps (a Gauss-Seidel form of the
@@ -188,8 +190,8 @@ typedef struct {
 
 /* f2m_info.gdp_kernel values */
 #define F2M_GDP_KERNEL_STREAMING 0     /* CSR read from global memory every sweep */
-#define F2M_GDP_KERNEL_TILED 1         /* shared-memory tiles, one sweep per barrier */
-#define F2M_GDP_KERNEL_TWO_SWEEP 2     /* shared-memory tiles, two sweeps per barrier */
+#define F2M_GDP_KERNEL_TILED 1         /* on-chip tiles, one sweep per exchange */
+#define F2M_GDP_KERNEL_TWO_SWEEP 2     /* on-chip tiles, two or more sweeps per exchange */
 #define F2M_GDP_KERNEL_TWO_SWEEP_PACKED 3  /* the same with 4-byte entries (larger tiles) */
 #define F2M_GDP_KERNEL_CLASSES 4       /* class-by-class sweeps */
 #define F2M_GDP_KERNEL_BATCH 5         /* batched, union CSR streamed */
@@ -234,9 +236,9 @@ f2m_status f2m_set_lambda(f2m_ctx* ctx, const int32_t* lambda, int32_t frac_bits
  * the finisher's supplies and demands are b_v.  Pricing is unchanged.
  *   b  [n] int32, host or device, copied; 1 <= b_v <= deg(v) - 1 for the
  *      graph held now (pricing only adds edges).  NULL restores b_v = 2.
- * Single-instance contexts only.  While b is set, GDP phases run on the
- * two-sweep shared-memory kernel (a sorted top-8 per row when every b_v < 8,
- * counting otherwise) or, where its tiles do not fit, the streaming kernel.
+ * Single-instance contexts only.  While b is set, GDP phases run on the tiled
+ * kernel (a sorted top-5 or top-8 per row when every b_v < 5 or < 8, counting
+ * otherwise) or, where its tiles do not fit, the streaming kernel.
  * Errors: INVALID_ARG (range, with the first offending node in
  * f2m_last_error; the previous b stays), OOM, CUDA. */
 f2m_status f2m_set_degrees(f2m_ctx* ctx, const int32_t* b);
@@ -258,8 +260,7 @@ f2m_status f2m_solve(f2m_ctx* ctx, f2m_info* info);
 
 /* One GDP phase (Eq. 9, Eq. 10, Jacobi): up to max_sweeps sweeps from the
  * current lambda (units 2^-F), stopping after the first sweep that changes no
- * lambda.  Runs as one persistent cooperative kernel with a device-wide
- * barrier per sweep.
+ * lambda.  Runs as one persistent cooperative kernel.
  *   sweeps         out: sweeps run.
  *   trace_bound2   NULL or [trace_cap] int64 (host or device): bound2 at the
  *                  lambda each sweep started from.

@@ -12,6 +12,7 @@
 #include <map>
 #include <mutex>
 #include <climits>
+#include <cmath>
 #include <cstdio>
 #include <cstring>
 #include <new>
@@ -345,9 +346,10 @@ extern "C" void f2m_destroy(f2m_ctx* c) {
   dfree(c->d_count); dfree(c->d_tile); dfree(c->d_deg); dfree(c->d_tmp_rp); dfree(c->d_new_rp);
   dfree(c->d_block_sums); dfree(c->d_tmp_col); dfree(c->d_out_a); dfree(c->d_out_b);
   dfree(c->d_check); dfree(c->d_scalar); dfree(c->d_bad); dfree(c->d_b); dfree(c->d_b_int);
+  dfree(c->d_ring_seg);
   free_finisher_buffers(c);
   if (c->fin_work) finisher_work_free(c->fin_work);
-  plan2_free(c->plan);
+  ring_free(c->ring);
   plan_free(c->plan);
   class_plan_free(c->classes);
   cut_state_free(c->cuts);
@@ -460,11 +462,7 @@ f2m_status f2m::create_internal(const int32_t* xy, int32_t n, const int32_t* row
     e = dalloc(&c->d_ec, c->ec_cap);
     if (e == cudaSuccess) e = launch_build_ec(c->d_xy, c->d_rp, d_col, n, c->d_ec, c->st);
     if (e == cudaSuccess) e = plan_renumber(c->d_xy, n, c->seg_off, c->plan, c->st);
-    if (e == cudaSuccess)
-      e = plan_build(c->d_rp, c->d_ec, n, c->nnz, c->num_sms, !(p.flags & F2M_FLAG_STREAMING_GDP),
-                     p.frac_bits, p.gdp_ctas_per_sm, c->plan, c->st);
-    if (e == cudaSuccess && seg_off.size() == 2 && !(p.flags & F2M_FLAG_ONE_SWEEP_GDP))
-      e = plan_build2(c->plan, p.frac_bits, c->st);
+    if (e == cudaSuccess) e = plan_build(c->d_rp, c->d_ec, n, c->nnz, c->plan, c->st);
     if (e == cudaSuccess && p.finisher) {
       e = alloc_finisher_buffers(c, c->ec_cap);
       c->fin_work = finisher_work_new();
@@ -598,6 +596,114 @@ const int32_t* f2m::cur_lambda(f2m_ctx* c, int32_t* fb) {
   return c->fb_cur == c->p.frac_bits ? c->d_lam[c->cur] : c->d_lam2;
 }
 
+// Sweeps per exchange of the GDP tiles, by own rows a tile: more rings cost more
+// rows, fewer more exchanges.  us a sweep with K = 1, 2, 3, 4: 66 rows 1.52, 0.93,
+// 0.79, 0.75; 132 rows 1.57, 1.07, 0.94, 0.92; 329 rows 1.78 at K = 2, 1.67 at 3, 1.93 at 4;
+// 658 rows 1.88, 1.58, 1.78, 1.82; 1,316 rows 3.00, 2.87, and K = 3 does not fit
+static int32_t ring_sweeps(int64_t own) { return own <= 200 ? 4 : (own <= 400 ? 3 : 2); }
+
+// A GDP phase on the shared-memory tiles; *ran false where no number of rings
+// fits (the caller takes the streaming kernel).
+static f2m_status ring_phase(f2m_ctx* c, int64_t max_sweeps, int64_t* sweeps, long long* tb, unsigned long long* tc,
+                             int64_t tcap, double* ms, bool* ran) {
+  *ran = true;
+  *sweeps = 0;
+  if (max_sweeps <= 0) return F2M_ERR_NOT_CONVERGED;
+  const bool half = c->p.gdp_ctas_per_sm == 2;  // 2 CTAs per SM
+  const bool one = half || (c->p.flags & F2M_FLAG_ONE_SWEEP_GDP);
+  // small graphs use fewer tiles, of 64 rows (1,000 points: 0.75 us a sweep with
+  // tiles of 64 rows, 0.77 with 32, 0.88 with 128, 1.19 with 256)
+  const int64_t most = (int64_t)c->num_sms * (half ? 2 : 1);
+  const int32_t tiles = (int32_t)std::max<int64_t>(1, std::min<int64_t>(most, c->n / 64));
+  const int32_t want = one ? 1 : ring_sweeps(c->n / tiles);
+  if (c->ring_k == 0) {
+    c->ring_k = want;
+    if (half || c->n / tiles > 1900) c->ring_reg = false;
+    // rows a thread: a guess (a ring of about 14 sqrt(own) rows), corrected below
+    const double own = (double)c->n / tiles, ring = tiles > 1 ? 14.0 * std::sqrt(own) + 30.0 : 0.0;
+    const double slices = own / 32.0 + (c->ring_k - 1) * (ring / 32.0 + 1.0);
+    c->ring_rows = slices <= 30.0 ? 1 : 2;
+  }
+  RingSeg h{};
+  for (;;) {
+    if (c->ring.version != c->plan.version || c->ring.K != c->ring_k) {
+      if (!c->d_ring_seg) {
+        const int32_t off[2] = {0, c->n};
+        CK(c, dalloc(&c->d_ring_seg, 2));
+        CK(c, cudaMemcpyAsync(c->d_ring_seg, off, sizeof(off), cudaMemcpyHostToDevice, c->st));
+      }
+      CK(c, ring_build(c->plan, c->d_ring_seg, nullptr, tiles, c->ring_k, c->p.frac_bits, c->nnz / tiles, c->ring,
+                       c->st));
+    }
+    int64_t limit = std::min<int64_t>(max_sweeps, kRingSweeps);
+    bool replay = false;
+    int32_t status = 0;
+    // in shared memory: traces, and the counting selection of large b_v
+    const bool reg = c->ring_reg && tcap == 0 && !(c->d_b && c->b_max >= 8);
+    for (;;) {
+      CK(c, ring_start(c->ring, c->n, 1, c->st));
+      if (tcap > 0 && !replay) {
+        CK(c, cudaMemsetAsync(tb, 0, sizeof(long long) * tcap, c->st));
+        CK(c, cudaMemsetAsync(tc, 0, sizeof(unsigned long long) * tcap, c->st));
+      }
+      CK(c, cudaEventRecord(c->ev0, c->st));
+      const cudaError_t e =
+          launch_gdp_ring(c->plan, c->ring, 0, tiles, c->d_lam[c->cur], c->d_lam[c->cur ^ 1], c->p.damping_shift,
+                          (int32_t)limit, tb, tc, replay ? 0 : tcap, c->p.barrier_budget_cycles, c->d_b_int, c->b_max,
+                          reg ? (RingForm)c->ring_rows : (half ? kRingHalf : kRingSmem), c->st);
+      if (e == cudaErrorCooperativeLaunchTooLarge) {  // not on this device now
+        cudaGetLastError();
+        *ran = false;
+        return F2M_OK;
+      }
+      CK(c, e);
+      CK(c, cudaEventRecord(c->ev1, c->st));
+      RingStats rs{};
+      CK(c, cudaMemcpyAsync(&status, c->ring.status, sizeof(status), cudaMemcpyDeviceToHost, c->st));
+      CK(c, cudaMemcpyAsync(&rs, c->ring.stats, sizeof(rs), cudaMemcpyDeviceToHost, c->st));
+      RingSeg q{};
+      CK(c, cudaMemcpyAsync(&q, c->ring.seg, sizeof(q), cudaMemcpyDeviceToHost, c->st));
+      CK(c, cudaStreamSynchronize(c->st));
+      if (ms) *ms += elapsed_ms(c);
+      if (status & kGdpTimeout) return fail(c, F2M_ERR_TIMEOUT, "a wait for another tile exceeded its budget");
+      if (reg) {  // what the tiles need, known now
+        const int fits = ring_reg_rows(rs), had = c->ring_rows;
+        if (fits) c->ring_rows = fits;
+        if ((status & kGdpNoFit) && fits && fits != had) continue;
+      }
+      if (status & kGdpNoFit) break;
+      const bool packed = reg ? c->ring_rows > 1 : rs.bytes8 > ring_smem(half);
+      c->gdp_kernel = c->ring.K == 1 ? F2M_GDP_KERNEL_TILED
+                                     : (packed ? F2M_GDP_KERNEL_TWO_SWEEP_PACKED : F2M_GDP_KERNEL_TWO_SWEEP);
+      if (replay) break;
+      h = q;
+      if (!q.overflow) break;
+      // the input of the sweep that overflowed: the sweeps before it again
+      replay = true;
+      limit = q.sweeps - 1;
+      if (limit == 0) break;
+    }
+    if (!(status & kGdpNoFit)) {
+      if (!(h.overflow && h.sweeps == 1)) c->cur ^= 1;  // else lambda stays at the input
+      break;
+    }
+    // fewer rings take fewer registers and less shared memory
+    if (c->ring_k > 1) {
+      c->ring_k -= 1;
+    } else if (reg) {
+      c->ring_reg = false;
+      c->ring_k = one ? 1 : 2;
+    } else {
+      c->ring_k = -1;
+      *ran = false;
+      return F2M_OK;
+    }
+  }
+  *sweeps = h.sweeps;
+  if (h.overflow) return fail(c, F2M_ERR_OVERFLOW, "|lambda| reached 2^29");
+  return h.fixed_point ? F2M_OK : F2M_ERR_NOT_CONVERGED;
+}
+
 f2m_status f2m::gdp_phase(f2m_ctx* c, int64_t max_sweeps, int64_t* sweeps, bool want_trace,
                             int64_t trace_cap, double* ms) {
   const int32_t F = c->p.frac_bits;
@@ -638,97 +744,36 @@ f2m_status f2m::gdp_phase(f2m_ctx* c, int64_t max_sweeps, int64_t* sweeps, bool 
     if (h.status & kGdpOverflow) return fail(c, F2M_ERR_OVERFLOW, "|lambda| reached 2^29");
     return h.fixed_point ? F2M_OK : F2M_ERR_NOT_CONVERGED;
   }
-  if (c->plan1_pending) {
-    CK(c, plan_build_tiles(c->num_sms, c->p.frac_bits, c->p.gdp_ctas_per_sm, c->plan, c->st));
-    c->plan1_pending = false;
-  }
-  if (c->plan2_pending) {
-    CK(c, plan_build2(c->plan, c->p.frac_bits, c->st));
-    c->plan2_pending = false;
+  if (!(c->p.flags & F2M_FLAG_STREAMING_GDP) && c->ring_k >= 0) {
+    bool ran = false;
+    f2m_status s = ring_phase(c, max_sweeps, sweeps, tb, tc, tcap, ms, &ran);
+    while (ran && s == F2M_ERR_NOT_CONVERGED && *sweeps < max_sweeps) {  // past one launch's sweeps
+      int64_t more = 0;
+      const int64_t at = *sweeps;
+      s = ring_phase(c, max_sweeps - at, &more, tb ? tb + std::min(at, tcap) : tb, tc ? tc + std::min(at, tcap) : tc,
+                     std::max<int64_t>(tcap - at, 0), ms, &ran);
+      *sweeps = at + more;
+    }
+    if (ran) return s;
   }
   CK(c, cudaMemsetAsync(c->d_gdp, 0, sizeof(GdpCtl), c->st));
   CK(c, cudaEventRecord(c->ev0, c->st));
-  // degree requirements run on the two-sweep kernel or the streaming one (the
-  // one-sweep tiled kernel holds Eq. 10's top-3 only)
-  bool two = c->plan.valid2;  // two sweeps per barrier
-  bool tiled = c->plan.valid && !c->d_b;
-  if (two) {
-    cudaError_t e = launch_gdp_tiled2(c->plan, c->d_lam[c->cur], c->p.damping_shift, max_sweeps, c->d_gdp, tb,
-                                      tc, tcap, c->p.barrier_budget_cycles, c->d_b_int, c->b_max, c->st);
-    if (e == cudaErrorCooperativeLaunchTooLarge) {
-      cudaGetLastError();
-      two = false;
-    } else {
-      CK(c, e);
-    }
-  }
-  if (!two && tiled) {
-    cudaError_t e = launch_gdp_tiled(c->plan, c->d_lam[c->cur], c->p.damping_shift, max_sweeps,
-                                     c->d_gdp, tb, tc, tcap, c->p.barrier_budget_cycles, c->st);
-    if (e == cudaErrorCooperativeLaunchTooLarge) {
-      cudaGetLastError();
-      tiled = false;  // the tiles do not fit on this device now: streaming kernel
-    } else {
-      CK(c, e);
-    }
-  }
-  if (!two && !tiled)
-    CK(c, launch_gdp(c->d_rp, c->d_ec, c->d_b, c->b_max, c->d_lam[c->cur], c->d_lam[c->cur ^ 1], c->n, F,
-                     c->p.damping_shift, max_sweeps, c->d_gdp, tb, tc, tcap,
-                     c->p.barrier_budget_cycles, c->num_sms, c->st));
+  CK(c, launch_gdp(c->d_rp, c->d_ec, c->d_b, c->b_max, c->d_lam[c->cur], c->d_lam[c->cur ^ 1], c->n, F,
+                   c->p.damping_shift, max_sweeps, c->d_gdp, tb, tc, tcap,
+                   c->p.barrier_budget_cycles, c->num_sms, c->st));
   CK(c, cudaEventRecord(c->ev1, c->st));
-  c->gdp_kernel = two ? (c->plan.packed2 ? F2M_GDP_KERNEL_TWO_SWEEP_PACKED : F2M_GDP_KERNEL_TWO_SWEEP)
-                      : (tiled ? F2M_GDP_KERNEL_TILED : F2M_GDP_KERNEL_STREAMING);
+  c->gdp_kernel = F2M_GDP_KERNEL_STREAMING;
   GdpCtl h{};
   CK(c, cudaMemcpyAsync(&h, c->d_gdp, sizeof(h), cudaMemcpyDeviceToHost, c->st));
   CK(c, cudaStreamSynchronize(c->st));
   if (ms) *ms += elapsed_ms(c);
-  if (two && !(h.status & kGdpTimeout)) {
-    CK(c, plan_scatter_lambda(c->plan, (int)h.pad1, c->d_lam[c->cur], c->st));
-    if (h.status & kGdpOddOverflow) {
-      // the second sweep of a round overflowed: replay that round from its
-      // input with the one-sweep kernel, which leaves lambda at the input of
-      // the overflowing sweep
-      const long long base = h.sweeps - 2;
-      CK(c, cudaMemsetAsync(c->d_gdp, 0, sizeof(GdpCtl), c->st));
-      GdpCtl h2{};
-      if (c->d_b) {  // with degree requirements: the streaming kernel replays the round
-        CK(c, launch_gdp(c->d_rp, c->d_ec, c->d_b, c->b_max, c->d_lam[c->cur], c->d_lam[c->cur ^ 1], c->n, F,
-                         c->p.damping_shift, 2, c->d_gdp, tb ? tb + base : nullptr, tc ? tc + base : nullptr,
-                         tcap > base ? tcap - base : 0, c->p.barrier_budget_cycles, c->num_sms, c->st));
-        CK(c, cudaMemcpyAsync(&h2, c->d_gdp, sizeof(h2), cudaMemcpyDeviceToHost, c->st));
-        CK(c, cudaStreamSynchronize(c->st));
-        const bool ovf2 = (h2.status & kGdpOverflow) != 0;
-        if (!(h2.status & kGdpTimeout) && ((ovf2 ? h2.sweeps - 1 : h2.sweeps) & 1)) c->cur ^= 1;
-      } else {
-        CK(c, launch_gdp_tiled(c->plan, c->d_lam[c->cur], c->p.damping_shift, 2, c->d_gdp,
-                               tb ? tb + base : nullptr, tc ? tc + base : nullptr,
-                               tcap > base ? tcap - base : 0, c->p.barrier_budget_cycles, c->st));
-        CK(c, cudaMemcpyAsync(&h2, c->d_gdp, sizeof(h2), cudaMemcpyDeviceToHost, c->st));
-        CK(c, cudaStreamSynchronize(c->st));
-        const bool ovf2 = (h2.status & kGdpOverflow) != 0;
-        if (!(h2.status & kGdpTimeout))
-          CK(c, plan_scatter_lambda(c->plan, (int)((ovf2 ? h2.sweeps - 1 : h2.sweeps) % 3), c->d_lam[c->cur], c->st));
-      }
-      h.status = (h.status & ~kGdpOddOverflow) | h2.status;
-      h.sweeps = base + h2.sweeps;
-      h.fixed_point = h2.fixed_point;
-    }
-  }
   *sweeps = h.sweeps;
   const bool ovf = (h.status & kGdpOverflow) != 0;
   // the sweep that overflowed leaves lambda at its input; otherwise the last output
-  const long long used = ovf ? h.sweeps - 1 : h.sweeps;
-  if (!two && tiled) {
-    if (!(h.status & kGdpTimeout))
-      CK(c, plan_scatter_lambda(c->plan, (int)(used % 3), c->d_lam[c->cur], c->st));
-  } else if (!two && (used & 1)) {
-    c->cur ^= 1;
-  }
+  if ((ovf ? h.sweeps - 1 : h.sweeps) & 1) c->cur ^= 1;
   if (h.status & kGdpTimeout) return fail(c, F2M_ERR_TIMEOUT, "device-wide barrier wait exceeded its budget");
   if (ovf) return fail(c, F2M_ERR_OVERFLOW, "|lambda| reached 2^29");
-  if (!h.fixed_point) return F2M_ERR_NOT_CONVERGED;
-  return F2M_OK;
+  return h.fixed_point ? F2M_OK : F2M_ERR_NOT_CONVERGED;
 }
 
 extern "C" f2m_status f2m_gdp(f2m_ctx* c, int64_t max_sweeps, int64_t* sweeps, int64_t* trace_bound2,
@@ -1108,14 +1153,10 @@ f2m_status f2m::merge_internal(f2m_ctx* c, const int2* d_pairs, int64_t npairs, 
   CK(c, read_check(c, &h));
   c->nnz = nnz_h;
   if (h.flags) return fail(c, F2M_ERR_INVALID_ARG, check_message(h.flags, h.first_bad));
-  // the internal CSR now (the finisher reads it); the tiles of the
-  // shared-memory GDP kernels only serve GDP phases: built when the next one
-  // starts (a merge before the finisher and the last scan needs none)
-  CK(c, plan_build(c->d_rp, c->d_ec, n, c->nnz, c->num_sms, false, c->p.frac_bits, c->p.gdp_ctas_per_sm,
-                   c->plan, c->st));
-  c->plan1_pending = c->seg_off.size() == 2 && !(c->p.flags & F2M_FLAG_STREAMING_GDP);
-  c->plan.valid2 = false;
-  c->plan2_pending = c->seg_off.size() == 2 && !(c->p.flags & F2M_FLAG_ONE_SWEEP_GDP);
+  // the internal CSR now (the finisher reads it); the GDP tiles only serve GDP
+  // phases: built when the next one starts (a merge before the finisher and the
+  // last scan needs none)
+  CK(c, plan_build(c->d_rp, c->d_ec, n, c->nnz, c->plan, c->st));
   CK(c, cudaEventRecord(c->ev1, c->st));
   if (ms) *ms += elapsed_ms(c);
   return F2M_OK;

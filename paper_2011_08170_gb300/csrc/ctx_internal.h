@@ -111,9 +111,12 @@ struct f2m_ctx {
   long long* d_scalar = nullptr;
   unsigned long long* d_bad = nullptr;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
-  f2m::GdpPlan plan;         // renumbering and tiles of the shared-memory GDP kernel
-  bool plan1_pending = false;  // the one-sweep tiles are built at the next GDP phase
-  bool plan2_pending = false;  // the two-sweep tiles are built at the next GDP phase
+  f2m::GdpPlan plan;         // renumbering, the CSR in that order
+  f2m::RingPlan ring;        // shared-memory tiles of the GDP kernel (built by the phase that needs them)
+  int32_t* d_ring_seg = nullptr;  // {0, n} on the device
+  int32_t ring_k = 0;        // rings of the tiles (0: not tried, -1: none fit, the streaming kernel runs)
+  int32_t ring_rows = 0;     // rows a thread in that form
+  bool ring_reg = true;      // the tiles' rows fit registers, as far as tried
   f2m::ClassPlan classes;    // colour classes of the class-by-class GDP
   // exact finisher: device scratch, host work arrays; the h_ arrays point into
   // the process's one pinned host mirror while a finisher call holds it

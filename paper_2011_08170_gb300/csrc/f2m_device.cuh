@@ -47,11 +47,38 @@ __device__ __forceinline__ long long gdp_step(int z2, int z3, int shift) {
   return s >= 0 ? (s >> shift) : -((-s) >> shift);
 }
 
+// The same step where |z2|, |z3| < 2^31 and it fits 32 bits, without 64-bit
+// arithmetic: with h = floor(s / 2) and r the bit lost, trunc(s / 2^shift) is
+// h >> (shift - 1) for s >= 0 and floor((s + 2^shift - 1) / 2^shift) for s < 0.
+__device__ __forceinline__ int gdp_step32(int z2, int z3, int shift) {
+  const int r = (z2 ^ z3) & 1, h = (z2 >> 1) + (z3 >> 1) + (z2 & z3 & 1);
+  return (h + (h < 0 ? (1 << (shift - 1)) - 1 + r : 0)) >> (shift - 1);
+}
+
 // Top-3 of two partial top-3 sets (each ascending): the 3 smallest of their union.
 __device__ __forceinline__ void top3_merge(int a1, int b1, int c1, int& a, int& b, int& c) {
   top3_insert_minmax(a1, a, b, c);
   top3_insert_minmax(b1, a, b, c);
   top3_insert_minmax(c1, a, b, c);
+}
+
+// Selection by merging, fewer operations and a shorter chain than insertion:
+// the three smallest of four values (9), and of two ascending triples (7).
+__device__ __forceinline__ void top3_of4(int z0, int z1, int z2, int z3, int& a, int& b, int& c) {
+  const int l1 = min(z0, z1), h1 = max(z0, z1), l2 = min(z2, z3), h2 = max(z2, z3);
+  const int t = max(l1, l2), u = min(h1, h2);
+  a = min(l1, l2);
+  b = min(t, u);
+  c = max(t, u);
+}
+// With m the larger of the firsts and q the smaller of the seconds: m < q makes
+// q the third; else it is m or the third of the triple with the smaller first
+// (the other's third is not below m).
+__device__ __forceinline__ void top3_join(int a1, int b1, int c1, int& a, int& b, int& c) {
+  const int m = max(a, a1), q = min(b, b1);
+  a = min(a, a1);
+  c = min(max(m, q), min(c, c1));
+  b = min(m, q);
 }
 
 // Load that bypasses L1: lambda is rewritten by other SMs between sweeps.

@@ -29,16 +29,11 @@ struct GdpCtl {
   long long slot_b2[3];        // per-sweep bound2 accumulators (ring of 3)
   unsigned long long slot_ch[3];  // per-sweep changed counts (ring of 3)
   long long sweeps;            // sweeps completed
-  long long pad1;
-  // ring of 4 per-sweep slots used by the tiled kernel (stop test lagged by two sweeps)
-  long long q_b2[4];
-  unsigned long long q_ch[4];
-  int q_ovf[4];
 };
 
 constexpr int kGdpOverflow = 1;
 constexpr int kGdpTimeout = 2;
-constexpr int kGdpOddOverflow = 4;  // two-sweep kernel: the second sweep of a round overflowed
+constexpr int kGdpNoFit = 4;        // shared-memory tiles: some tile does not fit
 
 // Validation result written by the create-time check kernel.
 struct CheckCtl {
@@ -219,64 +214,23 @@ cudaError_t launch_gdp_classes(const int32_t* rp, const int2* ec, const int32_t*
                                unsigned long long* trace_ch, int64_t trace_cap, long long budget,
                                int num_sms, cudaStream_t st);
 
-// ---- shared-memory tiled GDP (gdp_tiled.cu) ----------------------------------------
-// Spatial renumbering and per-CTA plan; see gdp_tiled.cu.
+// ---- spatial renumbering and the CSR in that order (plan.cu) --------------------
 struct GdpPlan {
   int32_t n = 0;
   int64_t nnz = 0;               // entries of the internal CSR
   int64_t version = 0;           // bumped whenever the internal CSR is rebuilt
-  bool valid = false;            // the tiled kernel can run this CSR
-  int32_t B = 0, threads = 0;    // CTAs (one node range each) and threads per CTA
-  int32_t maxO = 0, maxS = 0, maxH = 0;  // max own nodes, sliced entries, halo per CTA
-  int32_t halo_total = 0;
-  size_t smem = 0;               // dynamic shared memory per CTA
   int32_t* perm = nullptr;       // internal -> caller node
   int32_t* inv = nullptr;        // caller -> internal node
   int32_t* irp = nullptr;        // internal CSR offsets
   int2* iec = nullptr;           // internal {col, cost}
-  int2* lec = nullptr;           // sliced {local index, cost * 2^F} per CTA
-  int32_t* scount = nullptr;     // [B+1] sliced entries per CTA
-  int32_t* soff = nullptr;       // [B+1] their offsets
-  int32_t* order = nullptr;      // [n] node of each slot (degree-descending per CTA)
-  int2* slc = nullptr;           // [n] per-CTA slice table {offset, depth}
-  int32_t* part = nullptr;       // [B+1] node range of each CTA
-  int32_t* hoff = nullptr;       // [B+1] halo offsets
-  int32_t* hcount = nullptr;
-  int32_t* halo = nullptr;       // halo node ids (internal)
-  int32_t* tmp = nullptr;
-  int32_t* stats = nullptr;
-  int32_t* ilam[3] = {nullptr, nullptr, nullptr};  // lambda in internal order (ring of 3)
+  int32_t* ilam[2] = {nullptr, nullptr};  // lambda in internal order
   uint64_t* keys = nullptr;
   uint64_t* keys2 = nullptr;
   int32_t* idx = nullptr;
   void* sort_tmp = nullptr;
   int32_t* scan_tmp = nullptr;
-  int64_t irp_cap = 0, iec_cap = 0, lec_cap = 0, tmp_cap = 0, halo_cap = 0, scan_cap = 0;
-  int64_t order_cap = 0, slc_cap = 0;
-  int64_t cta_cap = 0;           // entries of part, hcount, scount, soff, hoff
-  int64_t ilam_cap[3] = {0, 0, 0};
-  // two-sweep form (gdp_tiled2.cu): H1 rows and the H2 ring per CTA
-  bool valid2 = false;
-  int32_t maxS2 = 0, maxSl2 = 0, maxL2 = 0, maxHH2 = 0;  // max sliced entries, slices, lambda slots, halo
-  size_t smem2 = 0;
-  int32_t* h2count = nullptr;    // [B+1] H2 per CTA
-  int32_t* hhcount = nullptr;    // [B+1] H1 + H2 per CTA
-  int32_t* s2count = nullptr;    // [B+1] sliced entries (own + H1 rows)
-  int32_t* nslc = nullptr;       // [B+1] slices (own + H1)
-  int32_t* hoff2 = nullptr;      // [B+1] offsets of the H1|H2 lists
-  int32_t* soff2 = nullptr;      // [B+1] offsets of the sliced entries
-  int32_t* sloff2 = nullptr;     // [B+1] slice offsets
-  int32_t* halo2 = nullptr;      // H1 then H2 node ids per CTA
-  int32_t* order2 = nullptr;     // local node of each slot
-  int2* slc2 = nullptr;          // {offset, depth} per slice
-  int2* lec2 = nullptr;          // sliced {local index, cost * 2^F}
-  uint32_t* lec2p = nullptr;     // the same packed as cost << 13 | local index (packed2)
-  int64_t lec2p_cap = 0;
-  bool packed2 = false;          // the kernel reads lec2p (the 8-byte tiles do not fit)
-  int32_t frac_bits2 = 8;        // F the entries were built with
-  int32_t* tmp2 = nullptr;       // H2 lists during the build
-  int32_t* stats2 = nullptr;
-  int64_t cap2_small = 0, halo2_cap = 0, order2_cap = 0, slc2_cap = 0, lec2_cap = 0, tmp2_cap = 0;
+  int64_t irp_cap = 0, iec_cap = 0, scan_cap = 0;
+  int64_t ilam_cap[2] = {0, 0};
 };
 cudaError_t sort_pairs_u64(void* temp, size_t& temp_bytes, const uint64_t* keys_in,
                            uint64_t* keys_out, const int32_t* vals_in, int32_t* vals_out,
@@ -284,31 +238,100 @@ cudaError_t sort_pairs_u64(void* temp, size_t& temp_bytes, const uint64_t* keys_
 // Morton renumbering inside each segment [seg_off[s], seg_off[s+1]) (segments stay contiguous)
 cudaError_t plan_renumber(const int2* xy, int32_t n, const std::vector<int32_t>& seg_off, GdpPlan& p,
                           cudaStream_t st);
-// internal CSR (always) and, if `tiles`, the per-CTA tiles of the shared-memory kernel
-cudaError_t plan_build(const int32_t* rp, const int2* ec, int32_t n, int64_t nnz, int num_sms,
-                       bool tiles, int32_t F, int32_t ctas_per_sm, GdpPlan& p, cudaStream_t st);
-// the per-CTA tiles alone, for the internal CSR plan_build made last
-cudaError_t plan_build_tiles(int num_sms, int32_t F, int32_t ctas_per_sm, GdpPlan& p, cudaStream_t st);
+// the CSR in the renumbered order
+cudaError_t plan_build(const int32_t* rp, const int2* ec, int32_t n, int64_t nnz, GdpPlan& p, cudaStream_t st);
 // dst[i] = src[perm[i]]  /  dst[perm[i]] = src[i]
 cudaError_t gather_perm(const int32_t* src, const int32_t* perm, int32_t n, int32_t* dst,
                         cudaStream_t st);
 cudaError_t scatter_perm(const int32_t* src, const int32_t* perm, int32_t n, int32_t* dst,
                          cudaStream_t st);
 void plan_free(GdpPlan& p);
-// gathers lam_in (caller order) into ilam[0], then one cooperative tiled launch
-cudaError_t launch_gdp_tiled(GdpPlan& p, const int32_t* lam_in, int32_t shift, int64_t max_sweeps,
-                             GdpCtl* ctl, long long* trace_b2, unsigned long long* trace_ch,
-                             int64_t trace_cap, long long budget, cudaStream_t st);
-// two-sweep form on top of a valid one-sweep plan of 1024-thread CTAs (valid2 false if it does not fit)
-cudaError_t plan_build2(GdpPlan& p, int32_t F, cudaStream_t st);
-void plan2_free(GdpPlan& p);
-// gathers lam_in into ilam[0], one cooperative launch; the result is in ilam[ctl->pad1].
-// bint: degree requirements in internal order (NULL: b_v = 2), bmax their largest
-cudaError_t launch_gdp_tiled2(GdpPlan& p, const int32_t* lam_in, int32_t shift, int64_t max_sweeps, GdpCtl* ctl,
-                              long long* trace_b2, unsigned long long* trace_ch, int64_t trace_cap,
-                              long long budget, const int32_t* bint, int32_t bmax, cudaStream_t st);
-// lam_out (caller order) = ilam[which]
-cudaError_t plan_scatter_lambda(const GdpPlan& p, int which, int32_t* lam_out, cudaStream_t st);
+// ---- GDP on shared-memory tiles (gdp_ring.cu) --------------------------------------
+constexpr int kRingMax = 6;          // rings around a tile: sweeps per exchange
+constexpr int kRingLocals = 8192;    // nodes a tile knows (own, rings, two padding slots)
+constexpr int kRingHalo = 4096;      // of them in rings
+constexpr int kRingSlots = 8192;     // rows it computes, in whole slices
+constexpr int kRingSlices = kRingSlots / 32;
+constexpr int kRingSweeps = 1 << 30;  // of one launch (a longer phase takes several)
+constexpr int kRingRing = 16;        // rounds whose stop-test slots are live
+constexpr int kRingBadSize = 1;      // RingStats::bad: some tile is too large
+struct RingTile {
+  int32_t seg, j, count;  // the j-th of the count tiles of an instance (segment)
+};
+struct RingHdr {
+  int32_t lo, own;        // first own node (internal), own nodes
+  int32_t halo;           // nodes of all rings
+  int32_t seg, count, first;
+  int32_t word0;          // its first word in the exchange
+  int32_t nsl, nent;      // slices, sliced entries
+  int32_t sec_end[kRingMax];  // slices of own rows, and of those of rings 1 .. k
+};
+struct RingStats {        // over all tiles of a plan
+  int32_t bytes8, bytes4;  // shared memory of the largest with 8- and 4-byte entries there,
+  int32_t bytes_reg;       // and with entries in registers
+  int32_t slices, maxcost;
+  int32_t bad;
+};
+struct RingSeg {          // per instance, zeroed per phase
+  unsigned long long slot[kRingRing];
+  unsigned int ovf[kRingRing];
+  long long sweeps;       // the result
+  int32_t fixed_point, overflow;
+};
+struct RingArgs {
+  const RingHdr* hdr;
+  const int32_t* halo;
+  const uint16_t* order;
+  const uint32_t* slc;
+  const int2* ent;
+  const RingStats* stats;
+  const int32_t* pos;      // by internal node: its word
+  RingSeg* seg;
+  unsigned* words[2];
+  int* status;
+  const int32_t* lam_in;   // caller order; lam_out must be another array
+  int32_t* lam_out;
+  const int32_t* perm;
+  const int32_t* bint;     // b_v in internal order (NULL: 2)
+  long long* trace_b2;     // zeroed
+  unsigned long long* trace_ch;
+  long long trace_cap, budget;
+  int32_t max_sweeps;      // at most kRingSweeps
+  int32_t first_tile, K, F, shift, ecap, smem;
+};
+struct RingPlan {
+  int64_t version = -1;    // GdpPlan::version it was built from
+  int32_t tiles = 0, K = 0, F = 0, ecap = 0;
+  RingHdr* hdr = nullptr;
+  int32_t* halo = nullptr;
+  uint16_t* order = nullptr;
+  uint32_t* slc = nullptr;
+  int2* ent = nullptr;
+  RingStats* stats = nullptr;
+  RingSeg* seg = nullptr;
+  int32_t* pos = nullptr;
+  unsigned* words = nullptr;  // the exchange: two buffers of words_n
+  int64_t words_n = 0;
+  int* status = nullptr;
+  int64_t hdr_cap = 0, halo_cap = 0, order_cap = 0, slc_cap = 0, ent_cap = 0, seg_cap = 0, words_cap = 0, pos_cap = 0;
+};
+void ring_free(RingPlan& p);
+// the tiles of K rings over the internal CSR: `tiles` equal shares of the one
+// segment (list NULL), or those of the device list; seg_off on the device
+cudaError_t ring_build(const GdpPlan& g, const int32_t* seg_off, const RingTile* list, int32_t tiles, int32_t K,
+                       int32_t F, int64_t entries_per_tile, RingPlan& p, cudaStream_t st);
+int32_t ring_smem(bool half);  // dynamic shared memory of a CTA
+// per phase: cleared segment records and status
+cudaError_t ring_start(RingPlan& p, int32_t n, int32_t nseg, cudaStream_t st);
+// Where the rows' entries are kept: registers (1 or 2 rows a thread, up to 1,984
+// rows a tile), shared memory, or shared memory with two CTAs per SM.
+enum RingForm { kRingHalf = -1, kRingSmem = 0, kRingReg1 = 1, kRingReg2 = 2 };
+int ring_reg_rows(const RingStats& st);  // rows a thread of the register form (0: does not fit)
+// one cooperative launch over tiles [first_tile, first_tile + tiles): whole instances
+cudaError_t launch_gdp_ring(const GdpPlan& g, RingPlan& p, int32_t first_tile, int32_t tiles, const int32_t* lam_in,
+                            int32_t* lam_out, int32_t shift, int32_t max_sweeps, long long* trace_b2,
+                            unsigned long long* trace_ch, int64_t trace_cap, long long budget, const int32_t* bint,
+                            int32_t bmax, RingForm form, cudaStream_t st);
 
 // ---- exact finisher (finisher_prep.cu on the device, finisher.cpp on the host) ---
 // twin[e] for every internal entry; *missing (zeroed by the caller) counts
