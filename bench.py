@@ -692,9 +692,13 @@ def run_batch(args, w, rank, world, local):
     sm_mhz = clk.get("sm_mhz") or peaks.get("sm_max_mhz", 2070.0)
     num_sms = torch.cuda.get_device_properties(local).multi_processor_count
     pr_rate = pairs / (ms_pr * 1e-3) if ms_pr > 0 else 0.0
-    roofline = {"kernel": "gdp_batch_kernel", "bound": "hbm", "achieved": gdp_gbs,
+    tiles = tot.gdp_kernel == 8  # F2M_GDP_KERNEL_BATCH_TILES
+    roofline = {"kernel": "gdp_ring_reg_kernel" if tiles else "gdp_batch_kernel", "bound": "hbm", "achieved": gdp_gbs,
                 "peak": peaks["hbm_gbs"], "unit": "GB/s", "frac": gdp_gbs / peaks["hbm_gbs"],
-                "traffic": load_traffic(args.workload).get("gdp_batch_kernel"),
+                "traffic": None if tiles else load_traffic(args.workload).get("gdp_batch_kernel"),
+                "note": "algorithmic bytes of the sweeps over their time" +
+                        ("; the tiles' rows stay in registers for a phase, so this is an effective rate (DRAM sees "
+                         "the graph once per phase)" if tiles else ""),
                 "peak_source": "MEASURED_PEAKS.json" if not peaks.get("_fallback") else "fallback",
                 "gdp_working_set_mb": float(np.sum(GDP_BYTES_PER_ENTRY * nnzs + GDP_BYTES_PER_NODE * ns)) / 1e6,
                 "pricing_tflops": pr_rate * PRICING_FLOPS_PER_PAIR / 1e12,
@@ -706,7 +710,7 @@ def run_batch(args, w, rank, world, local):
             "config": {"workload": workload_name(w) if not args.instances else
                        workload_name(w) + f" (first {len(ns)} instances)", "instances": int(len(ns)),
                        "sum_n": int(ns.sum()), "kernel_shape": int(tot.batch_shape), "graph": bool(tot.batch_graph),
-                       "gdp_path": "clusters" if args.batch_clusters else "streaming",
+                       "gdp_path": {8: "tiles", 6: "clusters"}.get(int(tot.gdp_kernel), "streaming"),
                        "max_iters": int(params.max_iters),
                        "sum_nnz": int(nnzs.sum()), "l2": "working set larger than L2; flushed before every step",
                        "parallelism": f"replicas x{world}"},

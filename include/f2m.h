@@ -86,10 +86,11 @@ typedef struct {
   int32_t gdp_lanes;            /* lanes per node in the tiled GDP kernel: 1 (one thread per node); 0 = auto */
   int32_t gdp_ctas_per_sm;      /* tiled GDP CTAs per SM: 1 (x1024 threads), 2 (x512, one sweep
                                    per exchange); 0 = auto */
-  int32_t batch_shape;          /* batched GDP kernel shape (threads, copy stages, CTAs per SM):
-                                   -1 = picked by the autotuner (default), 0..4 = a fixed one */
-  int32_t batch_graph;          /* 1 = replay each batched GDP phase from a captured CUDA graph
-                                   (default), 0 = launch directly; same results */
+  int32_t batch_shape;          /* batched GDP: -1 = on-chip tiles, or where they do not fit the
+                                   streaming kernel's shape (threads, copy stages, CTAs per SM)
+                                   picked by the autotuner (default), 0..11 = a fixed shape of it */
+  int32_t batch_graph;          /* 1 = replay the streaming kernel's phases from a captured CUDA
+                                   graph (default), 0 = launch directly; same results */
 } f2m_params;
 
 /* f2m_params.flags: run GDP with the streaming kernel (CSR read from global
@@ -120,9 +121,9 @@ typedef struct {
 #define F2M_FLAG_CLASS_SWEEPS 4u
 
 /* f2m_params.flags (batches, with batch_shape -1): run batched GDP phases on
- * thread-block clusters instead of the default streaming batch kernels (the
- * union CSR streamed from HBM every sweep, one device-wide barrier per sweep):
- * every instance gets a cluster of 1-16 CTAs that holds its rows and lambda in
+ * thread-block clusters instead of the default on-chip tiles (whole instances in
+ * waves; where they do not fit, the streaming kernels: the union CSR streamed
+ * from HBM every sweep, one device-wide barrier per sweep): every instance gets a cluster of 1-16 CTAs that holds its rows and lambda in
  * shared memory, with the hardware cluster barrier per sweep and neighbours'
  * lambda read through distributed shared memory.  A batch with an instance too
  * large for 16 CTAs (2048 nodes, 24,000 entries each) uses the streaming
@@ -197,6 +198,7 @@ typedef struct {
 #define F2M_GDP_KERNEL_BATCH 5         /* batched, union CSR streamed */
 #define F2M_GDP_KERNEL_BATCH_CLUSTERS 6  /* batched, one thread-block cluster per instance */
 #define F2M_GDP_KERNEL_CUTS 7          /* node and subtour-cut duals, streaming */
+#define F2M_GDP_KERNEL_BATCH_TILES 8   /* batched, on-chip tiles, whole instances in waves */
 
 /* Fills *p with the defaults above.  p must not be NULL. */
 void f2m_default_params(f2m_params* p);
@@ -412,8 +414,8 @@ f2m_status f2m_solve_subtour(f2m_ctx* ctx, int32_t rounds, f2m_subtour_info* inf
 typedef struct f2m_batch f2m_batch;  /* opaque, library-owned */
 
 /* Creates a batch of `count` instances, solved together: every device step of
- * f2m_solve_batch (one persistent GDP launch per phase, with instances that
- * reached their fixed point frozen, for max_iters sweeps at most; one pricing
+ * f2m_solve_batch (the GDP phases, each instance for max_iters sweeps at most or
+ * to its fixed point; one pricing
  * scan over the pair tiles of the
  * instances that need one; one merge; one extraction; one finisher call) covers
  * all instances, and each instance's lambda, x and bound are those of its own

@@ -269,7 +269,7 @@ struct RingHdr {
 struct RingStats {        // over all tiles of a plan
   int32_t bytes8, bytes4;  // shared memory of the largest with 8- and 4-byte entries there,
   int32_t bytes_reg;       // and with entries in registers
-  int32_t slices, maxcost;
+  int32_t slices, locals, maxcost;
   int32_t bad;
 };
 struct RingSeg {          // per instance, zeroed per phase
@@ -317,15 +317,16 @@ struct RingPlan {
 };
 void ring_free(RingPlan& p);
 // the tiles of K rings over the internal CSR: `tiles` equal shares of the one
-// segment (list NULL), or those of the device list; seg_off on the device
+// segment's nodes (list NULL), or those of the device list; seg_off on the device
 cudaError_t ring_build(const GdpPlan& g, const int32_t* seg_off, const RingTile* list, int32_t tiles, int32_t K,
                        int32_t F, int64_t entries_per_tile, RingPlan& p, cudaStream_t st);
 int32_t ring_smem(bool half);  // dynamic shared memory of a CTA
 // per phase: cleared segment records and status
 cudaError_t ring_start(RingPlan& p, int32_t n, int32_t nseg, cudaStream_t st);
 // Where the rows' entries are kept: registers (1 or 2 rows a thread, up to 1,984
-// rows a tile), shared memory, or shared memory with two CTAs per SM.
-enum RingForm { kRingHalf = -1, kRingSmem = 0, kRingReg1 = 1, kRingReg2 = 2 };
+// rows a tile), registers with two CTAs per SM (up to 960 rows a tile, b_v = 2),
+// shared memory, or shared memory with two CTAs per SM.
+enum RingForm { kRingHalf = -1, kRingSmem = 0, kRingReg1 = 1, kRingReg2 = 2, kRingPair = 3 };
 int ring_reg_rows(const RingStats& st);  // rows a thread of the register form (0: does not fit)
 // one cooperative launch over tiles [first_tile, first_tile + tiles): whole instances
 cudaError_t launch_gdp_ring(const GdpPlan& g, RingPlan& p, int32_t first_tile, int32_t tiles, const int32_t* lam_in,

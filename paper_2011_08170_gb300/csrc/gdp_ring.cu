@@ -57,11 +57,7 @@ namespace f2m {
 namespace {
 
 constexpr int kPlanThreads = 1024;
-constexpr int kRegThreads = 1024;           // register form: threads a tile,
-constexpr int kRegWarps = kRegThreads / 32 - 1;
-constexpr int kRegRows = 2;                 // most rows a thread in registers,
-constexpr int kRegEntries = 16;             // entries of a row in registers
-constexpr uint32_t kRegPadCost = (1u << 17) - 1;  // cost of a packed padding entry
+constexpr int kRegEntries = 16;             // register form: entries of a row in registers
 constexpr int kRingLamBytes = 4 * kRingLocals;    // between its two lambda arrays
 constexpr int kHash = 2 * kRingHalo;        // slots of the plan's table of outside nodes
 constexpr int kShallow = 12;                // entries of most rows (k = 10 graphs: three in four)
@@ -71,22 +67,6 @@ constexpr uint32_t kPackPadCost = (1u << (32 - kPackIdx)) - 1;  // cost of a pac
 // is about 2^30 - lambda_v, above every real one (as the 8-byte padding's)
 constexpr int kPackPadLam = -(1 << 30) + (1 << 27);
 static_assert(kRingLocals <= (1 << kPackIdx), "local indices fit the packed form");
-
-// first row in [a, b) whose offset is at or after target (irp nondecreasing);
-// the whole warp searches, 32 probes a step
-__device__ int warp_lower_bound(const int32_t* __restrict__ irp, int a, int b, long long target) {
-  const int lane = threadIdx.x & 31;
-  while (a < b) {
-    const int step = (b - a + 31) / 32, p = min(a + lane * step, b);
-    const bool below = p < b && irp[p] < target;
-    const int k = __popc(__ballot_sync(0xffffffffu, below));  // probes below the target come first
-    if (k == 0) return a;
-    const int lo = a + (k - 1) * step + 1;
-    b = min(a + k * step, b);
-    a = lo;
-  }
-  return a;
-}
 
 constexpr int kHashBits = 13;
 static_assert(kHash == 1 << kHashBits, "table size");
@@ -101,7 +81,7 @@ __device__ __forceinline__ int hash_find(const int* keys, const uint16_t* vals, 
 
 }  // namespace
 
-// One CTA per tile: its node range (an equal share of its instance's entries),
+// One CTA per tile: its node range (an equal share of its instance's nodes),
 // the rings (each sorted by node), the slots, the slice table and the sliced
 // entries.  A section (own rows, R1, ..., R(K-1)) starts a slice; its rows with
 // more than 12 entries come first, by falling degree, then the others in node
@@ -122,19 +102,13 @@ ring_plan_kernel(const int32_t* __restrict__ irp, const int2* __restrict__ iec, 
   uint16_t* deg = at_key + kRingHalo;                               // [kRingLocals] per row (own, then ring)
   uint16_t* ord = deg + kRingLocals;                                // [kRingSlots] row of a slot
   uint16_t* inv = ord + kRingSlots;                                 // [kRingLocals] slot of an own node
-  __shared__ int s_lo, s_hi, s_cnt, s_bad, s_hist[64], s_maxcost, s_tail;
+  __shared__ int s_cnt, s_bad, s_hist[64], s_maxcost, s_tail;
   __shared__ int s_sl[kRingSlices + 1];
   __shared__ int s_warp[33];
   const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   RingTile tl{0, b, tiles};
   if (list) tl = list[b];
-  const int n0 = seg_off[tl.seg], n1 = seg_off[tl.seg + 1];
-  const long long e0 = irp[n0], ne = irp[n1] - e0;
-  if (warp < 2) {
-    const int j = tl.j + warp;
-    const int v = j == 0 ? n0 : (j == tl.count ? n1 : warp_lower_bound(irp, n0, n1, e0 + ne * j / tl.count));
-    if (lane == 0) (warp ? s_hi : s_lo) = v;
-  }
+  const int n0 = seg_off[tl.seg], ns = seg_off[tl.seg + 1] - n0;
   for (int i = tid; i < kHash; i += kPlanThreads) keys[i] = -1;
   if (tid == 0) {
     s_cnt = 0;
@@ -143,7 +117,8 @@ ring_plan_kernel(const int32_t* __restrict__ irp, const int2* __restrict__ iec, 
     s_tail = 0;
   }
   __syncthreads();
-  const int lo = s_lo, hi = s_hi, own = hi - lo, ownp = (own + 31) & ~31;
+  const int lo = n0 + (int)((long long)ns * tl.j / tl.count), hi = n0 + (int)((long long)ns * (tl.j + 1) / tl.count);
+  const int own = hi - lo, ownp = (own + 31) & ~31;
   // ring nodes that fit beside own slots and the two padding slots
   const int room = min(kRingHalo, kRingLocals - 2 - ownp);
   RingHdr h{};
@@ -331,6 +306,7 @@ ring_plan_kernel(const int32_t* __restrict__ irp, const int2* __restrict__ iec, 
     atomicMax(&stats->bytes8, 8 * nent + rest);
     atomicMax(&stats->bytes4, 4 * nent + rest);
     atomicMax(&stats->slices, nsl);
+    atomicMax(&stats->locals, ownp + HH + 2);
     atomicMax(&stats->maxcost, s_maxcost);
     atomicMax(&stats->bytes_reg, 2 * kRingLamBytes + 4 * (HH + nsl) + 8 * s_tail + 64);
     if (bad) atomicOr(&stats->bad, bad);
@@ -556,15 +532,25 @@ struct SmemRows {
   }
 };
 
+// address bits of a packed entry in a register, by row warps; cost of a padding entry
+__host__ __device__ constexpr int reg_address_bits(int nw) { return nw < 16 ? 13 : 14; }
+__host__ __device__ constexpr int reg_pad_cost(int bits) { return (int)((1u << (32 - bits)) - 1u); }
+__host__ __device__ __forceinline__ bool reg_packs(const RingStats& st, int nw) {
+  const int bits = reg_address_bits(nw);
+  return st.locals <= 1 << (bits - 2) && st.maxcost < reg_pad_cost(bits);
+}
+
 // Rows whose entries stay in registers: R rows a thread, at most kRegEntries
-// entries each (deeper slices keep the rest in shared memory).  R = 1: an entry is the byte address of its lambda in the
-// tile's array and its cost; R = 2: both in one register, cost << 15 | address
-// (costs below 2^17 - 1).  The two lambda arrays lie a constant apart, so that a
-// gather is one load with an immediate offset (the two parities are compiled
-// separately).
+// entries each (deeper slices keep the rest in shared memory).  R = 1: an entry
+// is the byte address of its lambda in the tile's array and its cost; R = 2:
+// both in one register, cost << AB | address: 13 bits of address (2,048 nodes a
+// tile, costs below 2^19 - 1) with two CTAs per SM, 14 with one.  The two
+// lambda arrays lie a constant apart, so that a gather is one load with an
+// immediate offset (the two parities are compiled separately).
 template <int MODE, int R, int NW>
 struct RegRows {
   static constexpr bool PACKED = R > 1;
+  static constexpr int AB = reg_address_bits(NW);
   static constexpr int D = kRegEntries;
   static constexpr int NB = MODE == 1 ? 5 : 8;
   unsigned char* sm;
@@ -636,8 +622,8 @@ struct RegRows {
         if (k < depth) q = *reinterpret_cast<const int4*>(ent + at + k * 32);
         if constexpr (PACKED) {
           auto pack = [&](int at_, int c) {
-            return c == (1 << 30) ? kRegPadCost << 15 | (uint32_t)(zero_slot + 1) << 2
-                                  : (uint32_t)(c >> F) << 15 | (uint32_t)at_ << 2;
+            return c == (1 << 30) ? (uint32_t)reg_pad_cost(AB) << AB | (uint32_t)(zero_slot + 1) << 2
+                                  : (uint32_t)(c >> F) << AB | (uint32_t)at_ << 2;
           };
           ea[r][k] = pack(q.x, q.y);
           ea[r][k + 1] = pack(q.z, q.w);
@@ -655,8 +641,8 @@ struct RegRows {
   __device__ __forceinline__ int z_of(uint32_t a, int c, int lam_v) const {
     if constexpr (PACKED) {
       asm volatile("" : "+r"(a));  // keeps the unpacked form from being held in registers across sweeps
-      c = (int)(a >> 15) << F;
-      a &= 0x7FFCu;
+      c = (int)(a >> AB) << F;
+      a &= (1u << AB) - 1u;
     }
     return c - lam_v - *reinterpret_cast<const int*>(sm + PAR * kRingLamBytes + a);  // Eq. 9
   }
@@ -906,17 +892,18 @@ gdp_ring_smem_kernel(const __grid_constant__ RingArgs A) {
     ring_run<SmemRows<MODE, BOUND, true, T / 32 - 1>, T>(A, h, smem);
 }
 
-template <int MODE, int R>
-__global__ void __launch_bounds__(kRegThreads, 1)
+template <int MODE, int R, int T>
+__global__ void __launch_bounds__(T, 1024 / T)
 gdp_ring_reg_kernel(const __grid_constant__ RingArgs A) {
   extern __shared__ __align__(16) unsigned char smem[];
+  constexpr int NW = T / 32 - 1;
   const RingStats st = *A.stats;
-  if (st.bad || st.bytes_reg > A.smem || st.slices > R * kRegWarps || (R > 1 && (uint32_t)st.maxcost >= kRegPadCost)) {
+  if (st.bad || st.bytes_reg > A.smem || st.slices > R * NW || (R > 1 && !reg_packs(st, NW))) {
     if (threadIdx.x == 0) atomicOr(A.status, kGdpNoFit);
     return;
   }
   const RingHdr h = A.hdr[A.first_tile + blockIdx.x];
-  ring_run<RegRows<MODE, R, kRegWarps>, kRegThreads>(A, h, smem);
+  ring_run<RegRows<MODE, R, NW>, T>(A, h, smem);
 }
 
 // ---- host side -------------------------------------------------------------------------
@@ -947,9 +934,10 @@ void ring_free(RingPlan& p) {
 
 cudaError_t ring_build(const GdpPlan& g, const int32_t* seg_off, const RingTile* list, int32_t tiles, int32_t K,
                        int32_t F, int64_t entries_per_tile, RingPlan& p, cudaStream_t st) {
-  // room for a tile's sliced entries: its own and its rings', at most what the
-  // 4-byte form could hold in shared memory
-  const int64_t ecap = (entries_per_tile * 2 + 16384 < 49152 ? entries_per_tile * 2 + 16384 : 49152) / 64 * 64;
+  // room for a tile's sliced entries: its own and its inner rings', at most what
+  // the 4-byte form could hold in shared memory
+  const int64_t want = K > 1 ? entries_per_tile * 2 + 16384 : entries_per_tile * 3 / 2 + 4096;
+  const int64_t ecap = (want < 49152 ? want : 49152) / 64 * 64;
   p.version = -1;
   RCK(grow(&p.hdr, &p.hdr_cap, tiles));
   RCK(grow(&p.halo, &p.halo_cap, (int64_t)tiles * kRingHalo));
@@ -991,15 +979,15 @@ static const void* ring_kernel_of(bool bound) {
 
 template <int R>
 static const void* ring_reg_kernel_of(int mode) {
-  return mode == 0   ? (const void*)gdp_ring_reg_kernel<0, R>
-         : mode == 1 ? (const void*)gdp_ring_reg_kernel<1, R>
-                     : (const void*)gdp_ring_reg_kernel<2, R>;
+  return mode == 0   ? (const void*)gdp_ring_reg_kernel<0, R, 1024>
+         : mode == 1 ? (const void*)gdp_ring_reg_kernel<1, R, 1024>
+                     : (const void*)gdp_ring_reg_kernel<2, R, 1024>;
 }
 
 int ring_reg_rows(const RingStats& st) {
   if (st.bad || st.bytes_reg > ring_smem(false)) return 0;
-  if (st.slices <= kRegWarps) return 1;
-  return st.slices <= 2 * kRegWarps && (uint32_t)st.maxcost < kRegPadCost ? 2 : 0;
+  if (st.slices <= 31) return 1;
+  return st.slices <= 62 && reg_packs(st, 31) ? 2 : 0;
 }
 
 int32_t ring_smem(bool half) {
@@ -1016,12 +1004,13 @@ cudaError_t launch_gdp_ring(const GdpPlan& g, RingPlan& p, int32_t first_tile, i
                             int32_t* lam_out, int32_t shift, int32_t max_sweeps, long long* trace_b2,
                             unsigned long long* trace_ch, int64_t trace_cap, long long budget, const int32_t* bint,
                             int32_t bmax, RingForm form, cudaStream_t st) {
-  const bool bound = trace_cap > 0, half = form == kRingHalf, reg = form > 0;
+  const bool bound = trace_cap > 0, half = form == kRingHalf || form == kRingPair, reg = form > 0;
   const int mode = !bint ? 0 : (bmax < 5 ? 1 : (bmax < 8 ? 2 : 3));
-  if (reg && (bound || mode > 2)) return cudaErrorInvalidValue;
-  const int T = reg ? kRegThreads : (half || mode >= 2 ? 512 : 1024);
+  if (reg && (bound || mode > (form == kRingPair ? 0 : 2))) return cudaErrorInvalidValue;
+  const int T = reg ? (half ? 512 : 1024) : (half || mode >= 2 ? 512 : 1024);
   const void* kern = form == kRingReg1   ? ring_reg_kernel_of<1>(mode)
                      : form == kRingReg2 ? ring_reg_kernel_of<2>(mode)
+                     : form == kRingPair ? (const void*)gdp_ring_reg_kernel<0, 2, 512>
                      : half && mode == 0 ? ring_kernel_of<0, 512>(bound)
                      : mode == 0       ? ring_kernel_of<0, 1024>(bound)
                      : mode == 1       ? (half ? ring_kernel_of<1, 512>(bound) : ring_kernel_of<1, 1024>(bound))
