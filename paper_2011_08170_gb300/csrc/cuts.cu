@@ -27,18 +27,31 @@
 // form the cut set.  Cuts of one layer are disjoint.  Separation makes one
 // layer from the connected components of the support of x.
 //
-// Device layout (caller node order, like the streaming GDP kernel):
-//   comp [L][n] int32 labels; mu [2][M] int32 (Jacobi double buffer);
-//   mask [nnz] uint8 (bit l: the entry's two ends differ in layer l's label);
-//   cut lists: cut_ptr [M+1], items {row u, entry e} for every directed entry
-//   whose row lies in the cut and whose column does not (each crossing edge
-//   once per cut).
-// Kernel: one persistent cooperative launch per phase.  G = 4 lanes per node
-// stream its row (cut terms only on entries whose mask is set), then one warp
-// per cut streams its list (a whole block for a cut with 128 or more entries,
-// its warps' top-3s merged in shared memory); both from the same input, one
-// device-wide barrier per sweep.  z is computed in 64 bits (several duals per
-// edge).
+// Device layout.  Caller order: comp [L][n] int32 labels, mask [nnz] uint8 (bit
+// l: the entry's two ends differ in layer l's label) for the bound, rule (7) and
+// pricing.  Renumbered order, for the GDP kernel: cid [L][n] the cut that holds
+// a node (or -1), the mask again, cut lists cut_ptr [M+1] / items ({entry, row} of
+// the entries whose row lies in the cut and whose column does not: each crossing
+// edge once per cut); mu [2][M] (Jacobi double buffer).
+//
+// Kernel: one persistent cooperative launch per phase, one block per SM, one
+// device-wide barrier a sweep.  A block takes an equal share of the rows (4 lanes
+// each) and the cuts whose lists begin in its share of all lists (a warp each, the
+// whole block for a list above 1,024 entries), and computes z for both from
+// tables it builds once per phase in shared memory: its entries, and the distinct
+// nodes and cuts that they read (one bit each, the rank of a bit is its place),
+// whose lambda and mu it fetches once a sweep.  A block whose tables do not fit
+// reads global memory through L1 instead.
+//
+// Bound, at 20,000 points with 10 neighbours and two layers (sweep of 7.7 us):
+// issue and shared-memory latency of the 57 row groups and cuts of a block (4 us),
+// the fetch of some 1,200 values (1 us), the barrier and the slack of the fullest
+// block (2.5 us).  With one gather per entry, end and crossed cut from L2 (two
+// million a sweep, all past L1) the same sweep took 19 to 24 us; through L1 with
+// no tables 8 to 11 us.  Per sweep before and now with one layer: 3,000 points 16.6
+// and 5.2 us, 40,000 points 30 and 12, 100,000 points (no tables) 41 and 32.  z is kept in 32 bits in a sweep whose values allow it
+// (checked with the fetch), else in 64: the 64-bit compares had been half of the
+// instructions.  512 threads: with 1,024 the 64 registers a thread spill (9 us).
 #include <algorithm>
 #include <chrono>
 #include <climits>
@@ -74,13 +87,12 @@ struct CutState {
   int32_t* d_ptr = nullptr;    // [M + 1]
   int32_t* d_scan = nullptr;   // scan scratch
   int64_t ptr_cap = 0;
-  int2* d_items = nullptr;
+  int2* d_items = nullptr;     // {entry, row}, renumbered order
   int64_t item_cap = 0;
-  int64_t items = 0;
-  int32_t* d_lflag = nullptr;  // [ptr_cap] long-cut flags
-  int32_t* d_lpos = nullptr;   // [ptr_cap] their exclusive scan
-  int32_t* d_long = nullptr;   // [ptr_cap] the cuts a block takes
-  int32_t nlong = 0;
+  int32_t* d_cid = nullptr;    // [L][n] renumbered order
+  int64_t cid_cap = 0;
+  uint8_t* d_imask = nullptr;  // [nnz] mask in the renumbered order
+  int64_t imask_cap = 0;
   int64_t built_version = -1;  // graph version the mask and lists were built for
   int32_t built_L = -1;
   // separation and pricing scratch
@@ -103,8 +115,7 @@ void cut_state_free(CutState* s) {
   dfree(s->d_comp); dfree(s->d_mu[0]); dfree(s->d_mu[1]); dfree(s->d_mask); dfree(s->d_cnt);
   dfree(s->d_ptr); dfree(s->d_scan); dfree(s->d_items); dfree(s->d_lab); dfree(s->d_cross);
   dfree(s->d_flag); dfree(s->d_rank); dfree(s->d_small); dfree(s->d_lamp); dfree(s->d_keep);
-  dfree(s->d_kpos); dfree(s->d_pairs2); dfree(s->d_pscan); dfree(s->d_lflag); dfree(s->d_lpos);
-  dfree(s->d_long);
+  dfree(s->d_kpos); dfree(s->d_pairs2); dfree(s->d_pscan); dfree(s->d_cid); dfree(s->d_imask);
   delete s;
 }
 
@@ -113,7 +124,7 @@ int64_t cut_count(const f2m_ctx* c) { return c->cuts ? c->cuts->M : 0; }
 namespace {
 
 constexpr long long kInfZ = LLONG_MAX / 4;
-constexpr int kLongCut = 128;  // crossing entries from which a block, not a warp, takes a cut
+constexpr int kLongCut = 1024;  // crossing entries above which a block's cut warps take a cut together
 
 __device__ __forceinline__ void top3_ins_ll(long long z, long long& a, long long& b, long long& c) {
   if (z < c) {
@@ -168,41 +179,42 @@ __global__ void cut_mask_kernel(const int32_t* __restrict__ rp, const int2* __re
   }
 }
 
-// per cut: crossing entries whose row lies in the cut (count, or fill at the
-// cursor); a label outside [-1, ncuts) flags the layer as invalid
+// cid[l][i] = the cut of layer l that holds internal node i, or -1
+__global__ void cut_cid_kernel(CutArgs a, const int32_t* __restrict__ perm, int32_t* __restrict__ cid) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < a.n;
+       i += (long long)gridDim.x * blockDim.x)
+    for (int l = 0; l < a.L; ++l) {
+      const int s = a.comp[(long long)l * a.n + perm[i]];
+      cid[(long long)l * a.n + i] = s >= 0 ? a.off[l] + s : -1;
+    }
+}
+
+// per cut: crossing entries whose row lies in the cut (counts, with the entries'
+// masks, or the list filled at the cursors)
 template <bool FILL>
-__global__ void cut_list_kernel(const int32_t* __restrict__ rp, const int2* __restrict__ ec,
-                                const uint8_t* __restrict__ mask, CutArgs a, int32_t* cnt,
-                                const int32_t* __restrict__ ptr, int2* items) {
-  for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < a.n;
+__global__ void cut_list_kernel(const int32_t* __restrict__ irp, const int2* __restrict__ iec,
+                                const int32_t* __restrict__ cid, int32_t n, int32_t L, uint8_t* __restrict__ mask,
+                                int32_t* cnt, const int32_t* __restrict__ ptr, int2* items) {
+  for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < n;
        v += (long long)gridDim.x * blockDim.x) {
-    for (int e = rp[v]; e < rp[v + 1]; ++e) {
-      const unsigned m = mask[e];
-      if (!m) continue;
-      for (int l = 0; l < a.L; ++l) {
-        if (!((m >> l) & 1u)) continue;
-        const int s = a.comp[(long long)l * a.n + v];
-        if (s < 0) continue;
-        const int id = a.off[l] + s;
+    for (int e = irp[v]; e < irp[v + 1]; ++e) {
+      unsigned m = 0;
+      if (FILL) {
+        m = mask[e];
+      } else {
+        const int w = iec[e].x;
+        for (int l = 0; l < L; ++l)
+          if (cid[(long long)l * n + v] != cid[(long long)l * n + w]) m |= 1u << l;
+        mask[e] = (uint8_t)m;
+      }
+      for (; m; m &= m - 1) {
+        const int id = cid[(long long)(__ffs(m) - 1) * n + v];
+        if (id < 0) continue;
         const int k = atomicAdd(cnt + id, 1);
-        if (FILL) items[ptr[id] + k] = make_int2((int)v, e);
+        if (FILL) items[ptr[id] + k] = make_int2(e, (int)v);
       }
     }
   }
-}
-
-// 1 for a cut whose list holds at least kLongCut entries
-__global__ void cut_long_flag_kernel(const int32_t* __restrict__ cnt, int32_t M, int32_t* flag) {
-  for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < M;
-       s += (long long)gridDim.x * blockDim.x)
-    flag[s] = cnt[s] >= kLongCut;
-}
-
-__global__ void cut_long_list_kernel(const int32_t* __restrict__ flag, const int32_t* __restrict__ pos,
-                                     int32_t M, int32_t* out) {
-  for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < M;
-       s += (long long)gridDim.x * blockDim.x)
-    if (flag[s]) out[pos[s]] = (int32_t)s;
 }
 
 // labels of layer l in [-1, ncuts): else flag
@@ -222,168 +234,416 @@ __global__ void cut_short_kernel(const int32_t* __restrict__ cnt, int32_t M, int
     if (cnt[s] < 3) atomicMin(flag, (int)s);
 }
 
-template <int G>
-__global__ void __launch_bounds__(512)
-cut_gdp_kernel(const int32_t* __restrict__ rp, const int2* __restrict__ ec, const uint8_t* __restrict__ mask,
-               const __grid_constant__ CutArgs ca, const int32_t* __restrict__ cut_ptr, const int2* __restrict__ items,
-               int32_t M, const int32_t* __restrict__ long_cuts, int32_t nlong,
-               int32_t* lam0, int32_t* lam1, int32_t* mu0, int32_t* mu1, int32_t F, int32_t shift,
-               long long max_sweeps, GdpCtl* ctl, long long* trace_b2, unsigned long long* trace_ch,
-               long long trace_cap, long long budget) {
-  __shared__ long long s_b2[32];
-  __shared__ unsigned s_ch[32];
-  __shared__ int s_ovf[32];
-  __shared__ int s_stop;
-  __shared__ long long s_t3[32 * 3];
-  const int tid = threadIdx.x;
-  const int lane = tid & 31, warp = tid >> 5;
-  const int sub = lane & (G - 1);
-  const unsigned gmask = (G >= 32) ? 0xffffffffu : (((1u << G) - 1u) << (lane & ~(G - 1)));
-  const long long per_block = blockDim.x / G;
-  const long long gid = (long long)blockIdx.x * per_block + tid / G;
-  const long long ngroups = (long long)gridDim.x * per_block;
-  const int nwarps = blockDim.x >> 5;
-  const long long gwarp = (long long)blockIdx.x * nwarps + warp;
-  const long long twarps = (long long)gridDim.x * nwarps;
-  const int n = ca.n;
+struct CutGdp {
+  const int32_t* irp;
+  const int2* iec;
+  const int32_t* perm;
+  const int32_t* cid;
+  const uint8_t* mask;
+  const int32_t* cut_ptr;
+  const int2* items;
+  const int32_t* lam_in;   // caller order
+  int32_t* lam_out;
+  int32_t* lam[2];         // renumbered
+  int32_t* mu[2];
+  GdpCtl* ctl;
+  long long* trace_b2;
+  unsigned long long* trace_ch;
+  long long trace_cap, max_sweeps, budget;
+  int32_t n, L, M, F, shift;
+};
 
-  for (long long t = 0; t < max_sweeps; ++t) {
-    const int32_t* lin = (t & 1) ? lam1 : lam0;
-    int32_t* lout = (t & 1) ? lam0 : lam1;
-    const int32_t* min_ = (t & 1) ? mu1 : mu0;
-    int32_t* mout = (t & 1) ? mu0 : mu1;
+constexpr int kCutThreads = 512;
+constexpr int kCutGroup = 4;        // lanes of a row
+constexpr int kCutSmem = 208 << 10; // a block's tables
+
+template <typename Z>
+__device__ __forceinline__ void cut_top3(Z z, Z& a, Z& b, Z& c) {  // no branches: the lanes of a warp disagree
+  c = min(c, max(b, z));
+  b = min(b, max(a, z));
+  a = min(a, z);
+}
+
+// top-3 of the lanes of an aligned group of W
+template <int W, typename Z>
+__device__ __forceinline__ void cut_top3_group(unsigned gmask, Z& a, Z& b, Z& c) {
+#pragma unroll
+  for (int o = 1; o < W; o <<= 1) {
+    const Z a1 = __shfl_xor_sync(gmask, a, o), b1 = __shfl_xor_sync(gmask, b, o), c1 = __shfl_xor_sync(gmask, c, o);
+    // the third of the union: see top3_join
+    const Z m = max(a, a1), q = min(b, b1);
+    a = min(a, a1);
+    c = min(max(m, q), min(c, c1));
+    b = min(m, q);
+  }
+}
+
+// Entries k, k + step, ... below end of a row or (not ROW) a cut into the top-3 and
+// b2, from the tables in shared memory: tab {u, v, cost, 16 * (first pair) +
+// pairs}, nodes by their place in val (the sweep's lambdas and mus), a pair {cut
+// of u, cut of v} for each layer in which the ends differ; val[zero] is 0.
+template <bool ROW, typename Z>
+__device__ __forceinline__ void cut_scan_in(const CutGdp& A, const int4* tab, const int2* pairs, const int* val,
+                                            int k, int end, int step, int lu, Z& a, Z& b, Z& c,
+                                            long long& b2) {
+#pragma unroll 2
+  for (; k < end; k += step) {
+    const int4 it = tab[k];
+    Z z = (Z)it.z * (Z)(1 << A.F) - (Z)val[it.y] - (Z)(ROW ? lu : val[it.x]);
+    const int2* q = pairs + ((unsigned)it.w >> 4);
+    const int np = it.w & 15;
+    for (int l = 0; l < np; ++l) z -= (Z)(val[q[l].x] + val[q[l].y]);  // two duals, each below 2^29
+    if (ROW && z < 0) b2 += z;
+    cut_top3(z, a, b, c);
+  }
+}
+
+// The same from global memory.  Four at a time with every load unconditional (a
+// dual that is not there reads cut 0 and counts as 0): loads inside branches wait
+// for one another.  lambda and mu come through L1, which the acquire of the
+// sweep's barrier has emptied of the sweep before: a block reads the same few
+// nodes many times, and with every gather from L2 its rate bound the sweep.
+template <bool ROW>
+__device__ __forceinline__ void cut_scan_out(const CutGdp& A, int u, int k, int end, int step, const int32_t* lam,
+                                             const int32_t* mu, long long lu, long long& a, long long& b, long long& c,
+                                             long long& b2) {
+  constexpr int U = 4;
+  for (; k < end; k += U * step) {
+    int4 it[U];
+    long long z[U];
+#pragma unroll
+    for (int j = 0; j < U; ++j) {
+      const int e = k + j * step;
+      it[j] = make_int4(0, 0, 0, 0);
+      if (e >= end) continue;
+      const int2 w = ROW ? make_int2(e, u) : __ldg(A.items + e);
+      const int2 q = __ldg(A.iec + w.x);
+      it[j] = make_int4(w.y, q.x, q.y, __ldg(A.mask + w.x));
+    }
+#pragma unroll
+    for (int j = 0; j < U; ++j)
+      z[j] = ((long long)it[j].z << A.F) - lam[it[j].y] - (ROW ? lu : (long long)lam[it[j].x]);
+    for (int l = 0; l < A.L; ++l) {
+      const int32_t* row = A.cid + (long long)l * A.n;
+#pragma unroll
+      for (int j = 0; j < U; ++j) {
+        int x = -1, y = -1;
+        if ((unsigned)it[j].w >> l & 1u) {
+          x = __ldg(row + it[j].x);
+          y = __ldg(row + it[j].y);
+        }
+        const int mx = mu[max(x, 0)], my = mu[max(y, 0)];
+        z[j] -= (x >= 0 ? mx : 0) + (y >= 0 ? my : 0);
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < U; ++j) {
+      if (k + j * step >= end) z[j] = kInfZ;
+      if (ROW && z[j] < 0) b2 += z[j];
+      cut_top3(z[j], a, b, c);
+    }
+  }
+}
+
+// exclusive sum of v over the block's threads; the total in *total
+__device__ __forceinline__ int cut_block_scan(int v, int* total) {
+  __shared__ int s_w[32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int x = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31) s_w[warp] = x;
+  __syncthreads();
+  int before = 0, all = 0;
+  for (int w = 0; w < (int)blockDim.x / 32; ++w) {
+    if (w < warp) before += s_w[w];
+    all += s_w[w];
+  }
+  *total = all;
+  return before + x - v;
+}
+
+__global__ void __launch_bounds__(kCutThreads, 1) cut_gdp_kernel(const __grid_constant__ CutGdp A) {
+  constexpr int G = kCutGroup, RW = 32 / G, NW = kCutThreads / 32;
+  extern __shared__ int4 s_dyn[];
+  __shared__ long long s_t3[NW * 3];
+  __shared__ unsigned s_ch, s_pairs;
+  __shared__ int s_ovf, s_stop, s_cut[2];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, sub = lane & (G - 1);
+  const unsigned gmask = ((1u << G) - 1u) << (lane & ~(G - 1));
+  const int n = A.n, L = A.L, M = A.M, nb = gridDim.x, blk = blockIdx.x;
+  const int v0 = (int)((long long)n * blk / nb), v1 = (int)((long long)n * (blk + 1) / nb), nr = v1 - v0;
+  for (int i = v0 + tid; i < v1; i += kCutThreads) A.lam[0][i] = A.lam_in[__ldg(A.perm + i)];
+  // the block's cuts: those whose list begins in its share of all lists
+  if (tid < 2) {
+    const long long T = __ldg(A.cut_ptr + M);
+    int lo = 0, hi = M;
+    if (blk + tid == nb) lo = M;
+    while (lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      if ((long long)__ldg(A.cut_ptr + mid) * nb >= T * (blk + tid)) hi = mid; else lo = mid + 1;
+    }
+    s_cut[tid] = lo;
+  }
+  if (tid == 0) { s_ch = 0; s_ovf = 0; s_pairs = 0; }
+  __syncthreads();
+  const int s0 = s_cut[0], nc = s_cut[1] - s0;
+  const int e0 = __ldg(A.irp + v0), ne = __ldg(A.irp + v1) - e0;
+  const int k0 = __ldg(A.cut_ptr + s0), nk = __ldg(A.cut_ptr + s0 + nc) - k0;
+  // Tables of the block in shared memory: the offsets of its rows and cuts, the
+  // entries of both, the nodes and cuts they read (found with one bit each; a
+  // place is the rank of the bit) with their values, and the pairs.  One that
+  // does not fit leaves the block on global memory.
+  const int wn = (n + 31) / 32, nw = wn + (M + 31) / 32;  // words: nodes, then cuts
+  const int offs = (nr + 1 + nc + 1 + 3) & ~3;
+  const long long fixed = 16LL * ne + 16LL * nk + 4LL * offs + 8LL * nw;
+  bool in = fixed + 16 <= kCutSmem;
+  int4* rtab = s_dyn;
+  int4* ktab = rtab + (in ? ne : 0);
+  int32_t* s_rp = reinterpret_cast<int32_t*>(ktab + (in ? nk : 0));
+  int32_t* s_cp = s_rp + nr + 1;
+  unsigned* bits = reinterpret_cast<unsigned*>(s_rp + (in ? offs : 0));
+  int32_t* rank = reinterpret_cast<int32_t*>(bits + (in ? nw : 0));
+  int32_t* need = rank + (in ? nw : 0);  // bit of each place, its value behind
+  int32_t* val = need;
+  int2* pairs = nullptr;
+  int nneed = 0;
+  auto entry = [&](auto&& f) {  // f(place in the tables, entry, row)
+    for (int i = tid / G; i < nr; i += kCutThreads / G)
+      for (int e = __ldg(A.irp + v0 + i) + sub, end = __ldg(A.irp + v0 + i + 1); e < end; e += G) f(e - e0, e, v0 + i);
+    for (int k = tid; k < nk; k += kCutThreads) {
+      const int2 w = __ldg(A.items + k0 + k);
+      f(ne + k, w.x, w.y);
+    }
+  };
+  auto mark = [&](int b) { atomicOr(bits + (b >> 5), 1u << (b & 31)); };
+  auto place = [&](int b) { return rank[b >> 5] + __popc(bits[b >> 5] & ((1u << (b & 31)) - 1u)); };
+  if (in) {
+    for (int i = tid; i < nw; i += kCutThreads) bits[i] = 0;
+    for (int i = tid; i <= nr; i += kCutThreads) s_rp[i] = __ldg(A.irp + v0 + i) - e0;
+    for (int i = tid; i <= nc; i += kCutThreads) s_cp[i] = __ldg(A.cut_ptr + s0 + i) - k0;
+    __syncthreads();
+    for (int i = v0 + tid; i < v1; i += kCutThreads) mark(i);
+    for (int i = s0 + tid; i < s0 + nc; i += kCutThreads) mark(wn * 32 + i);
+    entry([&](int, int e, int u) {
+      const int v = __ldg(A.iec + e).x;
+      unsigned m = __ldg(A.mask + e);
+      mark(u);
+      mark(v);
+      if (m) atomicAdd(&s_pairs, __popc(m));
+      for (; m; m &= m - 1) {
+        const int32_t* row = A.cid + (long long)(__ffs(m) - 1) * n;
+        const int x = __ldg(row + u), y = __ldg(row + v);
+        if (x >= 0) mark(wn * 32 + x);
+        if (y >= 0) mark(wn * 32 + y);
+      }
+    });
+    __syncthreads();
+    const int per = (nw + kCutThreads - 1) / kCutThreads, w0 = min(nw, tid * per), w1 = min(nw, w0 + per);
+    int mine = 0;
+    for (int w = w0; w < w1; ++w) mine += __popc(bits[w]);
+    int r = cut_block_scan(mine, &nneed);
+    const long long npairs = s_pairs;
+    in = fixed + 8LL * (nneed + 2) + 8LL * npairs + 16 <= kCutSmem;
+    if (in) {
+      val = need + nneed + 1;
+      pairs = reinterpret_cast<int2*>(need + ((2 * nneed + 3) & ~1));
+      pairs = reinterpret_cast<int2*>((reinterpret_cast<uintptr_t>(pairs) + 7) & ~(uintptr_t)7);
+      for (int w = w0; w < w1; ++w) {
+        rank[w] = r;
+        for (unsigned m = bits[w]; m; m &= m - 1) need[r++] = w * 32 + __ffs(m) - 1;
+      }
+      if (tid == 0) val[nneed] = 0;
+      __syncthreads();
+      if (tid == 0) s_pairs = 0;
+      __syncthreads();
+      entry([&](int at, int e, int u) {
+        const int2 q = __ldg(A.iec + e);
+        unsigned m = __ldg(A.mask + e), w = 0;
+        if (m) {
+          unsigned p = atomicAdd(&s_pairs, __popc(m));
+          w = p << 4 | __popc(m);
+          for (; m; m &= m - 1) {
+            const int32_t* row = A.cid + (long long)(__ffs(m) - 1) * n;
+            const int x = __ldg(row + u), y = __ldg(row + q.x);
+            pairs[p++] = make_int2(x >= 0 ? place(wn * 32 + x) : nneed, y >= 0 ? place(wn * 32 + y) : nneed);
+          }
+        }
+        rtab[at] = make_int4(place(u), place(q.x), q.y, (int)w);
+      });
+    }
+  }
+  const int32_t* rp = in ? s_rp : A.irp + v0;
+  const int32_t* cp = in ? s_cp : A.cut_ptr + s0;
+  const int own = in ? place(v0 < n ? v0 : 0) : 0, own_cut = in && nc ? place(wn * 32 + s0) : 0;
+  // z fits 32 bits while the costs stay below 2^29 and the values below lim
+  const int lim = ((1 << 30) - 1 + (1 << 29)) / (2 + 2 * L);
+  bool cheap = true, any_long = false;
+  if (in)
+    for (int i = tid; i < ne + nk; i += kCutThreads) cheap &= ((long long)rtab[i].z << A.F) < (1 << 29);
+  cheap = __syncthreads_and(cheap);
+  for (int i = tid; i < nc; i += kCutThreads) any_long |= cp[i + 1] - cp[i] > kLongCut;
+  any_long = __syncthreads_or(any_long);
+  int par = 0;  // the buffers that hold the result
+  bool ok = grid_barrier_counted(&A.ctl->bar_count, gridDim.x, A.budget);
+  if (!ok && tid == 0) atomicOr(&A.ctl->status, kGdpTimeout);
+  for (long long t = 0; ok && t < A.max_sweeps; ++t) {
+    const int p = (int)(t & 1), sl = (int)(t % 3);
+    const int32_t *lam = A.lam[p], *mu = A.mu[p];
     long long b2 = 0;
     unsigned ch = 0;
     int ovf = 0;
-    // node duals: Section 3's gradient over delta(v)
-    for (long long v = gid; v < n; v += ngroups) {
-      const int beg = __ldg(rp + v), end = __ldg(rp + v + 1);
-      long long a = kInfZ, b = kInfZ, c = kInfZ;
-      for (int e = beg + sub; e < end; e += G) {
-        const long long z = entry_z(ca, lin, min_, __ldg(mask + e), (int)v, __ldg(ec + e), F);
-        if (z < 0) b2 += z;
-        top3_ins_ll(z, a, b, c);
+    bool narrow = false;
+    if (in) {
+      bool big = false;
+      for (int i = tid; i < nneed; i += kCutThreads) {
+        const int w = need[i], x = w < wn * 32 ? __ldcg(lam + w) : __ldcg(mu + w - wn * 32);
+        big |= x >= lim || x <= -lim;
+        val[i] = x;
       }
-      for (int o = 1; o < G; o <<= 1) {
-        const long long a1 = __shfl_xor_sync(gmask, a, o), b1 = __shfl_xor_sync(gmask, b, o),
-                        c1 = __shfl_xor_sync(gmask, c, o);
-        top3_ins_ll(a1, a, b, c);
-        top3_ins_ll(b1, a, b, c);
-        top3_ins_ll(c1, a, b, c);
-      }
-      if (sub == 0) {
-        const long long lv = ld_cg_i(lin + v);
-        const long long d = step_ll(b, c, shift);
-        const long long nl = lv + d;
-        ovf |= (nl >= kLamLimit || nl <= -kLamLimit);
-        lout[v] = (int32_t)nl;
-        ch += (d != 0);
-        b2 += 4 * lv;
-      }
+      narrow = cheap & !__syncthreads_or(big);
     }
-    // cut duals: Section 3's gradient over delta(S), projected onto mu >= 0.
-    // A cut with a long list is taken by a whole block (its warps' top-3s
-    // merged in shared memory), the others by one warp each.
-    auto cut_update = [&](long long s, long long a, long long b, long long c) {
-      const long long m = ld_cg_i(min_ + s);
-      long long nm = m + step_ll(b, c, shift + 2);
-      if (nm < 0) nm = 0;
+    auto new_lambda = [&](int i, long long lv, long long b, long long c) {
+      const long long d = step_ll(b, c, A.shift), nl = lv + d;
+      ovf |= (nl >= kLamLimit || nl <= -kLamLimit);
+      __stcg(A.lam[p ^ 1] + v0 + i, (int32_t)nl);
+      ch += (d != 0);
+      b2 += 4LL * lv;
+    };
+    auto new_mu = [&](int s, long long b, long long c) {
+      const long long m = in ? val[own_cut + s] : mu[s0 + s];
+      const long long nm = max(0LL, m + step_ll(b, c, A.shift + 2));
       ovf |= (nm >= kLamLimit);
-      mout[s] = (int32_t)nm;
+      __stcg(A.mu[p ^ 1] + s0 + s, (int32_t)nm);
       ch += (nm != m);
       b2 += 4 * m;
     };
-    for (long long q = blockIdx.x; q < nlong; q += gridDim.x) {
-      const int s = __ldg(long_cuts + q);
-      const int p0 = __ldg(cut_ptr + s), p1 = __ldg(cut_ptr + s + 1);
-      long long a = kInfZ, b = kInfZ, c = kInfZ;
-      for (int k = p0 + tid; k < p1; k += blockDim.x) {
-        const int2 it = __ldg(items + k);
-        top3_ins_ll(entry_z(ca, lin, min_, __ldg(mask + it.y), it.x, __ldg(ec + it.y), F), a, b, c);
+    // entries [k, end) of cut s at this stride: the top-3 of the warp
+    auto cut_scan = [&](int k, int end, int step, long long& a, long long& b, long long& c) {
+      a = b = c = kInfZ;
+      if (narrow) {
+        int a1 = INT_MAX, b1 = INT_MAX, c1 = INT_MAX;
+        cut_scan_in<false>(A, ktab, pairs, val, k, end, step, 0, a1, b1, c1, b2);
+        cut_top3_group<32>(0xffffffffu, a1, b1, c1);
+        if (a1 != INT_MAX) a = a1;
+        if (b1 != INT_MAX) b = b1;
+        if (c1 != INT_MAX) c = c1;
+        return;
       }
-      for (int o = 1; o < 32; o <<= 1) {
-        const long long a1 = __shfl_xor_sync(0xffffffffu, a, o), b1 = __shfl_xor_sync(0xffffffffu, b, o),
-                        c1 = __shfl_xor_sync(0xffffffffu, c, o);
-        top3_ins_ll(a1, a, b, c);
-        top3_ins_ll(b1, a, b, c);
-        top3_ins_ll(c1, a, b, c);
+      if (in)
+        cut_scan_in<false>(A, ktab, pairs, val, k, end, step, 0, a, b, c, b2);
+      else
+        cut_scan_out<false>(A, 0, k, end, step, lam, mu, 0, a, b, c, b2);
+      cut_top3_group<32>(0xffffffffu, a, b, c);
+    };
+    // A warp takes one cut or eight rows at a time, cuts first (they are the
+    // longer ones).
+    const int jobs = (nr + RW - 1) / RW;
+    for (int job = warp; job < nc + jobs; job += NW) {
+      if (job < nc) {
+        // cut duals: Section 3's gradient over delta(S), projected onto mu >= 0
+        const int k = cp[job], end = cp[job + 1];
+        if (end - k > kLongCut) continue;
+        long long a, b, c;
+        cut_scan(k + lane, end, 32, a, b, c);
+        if (lane == 0) new_mu(job, b, c);
+        continue;
       }
+      // node duals: Section 3's gradient over delta(v)
+      const int i = (job - nc) * RW + lane / G;
+      const bool has = i < nr;
+      const int k = has ? rp[i] + sub : 0, end = has ? rp[i + 1] : 0;
+      if (narrow) {
+        const int lv = has ? val[own + i] : 0;
+        int a = INT_MAX, b = INT_MAX, c = INT_MAX;
+        cut_scan_in<true>(A, rtab, pairs, val, k, end, G, lv, a, b, c, b2);
+        cut_top3_group<G>(gmask, a, b, c);
+        if (sub == 0 && has) new_lambda(i, lv, b == INT_MAX ? kInfZ : b, c == INT_MAX ? kInfZ : c);
+      } else {
+        const int lv = !has ? 0 : in ? val[own + i] : lam[v0 + i];
+        long long a = kInfZ, b = kInfZ, c = kInfZ;
+        if (in)
+          cut_scan_in<true>(A, rtab, pairs, val, k, end, G, lv, a, b, c, b2);
+        else
+          cut_scan_out<true>(A, v0 + i, k, end, G, lam, mu, lv, a, b, c, b2);
+        cut_top3_group<G>(gmask, a, b, c);
+        if (sub == 0 && has) new_lambda(i, lv, b, c);
+      }
+    }
+    // long cuts: all warps on one, their top-3s merged in shared memory
+    for (int s = 0; any_long && s < nc; ++s) {
+      const int k = cp[s], end = cp[s + 1];
+      if (end - k <= kLongCut) continue;
+      long long a, b, c;
+      cut_scan(k + tid, end, kCutThreads, a, b, c);
       if (lane == 0) { s_t3[3 * warp] = a; s_t3[3 * warp + 1] = b; s_t3[3 * warp + 2] = c; }
       __syncthreads();
       if (warp == 0) {
-        a = lane < nwarps ? s_t3[3 * lane] : kInfZ;
-        b = lane < nwarps ? s_t3[3 * lane + 1] : kInfZ;
-        c = lane < nwarps ? s_t3[3 * lane + 2] : kInfZ;
-        for (int o = 1; o < 32; o <<= 1) {
-          const long long a1 = __shfl_xor_sync(0xffffffffu, a, o), b1 = __shfl_xor_sync(0xffffffffu, b, o),
-                          c1 = __shfl_xor_sync(0xffffffffu, c, o);
-          top3_ins_ll(a1, a, b, c);
-          top3_ins_ll(b1, a, b, c);
-          top3_ins_ll(c1, a, b, c);
-        }
-        if (lane == 0) cut_update(s, a, b, c);
+        a = lane < NW ? s_t3[3 * lane] : kInfZ;
+        b = lane < NW ? s_t3[3 * lane + 1] : kInfZ;
+        c = lane < NW ? s_t3[3 * lane + 2] : kInfZ;
+        cut_top3_group<32>(0xffffffffu, a, b, c);
+        if (lane == 0) new_mu(s, b, c);
       }
       __syncthreads();
     }
-    for (long long s = gwarp; s < M; s += twarps) {
-      const int p0 = __ldg(cut_ptr + s), p1 = __ldg(cut_ptr + s + 1);
-      if (p1 - p0 >= kLongCut) continue;  // a block's
-      long long a = kInfZ, b = kInfZ, c = kInfZ;
-      for (int k = p0 + lane; k < p1; k += 32) {
-        const int2 it = __ldg(items + k);
-        top3_ins_ll(entry_z(ca, lin, min_, __ldg(mask + it.y), it.x, __ldg(ec + it.y), F), a, b, c);
-      }
-      for (int o = 1; o < 32; o <<= 1) {
-        const long long a1 = __shfl_xor_sync(0xffffffffu, a, o), b1 = __shfl_xor_sync(0xffffffffu, b, o),
-                        c1 = __shfl_xor_sync(0xffffffffu, c, o);
-        top3_ins_ll(a1, a, b, c);
-        top3_ins_ll(b1, a, b, c);
-        top3_ins_ll(c1, a, b, c);
-      }
-      if (lane == 0) cut_update(s, a, b, c);
+    if (t < A.trace_cap) {
+      b2 = warp_sum_ll(b2);
+      if (lane == 0 && b2) atomicAdd(reinterpret_cast<unsigned long long*>(&A.ctl->slot_b2[sl]), (unsigned long long)b2);
     }
-    b2 = warp_sum_ll(b2);
     ch = warp_sum_u(ch);
     ovf = __any_sync(0xffffffffu, ovf);
-    if (lane == 0) { s_b2[warp] = b2; s_ch[warp] = ch; s_ovf[warp] = ovf; }
+    if (lane == 0 && ch) atomicAdd(&s_ch, ch);
+    if (lane == 0 && ovf) s_ovf = 1;
     __syncthreads();
-    if (warp == 0) {
-      long long x = lane < nwarps ? s_b2[lane] : 0;
-      unsigned y = lane < nwarps ? s_ch[lane] : 0;
-      int o = lane < nwarps ? s_ovf[lane] : 0;
-      x = warp_sum_ll(x);
-      y = warp_sum_u(y);
-      o = __any_sync(0xffffffffu, o);
-      if (lane == 0) {
-        const int sl = (int)(t % 3);
-        atomicAdd(reinterpret_cast<unsigned long long*>(&ctl->slot_b2[sl]), (unsigned long long)x);
-        if (y) atomicAdd(&ctl->slot_ch[sl], (unsigned long long)y);
-        if (o) atomicOr(&ctl->status, kGdpOverflow);
-      }
-    }
-    const bool ok = grid_barrier(&ctl->bar_count, &ctl->bar_gen, gridDim.x, budget);
+    // The sweep's barrier carries its totals: arrivals in bits 0-15, blocks that
+    // overflowed in bits 16-31, changed duals above.  Its word is the sweep's
+    // own (of three), so that nobody adds to it before everyone has read it.
     if (tid == 0) {
-      if (!ok) atomicOr(&ctl->status, kGdpTimeout);
-      volatile GdpCtl* vc = ctl;
-      const int sl = (int)(t % 3);
-      const unsigned long long chg = vc->slot_ch[sl];
-      const int st = vc->status;
-      if (blockIdx.x == 0) {
-        if (t < trace_cap) {
-          trace_b2[t] = vc->slot_b2[sl];
-          trace_ch[t] = chg;
-        }
-        const int r = (int)((t + 2) % 3);  // read by everyone after the previous barrier
-        vc->slot_b2[r] = 0;
-        vc->slot_ch[r] = 0;
-        vc->sweeps = t + 1;
-        vc->fixed_point = (chg == 0);
+      unsigned long long* word = &A.ctl->slot_ch[sl];
+      unsigned long long x = 1ull | (s_ovf ? 1ull << 16 : 0ull) | (unsigned long long)s_ch << 32;
+      s_ch = 0;
+      s_ovf = 0;
+      asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(word), "l"(x) : "memory");
+      const long long c0 = clock64();
+      int stop = 0;
+      for (;;) {
+        asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(x) : "l"(word) : "memory");
+        if ((x & 0xffff) == (unsigned)nb) break;
+        if (clock64() - c0 > A.budget) { stop = 3; break; }
       }
-      s_stop = (st != 0) || (chg == 0);
+      const unsigned chg = (unsigned)(x >> 32);
+      if (stop == 3) {
+        atomicOr(&A.ctl->status, kGdpTimeout);
+      } else {
+        const bool over = ((x >> 16) & 0xffff) != 0;
+        stop = over ? 2 : chg == 0;
+        if (blk == 0) {
+          volatile GdpCtl* vc = A.ctl;
+          if (t < A.trace_cap) {
+            A.trace_b2[t] = vc->slot_b2[sl];
+            A.trace_ch[t] = chg;
+          }
+          const int r = (int)((t + 2) % 3);  // read by everyone before this barrier
+          vc->slot_b2[r] = 0;
+          vc->slot_ch[r] = 0;
+          vc->sweeps = t + 1;
+          vc->fixed_point = (chg == 0);
+          if (over) atomicOr(&A.ctl->status, kGdpOverflow);
+        }
+      }
+      s_stop = stop;
     }
     __syncthreads();
-    if (s_stop) break;
+    const int stop = s_stop;
+    // an overflowing sweep is not kept: the result stays in its input
+    if (stop < 2) par = p ^ 1;
+    if (stop) break;
   }
+  for (int i = v0 + tid; i < v1; i += kCutThreads) A.lam_out[__ldg(A.perm + i)] = __ldcg(A.lam[par] + i);
 }
 
 // bound2 at (lam, mu) with fb bits, and (x2 != NULL) rule (7) with the cut terms
@@ -577,42 +837,30 @@ f2m_status cut_lists(f2m_ctx* c) {
     dfree(S->d_cnt);
     dfree(S->d_ptr);
     dfree(S->d_scan);
-    dfree(S->d_lflag);
-    dfree(S->d_lpos);
-    dfree(S->d_long);
     S->ptr_cap = S->M + 1 + 1024;
     CK(c, dalloc(&S->d_cnt, S->ptr_cap));
     CK(c, dalloc(&S->d_ptr, S->ptr_cap));
     CK(c, dalloc(&S->d_scan, (int64_t)scan_scratch_ints((int32_t)S->ptr_cap)));
-    CK(c, dalloc(&S->d_lflag, S->ptr_cap));
-    CK(c, dalloc(&S->d_lpos, S->ptr_cap));
-    CK(c, dalloc(&S->d_long, S->ptr_cap));
   }
-  CK(c, cudaMemsetAsync(S->d_cnt, 0, sizeof(int32_t) * (S->M + 1), c->st));
-  cut_list_kernel<false><<<grid_of(c->n, 256), 256, 0, c->st>>>(c->d_rp, c->d_ec, S->d_mask, a, S->d_cnt,
-                                                                  nullptr, nullptr);
+  const int32_t n = c->n, L = S->L, M = (int32_t)S->M;
+  const GdpPlan& P = c->plan;
+  CK(c, grow(&S->d_cid, &S->cid_cap, (int64_t)L * n));
+  CK(c, grow(&S->d_imask, &S->imask_cap, c->nnz));
+  CK(c, grow(&S->d_items, &S->item_cap, L * c->nnz));  // an entry crosses a layer's cuts once per row
+  cut_cid_kernel<<<grid_of(n, 256), 256, 0, c->st>>>(a, P.perm, S->d_cid);
   count_launch();
-  CK(c, launch_scan(S->d_cnt, S->d_ptr, (int32_t)S->M, S->d_scan, c->st));
-  int32_t total = 0;
-  CK(c, cudaMemcpyAsync(&total, S->d_ptr + S->M, sizeof(int32_t), cudaMemcpyDeviceToHost, c->st));
-  CK(c, cudaStreamSynchronize(c->st));
-  CK(c, grow(&S->d_items, &S->item_cap, (int64_t)total));
-  CK(c, cudaMemsetAsync(S->d_cnt, 0, sizeof(int32_t) * (S->M + 1), c->st));
-  cut_list_kernel<true><<<grid_of(c->n, 256), 256, 0, c->st>>>(c->d_rp, c->d_ec, S->d_mask, a, S->d_cnt,
-                                                                 S->d_ptr, S->d_items);
-  count_launch();
-  CK(c, cudaGetLastError());
-  // the cuts with long lists, in index order
-  cut_long_flag_kernel<<<grid_of(S->M, 256), 256, 0, c->st>>>(S->d_cnt, (int32_t)S->M, S->d_lflag);
-  count_launch();
-  CK(c, launch_scan(S->d_lflag, S->d_lpos, (int32_t)S->M, S->d_scan, c->st));
-  cut_long_list_kernel<<<grid_of(S->M, 256), 256, 0, c->st>>>(S->d_lflag, S->d_lpos, (int32_t)S->M, S->d_long);
-  count_launch();
-  int32_t nlong = 0;
-  CK(c, cudaMemcpyAsync(&nlong, S->d_lpos + S->M, sizeof(int32_t), cudaMemcpyDeviceToHost, c->st));
-  CK(c, cudaStreamSynchronize(c->st));
-  S->nlong = nlong;
-  S->items = total;
+  for (int fill = 0; fill < 2; ++fill) {
+    CK(c, cudaMemsetAsync(S->d_cnt, 0, sizeof(int32_t) * (M + 1), c->st));
+    if (!fill)
+      cut_list_kernel<false><<<grid_of(n, 256), 256, 0, c->st>>>(P.irp, P.iec, S->d_cid, n, L, S->d_imask, S->d_cnt,
+                                                                 nullptr, nullptr);
+    else
+      cut_list_kernel<true><<<grid_of(n, 256), 256, 0, c->st>>>(P.irp, P.iec, S->d_cid, n, L, S->d_imask, S->d_cnt,
+                                                                S->d_ptr, S->d_items);
+    count_launch();
+    CK(c, cudaGetLastError());
+    if (!fill) CK(c, launch_scan(S->d_cnt, S->d_ptr, M, S->d_scan, c->st));
+  }
   S->built_version = c->plan.version;
   S->built_L = S->L;
   return F2M_OK;
@@ -624,35 +872,40 @@ f2m_status cut_gdp_phase(f2m_ctx* c, int64_t max_sweeps, int64_t* sweeps, long l
   c->lam_version += 1;
   f2m_status s = cut_lists(c);
   if (s != F2M_OK) return s;
-  const CutArgs a = cut_args(c);
-  const int threads = 512;
-  int per_sm = 0;
-  CK(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cut_gdp_kernel<4>, threads, 0));
-  if (per_sm < 1) return fail(c, F2M_ERR_CUDA, "cut GDP kernel does not fit an SM");
-  if (per_sm > 2) per_sm = 2;
-  const int grid = c->num_sms * per_sm;
+  *sweeps = 0;
+  if (max_sweeps <= 0) return F2M_ERR_NOT_CONVERGED;
   CK(c, cudaMemsetAsync(c->d_gdp, 0, sizeof(GdpCtl), c->st));
   cudaEvent_t e0 = c->ev0, e1 = c->ev1;
   CK(c, cudaEventRecord(e0, c->st));
-  const int32_t* rp = c->d_rp;
-  const int2* ec = c->d_ec;
-  const uint8_t* mask = S->d_mask;
-  const int32_t* ptr = S->d_ptr;
-  const int2* items = S->d_items;
-  int32_t M = (int32_t)S->M;
-  const int32_t* lcuts = S->d_long;
-  int32_t nlong = S->nlong;
-  int32_t* l0 = c->d_lam[c->cur];
-  int32_t* l1 = c->d_lam[c->cur ^ 1];
-  int32_t* m0 = S->d_mu[S->cur];
-  int32_t* m1 = S->d_mu[S->cur ^ 1];
-  int32_t F = c->p.frac_bits, shift = c->p.damping_shift;
-  long long msw = max_sweeps, tcl = tcap, budget = c->p.barrier_budget_cycles;
-  GdpCtl* ctl = c->d_gdp;
-  void* args[] = {(void*)&rp, (void*)&ec, (void*)&mask, (void*)&a, (void*)&ptr, (void*)&items, (void*)&M,
-                  (void*)&lcuts, (void*)&nlong, (void*)&l0, (void*)&l1, (void*)&m0, (void*)&m1, (void*)&F, (void*)&shift, (void*)&msw,
-                  (void*)&ctl, (void*)&tb, (void*)&tc, (void*)&tcl, (void*)&budget};
-  CK(c, cudaLaunchCooperativeKernel((const void*)cut_gdp_kernel<4>, dim3(grid), dim3(threads), args, 0, c->st));
+  const GdpPlan& P = c->plan;
+  CutGdp g{};
+  g.irp = P.irp;
+  g.iec = P.iec;
+  g.perm = P.perm;
+  g.cid = S->d_cid;
+  g.mask = S->d_imask;
+  g.cut_ptr = S->d_ptr;
+  g.items = S->d_items;
+  g.lam_in = c->d_lam[c->cur];
+  g.lam_out = c->d_lam[c->cur ^ 1];
+  g.lam[0] = P.ilam[0];
+  g.lam[1] = P.ilam[1];
+  g.mu[0] = S->d_mu[S->cur];
+  g.mu[1] = S->d_mu[S->cur ^ 1];
+  g.ctl = c->d_gdp;
+  g.trace_b2 = tb;
+  g.trace_ch = tc;
+  g.trace_cap = tcap;
+  g.max_sweeps = max_sweeps;
+  g.budget = c->p.barrier_budget_cycles;
+  g.n = c->n;
+  g.L = S->L;
+  g.M = (int32_t)S->M;
+  g.F = c->p.frac_bits;
+  g.shift = c->p.damping_shift;
+  void* args[] = {(void*)&g};
+  CK(c, cudaFuncSetAttribute((const void*)cut_gdp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kCutSmem));
+  CK(c, cudaLaunchCooperativeKernel((const void*)cut_gdp_kernel, dim3(c->num_sms), dim3(kCutThreads), args, kCutSmem, c->st));
   count_launch();
   CK(c, cudaEventRecord(e1, c->st));
   GdpCtl h{};
@@ -667,10 +920,8 @@ f2m_status cut_gdp_phase(f2m_ctx* c, int64_t max_sweeps, int64_t* sweeps, long l
   // the state after the last sweep that was kept: an overflowing sweep is not
   const bool ovf = (h.status & kGdpOverflow) != 0;
   const long long used = ovf ? h.sweeps - 1 : h.sweeps;
-  if (used & 1) {
-    c->cur ^= 1;
-    S->cur ^= 1;
-  }
+  if (!(h.status & kGdpTimeout)) c->cur ^= 1;  // written from the buffer kept
+  if (used & 1) S->cur ^= 1;
   c->gdp_kernel = F2M_GDP_KERNEL_CUTS;
   if (h.status & kGdpTimeout) return fail(c, F2M_ERR_TIMEOUT, "device-wide barrier wait exceeded its budget");
   if (ovf) return fail(c, F2M_ERR_OVERFLOW, "|lambda| or a cut dual reached 2^29");
@@ -769,16 +1020,10 @@ f2m_status cut_separate(f2m_ctx* c, int32_t* d_comp_out, int32_t* m_out) {
       dfree(S->d_cnt);
       dfree(S->d_ptr);
       dfree(S->d_scan);
-      dfree(S->d_lflag);
-      dfree(S->d_lpos);
-      dfree(S->d_long);
       S->ptr_cap = n + 1;
       CK(c, dalloc(&S->d_cnt, S->ptr_cap));
       CK(c, dalloc(&S->d_ptr, S->ptr_cap));
       CK(c, dalloc(&S->d_scan, (int64_t)scan_scratch_ints((int32_t)S->ptr_cap)));
-      CK(c, dalloc(&S->d_lflag, S->ptr_cap));
-      CK(c, dalloc(&S->d_lpos, S->ptr_cap));
-      CK(c, dalloc(&S->d_long, S->ptr_cap));
       S->built_version = -1;
     }
   }
