@@ -62,7 +62,6 @@ struct f2m_batch {
   long long* d_seg_b2 = nullptr;
   unsigned long long* d_seg_bad = nullptr;
   int32_t* d_tmp_a = nullptr;       // output staging
-  int32_t* d_tmp_b = nullptr;
   int64_t tmp_cap = 0;
   uint8_t* d_mask = nullptr;        // per-segment mask for the masked steps
   // results, snapshotted when an instance finishes (later steps for other
@@ -79,7 +78,7 @@ struct f2m_batch {
   uint8_t* d_snap_done = nullptr;   // [count] instances being copied
   int32_t* d_snap_ent = nullptr;    // [count + 1] first entry of each instance
   std::vector<int64_t> res_eoff, res_nnz, res_b2;
-  std::vector<int32_t> res_fb;
+  std::vector<int32_t> res_fb, res_r0;  // fractional bits; first entry in the union's offsets
   std::vector<uint8_t> res_done;
   // tiles (gdp_ring.cu): those of a phase's active instances, wave by wave
   bool ring_off = false;            // they don't fit: the streaming kernels
@@ -128,7 +127,7 @@ extern "C" void f2m_destroy_batch(f2m_batch* b) {
   if (b->h_tiles) cudaFreeHost(b->h_tiles);
   if (b->h_e1) cudaFreeHost(b->h_e1);
   if (b->h_chunk) cudaFreeHost(b->h_chunk);
-  dfree(b->d_seg_b2); dfree(b->d_seg_bad); dfree(b->d_tmp_a); dfree(b->d_tmp_b);
+  dfree(b->d_seg_b2); dfree(b->d_seg_bad); dfree(b->d_tmp_a);
   dfree(b->d_mask); dfree(b->d_res_lam); dfree(b->d_res_rp); dfree(b->d_res_ec); dfree(b->d_res_x2);
   if (b->gexec) cudaGraphExecDestroy(b->gexec);
   if (b->gs) cudaStreamDestroy(b->gs);
@@ -834,6 +833,7 @@ static f2m_status snapshot(f2m_batch* b, const std::vector<uint8_t>& done) {
     const int64_t nz = h_ent[s + 1] - h_ent[s];
     h_eoff[s] = b->res_used;
     b->res_eoff[s] = b->res_used;
+    b->res_r0[s] = h_ent[s];
     b->res_nnz[s] = nz;
     b->res_b2[s] = h_b2[s];
     b->res_fb[s] = fb;
@@ -866,6 +866,7 @@ extern "C" f2m_status f2m_solve_batch(f2m_batch* b, f2m_info* info_out, f2m_info
   b->res_nnz.assign(K, 0);
   b->res_b2.assign(K, 0);
   b->res_fb.assign(K, c->p.frac_bits);
+  b->res_r0.assign(K, 0);
   b->res_done.assign(K, 0);
   b->res_used = 0;
   f2m_info tot;
@@ -1053,22 +1054,19 @@ extern "C" f2m_status f2m_solve_batch(f2m_batch* b, f2m_info* info_out, f2m_info
   return status;
 }
 
-static f2m_status stage(f2m_batch* b, int64_t cap) {
-  f2m_ctx* c = b->u;
-  if (b->tmp_cap >= cap) return F2M_OK;
-  dfree(b->d_tmp_a);
-  dfree(b->d_tmp_b);
-  CK(c, dalloc(&b->d_tmp_a, cap));
-  CK(c, dalloc(&b->d_tmp_b, cap));
-  b->tmp_cap = cap;
-  return F2M_OK;
-}
-
-__global__ void f2m_offset_kernel(const int32_t* __restrict__ in, int64_t count, int32_t sub,
-                                  int32_t* __restrict__ out) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < count;
-       i += (long long)gridDim.x * blockDim.x)
-    out[i] = in[i] - sub;
+// An instance's row offsets, columns (in its own numbering) and x out of the
+// result arenas in one pass; any of the three outputs may be NULL.
+__global__ void __launch_bounds__(256)
+f2m_batch_read_kernel(const int32_t* __restrict__ rp, int32_t rows, int32_t r0, int32_t* __restrict__ rp_out,
+                      const int2* __restrict__ ec, const uint8_t* __restrict__ x2, int64_t nz, int32_t v0,
+                      int32_t* __restrict__ col_out, uint8_t* __restrict__ x2_out) {
+  const long long i0 = blockIdx.x * (long long)blockDim.x + threadIdx.x, step = (long long)gridDim.x * blockDim.x;
+  if (rp_out)
+    for (long long i = i0; i < rows; i += step) rp_out[i] = rp[i] - r0;
+  for (long long i = i0; i < nz; i += step) {
+    if (col_out) col_out[i] = ec[i].x - v0;
+    if (x2_out) x2_out[i] = x2[i];
+  }
 }
 
 extern "C" f2m_status f2m_batch_get_lambda(f2m_batch* b, int32_t i, int32_t* lambda, int32_t* frac_bits) {
@@ -1095,27 +1093,35 @@ extern "C" f2m_status f2m_batch_get_x(f2m_batch* b, int32_t i, int64_t* nnz_inou
   *nnz_inout = nz;
   if (!row_ptr && !col && !x2) return F2M_OK;
   if ((col || x2) && cap < nz) return bfail(b, F2M_ERR_INVALID_ARG, "capacity below nnz");
-  f2m_status s = stage(b, std::max<int64_t>(nz, b->n[i] + 1));
-  if (s != F2M_OK) return s;
-  const int32_t* rp = b->d_res_rp + c->seg_off[i] + i;
-  if (row_ptr) {
-    int32_t r0 = 0;
-    CK(c, cudaMemcpyAsync(&r0, rp, sizeof(int32_t), cudaMemcpyDeviceToHost, c->st));
-    CK(c, cudaStreamSynchronize(c->st));
-    f2m_offset_kernel<<<64, 256, 0, c->st>>>(rp, b->n[i] + 1, r0, b->d_tmp_a);
-    count_launch();
-    CK(c, cudaGetLastError());
-    CK(c, cudaMemcpyAsync(row_ptr, b->d_tmp_a, sizeof(int32_t) * (b->n[i] + 1), cudaMemcpyDefault, c->st));
-    CK(c, cudaStreamSynchronize(c->st));
+  // straight into the caller's device arrays; host arrays by way of a staging copy
+  const int32_t rows = b->n[i] + 1;
+  auto on_device = [](const void* p) {
+    cudaPointerAttributes q;
+    if (p && cudaPointerGetAttributes(&q, p) == cudaSuccess)
+      return q.type == cudaMemoryTypeDevice || q.type == cudaMemoryTypeManaged;
+    cudaGetLastError();
+    return false;
+  };
+  const bool drp = on_device(row_ptr), dcol = on_device(col), dx2 = on_device(x2);
+  if ((row_ptr && !drp) || (col && !dcol)) {
+    const int64_t need = (int64_t)rows + nz;
+    if (b->tmp_cap < need) {
+      dfree(b->d_tmp_a);
+      b->tmp_cap = need + need / 2;
+      CK(c, dalloc(&b->d_tmp_a, b->tmp_cap));
+    }
   }
-  if (col && nz) {
-    CK(c, launch_split_ec(b->d_res_ec + b->res_eoff[i], nz, b->d_tmp_b, nullptr, c->st));
-    f2m_offset_kernel<<<256, 256, 0, c->st>>>(b->d_tmp_b, nz, c->seg_off[i], b->d_tmp_a);
-    count_launch();
-    CK(c, cudaGetLastError());
-    CK(c, cudaMemcpyAsync(col, b->d_tmp_a, sizeof(int32_t) * nz, cudaMemcpyDefault, c->st));
-  }
-  if (x2 && nz) CK(c, cudaMemcpyAsync(x2, b->d_res_x2 + b->res_eoff[i], nz, cudaMemcpyDefault, c->st));
+  int32_t* o_rp = row_ptr ? (drp ? row_ptr : b->d_tmp_a) : nullptr;
+  int32_t* o_col = col ? (dcol ? col : b->d_tmp_a + rows) : nullptr;
+  const long long most = std::max<long long>(rows, nz);
+  f2m_batch_read_kernel<<<(unsigned)std::min<long long>((most + 255) / 256, 4096), 256, 0, c->st>>>(
+      b->d_res_rp + c->seg_off[i] + i, rows, b->res_r0[i], o_rp, b->d_res_ec + b->res_eoff[i],
+      b->d_res_x2 + b->res_eoff[i], nz, c->seg_off[i], o_col, dx2 ? x2 : nullptr);
+  count_launch();
+  CK(c, cudaGetLastError());
+  if (row_ptr && !drp) CK(c, cudaMemcpyAsync(row_ptr, o_rp, sizeof(int32_t) * rows, cudaMemcpyDefault, c->st));
+  if (col && !dcol && nz) CK(c, cudaMemcpyAsync(col, o_col, sizeof(int32_t) * nz, cudaMemcpyDefault, c->st));
+  if (x2 && !dx2 && nz) CK(c, cudaMemcpyAsync(x2, b->d_res_x2 + b->res_eoff[i], nz, cudaMemcpyDefault, c->st));
   CK(c, cudaStreamSynchronize(c->st));
   return F2M_OK;
 }
