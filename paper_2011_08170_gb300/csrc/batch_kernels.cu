@@ -735,29 +735,53 @@ cudaError_t launch_batch_scatter_final(const int32_t* lam0, const int32_t* lam1,
 // ---- segmented helpers -------------------------------------------------------------
 
 // per-segment bound2 at lam (units 2^-fb); for segments flagged in seg_write
-// (NULL = none) also x2 by rule (7) and the count of rows not summing to 4
+// (NULL = none) also x2 by rule (7) and the count of rows not summing to 4.
+// Eight lanes a row, and a warp whose rows are of one segment (all but those on
+// a border) adds its sum once: an atomic of every row on its segment's word had
+// bound the kernel, 0.36 -> 0.09 ms at 1.6 M points in 256 instances.
 __global__ void batch_extract_bound_kernel(const int32_t* __restrict__ rp, const int2* __restrict__ ec,
                                            const int32_t* __restrict__ lam, int32_t n, int32_t fb,
                                            const int32_t* __restrict__ seg_off, int32_t nseg,
                                            uint8_t* __restrict__ x2, long long* seg_b2,
                                            unsigned long long* seg_bad,
                                            const uint8_t* __restrict__ seg_write) {
-  F2M_GRID_STRIDE(v, n) {
-    const int sg = segment_of(seg_off, nseg, (int)v);
-    const int write_x = seg_write != nullptr && seg_write[sg];
-    const long long lv = lam[v];
-    long long acc = 4 * lv;
-    int s = 0;
-    for (int e = rp[v]; e < rp[v + 1]; ++e) {
-      const int2 q = ec[e];
-      const long long z = ((long long)q.y << fb) - lv - lam[q.x];
-      if (z < 0) acc += z;
-      const int x = z < 0 ? 2 : (z == 0 ? 1 : 0);
-      if (write_x) x2[e] = (uint8_t)x;
-      s += x;
+  const int rows_a_warp = 32 / kRowLanes, sub = threadIdx.x & (kRowLanes - 1), lane = threadIdx.x & 31;
+  // every lane of a warp makes the same number of turns
+  for (long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) / 32; w * rows_a_warp < n;
+       w += (long long)gridDim.x * blockDim.x / 32) {
+    const long long v = w * rows_a_warp + lane / kRowLanes;
+    int sg = -1;
+    long long acc = 0;
+    int bad = 0;
+    if (v < n) {
+      sg = segment_of(seg_off, nseg, (int)v);
+      const int write_x = seg_write != nullptr && seg_write[sg];
+      const long long lv = lam[v];
+      if (sub == 0) acc = 4 * lv;
+      int s = 0;
+      for (int e = rp[v] + sub, end = rp[v + 1]; e < end; e += kRowLanes) {
+        const int2 q = ec[e];
+        const long long z = ((long long)q.y << fb) - lv - lam[q.x];
+        if (z < 0) acc += z;
+        const int x = z < 0 ? 2 : (z == 0 ? 1 : 0);
+        if (write_x) x2[e] = (uint8_t)x;
+        s += x;
+      }
+      s = row_sum(s);
+      bad = write_x && s != 4 && sub == 0;
     }
-    atomicAdd(reinterpret_cast<unsigned long long*>(&seg_b2[sg]), (unsigned long long)acc);
-    if (write_x && s != 4) atomicAdd(&seg_bad[sg], 1ull);
+    const int first = __shfl_sync(0xffffffffu, sg, 0);
+    if (__all_sync(0xffffffffu, sg == first || sg < 0)) {
+      acc = warp_sum_ll(acc);
+      bad = __popc(__ballot_sync(0xffffffffu, bad));
+      if (lane == 0) {
+        atomicAdd(reinterpret_cast<unsigned long long*>(&seg_b2[first]), (unsigned long long)acc);
+        if (bad) atomicAdd(&seg_bad[first], (unsigned long long)bad);
+      }
+    } else if (sg >= 0) {
+      if (acc) atomicAdd(reinterpret_cast<unsigned long long*>(&seg_b2[sg]), (unsigned long long)acc);
+      if (bad) atomicAdd(&seg_bad[sg], 1ull);
+    }
   }
 }
 
@@ -768,7 +792,7 @@ cudaError_t launch_batch_extract_bound(const int32_t* rp, const int2* ec, const 
   cudaError_t e = cudaMemsetAsync(seg_b2, 0, sizeof(long long) * nseg, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(seg_bad, 0, sizeof(unsigned long long) * nseg, st);
   if (e != cudaSuccess) return e;
-  batch_extract_bound_kernel<<<grid_for(n, 256), 256, 0, st>>>(rp, ec, lam, n, fb, seg_off, nseg, x2,
+  batch_extract_bound_kernel<<<grid_for((long long)n * kRowLanes, 256), 256, 0, st>>>(rp, ec, lam, n, fb, seg_off, nseg, x2,
                                                                seg_b2, seg_bad, seg_write);
   count_launch();
   return cudaGetLastError();
