@@ -693,8 +693,8 @@ def f2m_features(xy, stream=None, device=None):
         xy_t = torch.as_tensor(np.asarray(xy, np.int32) if not hasattr(xy, "data_ptr") else xy,
                                device=device).to(torch.int32).contiguous()
         n = int(xy_t.shape[0])
-        feat = torch.zeros((n, 16), dtype=torch.float32, device=device)
-        scale = torch.zeros(n, dtype=torch.float32, device=device)
+        feat = torch.empty((n, 16), dtype=torch.float32, device=device)
+        scale = torch.empty(n, dtype=torch.float32, device=device)
         _gcheck(load().f2m_features(xy_t.data_ptr(), n, feat.data_ptr(), scale.data_ptr(),
                                     _stream_handle(stream)))
         return feat, scale

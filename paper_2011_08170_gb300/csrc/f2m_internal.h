@@ -464,10 +464,11 @@ cudaError_t launch_double(const int32_t* lam_in, int32_t* lam_out, int32_t n, cu
 // ---- k nearest neighbours and warm-start features (knn.cu) -------------------------
 constexpr int kKnnMax = 32;    // largest k of the k-NN kernel
 constexpr int kFeatures = 16;  // neighbour distances per node in the warm-start features
-// exact k-NN lists (ties by index): nbr [n][k], d2 [n][k] (may be NULL); device pointers
+// exact k-NN lists (ties by index): nbr [n][k], d2 [n][k] (may be NULL); device
+// pointers.  All three synchronise: their work space goes back to the cache.
 cudaError_t knn_device(const int2* d_xy, int32_t n, int32_t k, int32_t* d_nbr, long long* d_d2,
                        cudaStream_t st);
-// symmetrised k-NN CSR; d_col holds up to 2 n k entries; *nnz_out on the host (synchronises)
+// symmetrised k-NN CSR; d_col holds up to 2 n k entries; *nnz_out on the host
 cudaError_t knn_csr_device(const int2* d_xy, int32_t n, int32_t k, int32_t* d_row_ptr, int32_t* d_col,
                            int64_t* nnz_out, cudaStream_t st);
 // feat [n][16] = sorted 16-NN distances / s, s = max(1, their mean)

@@ -40,15 +40,16 @@ bool is_device_ptr(const void* p) {
 
 // A caller array seen from the device: the pointer itself if it is device
 // memory, else a stream-ordered staging copy (copied in on request, copied back
-// by flush()).
+// by flush()).  pooled: the copy comes from the library's cache of blocks, for
+// calls that wait for the stream before they return (they set synced).
 template <typename T>
 struct DevView {
   T* user = nullptr;
   T* d = nullptr;
   size_t count = 0;
-  bool staged = false;
+  bool staged = false, pooled = false, synced = false;
   cudaStream_t st = nullptr;
-  cudaError_t open(T* p, size_t cnt, bool copy_in, cudaStream_t s) {
+  cudaError_t open(T* p, size_t cnt, bool copy_in, cudaStream_t s, bool from_pool = false) {
     user = p;
     count = cnt;
     st = s;
@@ -57,7 +58,8 @@ struct DevView {
       return cudaSuccess;
     }
     staged = true;
-    cudaError_t e = cudaMallocAsync((void**)&d, sizeof(T) * (cnt ? cnt : 1), s);
+    pooled = from_pool;
+    cudaError_t e = pooled ? dalloc(&d, (int64_t)cnt) : cudaMallocAsync((void**)&d, sizeof(T) * (cnt ? cnt : 1), s);
     if (e == cudaSuccess && copy_in && cnt)
       e = cudaMemcpyAsync(d, p, sizeof(T) * cnt, cudaMemcpyHostToDevice, s);
     return e;
@@ -67,7 +69,10 @@ struct DevView {
     return cudaMemcpyAsync(user, d, sizeof(T) * count, cudaMemcpyDeviceToHost, st);
   }
   ~DevView() {
-    if (staged && d) cudaFreeAsync(d, st);
+    if (!staged || !d) return;
+    if (!pooled) cudaFreeAsync(d, st);
+    else if (synced) dfree_synced(d);
+    else dfree(d);
   }
 };
 
@@ -115,19 +120,18 @@ extern "C" f2m_status f2m_knn(const int32_t* xy, int32_t n, int32_t k, int32_t* 
   DevView<int2> vxy;
   DevView<int32_t> vn;
   DevView<int64_t> vd;
-  cudaError_t e = vxy.open((int2*)xy, n, true, st);
-  if (e == cudaSuccess) e = vn.open(nbr, (size_t)n * k, false, st);
-  if (e == cudaSuccess && d2) e = vd.open(d2, (size_t)n * k, false, st);
+  cudaError_t e = vxy.open((int2*)xy, n, true, st, true);
+  if (e == cudaSuccess) e = vn.open(nbr, (size_t)n * k, false, st, true);
+  if (e == cudaSuccess && d2) e = vd.open(d2, (size_t)n * k, false, st, true);
   if (e != cudaSuccess) return cuda_fail(nullptr, e, "f2m_knn: buffers");
   // coordinates must be inside the grid
-  CheckCtl* ctl = nullptr;
-  e = cudaMallocAsync((void**)&ctl, sizeof(CheckCtl), st);
   CheckCtl h{0, 0x7fffffff};
-  if (e == cudaSuccess) e = cudaMemcpyAsync(ctl, &h, sizeof h, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = launch_check_points(vxy.d, n, ctl, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&h, ctl, sizeof h, cudaMemcpyDeviceToHost, st);
+  DevView<CheckCtl> ctl;
+  e = ctl.open(&h, 1, true, st, true);
+  if (e == cudaSuccess) e = launch_check_points(vxy.d, n, ctl.d, st);
+  if (e == cudaSuccess) e = ctl.flush();
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  cudaFreeAsync(ctl, st);
+  ctl.synced = e == cudaSuccess;
   if (e != cudaSuccess) return cuda_fail(nullptr, e, "f2m_knn: check");
   if (h.flags) return fail(nullptr, F2M_ERR_INVALID_ARG, "coordinate outside [0, 2^20) at node " + std::to_string(h.first_bad));
   e = knn_device(vxy.d, n, k, vn.d, d2 ? (long long*)vd.d : nullptr, st);
@@ -135,6 +139,7 @@ extern "C" f2m_status f2m_knn(const int32_t* xy, int32_t n, int32_t k, int32_t* 
   if (e == cudaSuccess && d2) e = vd.flush();
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return cuda_fail(nullptr, e, "f2m_knn");
+  vxy.synced = vn.synced = vd.synced = true;
   return F2M_OK;
 }
 
@@ -146,18 +151,17 @@ extern "C" f2m_status f2m_knn_csr(const int32_t* xy, int32_t n, int32_t k, int32
   cudaStream_t st = (cudaStream_t)stream;
   DevView<int2> vxy;
   DevView<int32_t> vrp, vcol;
-  cudaError_t e = vxy.open((int2*)xy, n, true, st);
-  if (e == cudaSuccess) e = vrp.open(row_ptr, (size_t)n + 1, false, st);
-  if (e == cudaSuccess) e = vcol.open(col, 2 * (size_t)n * k, false, st);
+  cudaError_t e = vxy.open((int2*)xy, n, true, st, true);
+  if (e == cudaSuccess) e = vrp.open(row_ptr, (size_t)n + 1, false, st, true);
+  if (e == cudaSuccess) e = vcol.open(col, 2 * (size_t)n * k, false, st, true);
   if (e != cudaSuccess) return cuda_fail(nullptr, e, "f2m_knn_csr: buffers");
-  CheckCtl* ctl = nullptr;
-  e = cudaMallocAsync((void**)&ctl, sizeof(CheckCtl), st);
   CheckCtl h{0, 0x7fffffff};
-  if (e == cudaSuccess) e = cudaMemcpyAsync(ctl, &h, sizeof h, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = launch_check_points(vxy.d, n, ctl, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&h, ctl, sizeof h, cudaMemcpyDeviceToHost, st);
+  DevView<CheckCtl> ctl;
+  e = ctl.open(&h, 1, true, st, true);
+  if (e == cudaSuccess) e = launch_check_points(vxy.d, n, ctl.d, st);
+  if (e == cudaSuccess) e = ctl.flush();
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  cudaFreeAsync(ctl, st);
+  ctl.synced = e == cudaSuccess;
   if (e != cudaSuccess) return cuda_fail(nullptr, e, "f2m_knn_csr: check");
   if (h.flags) return fail(nullptr, F2M_ERR_INVALID_ARG, "coordinate outside [0, 2^20) at node " + std::to_string(h.first_bad));
   int64_t m = 0;
@@ -170,6 +174,7 @@ extern "C" f2m_status f2m_knn_csr(const int32_t* xy, int32_t n, int32_t k, int32
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return cuda_fail(nullptr, e, "f2m_knn_csr");
   *nnz = m;
+  vxy.synced = vrp.synced = vcol.synced = true;
   return F2M_OK;
 }
 
@@ -179,18 +184,17 @@ extern "C" f2m_status f2m_features(const int32_t* xy, int32_t n, float* feat, fl
   cudaStream_t st = (cudaStream_t)stream;
   DevView<int2> vxy;
   DevView<float> vf, vs;
-  cudaError_t e = vxy.open((int2*)xy, n, true, st);
-  if (e == cudaSuccess) e = vf.open(feat, (size_t)n * kFeatures, false, st);
-  if (e == cudaSuccess) e = vs.open(scale, (size_t)n, false, st);
+  cudaError_t e = vxy.open((int2*)xy, n, true, st, true);
+  if (e == cudaSuccess) e = vf.open(feat, (size_t)n * kFeatures, false, st, true);
+  if (e == cudaSuccess) e = vs.open(scale, (size_t)n, false, st, true);
   if (e != cudaSuccess) return cuda_fail(nullptr, e, "f2m_features: buffers");
-  CheckCtl* ctl = nullptr;
-  e = cudaMallocAsync((void**)&ctl, sizeof(CheckCtl), st);
   CheckCtl h{0, 0x7fffffff};
-  if (e == cudaSuccess) e = cudaMemcpyAsync(ctl, &h, sizeof h, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = launch_check_points(vxy.d, n, ctl, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&h, ctl, sizeof h, cudaMemcpyDeviceToHost, st);
+  DevView<CheckCtl> ctl;
+  e = ctl.open(&h, 1, true, st, true);
+  if (e == cudaSuccess) e = launch_check_points(vxy.d, n, ctl.d, st);
+  if (e == cudaSuccess) e = ctl.flush();
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  cudaFreeAsync(ctl, st);
+  ctl.synced = e == cudaSuccess;
   if (e != cudaSuccess) return cuda_fail(nullptr, e, "f2m_features: check");
   if (h.flags) return fail(nullptr, F2M_ERR_INVALID_ARG, "coordinate outside [0, 2^20) at node " + std::to_string(h.first_bad));
   e = features_device(vxy.d, n, vf.d, vs.d, st);
@@ -198,6 +202,7 @@ extern "C" f2m_status f2m_features(const int32_t* xy, int32_t n, float* feat, fl
   if (e == cudaSuccess) e = vs.flush();
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return cuda_fail(nullptr, e, "f2m_features");
+  vxy.synced = vf.synced = vs.synced = true;
   return F2M_OK;
 }
 
