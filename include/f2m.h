@@ -431,6 +431,11 @@ f2m_status f2m_create_batch(int32_t count, const int32_t* n, const int32_t* xy,
                             const int32_t* row_ptr, const int32_t* col, const f2m_params* params,
                             void* stream, f2m_batch** out);
 
+/* The same from one host array per instance and kind: xy[i], row_ptr[i], col[i]. */
+f2m_status f2m_create_batch_parts(int32_t count, const int32_t* n, const int32_t* const* xy,
+                                  const int32_t* const* row_ptr, const int32_t* const* col,
+                                  const f2m_params* params, void* stream, f2m_batch** out);
+
 /* Solves every instance.  info: NULL or [count] (host) per-instance results
  * (augmentations = -1: counted for the batch only); total: NULL or the batch
  * totals (ms_* for the whole batch, iterations = sum of sweeps, frac_bits = -1).

@@ -46,7 +46,7 @@ F2M_GDP_KERNEL_BATCH_TILES = 8
 EXPORTS = ["f2m_default_params", "f2m_create", "f2m_destroy", "f2m_set_lambda", "f2m_solve",
            "f2m_gdp", "f2m_price", "f2m_add_edges", "f2m_extract", "f2m_get_lambda",
            "f2m_get_bound", "f2m_get_x", "f2m_status_string", "f2m_last_error",
-           "f2m_kernel_launches", "f2m_gdp_noalloc", "f2m_create_batch", "f2m_solve_batch",
+           "f2m_kernel_launches", "f2m_gdp_noalloc", "f2m_create_batch", "f2m_create_batch_parts", "f2m_solve_batch",
            "f2m_batch_get_lambda", "f2m_batch_get_x", "f2m_batch_last_error", "f2m_destroy_batch",
            "f2m_knn", "f2m_knn_csr", "f2m_features", "f2m_mlp_create", "f2m_mlp_destroy",
            "f2m_mlp_get_params", "f2m_mlp_last_error", "f2m_mlp_forward", "f2m_mlp_grad",
@@ -152,6 +152,7 @@ def load(path: str = LIB_PATH):
     L.f2m_gdp_noalloc.argtypes = [vp, vp, i64, i32, i32, i32, i64, vp, C.POINTER(i64),
                                   C.POINTER(i64), vp, C.c_char_p, i64]
     L.f2m_gdp_noalloc.restype = C.c_int
+    L.f2m_create_batch_parts.argtypes = [i32, vp, vp, vp, vp, C.POINTER(f2m_params), vp, C.POINTER(vp)]
     L.f2m_create_batch.argtypes = [i32, vp, vp, vp, vp, C.POINTER(f2m_params), vp, C.POINTER(vp)]
     L.f2m_create_batch.restype = C.c_int
     L.f2m_solve_batch.argtypes = [vp, vp, C.POINTER(f2m_info)]
@@ -555,20 +556,39 @@ def _bcheck(b, st):
         raise F2MError(st, f"{name}: {(msg or b'').decode()}")
 
 
-def f2m_create_batch(instances, params: f2m_params | None = None, stream=None) -> Batch:
-    """instances: list of (xy [n, 2], row_ptr [n + 1], col [nnz]) numpy arrays."""
-    L = load()
-    ns = np.array([len(rp) - 1 for _, rp, _ in instances], dtype=np.int32)
-    xy = np.ascontiguousarray(np.concatenate([np.asarray(x, np.int32).reshape(-1, 2) for x, _, _ in instances]))
-    rp = np.ascontiguousarray(np.concatenate([np.asarray(r, np.int32) for _, r, _ in instances]))
-    col = np.ascontiguousarray(np.concatenate([np.asarray(c, np.int32) for _, _, c in instances]))
-    h = C.c_void_p()
-    st = L.f2m_create_batch(len(ns), ns.ctypes.data, xy.ctypes.data, rp.ctypes.data, col.ctypes.data,
-                            C.byref(params) if params is not None else None, _stream_handle(stream),
-                            C.byref(h))
+def _new_batch(st, h, ns):
     if st != F2M_OK:
+        L = load()
         raise F2MError(st, f"{L.f2m_status_string(st).decode()}: {L.f2m_last_error(None).decode()}")
     return Batch(h.value, ns)
+
+
+def f2m_create_batch(instances, params: f2m_params | None = None, stream=None) -> Batch:
+    """instances: list of (xy [n, 2], row_ptr [n + 1], col [nnz]) numpy arrays."""
+    arrays = [[np.ascontiguousarray(a, np.int32) for a in t] for t in instances]
+    if all(r.ndim == 1 and r.size > 1 and x.size == 2 * (r.size - 1) and c.size == r[-1] for x, r, c in arrays):
+        return f2m_create_batch_parts(arrays, params, stream)
+    # sizes that do not fit: the checks of the union say where
+    ns = np.array([len(rp) - 1 for _, rp, _ in arrays], dtype=np.int32)
+    xy, rp, col = [np.concatenate([t[j].reshape(shape) if shape else t[j] for t in arrays])
+                   for j, shape in enumerate([(-1, 2), None, None])]
+    h = C.c_void_p()
+    st = load().f2m_create_batch(len(ns), ns.ctypes.data, xy.ctypes.data, rp.ctypes.data, col.ctypes.data,
+                                 C.byref(params) if params is not None else None, _stream_handle(stream), C.byref(h))
+    return _new_batch(st, h, ns)
+
+
+def f2m_create_batch_parts(instances, params: f2m_params | None = None, stream=None) -> Batch:
+    """f2m_create_batch from contiguous int32 arrays whose sizes fit, one of each
+    kind per instance."""
+    ns = np.array([r.size - 1 for _, r, _ in instances], dtype=np.int32)
+    at = np.array([[a.__array_interface__["data"][0] for a in t] for t in instances], np.uintp).reshape(-1, 3)
+    ptrs = [np.ascontiguousarray(at[:, j]) for j in range(3)]
+    h = C.c_void_p()
+    st = load().f2m_create_batch_parts(len(ns), ns.ctypes.data, *[q.ctypes.data for q in ptrs],
+                                       C.byref(params) if params is not None else None, _stream_handle(stream),
+                                       C.byref(h))
+    return _new_batch(st, h, ns)
 
 
 def f2m_solve_batch(b: Batch, raise_on_error: bool = True):
@@ -677,12 +697,12 @@ def f2m_knn_csr(xy, k: int, stream=None):
     """(row_ptr, col) of the symmetrised k-NN candidate graph."""
     xy = np.ascontiguousarray(xy, dtype=np.int32)
     n = xy.shape[0]
-    rp = np.zeros(n + 1, np.int32)
-    col = np.zeros(2 * n * k, np.int32)
+    rp = np.empty(n + 1, np.int32)
+    col = np.empty(2 * n * k, np.int32)  # only the pages of the entries are ever touched
     nnz = C.c_int64()
     _gcheck(load().f2m_knn_csr(xy.ctypes.data, n, k, rp.ctypes.data, col.ctypes.data, C.byref(nnz),
                                _stream_handle(stream)))
-    return rp, col[:nnz.value].copy()
+    return rp, col[:nnz.value]
 
 
 def f2m_features(xy, stream=None, device=None):

@@ -47,6 +47,9 @@ std::multimap<size_t, void*> g_pin_free;       // size -> cached block
 std::map<void*, size_t> g_pin_size;            // every block handed out or cached
 size_t g_pin_cached = 0;
 constexpr size_t kPinCacheMax = (size_t)1 << 31;
+}  // namespace
+
+namespace f2m {
 
 cudaError_t pin_alloc(void** p, size_t bytes) {
   if (bytes == 0) bytes = 1;
@@ -81,6 +84,10 @@ void pin_free(void* p) {
     g_pin_size.erase(it);
   }
 }
+
+}  // namespace f2m
+
+namespace {
 
 // Device blocks: creating a context makes about sixty allocations, each
 // costing more than the kernel that fills it, so freed blocks are kept per
@@ -465,8 +472,7 @@ f2m_status f2m::create_internal(const int32_t* xy, int32_t n, const int32_t* row
     if (e == cudaSuccess) e = plan_build(c->d_rp, c->d_ec, n, c->nnz, c->plan, c->st);
     if (e == cudaSuccess && p.finisher) {
       e = alloc_finisher_buffers(c, c->ec_cap);
-      c->fin_work = finisher_work_new();
-      finisher_work_reserve(c->fin_work, n);
+      c->fin_work = finisher_work_take(n);
     }
     if (e == cudaSuccess) e = dalloc(&c->d_x2, c->ec_cap);
     c->x2_cap = c->ec_cap;
@@ -1294,7 +1300,7 @@ f2m_status f2m::finisher_internal(f2m_ctx* c, int64_t* aug, const uint8_t* h_inc
   GdpPlan& P = c->plan;
   const int32_t nseg = (int32_t)c->seg_off.size() - 1;
   if (c->fin_cap < c->nnz) CK(c, alloc_finisher_buffers(c, c->ec_cap));
-  if (!c->fin_work) c->fin_work = finisher_work_new();
+  if (!c->fin_work) c->fin_work = finisher_work_take(n);
   // the host mirror for this call; on any return the stream is drained
   // before the next call may take the mirror (no copy still reads or writes it)
   std::unique_lock<std::mutex> mirror_lock(g_mirror.mu);

@@ -121,27 +121,27 @@ extern "C" void f2m_destroy_batch(f2m_batch* b) {
   if (b->u) f2m_destroy(b->u);
   dfree(b->d_active); dfree(b->d_seg_ch); dfree(b->d_seg_sweeps); dfree(b->d_tiles); dfree(b->d_e1);
   dfree(b->d_snap_eoff); dfree(b->d_snap_done); dfree(b->d_snap_ent);
-  if (b->h_snap) cudaFreeHost(b->h_snap);
-  if (b->h_irp) cudaFreeHost(b->h_irp);
+  pin_free(b->h_snap);
+  pin_free(b->h_irp);
   dfree(b->d_chunk);
-  if (b->h_tiles) cudaFreeHost(b->h_tiles);
-  if (b->h_e1) cudaFreeHost(b->h_e1);
-  if (b->h_chunk) cudaFreeHost(b->h_chunk);
+  pin_free(b->h_tiles);
+  pin_free(b->h_e1);
+  pin_free(b->h_chunk);
   dfree(b->d_seg_b2); dfree(b->d_seg_bad); dfree(b->d_tmp_a);
   dfree(b->d_mask); dfree(b->d_res_lam); dfree(b->d_res_rp); dfree(b->d_res_ec); dfree(b->d_res_x2);
   if (b->gexec) cudaGraphExecDestroy(b->gexec);
   if (b->gs) cudaStreamDestroy(b->gs);
   if (b->e_in) cudaEventDestroy(b->e_in);
   if (b->e_out) cudaEventDestroy(b->e_out);
-  if (b->h_active) cudaFreeHost(b->h_active);
-  if (b->h_ctl) cudaFreeHost(b->h_ctl);
-  if (b->h_sw) cudaFreeHost(b->h_sw);
-  if (b->h_still) cudaFreeHost(b->h_still);
+  pin_free(b->h_active);
+  pin_free(b->h_ctl);
+  pin_free(b->h_sw);
+  pin_free(b->h_still);
   dfree(b->d_rlist);
-  if (b->h_rseg) cudaFreeHost(b->h_rseg);
+  pin_free(b->h_rseg);
   dfree(b->d_pk); dfree(b->d_cl_all); dfree(b->d_cl_list); dfree(b->d_cl_out);
-  if (b->h_cl_list) cudaFreeHost(b->h_cl_list);
-  if (b->h_cl_out) cudaFreeHost(b->h_cl_out);
+  pin_free(b->h_cl_list);
+  pin_free(b->h_cl_out);
   for (cudaStream_t& q : b->cl_st)
     if (q) cudaStreamDestroy(q);
   for (cudaEvent_t& q : b->cl_ev)
@@ -168,13 +168,25 @@ extern "C" f2m_status f2m_create_batch(int32_t count, const int32_t* n, const in
   // per-instance entry counts: the last offset of each local row_ptr
   std::vector<int32_t> eoff(count + 1, 0);
   {
-    std::vector<int32_t> rp_all(N + count);
-    cudaError_t e = cudaMemcpyAsync(rp_all.data(), row_ptr, sizeof(int32_t) * (N + count),
-                                    cudaMemcpyDefault, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) return cuda_fail(nullptr, e, "create_batch: read row_ptr");
+    cudaPointerAttributes where;
+    const bool known = cudaPointerGetAttributes(&where, row_ptr) == cudaSuccess;
+    if (!known) cudaGetLastError();
+    const bool host = known && (where.type == cudaMemoryTypeHost || where.type == cudaMemoryTypeUnregistered);
+    std::vector<int32_t> rp_all;
+    if (host) {
+      // what was copied here is read in stream order: so are the caller's writes
+      cudaError_t e = where.type == cudaMemoryTypeHost ? cudaStreamSynchronize(st) : cudaSuccess;
+      if (e != cudaSuccess) return cuda_fail(nullptr, e, "create_batch: read row_ptr");
+    } else {
+      rp_all.resize(N + count);
+      cudaError_t e = cudaMemcpyAsync(rp_all.data(), row_ptr, sizeof(int32_t) * (N + count),
+                                      cudaMemcpyDefault, st);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+      if (e != cudaSuccess) return cuda_fail(nullptr, e, "create_batch: read row_ptr");
+    }
+    const int32_t* rps = host ? row_ptr : rp_all.data();
     for (int32_t s = 0; s < count; ++s) {
-      const int64_t nz = rp_all[seg_off[s + 1] + s];
+      const int64_t nz = rps[seg_off[s + 1] + s];
       if (nz < 0 || (int64_t)eoff[s] + nz >= INT32_MAX)
         return fail(nullptr, F2M_ERR_INVALID_ARG, "instance " + std::to_string(s) + ": bad row_ptr");
       eoff[s + 1] = eoff[s] + (int32_t)nz;
@@ -234,11 +246,11 @@ extern "C" f2m_status f2m_create_batch(int32_t count, const int32_t* n, const in
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->gs, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->e_in, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->e_out, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaMallocHost((void**)&b->h_active, count);
-    if (e == cudaSuccess) e = cudaMallocHost((void**)&b->h_ctl, sizeof(GdpCtl));
-    if (e == cudaSuccess) e = cudaMallocHost((void**)&b->h_sw, sizeof(long long) * count);
-    if (e == cudaSuccess) e = cudaMallocHost((void**)&b->h_still, count);
-    if (e == cudaSuccess) e = cudaMallocHost((void**)&b->h_chunk, sizeof(BatchChunk));
+    if (e == cudaSuccess) e = pin_alloc((void**)&b->h_active, count);
+    if (e == cudaSuccess) e = pin_alloc((void**)&b->h_ctl, sizeof(GdpCtl));
+    if (e == cudaSuccess) e = pin_alloc((void**)&b->h_sw, sizeof(long long) * count);
+    if (e == cudaSuccess) e = pin_alloc((void**)&b->h_still, count);
+    if (e == cudaSuccess) e = pin_alloc((void**)&b->h_chunk, sizeof(BatchChunk));
     if (e == cudaSuccess) e = dalloc(&b->d_chunk, 1);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) { f2m_destroy_batch(b); s = cuda_fail(nullptr, e, "create_batch: setup"); break; }
@@ -246,6 +258,49 @@ extern "C" f2m_status f2m_create_batch(int32_t count, const int32_t* n, const in
   } while (0);
   dfree(d_rpl); dfree(d_coll); dfree(d_rp); dfree(d_col); dfree(d_so); dfree(d_eo); dfree(d_chk);
   return s;
+}
+
+extern "C" f2m_status f2m_create_batch_parts(int32_t count, const int32_t* n, const int32_t* const* xy,
+                                             const int32_t* const* row_ptr, const int32_t* const* col,
+                                             const f2m_params* params, void* stream, f2m_batch** out) {
+  if (!out) return fail(nullptr, F2M_ERR_INVALID_ARG, "out is NULL");
+  *out = nullptr;
+  if (count < 1 || !n || !xy || !row_ptr || !col)
+    return fail(nullptr, F2M_ERR_INVALID_ARG, "count < 1 or NULL array");
+  int64_t N = 0, nnz = 0;
+  for (int32_t s = 0; s < count; ++s) {
+    if (!xy[s] || !row_ptr[s] || !col[s]) return fail(nullptr, F2M_ERR_INVALID_ARG, "NULL array");
+    if (n[s] < 4) return fail(nullptr, F2M_ERR_INVALID_ARG, "instance " + std::to_string(s) + ": n < 4");
+    if (N + n[s] >= (1 << 24)) return fail(nullptr, F2M_ERR_INVALID_ARG, "total nodes must stay below 2^24");
+    N += n[s];
+  }
+  for (int32_t s = 0; s < count; ++s) {
+    const int64_t nz = row_ptr[s][n[s]];
+    if (nz < 0 || nnz + nz >= INT32_MAX)
+      return fail(nullptr, F2M_ERR_INVALID_ARG, "instance " + std::to_string(s) + ": bad row_ptr");
+    nnz += nz;
+  }
+  // back to back in one pinned block (an array of its own for the three would
+  // be touched anew on each call)
+  int32_t* h = nullptr;
+  const cudaError_t e = pin_alloc((void**)&h, sizeof(int32_t) * (size_t)(3 * N + count + nnz));
+  if (e != cudaSuccess) return cuda_fail(nullptr, e, "create_batch: staging");
+  int32_t *hx = h, *hr = h + 2 * N, *hc = hr + N + count, *x = hx, *r = hr, *q = hc;
+  std::vector<HostCopy> parts;
+  for (int32_t s = 0; s < count; ++s) {
+    const size_t nz = (size_t)row_ptr[s][n[s]];
+    parts.push_back({x, xy[s], sizeof(int32_t) * 2 * (size_t)n[s]});
+    parts.push_back({r, row_ptr[s], sizeof(int32_t) * ((size_t)n[s] + 1)});
+    parts.push_back({q, col[s], sizeof(int32_t) * nz});
+    x += 2 * (int64_t)n[s];
+    r += n[s] + 1;
+    q += nz;
+  }
+  host_copy(parts);
+  const f2m_status st = f2m_create_batch(count, n, hx, hr, hc, params, stream, out);
+  if (st != F2M_OK) cudaStreamSynchronize((cudaStream_t)stream);  // copies of a refused call may be under way
+  pin_free(h);
+  return st;
 }
 
 constexpr int32_t kBatchTileRows = 960;  // rows a tile: 15 warps of 2 slices
@@ -257,7 +312,7 @@ constexpr int32_t kBatchTileRows = 960;  // rows a tile: 15 warps of 2 slices
 static f2m_status batch_tiles(f2m_batch* b, int te, int tn, std::vector<int4>& tiles, std::vector<int32_t>& e1) {
   f2m_ctx* c = b->u;
   GdpPlan& P = c->plan;
-  if (!b->h_irp) CK(c, cudaMallocHost((void**)&b->h_irp, sizeof(int32_t) * (c->n + 1)));
+  if (!b->h_irp) CK(c, pin_alloc((void**)&b->h_irp, sizeof(int32_t) * (c->n + 1)));
   const int32_t* irp = b->h_irp;
   CK(c, cudaMemcpyAsync(b->h_irp, P.irp, sizeof(int32_t) * (c->n + 1), cudaMemcpyDeviceToHost, c->st));
   CK(c, cudaStreamSynchronize(c->st));
@@ -310,16 +365,16 @@ static f2m_status batch_list_reserve(f2m_batch* b, int32_t need) {
   if (need <= b->tiles_cap) return F2M_OK;
   CK(c, cudaStreamSynchronize(c->st));
   CK(c, cudaStreamSynchronize(b->gs));
-  if (b->h_tiles) cudaFreeHost(b->h_tiles);
-  if (b->h_e1) cudaFreeHost(b->h_e1);
+  pin_free(b->h_tiles);
+  pin_free(b->h_e1);
   b->h_tiles = nullptr;
   b->h_e1 = nullptr;
   dfree(b->d_tiles);
   dfree(b->d_e1);
   b->tiles_cap = 0;
   const int32_t cap = need + need / 8 + 64;
-  CK(c, cudaMallocHost((void**)&b->h_tiles, sizeof(int4) * cap));
-  CK(c, cudaMallocHost((void**)&b->h_e1, sizeof(int32_t) * cap));
+  CK(c, pin_alloc((void**)&b->h_tiles, sizeof(int4) * cap));
+  CK(c, pin_alloc((void**)&b->h_e1, sizeof(int32_t) * cap));
   CK(c, dalloc(&b->d_tiles, cap));
   CK(c, dalloc(&b->d_e1, cap));
   b->tiles_cap = cap;
@@ -508,8 +563,8 @@ static f2m_status cluster_plan(f2m_batch* b) {
     CK(c, dalloc(&b->d_cl_all, K));
     CK(c, dalloc(&b->d_cl_list, K));
     CK(c, dalloc(&b->d_cl_out, K));
-    CK(c, cudaMallocHost((void**)&b->h_cl_list, sizeof(ClusterInst) * K));
-    CK(c, cudaMallocHost((void**)&b->h_cl_out, sizeof(ClusterOut) * K));
+    CK(c, pin_alloc((void**)&b->h_cl_list, sizeof(ClusterInst) * K));
+    CK(c, pin_alloc((void**)&b->h_cl_out, sizeof(ClusterOut) * K));
     for (cudaStream_t& q : b->cl_st) CK(c, cudaStreamCreateWithFlags(&q, cudaStreamNonBlocking));
     for (cudaEvent_t& q : b->cl_ev) CK(c, cudaEventCreateWithFlags(&q, cudaEventDisableTiming));
   }
@@ -604,7 +659,7 @@ static f2m_status batch_ring_phase(f2m_batch* b, const std::vector<uint8_t>& act
     b->rlist_cap = tiles + tiles / 8 + 64;
     CK(c, dalloc(&b->d_rlist, b->rlist_cap));
   }
-  if (!b->h_rseg) CK(c, cudaMallocHost((void**)&b->h_rseg, sizeof(RingSeg) * b->count));
+  if (!b->h_rseg) CK(c, pin_alloc((void**)&b->h_rseg, sizeof(RingSeg) * b->count));
   CK(c, cudaMemcpyAsync(b->d_rlist, list.data(), sizeof(RingTile) * tiles, cudaMemcpyHostToDevice, c->st));
   CK(c, ring_build(c->plan, c->d_seg_off, b->d_rlist, tiles, K, c->p.frac_bits, rows * c->nnz / c->n, c->ring, c->st));
   CK(c, ring_start(c->ring, c->n, b->count, c->st));
@@ -788,7 +843,7 @@ static f2m_status snapshot(f2m_batch* b, const std::vector<uint8_t>& done) {
   int32_t fb = 0;
   const int32_t* lam = cur_lambda(c, &fb);
   if (!b->h_snap) {  // pinned staging: bounds and entry offsets down, mask and arena offsets up
-    CK(c, cudaMallocHost((void**)&b->h_snap, sizeof(long long) * K + sizeof(int32_t) * (K + 1) +
+    CK(c, pin_alloc((void**)&b->h_snap, sizeof(long long) * K + sizeof(int32_t) * (K + 1) +
                                               sizeof(long long) * K + K));
     CK(c, dalloc(&b->d_snap_eoff, K));
     CK(c, dalloc(&b->d_snap_done, K));

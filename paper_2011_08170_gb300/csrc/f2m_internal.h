@@ -424,7 +424,18 @@ FinisherWork* finisher_work_new();
 // call does not wait for them to wake
 void finisher_pool_wake(int32_t threads);
 void finisher_work_reserve(FinisherWork* w, int32_t n);  // host work arrays for n nodes
-void finisher_work_free(FinisherWork* w);
+FinisherWork* finisher_work_take(int32_t n);  // with room for n nodes, from the cache if it has one
+void finisher_work_free(FinisherWork* w);     // back to the cache
+// copies between host arrays, on the finisher's worker threads when they are idle
+struct HostCopy {
+  void* dst;
+  const void* src;
+  size_t bytes;
+};
+void host_copy(const std::vector<HostCopy>& parts);
+// pinned host blocks from a bounded cache (api.cu)
+cudaError_t pin_alloc(void** p, size_t bytes);
+void pin_free(void* p);
 // Min-cost flow on the bipartite double cover, internal node order; see
 // finisher.cpp.  y is the initial flow (updated to the optimal one), exl the
 // left surpluses, lam2 receives pi(L) - pi(R) (F+1 bits).  Blocks and segments
