@@ -22,7 +22,8 @@ struct f2m_mlp {
   float* partial = nullptr;  // per-CTA partial gradients [num_sms][kMlpParams + 1]
   float* grad = nullptr;     // [kMlpParams + 1]
   long long* step = nullptr; // Adam steps taken
-  int* status = nullptr;     // bit 0: a tensor-core wait gave up
+  int* status = nullptr;     // bit 0: a tensor-core wait gave up (the word behind the loss in grad)
+  float* h_out = nullptr;    // pinned: gradient, loss, status
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   std::string err;
 };
@@ -99,12 +100,17 @@ int device_sms() {
   return sms;
 }
 
-f2m_status check_status(f2m_mlp* m) {
+f2m_status status_read(f2m_mlp* m) {  // after a copy of the status word to h_out
   int h = 0;
-  MCK(m, cudaMemcpyAsync(&h, m->status, sizeof(int), cudaMemcpyDeviceToHost, m->st));
-  MCK(m, cudaStreamSynchronize(m->st));
+  memcpy(&h, m->h_out + kMlpParams + 1, sizeof h);
   if (h) return mlp_fail(m, F2M_ERR_TIMEOUT, "a tensor-core completion wait gave up");
   return F2M_OK;
+}
+
+f2m_status check_status(f2m_mlp* m) {
+  MCK(m, cudaMemcpyAsync(m->h_out + kMlpParams + 1, m->status, sizeof(int), cudaMemcpyDeviceToHost, m->st));
+  MCK(m, cudaStreamSynchronize(m->st));
+  return status_read(m);
 }
 
 }  // namespace
@@ -212,7 +218,8 @@ extern "C" void f2m_mlp_destroy(f2m_mlp* m) {
   if (!m) return;
   DevSyncedScope synced;  // one wait for the device, then every block goes to the cache
   dfree(m->master); dfree(m->m1); dfree(m->m2); dfree(m->img); dfree(m->partial);
-  dfree(m->grad); dfree(m->step); dfree(m->status);
+  dfree(m->grad); dfree(m->step);
+  pin_free(m->h_out);
   if (m->ev0) cudaEventDestroy(m->ev0);
   if (m->ev1) cudaEventDestroy(m->ev1);
   delete m;
@@ -236,9 +243,10 @@ extern "C" f2m_status f2m_mlp_create(const float* params, void* stream, f2m_mlp*
   if (e == cudaSuccess) e = dalloc(&m->m2, kMlpParams);
   if (e == cudaSuccess) e = dalloc(&m->img, kMlpImgBytes);
   if (e == cudaSuccess) e = dalloc(&m->partial, (int64_t)(m->num_sms > 0 ? m->num_sms : 1) * (kMlpParams + 1));
-  if (e == cudaSuccess) e = dalloc(&m->grad, kMlpParams + 1);
+  if (e == cudaSuccess) e = dalloc(&m->grad, kMlpParams + 2);
+  if (e == cudaSuccess) m->status = reinterpret_cast<int*>(m->grad + kMlpParams + 1);
+  if (e == cudaSuccess) e = pin_alloc((void**)&m->h_out, sizeof(float) * (kMlpParams + 2));
   if (e == cudaSuccess) e = dalloc(&m->step, 1);
-  if (e == cudaSuccess) e = dalloc(&m->status, 1);
   if (e == cudaSuccess) e = cudaEventCreate(&m->ev0);
   if (e == cudaSuccess) e = cudaEventCreate(&m->ev1);
   if (e != cudaSuccess) {
@@ -292,25 +300,32 @@ extern "C" f2m_status f2m_mlp_grad(f2m_mlp* m, const float* feat, const float* t
                                    float* grad, float* loss) {
   if (!m || !feat || !target || !grad) return mlp_fail(m, F2M_ERR_INVALID_ARG, "NULL argument");
   if (count < 1 || count >= (1LL << 31)) return mlp_fail(m, F2M_ERR_INVALID_ARG, "count must be in [1, 2^31)");
-  DevView<float> vf, vt, vg, vl;
+  DevView<float> vf, vt;
   MCK(m, vf.open((float*)feat, (size_t)count * kFeatures, true, m->st));
   MCK(m, vt.open((float*)target, (size_t)count, true, m->st));
-  MCK(m, vg.open(grad, kMlpParams, false, m->st));
+  // gradient, loss and status lie side by side: one copy, one wait
+  const bool host = !is_device_ptr(grad);
   const int grid = mlp_grid(m->num_sms, count);
   MCK(m, mlp_train_launch(m->img, m->master, vf.d, vt.d, nullptr, 0, count, 2.f / (float)count,
                           m->partial, grid, nullptr, m->status, m->st));
   MlpAdam hp{};
-  MCK(m, mlp_reduce_launch(m->partial, grid, vg.d, m->master, m->m1, m->m2, m->img, nullptr, hp,
+  MCK(m, mlp_reduce_launch(m->partial, grid, host ? m->grad : grad, m->master, m->m1, m->m2, m->img, nullptr, hp,
                            m->grad + kMlpParams, m->st));
-  MCK(m, vg.flush());
+  const int first = host ? 0 : kMlpParams;
+  MCK(m, cudaMemcpyAsync(m->h_out + first, m->grad + first, sizeof(float) * (kMlpParams + 2 - first),
+                         cudaMemcpyDeviceToHost, m->st));
+  MCK(m, cudaStreamSynchronize(m->st));
+  if (host) memcpy(grad, m->h_out, sizeof(float) * kMlpParams);
   if (loss) {
-    float ls = 0.f;
-    MCK(m, cudaMemcpyAsync(&ls, m->grad + kMlpParams, sizeof(float), cudaMemcpyDeviceToHost, m->st));
-    MCK(m, cudaStreamSynchronize(m->st));
-    const float mean = ls / (float)count;
-    MCK(m, cudaMemcpyAsync(loss, &mean, sizeof(float), cudaMemcpyDefault, m->st));
+    const float mean = m->h_out[kMlpParams] / (float)count;
+    if (is_device_ptr(loss)) {
+      MCK(m, cudaMemcpyAsync(loss, &mean, sizeof(float), cudaMemcpyHostToDevice, m->st));
+      MCK(m, cudaStreamSynchronize(m->st));
+    } else {
+      *loss = mean;
+    }
   }
-  return check_status(m);
+  return status_read(m);
 }
 
 extern "C" f2m_status f2m_mlp_train(f2m_mlp* m, const float* feat, const float* target, int64_t count,

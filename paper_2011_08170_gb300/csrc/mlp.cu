@@ -34,6 +34,7 @@ namespace {
 using tc::kmajor_off;
 
 constexpr int kTile = 128;
+constexpr int kTrainThreads = 512;  // four column groups of 32 a sample
 constexpr long long kWaitLimit = 1LL << 24;  // mbarrier polls before giving up
 
 // shared-memory layout of the training kernel (bytes)
@@ -95,7 +96,8 @@ __device__ __forceinline__ void store_col32(uint8_t* tile, int b, int c0, const 
     *reinterpret_cast<unsigned short*>(tile + kmajor_off(c0 + i, b, 128)) = tc::bf16_bits(v[i]);
 }
 
-// features of sample row b into F [128 x 16] (row b) and, if ft, into [F|1]^T (column b)
+// features of sample row b into F [128 x 16] (row b) and into [F|1]^T (column b);
+// either may be NULL
 __device__ __forceinline__ void load_features(const float* __restrict__ feat, long long s, bool valid,
                                               uint8_t* sF, uint8_t* sFT, int b) {
   float f[16];
@@ -111,7 +113,7 @@ __device__ __forceinline__ void load_features(const float* __restrict__ feat, lo
     for (int j = 0; j < 16; ++j) f[j] = 0.f;
   }
 #pragma unroll
-  for (int g = 0; g < 2; ++g) {
+  for (int g = 0; g < (sF ? 2 : 0); ++g) {
     uint4 q;
     q.x = tc::pack_bf16x2(f[8 * g + 0], f[8 * g + 1]);
     q.y = tc::pack_bf16x2(f[8 * g + 2], f[8 * g + 3]);
@@ -249,16 +251,25 @@ mlp_forward_kernel(const uint8_t* __restrict__ img, const float* __restrict__ ma
 }
 
 // --------------------------------------------------------------------------------------
-// forward + backward over the CTA's tiles of one step; partial gradient per CTA
+// forward + backward over the CTA's tiles of one step; partial gradient per CTA.
+//
+// 512 threads: thread (b, grp) owns columns 32 grp .. 32 grp + 31 of sample b in every
+// epilogue (a warp reads the tensor-memory lanes of its number mod 4).  The
+// epilogues bound the kernel (the products of a tile take a microsecond): with one
+// thread a sample, four warps on an SM, the two tiles of a step of 38,912 samples
+// took 53 us, now 36.  The sum over a sample's columns runs through the groups in
+// column order, so that every value has the bits it had.
 // --------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(128, 1)
+__global__ void __launch_bounds__(kTrainThreads, 1)
 mlp_train_kernel(const uint8_t* __restrict__ img, const float* __restrict__ master,
                  const float* __restrict__ feat, const float* __restrict__ target,
                  const int32_t* __restrict__ perm, long long s0, long long count, float two_over_b,
                  float* __restrict__ partial, long long* step_ctr, int* status) {
   extern __shared__ __align__(1024) uint8_t smem[];
   __shared__ int s_abort;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  __shared__ float s_y[kTile];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, b = tid & (kTile - 1), grp = tid / kTile;
+  const int quad = warp & 3;  // its quarter of the tensor-memory lanes
   uint8_t* sW1 = smem + kSW1;
   uint8_t* sW2 = smem + kSW2;
   uint8_t* sW2T = smem + kSW2T;
@@ -282,21 +293,24 @@ mlp_train_kernel(const uint8_t* __restrict__ img, const float* __restrict__ mast
     if (blockIdx.x == 0 && step_ctr) *step_ctr += 1;  // Adam step number read by the reduce kernel
   }
   if (warp == 0) tc::tmem_alloc(tc::smem_u32(tslot), 512);
-  copy16(sW1, img, kImgW1Bytes, tid, 128);
-  copy16(sW2, img + kImgW1Bytes, kImgW2Bytes, tid, 128);
-  copy16(sW2T, img + kImgW1Bytes + kImgW2Bytes, kImgW2Bytes, tid, 128);
-  sb1[tid] = master[kOb1 + tid];
-  sb2[tid] = master[kOb2 + tid];
-  sw3[tid] = master[kOw3 + tid];
+  copy16(sW1, img, kImgW1Bytes, tid, kTrainThreads);
+  copy16(sW2, img + kImgW1Bytes, kImgW2Bytes, tid, kTrainThreads);
+  copy16(sW2T, img + kImgW1Bytes + kImgW2Bytes, kImgW2Bytes, tid, kTrainThreads);
+  if (grp == 0) {
+    sb1[b] = master[kOb1 + b];
+    sb2[b] = master[kOb2 + b];
+    sw3[b] = master[kOw3 + b];
+  }
   const float b3 = master[kOb3];
   // constant rows: the ones row of [H1 | 1]^T (row 128) and [F | 1]^T (row 16),
   // zero rows 129..143, 17..31 and 1..15 of [dY | 0]^T
   const unsigned short one = tc::bf16_bits(1.f);
-  for (int r = 128; r < 144; ++r)
-    *reinterpret_cast<unsigned short*>(sH1T + kmajor_off(r, tid, 128)) = r == 128 ? one : 0;
-  for (int r = 16; r < 32; ++r)
-    *reinterpret_cast<unsigned short*>(sFT + kmajor_off(r, tid, 128)) = r == 16 ? one : 0;
-  for (int r = 1; r < 16; ++r) *reinterpret_cast<unsigned short*>(sDY + kmajor_off(r, tid, 128)) = 0;
+  for (int r = 128 + grp; r < 144; r += kTrainThreads / kTile)
+    *reinterpret_cast<unsigned short*>(sH1T + kmajor_off(r, b, 128)) = r == 128 ? one : 0;
+  for (int r = 16 + grp; r < 32; r += kTrainThreads / kTile)
+    *reinterpret_cast<unsigned short*>(sFT + kmajor_off(r, b, 128)) = r == 16 ? one : 0;
+  for (int r = 1 + grp; r < 16; r += kTrainThreads / kTile)
+    *reinterpret_cast<unsigned short*>(sDY + kmajor_off(r, b, 128)) = 0;
   tc::fence_before();
   __syncthreads();
   tc::fence_after();
@@ -312,10 +326,11 @@ mlp_train_kernel(const uint8_t* __restrict__ img, const float* __restrict__ mast
   bool any = false;
 
   for (long long t0 = (long long)blockIdx.x * kTile; t0 < count; t0 += (long long)gridDim.x * kTile) {
-    const long long pos = t0 + tid;
+    const long long pos = t0 + b;
     const bool valid = pos < count;
     const long long s = valid ? (perm ? (long long)perm[s0 + pos] : s0 + pos) : 0;
-    load_features(feat, s, valid, sF, sFT, tid);
+    if (grp == 0) load_features(feat, s, valid, sF, nullptr, b);
+    if (grp == 1) load_features(feat, s, valid, nullptr, sFT, b);
     const float tgt = valid ? target[s] : 0.f;
     tc::fence_proxy_async();
     __syncthreads();
@@ -326,21 +341,18 @@ mlp_train_kernel(const uint8_t* __restrict__ img, const float* __restrict__ mast
     }
     if (!wait_phase(mbar, phase, &s_abort, status)) break;
     // epilogue 1: z1 -> mask, h1 = bf16(relu(z1)) into H1 (row) and [H1 | 1]^T (column)
-    uint32_t mask1[4];
-#pragma unroll 1
-    for (int q = 0; q < 4; ++q) {
+    uint32_t mask1 = 0;
+    {
       float v[32];
-      tc::tmem_ld32(tmem_at(tmem, warp, kC_D1 + 32 * q), v);
-      uint32_t m = 0;
+      tc::tmem_ld32(tmem_at(tmem, quad, kC_D1 + 32 * grp), v);
 #pragma unroll
       for (int i = 0; i < 32; ++i) {
-        const float z = v[i] + sb1[32 * q + i];
-        m |= (z > 0.f ? 1u : 0u) << i;
+        const float z = v[i] + sb1[32 * grp + i];
+        mask1 |= (z > 0.f ? 1u : 0u) << i;
         v[i] = fmaxf(z, 0.f);
       }
-      mask1[q] = m;
-      store_row32(sR1, tid, 32 * q, v);
-      store_col32(sH1T, tid, 32 * q, v);
+      store_row32(sR1, b, 32 * grp, v);
+      store_col32(sH1T, b, 32 * grp, v);
     }
     tc::fence_before();
     tc::fence_proxy_async();
@@ -352,35 +364,42 @@ mlp_train_kernel(const uint8_t* __restrict__ img, const float* __restrict__ mast
     }
     if (!wait_phase(mbar, phase, &s_abort, status)) break;
     // epilogue 2: y, dy; h2 into H2^T; dz2 = bf16(dy w3 [z2 > 0]) into dZ2 (row) and dZ2^T (column)
-    float y = b3;
-    uint32_t mask2[4];
-#pragma unroll 1
-    for (int q = 0; q < 4; ++q) {
+    uint32_t mask2 = 0;
+    {
       float v[32];
-      tc::tmem_ld32(tmem_at(tmem, warp, kC_D2 + 32 * q), v);
-      uint32_t m = 0;
+      tc::tmem_ld32(tmem_at(tmem, quad, kC_D2 + 32 * grp), v);
 #pragma unroll
       for (int i = 0; i < 32; ++i) {
-        const float z = v[i] + sb2[32 * q + i];
-        m |= (z > 0.f ? 1u : 0u) << i;
+        const float z = v[i] + sb2[32 * grp + i];
+        mask2 |= (z > 0.f ? 1u : 0u) << i;
         v[i] = fmaxf(z, 0.f);
-        y = fmaf(v[i], sw3[32 * q + i], y);
       }
-      mask2[q] = m;
-      store_col32(sH2T, tid, 32 * q, v);
+      store_col32(sH2T, b, 32 * grp, v);
+#pragma unroll 1
+      for (int g = 0; g < kTrainThreads / kTile; ++g) {
+        if (g == grp) {
+          float y = g ? s_y[b] : b3;
+#pragma unroll
+          for (int i = 0; i < 32; ++i) y = fmaf(v[i], sw3[32 * grp + i], y);
+          s_y[b] = y;
+        }
+        __syncthreads();
+      }
     }
+    const float y = s_y[b];
     const float r = valid ? y - tgt : 0.f;
     const float dy = two_over_b * r;
-    loss = fmaf(r, r, loss);
-    db3 += dy;
-    *reinterpret_cast<unsigned short*>(sDY + kmajor_off(0, tid, 128)) = tc::bf16_bits(dy);
-#pragma unroll 1
-    for (int q = 0; q < 4; ++q) {
+    if (grp == 0) {
+      loss = fmaf(r, r, loss);
+      db3 += dy;
+      *reinterpret_cast<unsigned short*>(sDY + kmajor_off(0, b, 128)) = tc::bf16_bits(dy);
+    }
+    {
       float v[32];
 #pragma unroll
-      for (int i = 0; i < 32; ++i) v[i] = ((mask2[q] >> i) & 1u) ? dy * sw3[32 * q + i] : 0.f;
-      store_row32(sR1, tid, 32 * q, v);  // D2 is complete: H1 is no longer needed as an operand
-      store_col32(sR2, tid, 32 * q, v);
+      for (int i = 0; i < 32; ++i) v[i] = ((mask2 >> i) & 1u) ? dy * sw3[32 * grp + i] : 0.f;
+      store_row32(sR1, b, 32 * grp, v);  // D2 is complete: H1 is no longer needed as an operand
+      store_col32(sR2, b, 32 * grp, v);
     }
     tc::fence_before();
     tc::fence_proxy_async();
@@ -394,13 +413,12 @@ mlp_train_kernel(const uint8_t* __restrict__ img, const float* __restrict__ mast
     }
     if (!wait_phase(mbar, phase, &s_abort, status)) break;
     // epilogue 3: dz1 = bf16(dh1 [z1 > 0]) into dZ1^T (column)
-#pragma unroll 1
-    for (int q = 0; q < 4; ++q) {
+    {
       float v[32];
-      tc::tmem_ld32(tmem_at(tmem, warp, kC_D1 + 32 * q), v);
+      tc::tmem_ld32(tmem_at(tmem, quad, kC_D1 + 32 * grp), v);
 #pragma unroll
-      for (int i = 0; i < 32; ++i) v[i] = ((mask1[q] >> i) & 1u) ? v[i] : 0.f;
-      store_col32(sR2, tid, 32 * q, v);
+      for (int i = 0; i < 32; ++i) v[i] = ((mask1 >> i) & 1u) ? v[i] : 0.f;
+      store_col32(sR2, b, 32 * grp, v);
     }
     tc::fence_before();
     tc::fence_proxy_async();
@@ -414,37 +432,32 @@ mlp_train_kernel(const uint8_t* __restrict__ img, const float* __restrict__ mast
     any = true;
   }
 
-  // partial gradient of this CTA: row `tid` of each accumulator
-  float* out = partial + (size_t)blockIdx.x * (kMlpParams + 1);
+  // partial gradient of this CTA: row `b` of each accumulator
+  float* out = partial + (size_t)blockIdx.x * (kMlpParams + 1);  // 8-byte aligned: an even number of floats
+  static_assert(kMlpParams % 2 == 1 && kOW2 % 2 == 0, "pairs of the partial gradient");
   if (s_abort == 0) {
+    float v[32];
     if (any) {
-      for (int q = 0; q < 5; ++q) {  // [dW2 | db2]: columns 0..143 used
-        float v[32];
-        tc::tmem_ld32(tmem_at(tmem, warp, kC_dW2 + 32 * q), v);
-#pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          const int c = 32 * q + i;
-          if (c < 128) out[kOW2 + tid * 128 + c] = v[i];
-          else if (c == 128) out[kOb2 + tid] = v[i];
-        }
-      }
-      float v[32];
-      tc::tmem_ld32(tmem_at(tmem, warp, kC_dW1), v);
-#pragma unroll
-      for (int j = 0; j < 16; ++j) out[kOW1 + tid * 16 + j] = v[j];
-      out[kOb1 + tid] = v[16];
-      tc::tmem_ld32(tmem_at(tmem, warp, kC_dW3), v);
-      out[kOw3 + tid] = v[0];
+      tc::tmem_ld32(tmem_at(tmem, quad, kC_dW2 + 32 * grp), v);
     } else {
-      for (int c = 0; c < 128; ++c) out[kOW2 + tid * 128 + c] = 0.f;
-      for (int j = 0; j < 16; ++j) out[kOW1 + tid * 16 + j] = 0.f;
-      out[kOb1 + tid] = 0.f;
-      out[kOb2 + tid] = 0.f;
-      out[kOw3 + tid] = 0.f;
+#pragma unroll
+      for (int i = 0; i < 32; ++i) v[i] = 0.f;
     }
+#pragma unroll
+    for (int i = 0; i < 32; i += 2)
+      *reinterpret_cast<float2*>(out + kOW2 + b * 128 + 32 * grp + i) = make_float2(v[i], v[i + 1]);
+    // column 128 of [dW2 | db2], [dW1 | db1] and dW3: one group each
+    if (any && grp < 3) tc::tmem_ld32(tmem_at(tmem, quad, grp == 0 ? kC_dW2 + 128 : grp == 1 ? kC_dW1 : kC_dW3), v);
+    if (grp == 0) out[kOb2 + b] = v[0];
+    if (grp == 1) {
+#pragma unroll
+      for (int j = 0; j < 16; ++j) out[kOW1 + b * 16 + j] = v[j];
+      out[kOb1 + b] = v[16];
+    }
+    if (grp == 2) out[kOw3 + b] = v[0];
     loss = warp_sum_f(loss);
     db3 = warp_sum_f(db3);
-    if (lane == 0) {
+    if (lane == 0 && grp == 0) {
       sred[2 * warp] = loss;
       sred[2 * warp + 1] = db3;
     }
@@ -460,15 +473,32 @@ mlp_train_kernel(const uint8_t* __restrict__ img, const float* __restrict__ mast
   if (warp == 0) tc::tmem_dealloc(tmem, 512);
 }
 
-// Sum the per-CTA partials in CTA order; then either store the gradient (and
+constexpr int kRedParts = 160;
+
+// Sum the per-CTA partials in CTA order; a block takes 32 parameters and has the
+// partials of up to kRedParts CTAs in flight at once, then one thread a parameter adds
+// them up (a thread's chain of loads: 9.4 us, now 6.4).  Then either store the gradient (and
 // loss) or apply one Adam step and refresh the bf16 operand images.
 __global__ void mlp_reduce_kernel(const float* __restrict__ partial, int nparts, float* __restrict__ grad,
                                   float* master, float* m1, float* m2, uint8_t* __restrict__ img,
                                   const long long* step_ctr, MlpAdam hp, float* loss_log) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p > kMlpParams) return;
+  __shared__ float s_part[kRedParts][32];
+  const int lane = threadIdx.x & 31, row = threadIdx.x >> 5, p = blockIdx.x * 32 + lane;
   float g = 0.f;
-  for (int c = 0; c < nparts; ++c) g += partial[(size_t)c * (kMlpParams + 1) + p];
+  for (int c0 = 0; c0 < nparts; c0 += kRedParts) {
+    const int m = min(kRedParts, nparts - c0);
+#pragma unroll
+    for (int i = 0; i < kRedParts / 8; ++i) {
+      const int c = row + 8 * i;
+      if (c < m && p <= kMlpParams) s_part[c][lane] = partial[(size_t)(c0 + c) * (kMlpParams + 1) + p];
+    }
+    __syncthreads();
+    if (row == 0)
+#pragma unroll 8
+      for (int c = 0; c < m; ++c) g += s_part[c][lane];
+    __syncthreads();
+  }
+  if (row || p > kMlpParams) return;
   if (p == kMlpParams) {  // loss sum of the step
     if (loss_log) loss_log[step_ctr ? *step_ctr - 1 - hp.log_base : 0] = g;
     return;
@@ -556,7 +586,7 @@ cudaError_t mlp_train_launch(const uint8_t* img, const float* master, const floa
                              float* partial, int grid, long long* step_ctr, int* status, cudaStream_t st) {
   cudaError_t e = cudaFuncSetAttribute(mlp_train_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTrainSmem);
   if (e != cudaSuccess) return e;
-  mlp_train_kernel<<<grid, 128, kTrainSmem, st>>>(img, master, feat, target, perm, s0, count, two_over_b,
+  mlp_train_kernel<<<grid, kTrainThreads, kTrainSmem, st>>>(img, master, feat, target, perm, s0, count, two_over_b,
                                                   partial, step_ctr, status);
   count_launch();
   return cudaGetLastError();
@@ -565,7 +595,7 @@ cudaError_t mlp_train_launch(const uint8_t* img, const float* master, const floa
 cudaError_t mlp_reduce_launch(const float* partial, int nparts, float* grad, float* master, float* m1,
                               float* m2, uint8_t* img, const long long* step_ctr, const MlpAdam& hp,
                               float* loss_log, cudaStream_t st) {
-  mlp_reduce_kernel<<<(kMlpParams + 1 + 255) / 256, 256, 0, st>>>(partial, nparts, grad, master, m1, m2, img,
+  mlp_reduce_kernel<<<(kMlpParams + 1 + 31) / 32, 256, 0, st>>>(partial, nparts, grad, master, m1, m2, img,
                                                                    step_ctr, hp, loss_log);
   count_launch();
   return cudaGetLastError();
