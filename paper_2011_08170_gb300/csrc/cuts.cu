@@ -43,15 +43,16 @@
 // whose lambda and mu it fetches once a sweep.  A block whose tables do not fit
 // reads global memory through L1 instead.
 //
-// Bound, at 20,000 points with 10 neighbours and two layers (sweep of 7.7 us):
-// issue and shared-memory latency of the 57 row groups and cuts of a block (4 us),
-// the fetch of some 1,200 values (1 us), the barrier and the slack of the fullest
-// block (2.5 us).  With one gather per entry, end and crossed cut from L2 (two
-// million a sweep, all past L1) the same sweep took 19 to 24 us; through L1 with
-// no tables 8 to 11 us.  Per sweep before and now with one layer: 3,000 points 16.6
-// and 5.2 us, 40,000 points 30 and 12, 100,000 points (no tables) 41 and 32.  z is kept in 32 bits in a sweep whose values allow it
-// (checked with the fetch), else in 64: the 64-bit compares had been half of the
-// instructions.  512 threads: with 1,024 the 64 registers a thread spill (9 us).
+// Bound, at 20,000 points with 10 neighbours and two layers (sweep of 6.8 us):
+// issue and shared-memory latency of the 57 row groups and cuts of a block (3.5
+// us), the fetch of some 1,200 values (1 us), the barrier and the slack of the
+// fullest block (2.3 us).  With one gather per entry, end and crossed cut from L2
+// (two million a sweep, all past L1) the same sweep took 19 to 24 us; through L1
+// with no tables 8 to 11 us.  Per sweep before and now with one layer: 3,000 points
+// 16.6 and 5.4 us, 40,000 points 30 and 9.7, 100,000 points (no tables) 41 and 30.
+// z is kept in 32 bits in a sweep whose values allow it (checked with the fetch),
+// else in 64: the 64-bit compares had been half of the instructions.  768 threads:
+// 512 take 10 % longer, and with 1,024 the 64 registers a thread spill (9 us).
 #include <algorithm>
 #include <chrono>
 #include <climits>
@@ -253,7 +254,7 @@ struct CutGdp {
   int32_t n, L, M, F, shift;
 };
 
-constexpr int kCutThreads = 512;
+constexpr int kCutThreads = 768;
 constexpr int kCutGroup = 4;        // lanes of a row
 constexpr int kCutSmem = 208 << 10; // a block's tables
 
