@@ -133,6 +133,7 @@ struct PriceScan {
   long long cap;              // of pairs
   int32_t list_cap;
   int32_t nseg, n, fb;
+  int32_t split;              // CTAs that share a tile pair (set by the launchers)
 };
 // points, blocks and cleared counters of a scan of lambda sc.lam
 cudaError_t launch_pricing_prep(const PriceScan& sc, const int32_t* perm, int32_t nblocks, float4* pts, float4* box,

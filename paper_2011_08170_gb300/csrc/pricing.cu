@@ -63,6 +63,7 @@
 // ms; 1,000 points: 0.11 to 0.05 ms a scan.
 #include <cuda_fp16.h>
 
+#include <algorithm>
 #include <climits>
 #include <cmath>
 
@@ -354,7 +355,8 @@ pricing_kernel(const __grid_constant__ PriceScan sc) {
     __syncthreads();
     if (threadIdx.x == 0) s_tp = (int)atomicAdd(&sc.ctl->next, 1u);
     __syncthreads();
-    const int tp = s_tp;
+    // sc.split CTAs take a tile pair together, each every sc.split-th 32 j-points of it
+    const int tp = s_tp / sc.split, part = s_tp % sc.split;
     if (tp >= ntiles) break;
     // the tile pair: i in [i0, i1), j in [j0, j1), and its blocks
     int i0, i1, j0, j1, bi0, bj0;
@@ -426,6 +428,7 @@ pricing_kernel(const __grid_constant__ PriceScan sc) {
     // the tile's j-points, rounded up to four steps
     const int kend = (j1 - j0 + 31) / 32 * 32;
     for (int k = threadIdx.x; k < kend; k += T) {
+      if (sc.split > 1 && (k >> 5) % sc.split != part) continue;
       const uint4 w = (j0 + k < j1 ? row_of(sc.pts[j0 + k]) : price_row_far()).row_j();
       unsigned* d = s_j + (k & ~31) * 4 + 16 * (k & 7) + ((k >> 3) & 3);
       d[0] = w.x;
@@ -442,7 +445,7 @@ pricing_kernel(const __grid_constant__ PriceScan sc) {
       a[m][0] = wi[64 * m + lane];
       a[m][1] = wi[64 * m + 32 + lane];
     }
-    for (int k0 = 0; k0 < kend; k0 += 32) {
+    for (int k0 = 32 * part; k0 < kend; k0 += 32 * sc.split) {
       const uint4 bj = *reinterpret_cast<const uint4*>(s_j + k0 * 4 + 4 * lane);
       const unsigned bs[4] = {bj.x, bj.y, bj.z, bj.w};
 #pragma unroll
@@ -539,10 +542,16 @@ static cudaError_t price_grid(const void* kern, int threads, int num_sms, long l
 
 template <int FORM, int W, int J, int MINB>
 static cudaError_t price_launch(const PriceScan& sc, int num_sms, long long ntiles, cudaStream_t st) {
+  PriceScan s = sc;
+  // Few tile pairs leave most SMs idle, and a tile pair is 30 us of one warp, most
+  // of it pairs that pass test 1: up to two a SM four CTAs share one (1,000 points:
+  // 30 -> 13 us a scan), up to four a SM two do.  Beyond that the prologues cost
+  // more than the idle warps.
+  s.split = W > 1 ? 1 : ntiles <= 2LL * num_sms ? 4 : ntiles <= 4LL * num_sms ? 2 : 1;
   int grid = 0;
-  cudaError_t e = price_grid((const void*)pricing_kernel<FORM, W, J, MINB>, W * 32, num_sms, ntiles, &grid);
+  cudaError_t e = price_grid((const void*)pricing_kernel<FORM, W, J, MINB>, W * 32, num_sms, ntiles * s.split, &grid);
   if (e != cudaSuccess) return e;
-  pricing_kernel<FORM, W, J, MINB><<<grid, W * 32, 0, st>>>(sc);
+  pricing_kernel<FORM, W, J, MINB><<<grid, W * 32, 0, st>>>(s);
   count_launch();
   return cudaGetLastError();
 }
@@ -558,16 +567,20 @@ cudaError_t launch_pricing_full(const PriceScan& sc, bool large, long long ntile
 }
 
 cudaError_t launch_pricing_list(const PriceScan& sc, int num_sms, cudaStream_t st) {
-  return price_launch<kPriceList, 1, kPriceBlock, 20>(sc, num_sms, 1LL << 30, st);
+  // the number of block pairs is on the device: at most these
+  const long long nb = sc.n / kPriceBlock + sc.nseg;
+  return price_launch<kPriceList, 1, kPriceBlock, 20>(sc, num_sms, std::min<long long>(sc.list_cap, nb * (nb + 1) / 2),
+                                                      st);
 }
 
 cudaError_t launch_pricing_rows(const PriceScan& sc, int num_sms, cudaStream_t st) {
   // the number of rows is on the device: sized for a fifth of the nodes
   const long long large = (long long)((sc.n / 5 + kPriceLargeI - 1) / kPriceLargeI) *
                           ((sc.n + kPriceLargeJ - 1) / kPriceLargeJ);
+  const long long nb = (sc.n + kPriceBlock - 1) / kPriceBlock;  // at most these tile pairs
   return price_large_tiles(large, num_sms)
              ? price_launch<kPriceRows, 4, kPriceLargeJ, 6>(sc, num_sms, 1LL << 30, st)
-             : price_launch<kPriceRows, 1, kPriceBlock, 20>(sc, num_sms, 1LL << 30, st);
+             : price_launch<kPriceRows, 1, kPriceBlock, 20>(sc, num_sms, nb * nb, st);
 }
 
 // ---- The scan on the tensor cores ------------------------------------------------
