@@ -60,7 +60,8 @@
 // for the same test in packed fp32 (3 FADD2, 2 FFMA2 per 2 pairs, an FFMA2
 // taking 2.7 cycles: 4.7 pairs a cycle at best); HADD2 / HFMA2 run at the
 // packed fp32 rate and gained nothing.  200,000 clustered points: 2.03 to 1.45
-// ms; 1,000 points: 0.11 to 0.05 ms a scan.
+// ms; 1,000 points: 0.11 to 0.05 ms a scan (the kernel 30 us, 13 with four CTAs a
+// tile pair).
 #include <cuda_fp16.h>
 
 #include <algorithm>
