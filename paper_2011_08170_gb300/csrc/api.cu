@@ -1118,8 +1118,9 @@ extern "C" f2m_status f2m_price(f2m_ctx* c, int64_t* count, int32_t* pairs, int6
   return F2M_OK;
 }
 
-// CSR u pairs (device array of npairs int2)
-f2m_status f2m::merge_internal(f2m_ctx* c, const int2* d_pairs, int64_t npairs, double* ms) {
+// CSR u pairs (device array of npairs int2); fresh: they are distinct, valid and
+// outside the CSR (a scan's)
+f2m_status f2m::merge_internal(f2m_ctx* c, const int2* d_pairs, int64_t npairs, double* ms, bool fresh) {
   const int32_t n = c->n;
   if (!c->d_deg) {
     CK(c, dalloc(&c->d_deg, n + 1));
@@ -1135,10 +1136,12 @@ f2m_status f2m::merge_internal(f2m_ctx* c, const int2* d_pairs, int64_t npairs, 
     CK(c, dalloc(&c->d_tmp_col, c->tmp_col_cap));
   }
   MergeBuffers mb{c->d_deg, c->d_tmp_rp, c->d_tmp_col, c->d_new_rp, c->d_block_sums, c->d_check};
-  CK(c, reset_check(c));
+  if (!fresh) CK(c, reset_check(c));
   CK(c, cudaEventRecord(c->ev0, c->st));
-  CK(c, launch_merge_count(c->d_rp, d_pairs, npairs, n, mb, c->st));
-  CK(c, launch_merge_fill(c->d_rp, c->d_ec, d_pairs, npairs, n, mb, c->st));
+  if (!fresh) {
+    CK(c, launch_merge_count(c->d_rp, d_pairs, npairs, n, mb, c->st));
+    CK(c, launch_merge_fill(c->d_rp, c->d_ec, d_pairs, npairs, n, mb, c->st));
+  }
   if (need > c->ec_alt_cap) {  // the array the merged rows go to
     dfree(c->d_ec_alt);
     c->ec_alt_cap = need + (need >> 3);
@@ -1148,6 +1151,16 @@ f2m_status f2m::merge_internal(f2m_ctx* c, const int2* d_pairs, int64_t npairs, 
     dfree(c->d_x2);
     c->x2_cap = need + (need >> 3);
     CK(c, dalloc(&c->d_x2, c->x2_cap));
+  }
+  if (fresh) {
+    CK(c, plan_merge(c->d_xy, c->d_rp, c->d_ec, d_pairs, npairs, n, need, mb, c->d_ec_alt, c->plan, c->st));
+    std::swap(c->d_ec, c->d_ec_alt);
+    std::swap(c->ec_cap, c->ec_alt_cap);
+    CK(c, cudaMemcpyAsync(c->d_rp, c->d_new_rp, sizeof(int32_t) * (n + 1), cudaMemcpyDeviceToDevice, c->st));
+    c->nnz = need;
+    CK(c, cudaEventRecord(c->ev1, c->st));
+    if (ms) *ms += elapsed_ms(c);
+    return F2M_OK;
   }
   CK(c, launch_merge_finish(c->d_xy, c->d_rp, c->d_ec, n, mb, c->d_ec_alt, c->st));
   std::swap(c->d_ec, c->d_ec_alt);
@@ -1175,7 +1188,7 @@ extern "C" f2m_status f2m_add_edges(f2m_ctx* c, const int32_t* pairs, int64_t np
   CK(c, dalloc(&d, npairs));
   cudaError_t e = cudaMemcpyAsync(d, pairs, sizeof(int2) * npairs, cudaMemcpyDefault, c->st);
   if (e != cudaSuccess) { dfree(d); return cuda_fail(c, e, "add_edges: upload"); }
-  f2m_status s = merge_internal(c, d, npairs, nullptr);
+  f2m_status s = merge_internal(c, d, npairs, nullptr, false);
   cudaStreamSynchronize(c->st);
   dfree(d);
   return s;
@@ -1498,7 +1511,7 @@ extern "C" f2m_status f2m_solve(f2m_ctx* c, f2m_info* info_out) {
       last_pairs = c->npairs;
       if (c->npairs > 0) {
         const int64_t found = c->npairs;
-        s = merge_internal(c, c->d_pairs, c->npairs, &info.ms_merge);
+        s = merge_internal(c, c->d_pairs, c->npairs, &info.ms_merge, true);
         if (s != F2M_OK) { status = s; break; }
         info.edges_added += found;
         // another GDP phase, unless the first phase's scan found few pairs:
@@ -1542,7 +1555,7 @@ extern "C" f2m_status f2m_solve(f2m_ctx* c, f2m_info* info_out) {
     info.certifying_scans += c->last_scan_rows >= 0;
     last_pairs = c->npairs;
     if (c->npairs == 0) { info.certified = 2; break; }
-    s = merge_internal(c, c->d_pairs, c->npairs, &info.ms_merge);
+    s = merge_internal(c, c->d_pairs, c->npairs, &info.ms_merge, true);
     if (s != F2M_OK) { status = s; break; }
     info.edges_added += c->npairs;
     info.certified = 0;

@@ -975,7 +975,7 @@ extern "C" f2m_status f2m_solve_batch(f2m_batch* b, f2m_info* info_out, f2m_info
           }
         }
         if (c->npairs > 0) {
-          status = merge_internal(c, c->d_pairs, c->npairs, &tot.ms_merge);
+          status = merge_internal(c, c->d_pairs, c->npairs, &tot.ms_merge, true);
           if (status != F2M_OK) break;
           tot.edges_added += c->npairs;
         }
@@ -1061,7 +1061,7 @@ extern "C" f2m_status f2m_solve_batch(f2m_batch* b, f2m_info* info_out, f2m_info
     for (int32_t s = 0; s < K; ++s)
       if (done_now[s]) state[s] = DONE;
     if (any_scan && c->npairs > 0) {
-      status = merge_internal(c, c->d_pairs, c->npairs, &tot.ms_merge);
+      status = merge_internal(c, c->d_pairs, c->npairs, &tot.ms_merge, true);
       if (status != F2M_OK) break;
       tot.edges_added += c->npairs;
     }

@@ -193,7 +193,7 @@ f2m_status gdp_phase(f2m_ctx* c, int64_t max_sweeps, int64_t* sweeps, bool want_
                      int64_t trace_cap, double* ms);
 // lam_override (device, [n], units 2^-fb): scan with it in place of lambda
 f2m_status price_internal(f2m_ctx* c, double* ms, const int32_t* lam_override = nullptr);
-f2m_status merge_internal(f2m_ctx* c, const int2* d_pairs, int64_t npairs, double* ms);
+f2m_status merge_internal(f2m_ctx* c, const int2* d_pairs, int64_t npairs, double* ms, bool fresh);
 f2m_status extract_internal(f2m_ctx* c, int64_t* bad, double* ms);
 f2m_status bound_internal(f2m_ctx* c, int64_t* b2);
 // h_include (host, per segment; NULL = all): the segments the finisher works on

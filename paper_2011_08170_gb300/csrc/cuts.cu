@@ -1199,7 +1199,7 @@ extern "C" f2m_status f2m_solve_subtour(f2m_ctx* c, int32_t rounds, f2m_subtour_
       info.pricing_rounds += 1;
       if (c->npairs == 0) break;
       const int64_t found = c->npairs;
-      s = merge_internal(c, c->d_pairs, c->npairs, &info.ms_merge);
+      s = merge_internal(c, c->d_pairs, c->npairs, &info.ms_merge, true);
       if (s != F2M_OK) return s;
       info.edges_added += found;
     }

@@ -177,6 +177,9 @@ struct MergeBuffers {
   int32_t* block_sums; // scan scratch
   CheckCtl* ctl;
 };
+cudaError_t launch_merge_new(const int2* xy, const int32_t* rp, const int2* ec_in, const int2* pairs, int64_t npairs,
+                             int32_t n, MergeBuffers& mb, const int32_t* perm, const int32_t* inv, int32_t* isums,
+                             int2* ec_out, int32_t* irp, int2* iec, cudaStream_t st);
 cudaError_t launch_merge_count(const int32_t* rp, const int2* pairs, int64_t npairs, int32_t n,
                                MergeBuffers& mb, cudaStream_t st);
 cudaError_t launch_merge_fill(const int32_t* rp, const int2* ec, const int2* pairs, int64_t npairs,
@@ -239,6 +242,10 @@ cudaError_t sort_pairs_u64(void* temp, size_t& temp_bytes, const uint64_t* keys_
 // Morton renumbering inside each segment [seg_off[s], seg_off[s+1]) (segments stay contiguous)
 cudaError_t plan_renumber(const int2* xy, int32_t n, const std::vector<int32_t>& seg_off, GdpPlan& p,
                           cudaStream_t st);
+// merge of npairs pairs that are distinct and outside the CSR, into ec_out, mb.new_rp and the
+// renumbered CSR of `nnz` = old entries + 2 npairs (MergeBuffers: above)
+cudaError_t plan_merge(const int2* xy, const int32_t* rp, const int2* ec_in, const int2* pairs, int64_t npairs,
+                       int32_t n, int64_t nnz, MergeBuffers& mb, int2* ec_out, GdpPlan& p, cudaStream_t st);
 // the CSR in the renumbered order
 cudaError_t plan_build(const int32_t* rp, const int2* ec, int32_t n, int64_t nnz, GdpPlan& p, cudaStream_t st);
 // dst[i] = src[perm[i]]  /  dst[perm[i]] = src[i]

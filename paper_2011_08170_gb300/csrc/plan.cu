@@ -154,13 +154,28 @@ cudaError_t scatter_perm(const int32_t* src, const int32_t* perm, int32_t n, int
   return cudaGetLastError();
 }
 
-cudaError_t plan_build(const int32_t* rp, const int2* ec, int32_t n, int64_t nnz, GdpPlan& p, cudaStream_t st) {
-  p.version += 1;
+cudaError_t plan_room(int32_t n, int64_t nnz, GdpPlan& p) {
   PCK(grow(&p.irp, &p.irp_cap, (int64_t)n + 1));
   PCK(grow(&p.iec, &p.iec_cap, nnz));
   PCK(grow(&p.ilam[0], &p.ilam_cap[0], n));
   PCK(grow(&p.ilam[1], &p.ilam_cap[1], n));
   PCK(grow(&p.scan_tmp, &p.scan_cap, (int64_t)scan_scratch_ints(n) + 1));
+  return cudaSuccess;
+}
+
+cudaError_t plan_merge(const int2* xy, const int32_t* rp, const int2* ec_in, const int2* pairs, int64_t npairs,
+                       int32_t n, int64_t nnz, MergeBuffers& mb, int2* ec_out, GdpPlan& p, cudaStream_t st) {
+  PCK(plan_room(n, nnz, p));
+  PCK(launch_merge_new(xy, rp, ec_in, pairs, npairs, n, mb, p.perm, p.inv, p.scan_tmp, ec_out, p.irp, p.iec, st));
+  p.version += 1;
+  p.n = n;
+  p.nnz = nnz;
+  return cudaSuccess;
+}
+
+cudaError_t plan_build(const int32_t* rp, const int2* ec, int32_t n, int64_t nnz, GdpPlan& p, cudaStream_t st) {
+  p.version += 1;
+  PCK(plan_room(n, nnz, p));
   // internal CSR: rows in renumbered order, columns renumbered
   int32_t* ideg = p.ilam[1];  // free until the phase starts
   internal_degree_kernel<<<grid_for(n, 256), 256, 0, st>>>(rp, p.perm, n, ideg);
