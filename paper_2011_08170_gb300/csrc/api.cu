@@ -296,6 +296,16 @@ f2m_status cuda_fail(f2m_ctx* ctx, cudaError_t e, const char* what) {
 
 }  // namespace f2m
 
+// a small device record to the host, by way of the context's pinned block (a copy
+// into pageable memory is staged by the driver, 6 to 10 us each); waits
+static cudaError_t read_back(f2m_ctx* c, void* dst, const void* src, size_t bytes) {
+  if (!c->h_rb || bytes > kReadBack) return cudaErrorInvalidValue;
+  cudaError_t e = cudaMemcpyAsync(c->h_rb, src, bytes, cudaMemcpyDeviceToHost, c->st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(c->st);
+  if (e == cudaSuccess) std::memcpy(dst, c->h_rb, bytes);
+  return e;
+}
+
 static float elapsed_ms(f2m_ctx* c) {
   float ms = 0.f;
   cudaEventSynchronize(c->ev1);
@@ -354,6 +364,7 @@ extern "C" void f2m_destroy(f2m_ctx* c) {
   dfree(c->d_block_sums); dfree(c->d_tmp_col); dfree(c->d_out_a); dfree(c->d_out_b);
   dfree(c->d_check); dfree(c->d_scalar); dfree(c->d_bad); dfree(c->d_b); dfree(c->d_b_int);
   dfree(c->d_ring_seg);
+  pin_free(c->h_rb);
   free_finisher_buffers(c);
   if (c->fin_work) finisher_work_free(c->fin_work);
   ring_free(c->ring);
@@ -444,6 +455,7 @@ f2m_status f2m::create_internal(const int32_t* xy, int32_t n, const int32_t* row
     if (e == cudaSuccess) e = dalloc(&c->d_rp, n + 1);
     if (e == cudaSuccess) e = dalloc(&c->d_xy, n);
     if (e == cudaSuccess) e = dalloc(&c->d_check, 1);
+    if (e == cudaSuccess) e = pin_alloc(&c->h_rb, kReadBack);
     if (e == cudaSuccess) e = cudaMemcpyAsync(c->d_rp, row_ptr, sizeof(int32_t) * (n + 1), cudaMemcpyDefault, c->st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(c->d_xy, xy, sizeof(int2) * n, cudaMemcpyDefault, c->st);
     int32_t nnz_h = 0;
@@ -638,7 +650,7 @@ static f2m_status ring_phase(f2m_ctx* c, int64_t max_sweeps, int64_t* sweeps, lo
         CK(c, dalloc(&c->d_ring_seg, 2));
         CK(c, cudaMemcpyAsync(c->d_ring_seg, off, sizeof(off), cudaMemcpyHostToDevice, c->st));
       }
-      CK(c, ring_build(c->plan, c->d_ring_seg, nullptr, tiles, c->ring_k, c->p.frac_bits, c->nnz / tiles, c->ring,
+      CK(c, ring_build(c->plan, c->d_ring_seg, nullptr, tiles, c->ring_k, c->p.frac_bits, c->nnz / tiles, 1, c->ring,
                        c->st));
     }
     int64_t limit = std::min<int64_t>(max_sweeps, kRingSweeps);
@@ -664,12 +676,11 @@ static f2m_status ring_phase(f2m_ctx* c, int64_t max_sweeps, int64_t* sweeps, lo
       }
       CK(c, e);
       CK(c, cudaEventRecord(c->ev1, c->st));
-      RingStats rs{};
-      CK(c, cudaMemcpyAsync(&status, c->ring.status, sizeof(status), cudaMemcpyDeviceToHost, c->st));
-      CK(c, cudaMemcpyAsync(&rs, c->ring.stats, sizeof(rs), cudaMemcpyDeviceToHost, c->st));
-      RingSeg q{};
-      CK(c, cudaMemcpyAsync(&q, c->ring.seg, sizeof(q), cudaMemcpyDeviceToHost, c->st));
-      CK(c, cudaStreamSynchronize(c->st));
+      RingRecord rec;
+      CK(c, read_back(c, &rec, c->ring.rec, sizeof(rec)));
+      const RingStats& rs = rec.stats;
+      const RingSeg& q = rec.seg[0];
+      status = rec.status;
       if (ms) *ms += elapsed_ms(c);
       if (status & kGdpTimeout) return fail(c, F2M_ERR_TIMEOUT, "a wait for another tile exceeded its budget");
       if (reg) {  // what the tiles need, known now
@@ -1055,8 +1066,7 @@ f2m_status f2m::price_internal(f2m_ctx* c, double* ms, const int32_t* lam_overri
         CK(c, launch_pricing_full(sc, large, ntiles, c->num_sms, c->st));
       }
       CK(c, cudaEventRecord(c->ev1, c->st));
-      CK(c, cudaMemcpyAsync(&h, c->d_pctl, sizeof(h), cudaMemcpyDeviceToHost, c->st));
-      CK(c, cudaStreamSynchronize(c->st));
+      CK(c, read_back(c, &h, c->d_pctl, sizeof(h)));
       if (ms) *ms += elapsed_ms(c);
       s = price_grow(c, h, &again);
       if (s != F2M_OK) return s;
@@ -1202,8 +1212,7 @@ f2m_status f2m::extract_internal(f2m_ctx* c, int64_t* bad, double* ms) {
   CK(c, launch_extract(c->d_rp, c->d_ec, c->d_b, lam, c->n, fb, c->d_x2, c->d_bad, c->st));
   CK(c, cudaEventRecord(c->ev1, c->st));
   unsigned long long b = 0;
-  CK(c, cudaMemcpyAsync(&b, c->d_bad, sizeof(b), cudaMemcpyDeviceToHost, c->st));
-  CK(c, cudaStreamSynchronize(c->st));
+  CK(c, read_back(c, &b, c->d_bad, sizeof(b)));
   if (ms) *ms += elapsed_ms(c);
   *bad = (int64_t)b;
   return F2M_OK;
@@ -1226,8 +1235,7 @@ f2m_status f2m::bound_internal(f2m_ctx* c, int64_t* b2) {
   const int32_t* lam = cur_lambda(c, &fb);
   CK(c, launch_bound(c->d_rp, c->d_ec, c->d_b, lam, c->n, fb, c->d_scalar, c->st));
   long long h = 0;
-  CK(c, cudaMemcpyAsync(&h, c->d_scalar, sizeof(h), cudaMemcpyDeviceToHost, c->st));
-  CK(c, cudaStreamSynchronize(c->st));
+  CK(c, read_back(c, &h, c->d_scalar, sizeof(h)));
   *b2 = h;
   return F2M_OK;
 }

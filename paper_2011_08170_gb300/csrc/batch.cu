@@ -661,7 +661,8 @@ static f2m_status batch_ring_phase(f2m_batch* b, const std::vector<uint8_t>& act
   }
   if (!b->h_rseg) CK(c, pin_alloc((void**)&b->h_rseg, sizeof(RingSeg) * b->count));
   CK(c, cudaMemcpyAsync(b->d_rlist, list.data(), sizeof(RingTile) * tiles, cudaMemcpyHostToDevice, c->st));
-  CK(c, ring_build(c->plan, c->d_seg_off, b->d_rlist, tiles, K, c->p.frac_bits, rows * c->nnz / c->n, c->ring, c->st));
+  CK(c, ring_build(c->plan, c->d_seg_off, b->d_rlist, tiles, K, c->p.frac_bits, rows * c->nnz / c->n, b->count, c->ring,
+                   c->st));
   CK(c, ring_start(c->ring, c->n, b->count, c->st));
   // the instances left alone keep their lambda
   const int32_t* in = c->d_lam[c->cur];
@@ -681,8 +682,8 @@ static f2m_status batch_ring_phase(f2m_batch* b, const std::vector<uint8_t>& act
   }
   CK(c, cudaEventRecord(c->ev1, c->st));
   int32_t status = 0;
-  CK(c, cudaMemcpyAsync(&status, c->ring.status, sizeof(status), cudaMemcpyDeviceToHost, c->st));
-  CK(c, cudaMemcpyAsync(b->h_rseg, c->ring.seg, sizeof(RingSeg) * b->count, cudaMemcpyDeviceToHost, c->st));
+  CK(c, cudaMemcpyAsync(&status, &c->ring.rec->status, sizeof(status), cudaMemcpyDeviceToHost, c->st));
+  CK(c, cudaMemcpyAsync(b->h_rseg, c->ring.rec->seg, sizeof(RingSeg) * b->count, cudaMemcpyDeviceToHost, c->st));
   CK(c, cudaStreamSynchronize(c->st));
   if (status & kGdpNoFit) return F2M_OK;
   *ran = true;

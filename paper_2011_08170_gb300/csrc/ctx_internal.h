@@ -14,6 +14,8 @@ namespace f2m {
 struct CutState;  // subtour-elimination cuts (cuts.cu)
 }
 
+constexpr size_t kReadBack = 1024;
+
 struct f2m_ctx {
   // segments: contiguous node ranges that are separate instances (a batch);
   // one segment [0, n) for a single instance.  Pricing pairs stay inside a
@@ -133,6 +135,7 @@ struct f2m_ctx {
   int32_t* h_lam = nullptr;
   int32_t* h_lam2 = nullptr;
   f2m::FinisherWork* fin_work = nullptr;
+  void* h_rb = nullptr;  // pinned, kReadBack bytes: small results on their way to the host
   // the finisher's phase 1 on the GPU: node state of both copies, blocks, heaps
   long long* d_fpi = nullptr;
   long long* d_fdist = nullptr;

@@ -286,6 +286,11 @@ struct RingSeg {          // per instance, zeroed per phase
   long long sweeps;       // the result
   int32_t fixed_point, overflow;
 };
+struct RingRecord {       // what the host reads after a phase, in one copy
+  RingStats stats;        // zeroed per plan
+  int32_t status;         // from here on zeroed per phase
+  RingSeg seg[1];         // one per instance
+};
 struct RingArgs {
   const RingHdr* hdr;
   const int32_t* halo;
@@ -315,19 +320,17 @@ struct RingPlan {
   uint16_t* order = nullptr;
   uint32_t* slc = nullptr;
   int2* ent = nullptr;
-  RingStats* stats = nullptr;
-  RingSeg* seg = nullptr;
+  RingRecord* rec = nullptr;
   int32_t* pos = nullptr;
   unsigned* words = nullptr;  // the exchange: two buffers of words_n
   int64_t words_n = 0;
-  int* status = nullptr;
   int64_t hdr_cap = 0, halo_cap = 0, order_cap = 0, slc_cap = 0, ent_cap = 0, seg_cap = 0, words_cap = 0, pos_cap = 0;
 };
 void ring_free(RingPlan& p);
 // the tiles of K rings over the internal CSR: `tiles` equal shares of the one
 // segment's nodes (list NULL), or those of the device list; seg_off on the device
 cudaError_t ring_build(const GdpPlan& g, const int32_t* seg_off, const RingTile* list, int32_t tiles, int32_t K,
-                       int32_t F, int64_t entries_per_tile, RingPlan& p, cudaStream_t st);
+                       int32_t F, int64_t entries_per_tile, int32_t nseg, RingPlan& p, cudaStream_t st);
 int32_t ring_smem(bool half);  // dynamic shared memory of a CTA
 // per phase: cleared segment records and status
 cudaError_t ring_start(RingPlan& p, int32_t n, int32_t nseg, cudaStream_t st);

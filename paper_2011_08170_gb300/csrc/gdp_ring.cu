@@ -48,6 +48,7 @@
 // 1.78 / 1.0 to 0.95; merging triples instead of inserting was worth 5 % of the
 // instructions.
 #include <climits>
+#include <cstddef>
 
 #include "f2m_device.cuh"
 #include "f2m_internal.h"
@@ -926,14 +927,14 @@ static cudaError_t grow(T** p, int64_t* cap, int64_t need) {
 }
 
 void ring_free(RingPlan& p) {
-  void* ptrs[] = {p.hdr, p.halo, p.order, p.slc, p.ent, p.pos, p.stats, p.seg, p.words, p.status};
+  void* ptrs[] = {p.hdr, p.halo, p.order, p.slc, p.ent, p.pos, p.rec, p.words};
   for (void* q : ptrs)
     if (q) dev_free(q);
   p = RingPlan();
 }
 
 cudaError_t ring_build(const GdpPlan& g, const int32_t* seg_off, const RingTile* list, int32_t tiles, int32_t K,
-                       int32_t F, int64_t entries_per_tile, RingPlan& p, cudaStream_t st) {
+                       int32_t F, int64_t entries_per_tile, int32_t nseg, RingPlan& p, cudaStream_t st) {
   // room for a tile's sliced entries: its own and its inner rings', at most what
   // the 4-byte form could hold in shared memory
   const int64_t want = K > 1 ? entries_per_tile * 2 + 16384 : entries_per_tile * 3 / 2 + 4096;
@@ -945,12 +946,18 @@ cudaError_t ring_build(const GdpPlan& g, const int32_t* seg_off, const RingTile*
   RCK(grow(&p.order, &p.order_cap, (int64_t)tiles * kRingSlots));
   RCK(grow(&p.slc, &p.slc_cap, (int64_t)tiles * kRingSlices));
   RCK(grow(&p.ent, &p.ent_cap, (int64_t)tiles * ecap));
-  if (!p.stats) RCK(dev_malloc((void**)&p.stats, sizeof(RingStats)));
-  RCK(cudaMemsetAsync(p.stats, 0, sizeof(RingStats), st));
+  if (p.seg_cap < nseg) {
+    if (p.rec) dev_free(p.rec);
+    p.rec = nullptr;
+    p.seg_cap = 0;
+    RCK(dev_malloc((void**)&p.rec, sizeof(RingRecord) + sizeof(RingSeg) * (size_t)nseg));
+    p.seg_cap = nseg;
+  }
+  RCK(cudaMemsetAsync(&p.rec->stats, 0, sizeof(RingStats), st));
   constexpr size_t smem = 4 * (kHash + 2 * kRingHalo) + 2 * (kHash + kRingHalo + 2 * kRingLocals + kRingSlots);
   RCK(cudaFuncSetAttribute(ring_plan_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   ring_plan_kernel<<<tiles, kPlanThreads, smem, st>>>(g.irp, g.iec, list, seg_off, tiles, K, F, (int32_t)ecap, p.hdr,
-                                                      p.halo, p.order, p.slc, p.ent, p.pos, p.stats);
+                                                      p.halo, p.order, p.slc, p.ent, p.pos, &p.rec->stats);
   count_launch();
   RCK(cudaGetLastError());
   p.ecap = (int32_t)ecap;
@@ -962,14 +969,13 @@ cudaError_t ring_build(const GdpPlan& g, const int32_t* seg_off, const RingTile*
 }
 
 cudaError_t ring_start(RingPlan& p, int32_t n, int32_t nseg, cudaStream_t st) {
-  if (!p.status) RCK(dev_malloc((void**)&p.status, sizeof(int)));
-  RCK(grow(&p.seg, &p.seg_cap, nseg));
+  if (p.seg_cap < nseg) return cudaErrorInvalidValue;
   const int64_t m = (int64_t)n + 32LL * p.tiles;  // a tile's own slots are whole slices
   RCK(grow(&p.words, &p.words_cap, 2 * m));
   p.words_n = m;
   RCK(cudaMemsetAsync(p.words, 0, sizeof(unsigned) * 2 * m, st));
-  RCK(cudaMemsetAsync(p.seg, 0, sizeof(RingSeg) * nseg, st));
-  return cudaMemsetAsync(p.status, 0, sizeof(int), st);
+  return cudaMemsetAsync(&p.rec->status, 0,
+                         offsetof(RingRecord, seg) - offsetof(RingRecord, status) + sizeof(RingSeg) * nseg, st);
 }
 
 template <int MODE, int T>
@@ -1024,12 +1030,12 @@ cudaError_t launch_gdp_ring(const GdpPlan& g, RingPlan& p, int32_t first_tile, i
   a.order = p.order;
   a.slc = p.slc;
   a.ent = p.ent;
-  a.stats = p.stats;
-  a.seg = p.seg;
+  a.stats = &p.rec->stats;
+  a.seg = p.rec->seg;
   a.words[0] = p.words;
   a.words[1] = p.words + p.words_n;
   a.pos = p.pos;
-  a.status = p.status;
+  a.status = &p.rec->status;
   a.lam_in = lam_in;
   a.lam_out = lam_out;
   a.perm = g.perm;
