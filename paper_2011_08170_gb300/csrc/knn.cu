@@ -27,6 +27,7 @@
 // with a coarser level per point (627: a level is four times too coarse near the
 // edge of a cluster).
 #include <climits>
+#include <cstdint>
 #include <vector>
 
 #include <cub/cub.cuh>
@@ -121,9 +122,15 @@ __device__ __forceinline__ void write_features(const long long (&d2)[kFeatures],
     for (int j = 0; j < kFeatures; ++j) hi[j] = (float)(sqrt((double)d2[j]) / s);
     sh = (float)s;
   }
+  // the caller's array may begin at any float
+  if ((reinterpret_cast<uintptr_t>(feat) & 15) == 0) {
 #pragma unroll
-  for (int j = 0; j < kFeatures; j += 4)
-    *reinterpret_cast<float4*>(feat + j) = make_float4(hi[j], hi[j + 1], hi[j + 2], hi[j + 3]);
+    for (int j = 0; j < kFeatures; j += 4)
+      *reinterpret_cast<float4*>(feat + j) = make_float4(hi[j], hi[j + 1], hi[j + 2], hi[j + 3]);
+  } else {
+#pragma unroll
+    for (int j = 0; j < kFeatures; ++j) feat[j] = hi[j];
+  }
   *scale = sh;
 }
 

@@ -78,3 +78,15 @@ def test_features_are_the_64_bit_ones(lib, oracle_lib, kind):
     s = np.maximum(1.0, s / 16)
     assert np.array_equal(scale, s.astype(np.float32))
     assert np.array_equal(feat, (d / s[:, None]).astype(np.float32))
+
+
+def test_features_into_any_float(lib):
+    import torch
+    xy = I.uniform_points(500, 6)
+    feat, scale = f2m.f2m_features(xy)
+    d = torch.from_numpy(xy).cuda()
+    f, s = torch.zeros(500 * 16 + 3, device="cuda"), torch.zeros(501, device="cuda")
+    for o in (0, 1, 2, 3):
+        assert lib.f2m_features(d.data_ptr(), 500, f[o:].data_ptr(), s[1:].data_ptr(), None) == f2m.F2M_OK
+        assert np.array_equal(f[o:o + 8000].cpu().numpy().reshape(500, 16), feat)
+        assert np.array_equal(s[1:].cpu().numpy(), scale)
