@@ -409,15 +409,11 @@ static std::string check_message(int flags, int first) {
 }
 
 static cudaError_t reset_check(f2m_ctx* c) {
-  CheckCtl h{0, INT_MAX};
-  return cudaMemcpyAsync(c->d_check, &h, sizeof(h), cudaMemcpyHostToDevice, c->st);
+  return cudaMemcpyAsync(c->d_check, static_cast<char*>(c->h_rb) + kReadBack, sizeof(CheckCtl), cudaMemcpyHostToDevice,
+                         c->st);
 }
 
-static cudaError_t read_check(f2m_ctx* c, CheckCtl* h) {
-  cudaError_t e = cudaMemcpyAsync(h, c->d_check, sizeof(*h), cudaMemcpyDeviceToHost, c->st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(c->st);
-  return e;
-}
+static cudaError_t read_check(f2m_ctx* c, CheckCtl* h) { return read_back(c, h, c->d_check, sizeof(*h)); }
 
 extern "C" f2m_status f2m_create(const int32_t* xy, int32_t n, const int32_t* row_ptr,
                                  const int32_t* col, const f2m_params* params, void* stream,
@@ -454,26 +450,29 @@ f2m_status f2m::create_internal(const int32_t* xy, int32_t n, const int32_t* row
     if (e == cudaSuccess) e = cudaEventCreate(&c->ev1);
     if (e == cudaSuccess) e = dalloc(&c->d_rp, n + 1);
     if (e == cudaSuccess) e = dalloc(&c->d_xy, n);
-    if (e == cudaSuccess) e = dalloc(&c->d_check, 1);
-    if (e == cudaSuccess) e = pin_alloc(&c->h_rb, kReadBack);
+    if (e == cudaSuccess) e = dalloc(&c->d_check, 2);  // and the entry count that the first check reads
+    if (e == cudaSuccess) e = pin_alloc(&c->h_rb, kReadBack + sizeof(CheckCtl));
+    if (e == cudaSuccess) {
+      const CheckCtl none{0, INT_MAX};  // a cleared record, behind the results
+      std::memcpy(static_cast<char*>(c->h_rb) + kReadBack, &none, sizeof(none));
+    }
     if (e == cudaSuccess) e = cudaMemcpyAsync(c->d_rp, row_ptr, sizeof(int32_t) * (n + 1), cudaMemcpyDefault, c->st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(c->d_xy, xy, sizeof(int2) * n, cudaMemcpyDefault, c->st);
-    int32_t nnz_h = 0;
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&nnz_h, c->d_rp + n, sizeof(int32_t), cudaMemcpyDeviceToHost, c->st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(c->st);
-    if (e != cudaSuccess) { s = cuda_fail(nullptr, e, "create: upload"); break; }
+    // the offsets' check, which also hands back their last, the entry count
+    if (e == cudaSuccess) e = reset_check(c);
+    if (e == cudaSuccess) e = launch_check(c->d_xy, c->d_rp, nullptr, n, c->d_check, c->st);
+    CheckCtl rec[2] = {};
+    if (e == cudaSuccess) e = read_back(c, rec, c->d_check, sizeof(rec));
+    if (e != cudaSuccess) { s = cuda_fail(nullptr, e, "create: upload and check row_ptr"); break; }
+    CheckCtl h = rec[0];
+    const int32_t nnz_h = rec[1].flags;
     if (nnz_h < 3 * (int64_t)n) { s = fail(nullptr, F2M_ERR_INVALID_ARG, "row_ptr[n] < 3n: some node has degree below 3"); break; }
     c->nnz = nnz_h;
-    e = reset_check(c);
-    if (e == cudaSuccess) e = launch_check(c->d_xy, c->d_rp, nullptr, n, c->nnz, c->d_check, c->st);
-    CheckCtl h{};
-    if (e == cudaSuccess) e = read_check(c, &h);
-    if (e != cudaSuccess) { s = cuda_fail(nullptr, e, "create: check row_ptr"); break; }
     if (h.flags) { s = fail(nullptr, F2M_ERR_INVALID_ARG, check_message(h.flags, h.first_bad)); break; }
     e = dalloc(&d_col, c->nnz);
     if (e == cudaSuccess) e = cudaMemcpyAsync(d_col, col, sizeof(int32_t) * c->nnz, cudaMemcpyDefault, c->st);
     if (e == cudaSuccess) e = reset_check(c);
-    if (e == cudaSuccess) e = launch_check(c->d_xy, c->d_rp, d_col, n, c->nnz, c->d_check, c->st);
+    if (e == cudaSuccess) e = launch_check(c->d_xy, c->d_rp, d_col, n, c->d_check, c->st);
     if (e == cudaSuccess) e = read_check(c, &h);
     if (e != cudaSuccess) { s = cuda_fail(nullptr, e, "create: check rows"); break; }
     if (h.flags) { s = fail(nullptr, F2M_ERR_INVALID_ARG, check_message(h.flags, h.first_bad)); break; }

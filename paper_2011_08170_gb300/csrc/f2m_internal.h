@@ -72,9 +72,10 @@ void count_launches(long long k);  // k launches replayed from a captured graph
 
 // ---- launchers (each enqueues on `st`) -------------------------------------
 
-// validation of the input CSR and points; ctl must be zeroed (first_bad = INT_MAX)
-cudaError_t launch_check(const int2* xy, const int32_t* rp, const int32_t* col, int32_t n,
-                         int64_t nnz, CheckCtl* ctl, cudaStream_t st);
+// validation of the input CSR and points; ctl must be zeroed (first_bad = INT_MAX).
+// Without col: offsets and points, and rp[n] into the record after ctl.
+cudaError_t launch_check(const int2* xy, const int32_t* rp, const int32_t* col, int32_t n, CheckCtl* ctl,
+                         cudaStream_t st);
 // coordinates in [0, 2^20) (flag kBadCoord); ctl zeroed with first_bad = INT_MAX
 cudaError_t launch_check_points(const int2* xy, int32_t n, CheckCtl* ctl, cudaStream_t st);
 // degree requirements 1 <= b_v <= deg(v) - 1 (flag kBadDegreeReq); the

@@ -24,12 +24,14 @@ __device__ __forceinline__ void flag(CheckCtl* ctl, int bit, long long where) {
   atomicMin(&ctl->first_bad, (int)(where < INT_MAX ? where : INT_MAX));
 }
 
-// pass 1: row offsets monotone and in [0, nnz], coordinates in range
-__global__ void check_rowptr_kernel(const int2* xy, const int32_t* rp, int32_t n, int64_t nnz,
-                                    CheckCtl* ctl) {
+// pass 1: row offsets monotone and in [0, nnz], coordinates in range; nnz = rp[n]
+// goes to the host with the verdict
+__global__ void check_rowptr_kernel(const int2* xy, const int32_t* rp, int32_t n, CheckCtl* ctl) {
+  const int32_t nnz = rp[n];
+  if (blockIdx.x == 0 && threadIdx.x == 0) ctl[1].flags = nnz;
   F2M_GRID_STRIDE(v, n) {
     const int a = rp[v], b = rp[v + 1];
-    if (a < 0 || b < a || (long long)b > nnz || (v == 0 && a != 0) || (v == n - 1 && b != nnz))
+    if (a < 0 || b < a || b > nnz || (v == 0 && a != 0))
       flag(ctl, kBadRowPtr, v);
     const int2 p = xy[v];
     if (p.x < 0 || p.y < 0 || p.x >= kCoordLimit || p.y >= kCoordLimit) flag(ctl, kBadCoord, v);
@@ -99,11 +101,11 @@ cudaError_t launch_check_degrees(const int32_t* rp, const int32_t* bdeg, int32_t
   return cudaGetLastError();
 }
 
-cudaError_t launch_check(const int2* xy, const int32_t* rp, const int32_t* col, int32_t n,
-                         int64_t nnz, CheckCtl* ctl, cudaStream_t st) {
+cudaError_t launch_check(const int2* xy, const int32_t* rp, const int32_t* col, int32_t n, CheckCtl* ctl,
+                         cudaStream_t st) {
   // two passes; the host reads ctl between them (pass 2 trusts the row offsets)
   if (col == nullptr) {
-    check_rowptr_kernel<<<grid_for(n, 256), 256, 0, st>>>(xy, rp, n, nnz, ctl);
+    check_rowptr_kernel<<<grid_for(n, 256), 256, 0, st>>>(xy, rp, n, ctl);
     count_launch();
   } else {
     check_rows_kernel<<<grid_for((long long)n * kRowLanes, 256), 256, 0, st>>>(rp, col, n, ctl);

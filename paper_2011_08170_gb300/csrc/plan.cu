@@ -110,11 +110,13 @@ cudaError_t plan_renumber(const int2* xy, int32_t n, const std::vector<int32_t>&
                           cudaStream_t st) {
   int64_t cap = 0;
   const int32_t nseg = (int32_t)seg_off.size() - 1;
-  int32_t* d_seg = nullptr;
-  PCK(dev_malloc((void**)&d_seg, sizeof(int32_t) * seg_off.size()));
-  cudaError_t e0 = cudaMemcpyAsync(d_seg, seg_off.data(), sizeof(int32_t) * seg_off.size(),
-                                   cudaMemcpyHostToDevice, st);
-  if (e0 != cudaSuccess) { dev_free(d_seg); return e0; }
+  int32_t* d_seg = nullptr;  // not read for one segment
+  if (nseg > 1) {
+    PCK(dev_malloc((void**)&d_seg, sizeof(int32_t) * seg_off.size()));
+    cudaError_t e0 = cudaMemcpyAsync(d_seg, seg_off.data(), sizeof(int32_t) * seg_off.size(),
+                                     cudaMemcpyHostToDevice, st);
+    if (e0 != cudaSuccess) { dev_free(d_seg); return e0; }
+  }
   int end_bit = 40;
   while ((1LL << (end_bit - 40)) < nseg) ++end_bit;
   PCK(grow(&p.perm, &cap, n)); cap = 0;
@@ -125,8 +127,10 @@ cudaError_t plan_renumber(const int2* xy, int32_t n, const std::vector<int32_t>&
   morton_kernel<<<grid_for(n, 256), 256, 0, st>>>(xy, n, d_seg, nseg, p.keys, p.idx);
   count_launch();
   cudaError_t e1 = cudaGetLastError();
-  if (e1 == cudaSuccess) e1 = cudaStreamSynchronize(st);
-  dev_free(d_seg);
+  if (d_seg) {
+    if (e1 == cudaSuccess) e1 = cudaStreamSynchronize(st);
+    dev_free(d_seg);
+  }
   PCK(e1);
   size_t bytes = 0;
   PCK(sort_pairs_u64(nullptr, bytes, p.keys, p.keys2, p.idx, p.perm, n, end_bit, st));
