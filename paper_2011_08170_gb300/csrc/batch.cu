@@ -1149,12 +1149,14 @@ extern "C" f2m_status f2m_batch_get_x(f2m_batch* b, int32_t i, int64_t* nnz_inou
   *nnz_inout = nz;
   if (!row_ptr && !col && !x2) return F2M_OK;
   if ((col || x2) && cap < nz) return bfail(b, F2M_ERR_INVALID_ARG, "capacity below nnz");
-  // straight into the caller's device arrays; host arrays by way of a staging copy
+  // straight into the caller's arrays on this device; those of the host and of
+  // another GPU by way of a staging copy
   const int32_t rows = b->n[i] + 1;
-  auto on_device = [](const void* p) {
+  int dev = 0;
+  CK(c, cudaGetDevice(&dev));
+  auto on_device = [dev](const void* p) {
     cudaPointerAttributes q;
-    if (p && cudaPointerGetAttributes(&q, p) == cudaSuccess)
-      return q.type == cudaMemoryTypeDevice || q.type == cudaMemoryTypeManaged;
+    if (p && cudaPointerGetAttributes(&q, p) == cudaSuccess) return kernel_reaches(q.type, q.device, dev);
     cudaGetLastError();
     return false;
   };

@@ -60,6 +60,11 @@ enum CheckBits {
 cudaError_t dev_malloc(void** p, size_t bytes);
 void dev_free(void* p);
 void dev_free_synced(void* p);
+// whether a kernel on device `current` may write to memory of this kind on `device`
+// (another GPU's memory only by a copy)
+inline bool kernel_reaches(cudaMemoryType type, int device, int current) {
+  return type == cudaMemoryTypeManaged || (type == cudaMemoryTypeDevice && device == current);
+}
 // waits for the device once; while it lives, dev_free on this thread waits no more
 struct DevSyncedScope {
   DevSyncedScope();
