@@ -731,6 +731,7 @@ f2m_status f2m::gdp_phase(f2m_ctx* c, int64_t max_sweeps, int64_t* sweeps, bool 
   if (want_trace && trace_cap > c->trace_cap) {
     dfree(c->d_trace_b2);
     dfree(c->d_trace_ch);
+    c->trace_cap = 0;
     CK(c, dalloc(&c->d_trace_b2, trace_cap));
     CK(c, dalloc(&c->d_trace_ch, trace_cap));
     c->trace_cap = trace_cap;
@@ -840,8 +841,7 @@ static void build_mma_tiles(const f2m_ctx* c, std::vector<int4>& tiles, std::vec
 static f2m_status price_setup(f2m_ctx* c) {
   const int32_t nseg = (int32_t)c->seg_off.size() - 1;
   if (!c->d_pairs) {
-    c->pairs_cap = c->p.pricing_cap;
-    CK(c, dalloc(&c->d_pairs, c->pairs_cap));
+    CK(c, dgrow(&c->d_pairs, &c->pairs_cap, 1, c->p.pricing_cap));
   }
   if (c->d_pseg) return F2M_OK;
   std::vector<int32_t> h(c->seg_off.begin(), c->seg_off.end());
@@ -867,15 +867,12 @@ static f2m_status price_setup(f2m_ctx* c) {
 static f2m_status price_grow(f2m_ctx* c, const PriceCtl& h, bool* again) {
   *again = false;
   if ((int64_t)h.count > c->pairs_cap) {
-    dfree(c->d_pairs);
-    c->pairs_cap = (int64_t)h.count + ((int64_t)h.count >> 2) + 1024;
-    CK(c, dalloc(&c->d_pairs, c->pairs_cap));
+    CK(c, dgrow(&c->d_pairs, &c->pairs_cap, (int64_t)h.count, (int64_t)h.count + ((int64_t)h.count >> 2) + 1024));
     *again = true;
   }
   if ((int64_t)h.listed > c->plist_cap) {
-    dfree(c->d_plist);
-    c->plist_cap = std::min<int64_t>((int64_t)h.listed + ((int64_t)h.listed >> 3) + 1024, INT_MAX);
-    CK(c, dalloc(&c->d_plist, c->plist_cap));
+    CK(c, dgrow(&c->d_plist, &c->plist_cap, (int64_t)h.listed,
+                std::min<int64_t>((int64_t)h.listed + ((int64_t)h.listed >> 3) + 1024, INT_MAX)));
     *again = true;
   }
   return F2M_OK;
@@ -885,36 +882,38 @@ static f2m_status price_grow(f2m_ctx* c, const PriceCtl& h, bool* again) {
 static f2m_status price_mma(f2m_ctx* c, const int32_t* lam, int32_t fb, double* ms) {
   // the tile-pair list depends only on the segments scanned: it stays on the
   // device from one scan to the next while they are the same
-  if (!c->d_pts4) {
-    CK(c, dalloc(&c->d_count, 1));
-    CK(c, dalloc(&c->d_tile, 1));
-    CK(c, dalloc(&c->d_pts4, c->n));
-    CK(c, dalloc(&c->d_pstat, 1));
-    CK(c, dalloc(&c->d_mncand, 1));
-    c->mcand_cap = std::max<int64_t>(4LL * c->n, 1 << 20);
-    CK(c, dalloc(&c->d_mcand, c->mcand_cap));
-  }
+  if (!c->d_count) CK(c, dalloc(&c->d_count, 1));
+  if (!c->d_tile) CK(c, dalloc(&c->d_tile, 1));
+  if (!c->d_pts4) CK(c, dalloc(&c->d_pts4, c->n));
+  if (!c->d_pstat) CK(c, dalloc(&c->d_pstat, 1));
+  if (!c->d_mncand) CK(c, dalloc(&c->d_mncand, 1));
+  if (!c->d_mcand) CK(c, dgrow(&c->d_mcand, &c->mcand_cap, 1, std::max<int64_t>(4LL * c->n, 1 << 20)));
   if (!(c->tiles_valid && c->tiles_seg_scan == c->seg_scan)) {
     std::vector<int4> tiles, tblk;
     std::vector<int2> ranges;
     build_mma_tiles(c, tiles, tblk, ranges);
+    c->tiles_valid = false;
     if ((int64_t)ranges.size() > c->mblocks_cap) {
       dfree(c->d_mranges);
       dfree(c->d_mbox);
       dfree(c->d_mlmax);
-      c->mblocks_cap = (int64_t)ranges.size() + 64;
-      CK(c, dalloc(&c->d_mranges, c->mblocks_cap));
-      CK(c, dalloc(&c->d_mbox, c->mblocks_cap));
-      CK(c, dalloc(&c->d_mlmax, c->mblocks_cap));
+      c->mblocks_cap = 0;
+      const int64_t room = (int64_t)ranges.size() + 64;
+      CK(c, dalloc(&c->d_mranges, room));
+      CK(c, dalloc(&c->d_mbox, room));
+      CK(c, dalloc(&c->d_mlmax, room));
+      c->mblocks_cap = room;
     }
     if ((int64_t)tiles.size() > c->mtiles_cap) {
       dfree(c->d_tiles);
       dfree(c->d_mtblk);
       dfree(c->d_mframes);
-      c->mtiles_cap = (int64_t)tiles.size() + 64;
-      CK(c, dalloc(&c->d_tiles, c->mtiles_cap));
-      CK(c, dalloc(&c->d_mtblk, c->mtiles_cap));
-      CK(c, dalloc(&c->d_mframes, c->mtiles_cap));
+      c->mtiles_cap = 0;
+      const int64_t room = (int64_t)tiles.size() + 64;
+      CK(c, dalloc(&c->d_tiles, room));
+      CK(c, dalloc(&c->d_mtblk, room));
+      CK(c, dalloc(&c->d_mframes, room));
+      c->mtiles_cap = room;
     }
     if (!tiles.empty()) {
       CK(c, cudaMemcpyAsync(c->d_mranges, ranges.data(), sizeof(int2) * ranges.size(), cudaMemcpyHostToDevice, c->st));
@@ -944,9 +943,7 @@ static f2m_status price_mma(f2m_ctx* c, const int32_t* lam, int32_t fb, double* 
     if (ms) *ms += elapsed_ms(c);
     if (pstat) return fail(c, F2M_ERR_TIMEOUT, "pricing scan: a tensor-core wait ran past its budget");
     if ((int64_t)ncand > c->mcand_cap) {  // the candidate list overflowed: grow it, scan again
-      dfree(c->d_mcand);
-      c->mcand_cap = (int64_t)ncand + ((int64_t)ncand >> 2) + 1024;
-      CK(c, dalloc(&c->d_mcand, c->mcand_cap));
+      CK(c, dgrow(&c->d_mcand, &c->mcand_cap, (int64_t)ncand, (int64_t)ncand + ((int64_t)ncand >> 2) + 1024));
       continue;
     }
     c->npairs = (int64_t)cnt;
@@ -1019,10 +1016,7 @@ f2m_status f2m::price_internal(f2m_ctx* c, double* ms, const int32_t* lam_overri
       }
     }
     if (culled) {
-      if (!c->d_plist) {
-        c->plist_cap = 64LL * c->price_blocks + 4096;
-        CK(c, dalloc(&c->d_plist, c->plist_cap));
-      }
+      if (!c->d_plist) CK(c, dgrow(&c->d_plist, &c->plist_cap, 1, 64LL * c->price_blocks + 4096));
       if (!c->seg_scan.empty())
         CK(c, cudaMemcpyAsync(d_scan, c->seg_scan.data(), nseg, cudaMemcpyHostToDevice, c->st));
     }
@@ -1131,19 +1125,13 @@ extern "C" f2m_status f2m_price(f2m_ctx* c, int64_t* count, int32_t* pairs, int6
 // outside the CSR (a scan's)
 f2m_status f2m::merge_internal(f2m_ctx* c, const int2* d_pairs, int64_t npairs, double* ms, bool fresh) {
   const int32_t n = c->n;
-  if (!c->d_deg) {
-    CK(c, dalloc(&c->d_deg, n + 1));
-    CK(c, dalloc(&c->d_tmp_rp, n + 1));
-    CK(c, dalloc(&c->d_new_rp, n + 1));
-    CK(c, dalloc(&c->d_block_sums, (int64_t)scan_scratch_ints(n)));
-  }
+  if (!c->d_deg) CK(c, dalloc(&c->d_deg, n + 1));
+  if (!c->d_tmp_rp) CK(c, dalloc(&c->d_tmp_rp, n + 1));
+  if (!c->d_new_rp) CK(c, dalloc(&c->d_new_rp, n + 1));
+  if (!c->d_block_sums) CK(c, dalloc(&c->d_block_sums, (int64_t)scan_scratch_ints(n)));
   const int64_t need = c->nnz + 2 * npairs;
   if (need >= INT_MAX) return fail(c, F2M_ERR_INVALID_ARG, "graph would exceed 2^31 entries");
-  if (need > c->tmp_col_cap) {
-    dfree(c->d_tmp_col);
-    c->tmp_col_cap = need + (need >> 3);
-    CK(c, dalloc(&c->d_tmp_col, c->tmp_col_cap));
-  }
+  CK(c, dgrow(&c->d_tmp_col, &c->tmp_col_cap, need, need + (need >> 3)));
   MergeBuffers mb{c->d_deg, c->d_tmp_rp, c->d_tmp_col, c->d_new_rp, c->d_block_sums, c->d_check};
   if (!fresh) CK(c, reset_check(c));
   CK(c, cudaEventRecord(c->ev0, c->st));
@@ -1151,16 +1139,8 @@ f2m_status f2m::merge_internal(f2m_ctx* c, const int2* d_pairs, int64_t npairs, 
     CK(c, launch_merge_count(c->d_rp, d_pairs, npairs, n, mb, c->st));
     CK(c, launch_merge_fill(c->d_rp, c->d_ec, d_pairs, npairs, n, mb, c->st));
   }
-  if (need > c->ec_alt_cap) {  // the array the merged rows go to
-    dfree(c->d_ec_alt);
-    c->ec_alt_cap = need + (need >> 3);
-    CK(c, dalloc(&c->d_ec_alt, c->ec_alt_cap));
-  }
-  if (need > c->x2_cap) {
-    dfree(c->d_x2);
-    c->x2_cap = need + (need >> 3);
-    CK(c, dalloc(&c->d_x2, c->x2_cap));
-  }
+  CK(c, dgrow(&c->d_ec_alt, &c->ec_alt_cap, need, need + (need >> 3)));  // the merged rows go there
+  CK(c, dgrow(&c->d_x2, &c->x2_cap, need, need + (need >> 3)));
   if (fresh) {
     CK(c, plan_merge(c->d_xy, c->d_rp, c->d_ec, d_pairs, npairs, n, need, mb, c->d_ec_alt, c->plan, c->st));
     std::swap(c->d_ec, c->d_ec_alt);
@@ -1247,29 +1227,30 @@ static f2m_status fin_gpu_phase1(f2m_ctx* c, const std::vector<int2>& fblocks, c
   const int32_t n = c->n;
   const int32_t nb = (int32_t)fblocks.size();
   GdpPlan& P = c->plan;
-  if (!c->d_fpi) {  // node-sized state, both copies of every node
-    CK(c, dalloc(&c->d_fpi, 2LL * n));
-    CK(c, dalloc(&c->d_fdist, 2LL * n));
-    CK(c, dalloc(&c->d_fex, 2LL * n));
-    CK(c, dalloc(&c->d_fvia, 2LL * n));
-    CK(c, dalloc(&c->d_fpred, 2LL * n));
-    CK(c, dalloc(&c->d_freach, 2LL * n));
-    CK(c, dalloc(&c->d_fclos, 2LL * n));
-    CK(c, dalloc(&c->d_forder, 2LL * n));
-    CK(c, dalloc(&c->d_fstat, 1));
-    CK(c, pin_alloc((void**)&c->h_fpi, sizeof(int64_t) * 2 * (size_t)n));
-    CK(c, pin_alloc((void**)&c->h_fex, sizeof(int32_t) * 2 * (size_t)n));
-  }
+  // node-sized state, both copies of every node
+  if (!c->d_fpi) CK(c, dalloc(&c->d_fpi, 2LL * n));
+  if (!c->d_fdist) CK(c, dalloc(&c->d_fdist, 2LL * n));
+  if (!c->d_fex) CK(c, dalloc(&c->d_fex, 2LL * n));
+  if (!c->d_fvia) CK(c, dalloc(&c->d_fvia, 2LL * n));
+  if (!c->d_fpred) CK(c, dalloc(&c->d_fpred, 2LL * n));
+  if (!c->d_freach) CK(c, dalloc(&c->d_freach, 2LL * n));
+  if (!c->d_fclos) CK(c, dalloc(&c->d_fclos, 2LL * n));
+  if (!c->d_forder) CK(c, dalloc(&c->d_forder, 2LL * n));
+  if (!c->d_fstat) CK(c, dalloc(&c->d_fstat, 1));
+  if (!c->h_fpi) CK(c, pin_alloc((void**)&c->h_fpi, sizeof(int64_t) * 2 * (size_t)n));
+  if (!c->h_fex) CK(c, pin_alloc((void**)&c->h_fex, sizeof(int32_t) * 2 * (size_t)n));
   if (nb > c->fblk_cap) {
     dfree(c->d_fblk);
     dfree(c->d_fcaps);
     dfree(c->d_fheap_off);
     dfree(c->d_fpush);
-    c->fblk_cap = nb + nb / 4 + 16;
-    CK(c, dalloc(&c->d_fblk, c->fblk_cap));
-    CK(c, dalloc(&c->d_fcaps, c->fblk_cap));
-    CK(c, dalloc(&c->d_fheap_off, c->fblk_cap + 1));
-    CK(c, dalloc(&c->d_fpush, c->fblk_cap));
+    c->fblk_cap = 0;
+    const int64_t room = nb + nb / 4 + 16;
+    CK(c, dalloc(&c->d_fblk, room));
+    CK(c, dalloc(&c->d_fcaps, room));
+    CK(c, dalloc(&c->d_fheap_off, room + 1));
+    CK(c, dalloc(&c->d_fpush, room));
+    c->fblk_cap = room;
   }
   CK(c, cudaMemcpyAsync(c->d_fblk, fblocks.data(), sizeof(int2) * nb, cudaMemcpyHostToDevice, c->st));
   CK(c, launch_fin_block_caps(c->d_fblk, nb, P.irp, c->d_fcaps, c->st));
@@ -1282,8 +1263,10 @@ static f2m_status fin_gpu_phase1(f2m_ctx* c, const std::vector<int2>& fblocks, c
   const size_t item = fin_heap_item_bytes();
   if ((int64_t)off[nb] > c->fheap_cap) {
     dfree(c->d_fheap);
-    c->fheap_cap = off[nb] + off[nb] / 4 + 1024;
-    CK(c, dalloc(&c->d_fheap, (int64_t)(c->fheap_cap * item)));
+    c->fheap_cap = 0;
+    const int64_t room = off[nb] + off[nb] / 4 + 1024;
+    CK(c, dalloc(&c->d_fheap, (int64_t)(room * item)));
+    c->fheap_cap = room;
   }
   CK(c, cudaMemcpyAsync(c->d_fheap_off, off.data(), sizeof(long long) * (nb + 1), cudaMemcpyHostToDevice, c->st));
   CK(c, cudaMemsetAsync(c->d_fstat, 0, sizeof(int32_t), c->st));
@@ -1613,9 +1596,10 @@ extern "C" f2m_status f2m_get_x(f2m_ctx* c, int64_t* nnz_inout, int32_t* row_ptr
     if (c->out_cap < c->nnz) {
       dfree(c->d_out_a);
       dfree(c->d_out_b);
+      c->out_cap = 0;
+      CK(c, dalloc(&c->d_out_a, c->nnz));
+      CK(c, dalloc(&c->d_out_b, c->nnz));
       c->out_cap = c->nnz;
-      CK(c, dalloc(&c->d_out_a, c->out_cap));
-      CK(c, dalloc(&c->d_out_b, c->out_cap));
     }
     CK(c, launch_split_ec(c->d_ec, c->nnz, c->d_out_a, c->d_out_b, c->st));
     if (col) CK(c, cudaMemcpyAsync(col, c->d_out_a, sizeof(int32_t) * c->nnz, cudaMemcpyDefault, c->st));

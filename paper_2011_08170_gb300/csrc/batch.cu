@@ -568,11 +568,7 @@ static f2m_status cluster_plan(f2m_batch* b) {
     for (cudaStream_t& q : b->cl_st) CK(c, cudaStreamCreateWithFlags(&q, cudaStreamNonBlocking));
     for (cudaEvent_t& q : b->cl_ev) CK(c, cudaEventCreateWithFlags(&q, cudaEventDisableTiming));
   }
-  if (b->pk_cap < c->nnz) {
-    dfree(b->d_pk);
-    b->pk_cap = c->ec_cap;
-    CK(c, dalloc(&b->d_pk, b->pk_cap));
-  }
+  CK(c, dgrow(&b->d_pk, &b->pk_cap, c->nnz, c->ec_cap));
   CK(c, cudaMemcpyAsync(b->d_cl_all, b->cl_inst.data(), sizeof(ClusterInst) * K, cudaMemcpyHostToDevice, c->st));
   CK(c, cluster_pack(P.irp, P.iec, b->d_cl_all, K, c->p.frac_bits, b->d_pk, c->st));
   CK(c, cudaStreamSynchronize(c->st));
@@ -654,11 +650,7 @@ static f2m_status batch_ring_phase(f2m_batch* b, const std::vector<uint8_t>& act
   }
   waves.push_back((int32_t)list.size());
   const int32_t tiles = (int32_t)list.size();
-  if (b->rlist_cap < tiles) {
-    dfree(b->d_rlist);
-    b->rlist_cap = tiles + tiles / 8 + 64;
-    CK(c, dalloc(&b->d_rlist, b->rlist_cap));
-  }
+  CK(c, dgrow(&b->d_rlist, &b->rlist_cap, tiles, tiles + tiles / 8 + 64));
   if (!b->h_rseg) CK(c, pin_alloc((void**)&b->h_rseg, sizeof(RingSeg) * b->count));
   CK(c, cudaMemcpyAsync(b->d_rlist, list.data(), sizeof(RingTile) * tiles, cudaMemcpyHostToDevice, c->st));
   CK(c, ring_build(c->plan, c->d_seg_off, b->d_rlist, tiles, K, c->p.frac_bits, rows * c->nnz / c->n, b->count, c->ring,
@@ -1163,11 +1155,7 @@ extern "C" f2m_status f2m_batch_get_x(f2m_batch* b, int32_t i, int64_t* nnz_inou
   const bool drp = on_device(row_ptr), dcol = on_device(col), dx2 = on_device(x2);
   if ((row_ptr && !drp) || (col && !dcol)) {
     const int64_t need = (int64_t)rows + nz;
-    if (b->tmp_cap < need) {
-      dfree(b->d_tmp_a);
-      b->tmp_cap = need + need / 2;
-      CK(c, dalloc(&b->d_tmp_a, b->tmp_cap));
-    }
+    CK(c, dgrow(&b->d_tmp_a, &b->tmp_cap, need, need + need / 2));
   }
   int32_t* o_rp = row_ptr ? (drp ? row_ptr : b->d_tmp_a) : nullptr;
   int32_t* o_col = col ? (dcol ? col : b->d_tmp_a + rows) : nullptr;

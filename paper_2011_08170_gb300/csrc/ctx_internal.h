@@ -183,6 +183,18 @@ void dfree(T*& p) {
   p = nullptr;
 }
 
+// room for `need` items in *p: kept, or replaced by a block of `room`.  The capacity
+// is what *p holds at any time, so that a call after a failed one tries again
+template <typename T>
+cudaError_t dgrow(T** p, int64_t* cap, int64_t need, int64_t room) {
+  if (*p && *cap >= need) return cudaSuccess;
+  dfree(*p);
+  *cap = 0;
+  const cudaError_t e = dalloc(p, room);
+  if (e == cudaSuccess) *cap = room;
+  return e;
+}
+
 // for a caller that has already waited for every use of the block
 template <typename T>
 void dfree_synced(T*& p) {

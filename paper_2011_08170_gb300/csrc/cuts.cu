@@ -818,10 +818,7 @@ CutArgs cut_args(const f2m_ctx* c) {
 
 template <typename T>
 cudaError_t grow(T** p, int64_t* cap, int64_t need) {
-  if (need <= *cap) return cudaSuccess;
-  dfree(*p);
-  *cap = need + need / 4 + 16;
-  return dalloc(p, *cap);
+  return dgrow(p, cap, need, need + need / 4 + 16);
 }
 
 }  // namespace
@@ -838,10 +835,12 @@ f2m_status cut_lists(f2m_ctx* c) {
     dfree(S->d_cnt);
     dfree(S->d_ptr);
     dfree(S->d_scan);
-    S->ptr_cap = S->M + 1 + 1024;
-    CK(c, dalloc(&S->d_cnt, S->ptr_cap));
-    CK(c, dalloc(&S->d_ptr, S->ptr_cap));
-    CK(c, dalloc(&S->d_scan, (int64_t)scan_scratch_ints((int32_t)S->ptr_cap)));
+    S->ptr_cap = 0;
+    const int64_t room = S->M + 1 + 1024;
+    CK(c, dalloc(&S->d_cnt, room));
+    CK(c, dalloc(&S->d_ptr, room));
+    CK(c, dalloc(&S->d_scan, (int64_t)scan_scratch_ints((int32_t)room)));
+    S->ptr_cap = room;
   }
   const int32_t n = c->n, L = S->L, M = (int32_t)S->M;
   const GdpPlan& P = c->plan;
@@ -960,10 +959,8 @@ f2m_status cut_price(f2m_ctx* c, double* ms) {
   const int32_t* lam = cur_lambda(c, &fb);
   if (fb != c->p.frac_bits) return fail(c, F2M_ERR_INVALID_ARG, "cut duals are held at F bits");
   const int64_t n1 = c->n + 1;
-  if (!S->d_lamp) {
-    CK(c, dalloc(&S->d_lamp, c->n));
-    CK(c, dalloc(&S->d_small, 4));
-  }
+  if (!S->d_lamp) CK(c, dalloc(&S->d_lamp, c->n));
+  if (!S->d_small) CK(c, dalloc(&S->d_small, 4));
   const CutArgs a = cut_args(c);
   CK(c, cudaMemsetAsync(S->d_small, 0, sizeof(int32_t), c->st));
   cut_lamp_kernel<<<grid_of(c->n, 256), 256, 0, c->st>>>(a, lam, S->d_mu[S->cur], S->d_lamp, S->d_small);
@@ -981,12 +978,14 @@ f2m_status cut_price(f2m_ctx* c, double* ms) {
     dfree(S->d_kpos);
     dfree(S->d_pairs2);
     dfree(S->d_pscan);
-    S->pair_cap = np + np / 4 + 1024;
-    if (S->pair_cap >= INT_MAX) return fail(c, F2M_ERR_INVALID_ARG, "too many pricing pairs");
-    CK(c, dalloc(&S->d_keep, S->pair_cap + 1));
-    CK(c, dalloc(&S->d_kpos, S->pair_cap + 1));
-    CK(c, dalloc(&S->d_pairs2, S->pair_cap));
-    CK(c, dalloc(&S->d_pscan, (int64_t)scan_scratch_ints((int32_t)S->pair_cap + 1)));
+    S->pair_cap = 0;
+    const int64_t room = np + np / 4 + 1024;
+    if (room >= INT_MAX) return fail(c, F2M_ERR_INVALID_ARG, "too many pricing pairs");
+    CK(c, dalloc(&S->d_keep, room + 1));
+    CK(c, dalloc(&S->d_kpos, room + 1));
+    CK(c, dalloc(&S->d_pairs2, room));
+    CK(c, dalloc(&S->d_pscan, (int64_t)scan_scratch_ints((int32_t)room + 1)));
+    S->pair_cap = room;
   }
   (void)n1;
   cut_pair_keep_kernel<<<grid_of(np, 256), 256, 0, c->st>>>(c->d_pairs, np, c->d_xy, a, lam, S->d_mu[S->cur], fb,
@@ -1011,22 +1010,21 @@ f2m_status cut_separate(f2m_ctx* c, int32_t* d_comp_out, int32_t* m_out) {
   if (!c->cuts) c->cuts = new CutState();
   CutState* S = c->cuts;
   const int32_t n = c->n;
-  if (!S->d_lab) {
-    CK(c, dalloc(&S->d_lab, n));
-    CK(c, dalloc(&S->d_cross, n));
-    CK(c, dalloc(&S->d_flag, n + 1));
-    CK(c, dalloc(&S->d_rank, n + 1));
-    if (!S->d_small) CK(c, dalloc(&S->d_small, 4));
-    if (S->ptr_cap < n + 1) {
-      dfree(S->d_cnt);
-      dfree(S->d_ptr);
-      dfree(S->d_scan);
-      S->ptr_cap = n + 1;
-      CK(c, dalloc(&S->d_cnt, S->ptr_cap));
-      CK(c, dalloc(&S->d_ptr, S->ptr_cap));
-      CK(c, dalloc(&S->d_scan, (int64_t)scan_scratch_ints((int32_t)S->ptr_cap)));
-      S->built_version = -1;
-    }
+  if (!S->d_lab) CK(c, dalloc(&S->d_lab, n));
+  if (!S->d_cross) CK(c, dalloc(&S->d_cross, n));
+  if (!S->d_flag) CK(c, dalloc(&S->d_flag, n + 1));
+  if (!S->d_rank) CK(c, dalloc(&S->d_rank, n + 1));
+  if (!S->d_small) CK(c, dalloc(&S->d_small, 4));
+  if (S->ptr_cap < n + 1) {
+    dfree(S->d_cnt);
+    dfree(S->d_ptr);
+    dfree(S->d_scan);
+    S->ptr_cap = 0;
+    S->built_version = -1;
+    CK(c, dalloc(&S->d_cnt, n + 1));
+    CK(c, dalloc(&S->d_ptr, n + 1));
+    CK(c, dalloc(&S->d_scan, (int64_t)scan_scratch_ints(n + 1)));
+    S->ptr_cap = n + 1;
   }
   const int g = grid_of(n, 256);
   cc_init_kernel<<<g, 256, 0, c->st>>>(S->d_lab, n);

@@ -1,5 +1,5 @@
 """Decisions that the library makes on the host, without a GPU: which arrays a kernel
-may write to."""
+may write to, and what a work array says of itself after an allocation failed."""
 import ctypes as C
 import os
 import shutil
@@ -34,3 +34,27 @@ UNREGISTERED, HOST, DEVICE, MANAGED = 0, 1, 2, 3  # cudaMemoryType
 def test_kernels_write_only_where_they_reach(rules, kind, device, current, want):
     # a read-out's kernel stores to arrays on its own GPU; another GPU's take a copy
     assert bool(rules.shim_kernel_reaches(kind, device, current)) == want
+
+
+OK, HELD, COVERS = 1, 2, 4
+
+
+@pytest.mark.parametrize("had,need,room,blocks,want", [
+    (0, 10, 15, 1, OK | HELD | COVERS),   # the first block
+    (20, 10, 15, 0, OK | HELD | COVERS),  # large enough
+    (5, 10, 15, 1, OK | HELD | COVERS),   # replaced
+    (5, 10, 15, 0, 0),                    # no memory: nothing held, and none claimed
+    (0, 10, 15, 0, 0)])
+def test_a_failed_allocation_claims_no_room(rules, had, need, room, blocks, want):
+    # a capacity noted before the allocation had the next call write through a null pointer
+    rules.shim_grow.argtypes = [C.c_longlong] * 3 + [C.c_int]
+    assert rules.shim_grow(had, need, room, blocks) == want
+
+
+def test_no_capacity_is_noted_before_its_allocation():
+    # the sources: a member's capacity is assigned from its size only after the block is there
+    import re
+    for name in ("api.cu", "batch.cu", "cuts.cu"):
+        src = open(os.path.join(CSRC, name)).read()
+        for m in re.finditer(r"(\w+->(\w+)_cap) = (?!0;)[^;]*;\s*CK\(c, dalloc\(&\w+->d_\w+, \1\)\)", src):
+            raise AssertionError(f"{name}: {m.group(0)}")
