@@ -377,7 +377,7 @@ extern "C" void f2m_destroy(f2m_ctx* c) {
 }
 
 f2m_status f2m::check_params_internal(const f2m_params& p) {
-  if (p.frac_bits < 1 || p.frac_bits > 8) return fail(nullptr, F2M_ERR_INVALID_ARG, "frac_bits must be in 1..8");
+  if (p.frac_bits < 1 || p.frac_bits > kMaxFracBits) return fail(nullptr, F2M_ERR_INVALID_ARG, "frac_bits must be in 1..8");
   if (p.damping_shift < 1 || p.damping_shift > 8) return fail(nullptr, F2M_ERR_INVALID_ARG, "damping_shift must be in 1..8");
   if (p.gdp_lanes != 0 && p.gdp_lanes != 1)
     return fail(nullptr, F2M_ERR_INVALID_ARG, "gdp_lanes must be 0 or 1");

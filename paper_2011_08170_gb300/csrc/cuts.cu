@@ -480,12 +480,12 @@ __global__ void __launch_bounds__(kCutThreads, 1) cut_gdp_kernel(const __grid_co
   const int32_t* rp = in ? s_rp : A.irp + v0;
   const int32_t* cp = in ? s_cp : A.cut_ptr + s0;
   const int own = in ? place(v0 < n ? v0 : 0) : 0, own_cut = in && nc ? place(wn * 32 + s0) : 0;
-  // z fits 32 bits while the costs stay below 2^29 and the values below lim
+  // z fits 32 bits while the values stay below lim: a cost times 2^F is below 2^29
+  // whatever the points
+  static_assert(2LL * kCoordLimit * kCoordLimit << 2 * kMaxFracBits < 1LL << 58, "costs in units 2^-F");
   const int lim = ((1 << 30) - 1 + (1 << 29)) / (2 + 2 * L);
-  bool cheap = true, any_long = false;
-  if (in)
-    for (int i = tid; i < ne + nk; i += kCutThreads) cheap &= ((long long)rtab[i].z << A.F) < (1 << 29);
-  cheap = __syncthreads_and(cheap);
+  bool any_long = false;
+  __syncthreads();  // the tables are complete
   for (int i = tid; i < nc; i += kCutThreads) any_long |= cp[i + 1] - cp[i] > kLongCut;
   any_long = __syncthreads_or(any_long);
   int par = 0;  // the buffers that hold the result
@@ -505,7 +505,7 @@ __global__ void __launch_bounds__(kCutThreads, 1) cut_gdp_kernel(const __grid_co
         big |= x >= lim || x <= -lim;
         val[i] = x;
       }
-      narrow = cheap & !__syncthreads_or(big);
+      narrow = !__syncthreads_or(big);
     }
     auto new_lambda = [&](int i, long long lv, long long b, long long c) {
       const long long d = step_ll(b, c, A.shift), nl = lv + d;
