@@ -870,9 +870,10 @@ static f2m_status price_grow(f2m_ctx* c, const PriceCtl& h, bool* again) {
     CK(c, dgrow(&c->d_pairs, &c->pairs_cap, (int64_t)h.count, (int64_t)h.count + ((int64_t)h.count >> 2) + 1024));
     *again = true;
   }
-  if ((int64_t)h.listed > c->plist_cap) {
-    CK(c, dgrow(&c->d_plist, &c->plist_cap, (int64_t)h.listed,
-                std::min<int64_t>((int64_t)h.listed + ((int64_t)h.listed >> 3) + 1024, INT_MAX)));
+  if (h.listed > (unsigned long long)c->plist_cap) {
+    const int64_t room = price_list_room(h.listed);
+    if (!room) return fail(c, F2M_ERR_INVALID_ARG, "too many pricing tile pairs");
+    CK(c, dgrow(&c->d_plist, &c->plist_cap, (int64_t)h.listed, room));
     *again = true;
   }
   return F2M_OK;

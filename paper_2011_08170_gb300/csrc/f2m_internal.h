@@ -115,8 +115,8 @@ constexpr int kPriceLargeI = 512;  // the large tile
 constexpr int kPriceLargeJ = 512;
 struct PriceCtl {
   unsigned long long count;  // pairs found (past the capacity too)
+  unsigned long long listed; // block pairs of the culled scan's list (past its capacity too)
   unsigned int next;         // tile pairs handed out
-  unsigned int listed;       // block pairs of the culled scan's list (past its capacity too)
   unsigned int rows;         // i-points of a scan of some rows
 };
 struct PriceScan {
@@ -142,6 +142,12 @@ struct PriceScan {
   int32_t nseg, n, fb;
   int32_t split;              // CTAs that share a tile pair (set by the launchers)
 };
+// room for a list of `listed` block pairs, which the scan hands out by 32-bit
+// numbers; 0: too many
+inline long long price_list_room(unsigned long long listed) {
+  const unsigned long long most = 0x7fffffffull, room = listed + (listed >> 3) + 1024;
+  return listed >= most ? 0 : (long long)(room < most ? room : most);
+}
 // points, blocks and cleared counters of a scan of lambda sc.lam
 cudaError_t launch_pricing_prep(const PriceScan& sc, const int32_t* perm, int32_t nblocks, float4* pts, float4* box,
                                 float* smax, cudaStream_t st);

@@ -193,10 +193,10 @@ pricing_cull_kernel(const float4* __restrict__ box, const float* __restrict__ sm
     }
     const unsigned m = __ballot_sync(0xffffffffu, keep);
     if (!m) continue;
-    unsigned base = 0;
-    if (lane == 0) base = atomicAdd(&ctl->listed, (unsigned)__popc(m));
+    unsigned long long base = 0;
+    if (lane == 0) base = atomicAdd(&ctl->listed, (unsigned long long)__popc(m));
     base = __shfl_sync(0xffffffffu, base, 0) + __popc(m & ((1u << lane) - 1u));
-    if (keep && base < (unsigned)cap) list[base] = make_int2(bi, bj);
+    if (keep && base < (unsigned long long)cap) list[base] = make_int2(bi, bj);
   }
 }
 
@@ -350,7 +350,8 @@ pricing_kernel(const __grid_constant__ PriceScan sc) {
   const int rows = FORM == kPriceRows ? (int)sc.ctl->rows : 0;
   const int nj_tiles = (sc.n + J - 1) / J;
   const long long ntiles = FORM == kPriceFull  ? sc.seg_tile[sc.nseg]
-                           : FORM == kPriceList ? min((int)sc.ctl->listed, sc.list_cap)
+                           // (a list that outgrew its room is scanned once it has the room)
+                           : FORM == kPriceList ? (sc.ctl->listed <= (unsigned long long)sc.list_cap ? (int)sc.ctl->listed : 0)
                                                 : (long long)((rows + I - 1) / I) * nj_tiles;
   for (;;) {
     __syncthreads();

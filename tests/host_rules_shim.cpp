@@ -34,3 +34,5 @@ extern "C" int shim_grow(long long had, long long need, long long room, int bloc
   std::free(p);
   return r;
 }
+
+extern "C" long long shim_price_list_room(unsigned long long listed) { return f2m::price_list_room(listed); }

@@ -1,5 +1,6 @@
 """Decisions that the library makes on the host, without a GPU: which arrays a kernel
-may write to, and what a work array says of itself after an allocation failed."""
+may write to, what a work array says of itself after an allocation failed, and how
+many block pairs a culled scan lists."""
 import ctypes as C
 import os
 import shutil
@@ -58,3 +59,17 @@ def test_no_capacity_is_noted_before_its_allocation():
         src = open(os.path.join(CSRC, name)).read()
         for m in re.finditer(r"(\w+->(\w+)_cap) = (?!0;)[^;]*;\s*CK\(c, dalloc\(&\w+->d_\w+, \1\)\)", src):
             raise AssertionError(f"{name}: {m.group(0)}")
+
+
+@pytest.mark.parametrize("listed", [0, 1, 4096, 1 << 20, (1 << 31) - 2])
+def test_a_listed_scan_gets_room(rules, listed):
+    rules.shim_price_list_room.argtypes, rules.shim_price_list_room.restype = [C.c_ulonglong], C.c_longlong
+    assert listed <= rules.shim_price_list_room(listed) < 1 << 31
+
+
+@pytest.mark.parametrize("listed", [(1 << 31) - 1, 1 << 31, (1 << 32) - 1, 1 << 32, (1 << 32) + 5, 8_590_000_128])
+def test_a_list_past_the_handed_out_numbers_is_refused(rules, listed):
+    # 2^24 points make 131,072 blocks, 8.6e9 pairs of them: clamped to 2^31 - 1 the
+    # scan and its list never met, and past 2^32 a 32-bit count wrapped
+    rules.shim_price_list_room.argtypes, rules.shim_price_list_room.restype = [C.c_ulonglong], C.c_longlong
+    assert rules.shim_price_list_room(listed) == 0
