@@ -223,17 +223,27 @@ void finisher_pool_wake(int32_t threads) {
   if (turn.owns_lock()) worker_pool().wake(threads);  // (busy with another job: nothing to do)
 }
 
-// Work arrays outlive their context, up to kWorkCacheMax bytes in all: their pages
-// (88 bytes a node) took longer to touch anew than most of what a create does
-// (6.5 ms at 1.6 M nodes, 0.2 ms at 100,000).  A search trusts only what carries its
-// own stamp, and an array's stamps go on counting from one context to the next.
+// Work arrays outlive their context, up to kWorkCacheMax bytes in all, the searchers'
+// heaps and lists counted: their pages (88 bytes a node) took longer to touch anew
+// than most of what a create does (6.5 ms at 1.6 M nodes, 0.2 ms at 100,000).  A
+// context takes arrays of up to twice its own size (of any size up to
+// kWorkSmall nodes), so that a small one does not hold a large one's.  A search
+// trusts only what carries its own stamp, and an array's stamps go on counting
+// from one context to the next.
 namespace {
 std::mutex g_work_mu;
 std::vector<FinisherWork*> g_work_free;
 size_t g_work_bytes = 0;
 constexpr size_t kWorkCacheMax = (size_t)1 << 28;
 
-size_t work_bytes(const FinisherWork* w) { return w->pi.capacity() * 44; }
+constexpr size_t kWorkSmall = (size_t)1 << 14;
+
+size_t work_bytes(const FinisherWork* w) {
+  size_t b = sizeof(*w) + w->pi.capacity() * 44 + w->workers.capacity() * sizeof(Searcher);
+  for (const Searcher& s : w->workers)
+    b += s.heap.capacity() * sizeof(Searcher::Item) + s.order.capacity() * sizeof(int32_t);
+  return b;
+}
 }  // namespace
 
 FinisherWork* finisher_work_new() { return new FinisherWork(); }
@@ -243,8 +253,9 @@ FinisherWork* finisher_work_take(int32_t n) {
   {
     std::lock_guard<std::mutex> lk(g_work_mu);
     size_t best = g_work_free.size();
+    const size_t most = 2 * std::max(2 * (size_t)n, kWorkSmall);
     for (size_t i = 0; i < g_work_free.size(); ++i)
-      if (g_work_free[i]->pi.size() >= 2 * (size_t)n &&
+      if (g_work_free[i]->pi.size() >= 2 * (size_t)n && g_work_free[i]->pi.size() <= most &&
           (best == g_work_free.size() || g_work_free[i]->pi.size() < g_work_free[best]->pi.size()))
         best = i;
     if (best < g_work_free.size()) {
@@ -259,10 +270,11 @@ FinisherWork* finisher_work_take(int32_t n) {
 }
 
 void finisher_work_free(FinisherWork* w) {
+  const size_t bytes = work_bytes(w);
   {
     std::lock_guard<std::mutex> lk(g_work_mu);
-    if (g_work_bytes + work_bytes(w) <= kWorkCacheMax && g_work_free.size() < 64) {
-      g_work_bytes += work_bytes(w);
+    if (g_work_bytes + bytes <= kWorkCacheMax && g_work_free.size() < 64) {
+      g_work_bytes += bytes;
       g_work_free.push_back(w);
       return;
     }
