@@ -51,6 +51,7 @@
 #include <cstring>
 #include <functional>
 #include <mutex>
+#include <system_error>
 #include <thread>
 #include <vector>
 
@@ -296,10 +297,14 @@ void host_copy(const std::vector<HostCopy>& parts) {
   };
   const int32_t threads = std::min<int32_t>(8, std::max<int32_t>(1, (int32_t)std::thread::hardware_concurrency()));
   std::unique_lock<std::mutex> turn(g_pool_turn, std::try_to_lock);
-  if (turn.owns_lock() && threads > 1 && pieces.size() >= 16)
-    worker_pool().run(threads, work);
-  else
-    work(0);  // small, or the workers are busy with another job
+  if (turn.owns_lock() && threads > 1 && pieces.size() >= 16) {
+    try {
+      worker_pool().run(threads, work);
+      return;
+    } catch (const std::system_error&) {  // no threads to be had: nothing has run yet
+    }
+  }
+  work(0);  // also small, or the workers are busy with another job
 }
 
 void finisher_work_reserve(FinisherWork* w, int32_t n) {

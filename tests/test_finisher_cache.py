@@ -48,3 +48,16 @@ def test_the_bound_covers_heaps_and_lists(cache):
     for w in works:
         cache.shim_free(w)
     assert 0 < cache.shim_cached_search_bytes() <= cache.shim_cache_max()
+
+
+def test_copies_without_threads(tmp_path):
+    # an exception out of a C entry point would end the caller's process
+    inc, cxx = "/usr/local/cuda/include", shutil.which("g++")
+    if not os.path.exists(os.path.join(inc, "cuda_runtime.h")) or cxx is None or (os.cpu_count() or 1) < 2:
+        pytest.skip("needs g++, the CUDA headers and a second core")
+    exe = str(tmp_path / "copy")
+    subprocess.run([cxx, "-O1", "-std=c++17", "-pthread", "-I", CSRC, "-I", inc,
+                    os.path.join(os.path.dirname(__file__), "host_copy_main.cpp"), os.path.join(CSRC, "finisher.cpp"),
+                    "-o", exe], check=True, capture_output=True)
+    r = subprocess.run([exe], capture_output=True, text=True, timeout=60)
+    assert r.returncode == 0 and r.stdout == "copied\n", (r.returncode, r.stderr)
