@@ -281,25 +281,34 @@ extern "C" f2m_status f2m_create_batch_parts(int32_t count, const int32_t* n, co
     nnz += nz;
   }
   // back to back in one pinned block (an array of its own for the three would
-  // be touched anew on each call)
-  int32_t* h = nullptr;
-  const cudaError_t e = pin_alloc((void**)&h, sizeof(int32_t) * (size_t)(3 * N + count + nnz));
-  if (e != cudaSuccess) return cuda_fail(nullptr, e, "create_batch: staging");
-  int32_t *hx = h, *hr = h + 2 * N, *hc = hr + N + count, *x = hx, *r = hr, *q = hc;
-  std::vector<HostCopy> parts;
-  for (int32_t s = 0; s < count; ++s) {
-    const size_t nz = (size_t)row_ptr[s][n[s]];
-    parts.push_back({x, xy[s], sizeof(int32_t) * 2 * (size_t)n[s]});
-    parts.push_back({r, row_ptr[s], sizeof(int32_t) * ((size_t)n[s] + 1)});
-    parts.push_back({q, col[s], sizeof(int32_t) * nz});
-    x += 2 * (int64_t)n[s];
-    r += n[s] + 1;
-    q += nz;
+  // be touched anew on each call; where there is no more to pin, one all the same)
+  const size_t ints = (size_t)(3 * N + count + nnz);
+  int32_t *h = nullptr, *pageable = nullptr;
+  if (pin_alloc((void**)&h, sizeof(int32_t) * ints) != cudaSuccess) {
+    cudaGetLastError();
+    h = pageable = new (std::nothrow) int32_t[ints];
+    if (!h) return fail(nullptr, F2M_ERR_OOM, "create_batch: staging");
   }
-  host_copy(parts);
-  const f2m_status st = f2m_create_batch(count, n, hx, hr, hc, params, stream, out);
+  int32_t *hx = h, *hr = h + 2 * N, *hc = hr + N + count, *x = hx, *r = hr, *q = hc;
+  f2m_status st = F2M_OK;
+  try {
+    std::vector<HostCopy> parts;
+    for (int32_t s = 0; s < count; ++s) {
+      const size_t nz = (size_t)row_ptr[s][n[s]];
+      parts.push_back({x, xy[s], sizeof(int32_t) * 2 * (size_t)n[s]});
+      parts.push_back({r, row_ptr[s], sizeof(int32_t) * ((size_t)n[s] + 1)});
+      parts.push_back({q, col[s], sizeof(int32_t) * nz});
+      x += 2 * (int64_t)n[s];
+      r += n[s] + 1;
+      q += nz;
+    }
+    host_copy(parts);
+    st = f2m_create_batch(count, n, hx, hr, hc, params, stream, out);
+  } catch (const std::bad_alloc&) {
+    st = fail(nullptr, F2M_ERR_OOM, "create_batch: host allocation");
+  }
   if (st != F2M_OK) cudaStreamSynchronize((cudaStream_t)stream);  // copies of a refused call may be under way
-  pin_free(h);
+  if (pageable) delete[] pageable; else pin_free(h);
   return st;
 }
 

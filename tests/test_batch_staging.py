@@ -1,0 +1,21 @@
+"""f2m_create_batch_parts where no memory can be pinned (here: no GPU at all): the call
+goes on with pageable memory, to where the union is put on the device."""
+import numpy as np
+import pytest
+
+import paper_2011_08170_gb300 as f2m
+from paper_2011_08170_gb300 import build as B
+
+
+def test_staging_does_not_need_pinned_memory():
+    import torch
+    if torch.cuda.is_available():
+        pytest.skip("memory can be pinned here")
+    B.build()
+    f2m.load()
+    xy = np.array([[0, 0], [3, 0], [0, 4], [5, 5], [9, 1]], np.int32)
+    rp = np.arange(0, 21, 4, dtype=np.int32)
+    col = np.array([[c for c in range(5) if c != v] for v in range(5)], np.int32).ravel()
+    with pytest.raises(f2m.F2MError) as e:
+        f2m.f2m_create_batch_parts([[xy, rp, col]] * 2)
+    assert "staging" not in str(e.value) and "row_ptr" in str(e.value)
