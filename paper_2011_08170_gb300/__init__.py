@@ -566,8 +566,8 @@ def _new_batch(st, h, ns):
 def f2m_create_batch(instances, params: f2m_params | None = None, stream=None) -> Batch:
     """instances: list of (xy [n, 2], row_ptr [n + 1], col [nnz]) numpy arrays."""
     arrays = [[np.ascontiguousarray(a, np.int32) for a in t] for t in instances]
-    if all(r.ndim == 1 and r.size > 1 and x.size == 2 * (r.size - 1) and c.size == r[-1] for x, r, c in arrays):
-        return f2m_create_batch_parts(arrays, params, stream)
+    if _parts_fit(arrays):
+        return _create_parts(arrays, params, stream)
     # sizes that do not fit: the checks of the union say where
     ns = np.array([len(rp) - 1 for _, rp, _ in arrays], dtype=np.int32)
     xy, rp, col = [np.concatenate([t[j].reshape(shape) if shape else t[j] for t in arrays])
@@ -580,7 +580,19 @@ def f2m_create_batch(instances, params: f2m_params | None = None, stream=None) -
 
 def f2m_create_batch_parts(instances, params: f2m_params | None = None, stream=None) -> Batch:
     """f2m_create_batch from contiguous int32 arrays whose sizes fit, one of each
-    kind per instance."""
+    kind per instance; ValueError on others (the library reads as many entries as
+    the row offsets say)."""
+    if not (all(isinstance(a, np.ndarray) and a.dtype == np.int32 and a.flags.c_contiguous
+                for t in instances for a in t) and _parts_fit(instances)):
+        raise ValueError("f2m_create_batch_parts: contiguous int32 arrays of fitting sizes needed")
+    return _create_parts(instances, params, stream)
+
+
+def _parts_fit(arrays) -> bool:
+    return all(r.ndim == 1 and r.size > 1 and x.size == 2 * (r.size - 1) and c.size == r[-1] for x, r, c in arrays)
+
+
+def _create_parts(instances, params, stream) -> Batch:
     ns = np.array([r.size - 1 for _, r, _ in instances], dtype=np.int32)
     at = np.array([[a.__array_interface__["data"][0] for a in t] for t in instances], np.uintp).reshape(-1, 3)
     ptrs = [np.ascontiguousarray(at[:, j]) for j in range(3)]

@@ -19,3 +19,19 @@ def test_staging_does_not_need_pinned_memory():
     with pytest.raises(f2m.F2MError) as e:
         f2m.f2m_create_batch_parts([[xy, rp, col]] * 2)
     assert "staging" not in str(e.value) and "row_ptr" in str(e.value)
+
+
+@pytest.mark.parametrize("bad", [
+    lambda x, r, c: (x, r, c[:-1]),                      # fewer columns than the offsets say
+    lambda x, r, c: (x[:-1], r, c),
+    lambda x, r, c: (x, r, c.astype(np.int64)),
+    lambda x, r, c: (x, np.repeat(r, 2)[::2], c),        # not contiguous
+    lambda x, r, c: (x, r[:1], c),
+    lambda x, r, c: (x, r.tolist(), c)])
+def test_parts_that_do_not_fit_are_refused(bad):
+    B.build()
+    xy = np.array([[0, 0], [3, 0], [0, 4], [5, 5], [9, 1]], np.int32)
+    rp = np.arange(0, 21, 4, dtype=np.int32)
+    col = np.array([[c for c in range(5) if c != v] for v in range(5)], np.int32).ravel()
+    with pytest.raises(ValueError):
+        f2m.f2m_create_batch_parts([(xy, rp, col), bad(xy, rp, col)])
