@@ -626,6 +626,20 @@ static f2m_status ring_phase(f2m_ctx* c, int64_t max_sweeps, int64_t* sweeps, lo
   *ran = true;
   *sweeps = 0;
   if (max_sweeps <= 0) return F2M_ERR_NOT_CONVERGED;
+  // what fits is remembered for later phases, but not what a traced one found: its
+  // rows are in shared memory in any case
+  struct Keep {
+    f2m_ctx* c;
+    bool traced;
+    int32_t k, rows;
+    bool reg;
+    ~Keep() {
+      if (!traced) return;
+      c->ring_k = k;
+      c->ring_rows = rows;
+      c->ring_reg = reg;
+    }
+  } keep{c, tcap > 0, c->ring_k, c->ring_rows, c->ring_reg};
   const bool half = c->p.gdp_ctas_per_sm == 2;  // 2 CTAs per SM
   const bool one = half || (c->p.flags & F2M_FLAG_ONE_SWEEP_GDP);
   // small graphs use fewer tiles, of 64 rows (1,000 points: 0.75 us a sweep with
@@ -688,7 +702,7 @@ static f2m_status ring_phase(f2m_ctx* c, int64_t max_sweeps, int64_t* sweeps, lo
         if ((status & kGdpNoFit) && fits && fits != had) continue;
       }
       if (status & kGdpNoFit) break;
-      const bool packed = reg ? c->ring_rows > 1 : rs.bytes8 > ring_smem(half);
+      const bool packed = reg ? c->ring_rows > 1 : rs.bytes8 > ring_smem(half, tcap > 0);
       c->gdp_kernel = c->ring.K == 1 ? F2M_GDP_KERNEL_TILED
                                      : (packed ? F2M_GDP_KERNEL_TWO_SWEEP_PACKED : F2M_GDP_KERNEL_TWO_SWEEP);
       if (replay) break;

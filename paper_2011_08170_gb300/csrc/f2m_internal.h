@@ -344,7 +344,7 @@ void ring_free(RingPlan& p);
 // segment's nodes (list NULL), or those of the device list; seg_off on the device
 cudaError_t ring_build(const GdpPlan& g, const int32_t* seg_off, const RingTile* list, int32_t tiles, int32_t K,
                        int32_t F, int64_t entries_per_tile, int32_t nseg, RingPlan& p, cudaStream_t st);
-int32_t ring_smem(bool half);  // dynamic shared memory of a CTA
+int32_t ring_smem(bool half, bool traced);  // dynamic shared memory of a CTA
 // per phase: cleared segment records and status
 cudaError_t ring_start(RingPlan& p, int32_t n, int32_t nseg, cudaStream_t st);
 // Where the rows' entries are kept: registers (1 or 2 rows a thread, up to 1,984

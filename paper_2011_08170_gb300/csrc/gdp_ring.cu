@@ -449,6 +449,16 @@ struct RowOut {
   }
 };
 
+// A traced sweep's sums of the row warps' own rows, by the sweep's parity: written
+// before the barrier that ends sweep t, read by the warp beside them behind it,
+// and written again after the next one.  One atomic a tile, sweep and word: an
+// atomic of every row on the sweep's two words had taken 7.6 ms for 128 sweeps of
+// 100,000 points, now TRACE_NEW (and TRACE_BARE without a trace).
+struct RingTrace {
+  long long b2[2][32];
+  unsigned ch[2][32];
+};
+
 // Rows whose entries stay in shared memory (any number that fits).
 // MODE 0: b_v = 2 (top-3); 1: every b_v < 5; 2: every b_v < 8; 3: any b_v.
 template <int MODE, bool BOUND, bool PACKED, int NW>
@@ -497,11 +507,13 @@ struct SmemRows {
   __device__ __forceinline__ const int* ring() const { return s_ring; }
 
   __device__ __forceinline__ unsigned sweep(const RingArgs& A, int par, int end, int sown, bool last,
-                                            unsigned* pub, unsigned tag, int t) {
+                                            unsigned* pub, unsigned tag, RingTrace* trace, int t) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int* in = lam(par);
     int* out = lam(par ^ 1);
     RowOut o;
+    long long b2 = 0;
+    unsigned ch = 0;
     for (int sl = warp; sl < end; sl += NW) {
       const uint32_t od = s_slc[sl];
       const int row = s_ord[sl * 32 + lane];
@@ -522,10 +534,18 @@ struct SmemRows {
         o.own(nl, lv);
         if (last) st_word(pub + vl, word_of(nl, tag));
         if constexpr (BOUND) {
-          if (t < A.trace_cap) {
-            atomicAdd(reinterpret_cast<unsigned long long*>(A.trace_b2 + t), (unsigned long long)(neg + 2LL * bv * lv));
-            if (nl != lv) atomicAdd(A.trace_ch + t, 1ull);
-          }
+          b2 += neg + 2LL * bv * lv;
+          ch += nl != lv;
+        }
+      }
+    }
+    if constexpr (BOUND) {
+      if (warp < sown) {  // the same warps every sweep: the others' sums stay 0
+        b2 = warp_sum_ll(b2);
+        ch = warp_sum_u(ch);
+        if (lane == 0) {
+          trace->b2[t & 1][warp] = b2;
+          trace->ch[t & 1][warp] = ch;
         }
       }
     }
@@ -729,7 +749,7 @@ struct RegRows {
     return o.flags;
   }
   __device__ __forceinline__ unsigned sweep(const RingArgs& A, int par, int end, int sown, bool last,
-                                            unsigned* pub, unsigned tag, int) {
+                                            unsigned* pub, unsigned tag, RingTrace*, int) {
     return par ? sweep_p<1>(A, end, sown, last, pub, tag) : sweep_p<0>(A, end, sown, last, pub, tag);
   }
 };
@@ -742,8 +762,10 @@ struct RingShared {
   int end[kRingMax];
 };
 
-// The stop test, by one warp beside those with the rows: the same barriers.
-__device__ __noinline__ void ring_boss(const RingArgs& A, const RingHdr& h, RingShared& S) {
+// The stop test (and the trace's totals), by one warp beside those with the rows: the
+// same barriers.
+template <int NW>
+__device__ __noinline__ void ring_boss(const RingArgs& A, const RingHdr& h, RingShared& S, const RingTrace* trace) {
   const int lane = threadIdx.x & 31, K = A.K, max_sweeps = A.max_sweeps;
   RingSeg* sg = A.seg + h.seg;
   const int width = 48 / K;  // bits of a slot's count of tiles a sweep changed, after 16 of arrivals
@@ -764,6 +786,15 @@ __device__ __noinline__ void ring_boss(const RingArgs& A, const RingHdr& h, Ring
         return true;
       }
       if (wait.give_up()) return false;
+    }
+  };
+  auto add_trace = [&](int t) {  // behind the barrier that ends sweep t
+    if (!trace || t >= A.trace_cap) return;
+    const long long b2 = warp_sum_ll(lane < NW ? trace->b2[t & 1][lane] : 0);
+    const unsigned ch = warp_sum_u(lane < NW ? trace->ch[t & 1][lane] : 0u);
+    if (lane == 0) {
+      if (b2) atomicAdd(reinterpret_cast<unsigned long long*>(A.trace_b2 + t), (unsigned long long)b2);
+      if (ch) atomicAdd(A.trace_ch + t, (unsigned long long)ch);
     }
   };
   int r = 0;
@@ -793,8 +824,13 @@ __device__ __noinline__ void ring_boss(const RingArgs& A, const RingHdr& h, Ring
       if (f >> 16) atomicOr(&sg->ovf[(r - 1) % kRingRing], f >> 16);
       add_slot(&sg->slot[(r - 1) % kRingRing], v);
     }
+    __syncwarp();
+    if (r >= 1) add_trace(min(r * K, max_sweeps) - 1);
     if (S.stop[r & 1]) break;
-    for (int s = 1; s < kk; ++s) __syncthreads();
+    for (int s = 1; s < kk; ++s) {
+      __syncthreads();
+      add_trace(r * K + s - 1);
+    }
   }
   // a phase that ran to its cap: the verdict of the last rounds
   if (lane == 0 && h.first) {
@@ -808,7 +844,8 @@ __device__ __noinline__ void ring_boss(const RingArgs& A, const RingHdr& h, Ring
 
 // The rounds of one tile: the last warp runs the stop test, the others hold the rows.
 template <typename Rows, int T>
-__device__ __forceinline__ void ring_run(const RingArgs& A, const RingHdr& h, unsigned char* smem) {
+__device__ __forceinline__ void ring_run(const RingArgs& A, const RingHdr& h, unsigned char* smem,
+                                         RingTrace* trace = nullptr) {
   constexpr int NW = T / 32 - 1;  // warps with rows
   __shared__ RingShared S;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, b = A.first_tile + blockIdx.x;
@@ -824,9 +861,13 @@ __device__ __forceinline__ void ring_run(const RingArgs& A, const RingHdr& h, un
   for (int i = tid; i < h.halo; i += T) rows.lam(0)[ownp + i] = A.lam_in[A.perm[halo[i]]];
   if (tid < kRingMax) S.end[tid] = A.hdr[b].sec_end[tid];
   if (tid < 2) S.abort[tid] = S.flags[tid] = 0;
+  if (trace && tid < 64) {
+    trace->b2[tid & 1][tid >> 1] = 0;
+    trace->ch[tid & 1][tid >> 1] = 0;
+  }
   __syncthreads();
   if (warp == NW) {
-    ring_boss(A, h, S);
+    ring_boss<NW>(A, h, S, trace);
     return;
   }
   const int* s_ring = rows.ring();
@@ -858,7 +899,8 @@ __device__ __forceinline__ void ring_run(const RingArgs& A, const RingHdr& h, un
       const bool last = s == kk - 1;
       const int sown = S.end[0], end = last ? sown : S.end[K - 1 - s];
       if (warp < end) {
-        unsigned flags = rows.sweep(A, par, end, sown, last, A.words[(r + 1) & 1] + h.word0, word_tag(r + 1), r * K + s);
+        unsigned flags = rows.sweep(A, par, end, sown, last, A.words[(r + 1) & 1] + h.word0, word_tag(r + 1), trace,
+                                    r * K + s);
         flags = __reduce_or_sync(0xffffffffu, flags);
         if (lane == 0 && flags) atomicOr(&S.flags[r & 1], flags << s);
       }
@@ -887,10 +929,15 @@ gdp_ring_smem_kernel(const __grid_constant__ RingArgs A) {
     return;
   }
   const RingHdr h = A.hdr[A.first_tile + blockIdx.x];
+  RingTrace* trace = nullptr;
+  if constexpr (BOUND) {
+    __shared__ RingTrace s_trace;
+    trace = &s_trace;
+  }
   if (wide)
-    ring_run<SmemRows<MODE, BOUND, false, T / 32 - 1>, T>(A, h, smem);
+    ring_run<SmemRows<MODE, BOUND, false, T / 32 - 1>, T>(A, h, smem, trace);
   else
-    ring_run<SmemRows<MODE, BOUND, true, T / 32 - 1>, T>(A, h, smem);
+    ring_run<SmemRows<MODE, BOUND, true, T / 32 - 1>, T>(A, h, smem, trace);
 }
 
 template <int MODE, int R, int T>
@@ -991,19 +1038,19 @@ static const void* ring_reg_kernel_of(int mode) {
 }
 
 int ring_reg_rows(const RingStats& st) {
-  if (st.bad || st.bytes_reg > ring_smem(false)) return 0;
+  if (st.bad || st.bytes_reg > ring_smem(false, false)) return 0;
   if (st.slices <= 31) return 1;
   return st.slices <= 62 && reg_packs(st, 31) ? 2 : 0;
 }
 
-int32_t ring_smem(bool half) {
+int32_t ring_smem(bool half, bool traced) {
   int dev = 0, optin = 0, sm = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess)
     return 0;
   // less what the kernel holds statically, and what the system keeps of each CTA
-  return ((half ? sm / 2 - 1024 : optin) - 128) & ~15;
+  return ((half ? sm / 2 - 1024 : optin) - 128 - (traced ? (int)sizeof(RingTrace) : 0)) & ~15;
 }
 
 cudaError_t launch_gdp_ring(const GdpPlan& g, RingPlan& p, int32_t first_tile, int32_t tiles, const int32_t* lam_in,
@@ -1022,7 +1069,7 @@ cudaError_t launch_gdp_ring(const GdpPlan& g, RingPlan& p, int32_t first_tile, i
                      : mode == 1       ? (half ? ring_kernel_of<1, 512>(bound) : ring_kernel_of<1, 1024>(bound))
                      : mode == 2       ? ring_kernel_of<2, 512>(bound)
                                        : ring_kernel_of<3, 512>(bound);
-  const int dyn = ring_smem(half);
+  const int dyn = ring_smem(half, bound);
   RCK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
   RingArgs a{};
   a.hdr = p.hdr;
