@@ -663,12 +663,13 @@ static f2m_status ring_phase(f2m_ctx* c, int64_t max_sweeps, int64_t* sweeps, lo
         CK(c, dalloc(&c->d_ring_seg, 2));
         CK(c, cudaMemcpyAsync(c->d_ring_seg, off, sizeof(off), cudaMemcpyHostToDevice, c->st));
       }
-      CK(c, ring_build(c->plan, c->d_ring_seg, nullptr, tiles, c->ring_k, c->p.frac_bits, c->nnz / tiles, 1, c->ring,
+      CK(c, ring_build(c->plan, c->d_ring_seg, nullptr, tiles, c->ring_k, c->p.frac_bits, c->ring_room ? -1 : c->nnz / tiles,
+                       kRingDepth, 1, c->ring,
                        c->st));
     }
     int64_t limit = std::min<int64_t>(max_sweeps, kRingSweeps);
     bool replay = false;
-    int32_t status = 0;
+    int32_t status = 0, bad = 0;
     // in shared memory: traces, and the counting selection of large b_v
     const bool reg = c->ring_reg && tcap == 0 && !(c->d_b && c->b_max >= 8);
     for (;;) {
@@ -681,7 +682,7 @@ static f2m_status ring_phase(f2m_ctx* c, int64_t max_sweeps, int64_t* sweeps, lo
       const cudaError_t e =
           launch_gdp_ring(c->plan, c->ring, 0, tiles, c->d_lam[c->cur], c->d_lam[c->cur ^ 1], c->p.damping_shift,
                           (int32_t)limit, tb, tc, replay ? 0 : tcap, c->p.barrier_budget_cycles, c->d_b_int, c->b_max,
-                          reg ? (RingForm)c->ring_rows : (half ? kRingHalf : kRingSmem), c->st);
+                          reg ? (RingForm)c->ring_rows : (half ? kRingHalf : kRingSmem), c->ring_longs, c->st);
       if (e == cudaErrorCooperativeLaunchTooLarge) {  // not on this device now
         cudaGetLastError();
         *ran = false;
@@ -694,12 +695,15 @@ static f2m_status ring_phase(f2m_ctx* c, int64_t max_sweeps, int64_t* sweeps, lo
       const RingStats& rs = rec.stats;
       const RingSeg& q = rec.seg[0];
       status = rec.status;
+      bad = rs.bad;
       if (ms) *ms += elapsed_ms(c);
       if (status & kGdpTimeout) return fail(c, F2M_ERR_TIMEOUT, "a wait for another tile exceeded its budget");
       if (reg) {  // what the tiles need, known now
         const int fits = ring_reg_rows(rs), had = c->ring_rows;
+        const bool longs = rs.longs && !c->d_b, other = longs != c->ring_longs;
         if (fits) c->ring_rows = fits;
-        if ((status & kGdpNoFit) && fits && fits != had) continue;
+        c->ring_longs = longs;
+        if ((status & kGdpNoFit) && fits && (fits != had || other)) continue;
       }
       if (status & kGdpNoFit) break;
       const bool packed = reg ? c->ring_rows > 1 : rs.bytes8 > ring_smem(half, tcap > 0);
@@ -717,9 +721,13 @@ static f2m_status ring_phase(f2m_ctx* c, int64_t max_sweeps, int64_t* sweeps, lo
       if (!(h.overflow && h.sweeps == 1)) c->cur ^= 1;  // else lambda stays at the input
       break;
     }
-    // fewer rings take fewer registers and less shared memory
-    if (c->ring_k > 1) {
-      c->ring_k -= 1;
+    // fewer rings take fewer registers and less shared memory; long rows, whose
+    // slices are mostly padding, more room
+    if (c->ring_k <= 2 && !c->ring_room && bad == kRingBadRoom) {
+      c->ring_room = true;
+      c->ring.version = -1;
+    } else if (c->ring_k > 1) {
+      c->ring_k = bad ? std::min(c->ring_k - 1, 2) : c->ring_k - 1;  // rings around long rows grow with their number
     } else if (reg) {
       c->ring_reg = false;
       c->ring_k = one ? 1 : 2;

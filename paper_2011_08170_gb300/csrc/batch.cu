@@ -312,6 +312,7 @@ extern "C" f2m_status f2m_create_batch_parts(int32_t count, const int32_t* n, co
   return st;
 }
 
+constexpr int32_t kBatchRowEntries = 254;  // the longest row of a tile (the streaming kernels' smallest shape takes 256)
 constexpr int32_t kBatchTileRows = 960;  // rows a tile: 15 warps of 2 slices
 
 // ---- GDP phase: tiles, kernel shape (autotuned), captured launch ----------------------
@@ -662,7 +663,7 @@ static f2m_status batch_ring_phase(f2m_batch* b, const std::vector<uint8_t>& act
   CK(c, dgrow(&b->d_rlist, &b->rlist_cap, tiles, tiles + tiles / 8 + 64));
   if (!b->h_rseg) CK(c, pin_alloc((void**)&b->h_rseg, sizeof(RingSeg) * b->count));
   CK(c, cudaMemcpyAsync(b->d_rlist, list.data(), sizeof(RingTile) * tiles, cudaMemcpyHostToDevice, c->st));
-  CK(c, ring_build(c->plan, c->d_seg_off, b->d_rlist, tiles, K, c->p.frac_bits, rows * c->nnz / c->n, b->count, c->ring,
+  CK(c, ring_build(c->plan, c->d_seg_off, b->d_rlist, tiles, K, c->p.frac_bits, rows * c->nnz / c->n, kBatchRowEntries, b->count, c->ring,
                    c->st));
   CK(c, ring_start(c->ring, c->n, b->count, c->st));
   // the instances left alone keep their lambda
@@ -673,7 +674,7 @@ static f2m_status batch_ring_phase(f2m_batch* b, const std::vector<uint8_t>& act
   for (size_t w = 0; w + 1 < waves.size(); ++w) {
     const cudaError_t e = launch_gdp_ring(c->plan, c->ring, waves[w], waves[w + 1] - waves[w], in, out,
                                           c->p.damping_shift, (int32_t)c->p.max_iters, nullptr, nullptr, 0,
-                                          c->p.barrier_budget_cycles, nullptr, 2, kRingPair, c->st);
+                                          c->p.barrier_budget_cycles, nullptr, 2, kRingPair, false, c->st);
     if (e == cudaErrorCooperativeLaunchTooLarge) {
       cudaGetLastError();
       CK(c, cudaStreamSynchronize(c->st));

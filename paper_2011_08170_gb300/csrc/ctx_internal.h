@@ -119,6 +119,8 @@ struct f2m_ctx {
   int32_t ring_k = 0;        // rings of the tiles (0: not tried, -1: none fit, the streaming kernel runs)
   int32_t ring_rows = 0;     // rows a thread in that form
   bool ring_reg = true;      // the tiles' rows fit registers, as far as tried
+  bool ring_longs = false;   // some tile has rows of more than kRingLong entries
+  bool ring_room = false;    // the tiles have as much room for entries as any can use
   f2m::ClassPlan classes;    // colour classes of the class-by-class GDP
   // exact finisher: device scratch, host work arrays; the h_ arrays point into
   // the process's one pinned host mirror while a finisher call holds it

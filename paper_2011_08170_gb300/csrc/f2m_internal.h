@@ -271,11 +271,19 @@ void plan_free(GdpPlan& p);
 constexpr int kRingMax = 6;          // rings around a tile: sweeps per exchange
 constexpr int kRingLocals = 8192;    // nodes a tile knows (own, rings, two padding slots)
 constexpr int kRingHalo = 4096;      // of them in rings
+constexpr int kRingDepth = 1536;     // entries of a row at most: 32 such rows are all that a tile can hold
+// A slice with a row of more than kRingLong entries leaves all but the first
+// kRingTail of each of its rows to the warp (where lanes and warp cost the same: rows
+// of 100 entries 405 against 416 us for 128 sweeps, of 66 301 against 400, of 256 826
+// against 355)
+constexpr int kRingLong = 112;
+constexpr int kRingTail = 32;
 constexpr int kRingSlots = 8192;     // rows it computes, in whole slices
 constexpr int kRingSlices = kRingSlots / 32;
 constexpr int kRingSweeps = 1 << 30;  // of one launch (a longer phase takes several)
 constexpr int kRingRing = 16;        // rounds whose stop-test slots are live
-constexpr int kRingBadSize = 1;      // RingStats::bad: some tile is too large
+constexpr int kRingBadSize = 1;      // RingStats::bad: some tile is too large,
+constexpr int kRingBadRoom = 2;      // or has more sliced entries than the arrays have room for
 struct RingTile {
   int32_t seg, j, count;  // the j-th of the count tiles of an instance (segment)
 };
@@ -291,6 +299,7 @@ struct RingStats {        // over all tiles of a plan
   int32_t bytes8, bytes4;  // shared memory of the largest with 8- and 4-byte entries there,
   int32_t bytes_reg;       // and with entries in registers
   int32_t slices, locals, maxcost;
+  int32_t longs;           // some row has more than kRingLong entries
   int32_t bad;
 };
 struct RingSeg {          // per instance, zeroed per phase
@@ -309,6 +318,7 @@ struct RingArgs {
   const int32_t* halo;
   const uint16_t* order;
   const uint32_t* slc;
+  const uint32_t* longs;   // per slice with a row of more than kRingLong entries: those past kRingTail
   const int2* ent;
   const RingStats* stats;
   const int32_t* pos;      // by internal node: its word
@@ -332,18 +342,21 @@ struct RingPlan {
   int32_t* halo = nullptr;
   uint16_t* order = nullptr;
   uint32_t* slc = nullptr;
+  uint32_t* longs = nullptr;
   int2* ent = nullptr;
   RingRecord* rec = nullptr;
   int32_t* pos = nullptr;
   unsigned* words = nullptr;  // the exchange: two buffers of words_n
   int64_t words_n = 0;
-  int64_t hdr_cap = 0, halo_cap = 0, order_cap = 0, slc_cap = 0, ent_cap = 0, seg_cap = 0, words_cap = 0, pos_cap = 0;
+  int64_t hdr_cap = 0, halo_cap = 0, order_cap = 0, slc_cap = 0, longs_cap = 0, ent_cap = 0, seg_cap = 0, words_cap = 0, pos_cap = 0;
 };
 void ring_free(RingPlan& p);
 // the tiles of K rings over the internal CSR: `tiles` equal shares of the one
-// segment's nodes (list NULL), or those of the device list; seg_off on the device
+// segment's nodes (list NULL), or those of the device list; seg_off on the device;
+// maxdeg: the longest row a tile takes, at most kRingDepth; entries_per_tile: their
+// mean (a tile's room is what near-even tiles need), -1: the most a tile can hold
 cudaError_t ring_build(const GdpPlan& g, const int32_t* seg_off, const RingTile* list, int32_t tiles, int32_t K,
-                       int32_t F, int64_t entries_per_tile, int32_t nseg, RingPlan& p, cudaStream_t st);
+                       int32_t F, int64_t entries_per_tile, int32_t maxdeg, int32_t nseg, RingPlan& p, cudaStream_t st);
 int32_t ring_smem(bool half, bool traced);  // dynamic shared memory of a CTA
 // per phase: cleared segment records and status
 cudaError_t ring_start(RingPlan& p, int32_t n, int32_t nseg, cudaStream_t st);
@@ -352,11 +365,12 @@ cudaError_t ring_start(RingPlan& p, int32_t n, int32_t nseg, cudaStream_t st);
 // shared memory, or shared memory with two CTAs per SM.
 enum RingForm { kRingHalf = -1, kRingSmem = 0, kRingReg1 = 1, kRingReg2 = 2, kRingPair = 3 };
 int ring_reg_rows(const RingStats& st);  // rows a thread of the register form (0: does not fit)
+// (longs: the register form for graphs with rows past kRingLong entries, b_v = 2)
 // one cooperative launch over tiles [first_tile, first_tile + tiles): whole instances
 cudaError_t launch_gdp_ring(const GdpPlan& g, RingPlan& p, int32_t first_tile, int32_t tiles, const int32_t* lam_in,
                             int32_t* lam_out, int32_t shift, int32_t max_sweeps, long long* trace_b2,
                             unsigned long long* trace_ch, int64_t trace_cap, long long budget, const int32_t* bint,
-                            int32_t bmax, RingForm form, cudaStream_t st);
+                            int32_t bmax, RingForm form, bool longs, cudaStream_t st);
 
 // ---- exact finisher (finisher_prep.cu on the device, finisher.cpp on the host) ---
 // twin[e] for every internal entry; *missing (zeroed by the caller) counts

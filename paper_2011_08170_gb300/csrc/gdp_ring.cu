@@ -63,6 +63,12 @@ constexpr int kRingLamBytes = 4 * kRingLocals;    // between its two lambda arra
 constexpr int kHash = 2 * kRingHalo;        // slots of the plan's table of outside nodes
 constexpr int kShallow = 12;                // entries of most rows (k = 10 graphs: three in four)
 constexpr int kPackIdx = 13;                // bits of a packed local index
+constexpr int kMaxEntries = 49152;          // sliced entries of a tile: what 4 bytes each could hold in shared memory
+constexpr int kDepthBits = 11;              // a slice's word: its first entry << kDepthBits | its depth
+constexpr int kDepthMask = (1 << kDepthBits) - 1;
+static_assert(kRingDepth <= kDepthMask - 1 && kMaxEntries < 1 << (31 - kDepthBits), "a slice's word");
+static_assert(kRingDepth % 2 == 0 && kRingLong % 2 == 0 && kRingTail % 2 == 0, "a depth is even");
+static_assert(kRingTail >= kRegEntries && kRingTail < kRingLong, "what a lane keeps");
 constexpr uint32_t kPackPadCost = (1u << (32 - kPackIdx)) - 1;  // cost of a packed padding entry
 // lambda of the padding slot in the packed form: with cost kPackPadCost its z
 // is about 2^30 - lambda_v, above every real one (as the 8-byte padding's)
@@ -91,9 +97,10 @@ __device__ __forceinline__ int hash_find(const int* keys, const uint16_t* vals, 
 // a ring node's ownp + its position (ownp: own slots, whole slices).
 __global__ void __launch_bounds__(kPlanThreads, 1)
 ring_plan_kernel(const int32_t* __restrict__ irp, const int2* __restrict__ iec, const RingTile* __restrict__ list,
-                 const int32_t* __restrict__ seg_off, int32_t tiles, int32_t K, int32_t F, int32_t ecap,
+                 const int32_t* __restrict__ seg_off, int32_t tiles, int32_t K, int32_t F, int32_t ecap, int32_t maxdeg,
                  RingHdr* __restrict__ hdr, int32_t* __restrict__ halo, uint16_t* __restrict__ order,
-                 uint32_t* __restrict__ slc, int2* __restrict__ ent, int32_t* __restrict__ pos, RingStats* stats) {
+                 uint32_t* __restrict__ slc, uint32_t* __restrict__ longs, int2* __restrict__ ent,
+                 int32_t* __restrict__ pos, RingStats* stats) {
   extern __shared__ __align__(16) unsigned char smem[];
   int* keys = reinterpret_cast<int*>(smem);                         // [kHash] outside nodes
   int* ring = keys + kHash;                                         // [kRingHalo] in ring order
@@ -103,7 +110,7 @@ ring_plan_kernel(const int32_t* __restrict__ irp, const int2* __restrict__ iec, 
   uint16_t* deg = at_key + kRingHalo;                               // [kRingLocals] per row (own, then ring)
   uint16_t* ord = deg + kRingLocals;                                // [kRingSlots] row of a slot
   uint16_t* inv = ord + kRingSlots;                                 // [kRingLocals] slot of an own node
-  __shared__ int s_cnt, s_bad, s_hist[64], s_maxcost, s_tail;
+  __shared__ int s_cnt, s_bad, s_hist[64], s_maxcost, s_tail, s_long;
   __shared__ int s_sl[kRingSlices + 1];
   __shared__ int s_warp[33];
   const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -116,6 +123,7 @@ ring_plan_kernel(const int32_t* __restrict__ irp, const int2* __restrict__ iec, 
     s_bad = 0;
     s_maxcost = 0;
     s_tail = 0;
+    s_long = 0;
   }
   __syncthreads();
   const int lo = n0 + (int)((long long)ns * tl.j / tl.count), hi = n0 + (int)((long long)ns * (tl.j + 1) / tl.count);
@@ -188,8 +196,8 @@ ring_plan_kernel(const int32_t* __restrict__ irp, const int2* __restrict__ iec, 
   if (!bad) {
     for (int l = tid; l < rows; l += kPlanThreads) {
       const int g = node_of(l), d = irp[g + 1] - irp[g];
-      if (d > 254) atomicOr(&s_bad, kRingBadSize);  // a slice's depth takes 8 bits
-      deg[l] = (uint16_t)min(d, 254);
+      if (d > maxdeg) atomicOr(&s_bad, kRingBadSize);
+      deg[l] = (uint16_t)min(d, maxdeg);
     }
     for (int h2 = tid; h2 < HH; h2 += kPlanThreads) halo[(size_t)b * kRingHalo + h2] = ring[h2];
   }
@@ -245,10 +253,13 @@ ring_plan_kernel(const int32_t* __restrict__ irp, const int2* __restrict__ iec, 
   // depth of a slice (even), offsets
   for (int s = warp; s < nsl; s += kPlanThreads / 32) {
     const int l = ord[s * 32 + lane];
-    const int d = __reduce_max_sync(0xffffffffu, l == 0xFFFF ? 0 : (int)deg[l]);
+    const int dl = l == 0xFFFF ? 0 : (int)deg[l], d = __reduce_max_sync(0xffffffffu, dl);
+    const unsigned longs_of = d > kRingLong ? __ballot_sync(0xffffffffu, dl > kRingTail) : 0u;
     if (lane == 0) {
       s_sl[s] = (d + 1) & ~1;
+      longs[(size_t)b * kRingSlices + s] = longs_of;
       if (d > kRegEntries) atomicAdd(&s_tail, 32 * (((d + 1) & ~1) - kRegEntries));
+      if (longs_of) s_long = 1;
     }
   }
   __syncthreads();
@@ -256,10 +267,10 @@ ring_plan_kernel(const int32_t* __restrict__ irp, const int2* __restrict__ iec, 
   int nent = 0;
   const int off = block_exclusive_scan(32 * depth, s_warp, nent);
   static_assert(kRingSlices <= kPlanThreads, "one thread per slice");
-  if (nent > ecap) bad = kRingBadSize;
+  if (nent > ecap) bad = kRingBadRoom;
   if (tid < nsl && !bad) {
-    s_sl[tid] = off << 8 | depth;
-    slc[(size_t)b * kRingSlices + tid] = (uint32_t)(off << 8 | depth);
+    s_sl[tid] = off << kDepthBits | depth;
+    slc[(size_t)b * kRingSlices + tid] = (uint32_t)(off << kDepthBits | depth);
   }
   __syncthreads();
   // entries
@@ -271,7 +282,7 @@ ring_plan_kernel(const int32_t* __restrict__ irp, const int2* __restrict__ iec, 
     for (int l = tid; l < own; l += kPlanThreads) pos[lo + l] = h.word0 + inv[l];
     auto local_of = [&](int c) { return c >= lo && c < hi ? (int)inv[c - lo] : ownp + hash_find(keys, vals, c); };
     for (int s = warp; s < nsl; s += kPlanThreads / 32) {
-      const int l = ord[s * 32 + lane], o = s_sl[s] >> 8, dep = s_sl[s] & 255;
+      const int l = ord[s * 32 + lane], o = s_sl[s] >> kDepthBits, dep = s_sl[s] & kDepthMask;
       const int g = l == 0xFFFF ? -1 : node_of(l);
       const int a = g >= 0 ? irp[g] : 0, d = g >= 0 ? irp[g + 1] - a : 0;
       for (int k = 0; k < dep; k += 2) {
@@ -307,6 +318,7 @@ ring_plan_kernel(const int32_t* __restrict__ irp, const int2* __restrict__ iec, 
     atomicMax(&stats->bytes8, 8 * nent + rest);
     atomicMax(&stats->bytes4, 4 * nent + rest);
     atomicMax(&stats->slices, nsl);
+    if (s_long) stats->longs = 1;
     atomicMax(&stats->locals, ownp + HH + 2);
     atomicMax(&stats->maxcost, s_maxcost);
     atomicMax(&stats->bytes_reg, 2 * kRingLamBytes + 4 * (HH + nsl) + 8 * s_tail + 64);
@@ -328,16 +340,52 @@ __device__ __forceinline__ int4 two_entries(const void* ent, int at, int F) {
   }
 }
 
+// Entries from kRingTail on of the slice's rows flagged in `rows`: the warp takes one
+// row after the other, its lanes pairs of that row's entries, whose top-3 (and
+// sum of min(0, z)) go to the row's lane.  As one lane's chain an entry cost 40
+// cycles, and every tile waits for the one with the longest row: 128 sweeps of 3,000
+// points, one with 256 neighbours, 826 us, so 355; 100,000 points, one with 300,
+// 1,016 and 474 (the streaming kernel 2,150).  All lanes of the warp call it.
+template <bool BOUND, typename Two>
+__device__ __forceinline__ void long_rows(unsigned rows, int depth, int lv, const Two& two, const int* s_in, int& a,
+                                          int& zb, int& zc, long long& neg) {
+  const int lane = threadIdx.x & 31;
+  for (; rows; rows &= rows - 1) {
+    const int row = __ffs(rows) - 1, l = __shfl_sync(0xffffffffu, lv, row);
+    int x = INT_MAX, y = INT_MAX, w = INT_MAX;
+    long long sum = 0;
+    for (int k = kRingTail + 2 * lane; k < depth; k += 64) {
+      const int4 q = two(k, row);
+      const int z = q.y - l - s_in[q.x], z1 = q.w - l - s_in[q.z];
+      if (BOUND) sum += min(z, 0) + min(z1, 0);
+      top3_insert_minmax(z, x, y, w);
+      top3_insert_minmax(z1, x, y, w);
+    }
+#pragma unroll 1
+    for (int o = 1; o < 32; o <<= 1) {
+      const int x1 = __shfl_xor_sync(0xffffffffu, x, o), y1 = __shfl_xor_sync(0xffffffffu, y, o),
+                w1 = __shfl_xor_sync(0xffffffffu, w, o);
+      top3_merge(x1, y1, w1, x, y, w);
+    }
+    if (BOUND) sum = warp_sum_ll(sum);
+    if (lane == row) {
+      top3_merge(x, y, w, a, zb, zc);
+      if (BOUND) neg += sum;
+    }
+  }
+}
+
 // z(2) and z(3) of one row (Eq. 10): two top-3 chains over alternate entries,
 // merged; if BOUND, also the row's sum of min(0, z)
 template <bool PACKED, bool BOUND>
-__device__ __forceinline__ void row_top3(const void* ent, int at, int depth, int F, int lv, const int* s_in, int& zb,
-                                         int& zc, long long& neg) {
+__device__ __forceinline__ void row_top3(const void* ent, int at, int depth, int F, int lv, const int* s_in,
+                                         const uint32_t* longs, int& zb, int& zc, long long& neg) {
   int a = INT_MAX, a1 = INT_MAX, b1 = INT_MAX, c1 = INT_MAX;
   zb = INT_MAX;
   zc = INT_MAX;
+  const int stop = depth > kRingLong ? kRingTail : depth;
 #pragma unroll 4
-  for (int k = 0; k < depth; k += 2) {
+  for (int k = 0; k < stop; k += 2) {
     const int4 q = two_entries<PACKED>(ent, at + k * 32, F);
     const int z = q.y - lv - s_in[q.x];  // Eq. 9
     const int z1 = q.w - lv - s_in[q.z];
@@ -346,6 +394,11 @@ __device__ __forceinline__ void row_top3(const void* ent, int at, int depth, int
     top3_insert_minmax(z1, a1, b1, c1);
   }
   top3_merge(a1, b1, c1, a, zb, zc);
+  if (depth > kRingLong) {
+    const int row0 = at - (threadIdx.x & 31) * 2;
+    long_rows<BOUND>(*longs, depth, lv, [&](int k, int row) { return two_entries<PACKED>(ent, row0 + k * 32 + row * 2, F); },
+                     s_in, a, zb, zc, neg);
+  }
 }
 
 // Degree requirements b_v (Section 3 with Eq. 8): z(b_v) and z(b_v + 1) of one
@@ -476,6 +529,7 @@ struct SmemRows {
   const int* s_ring;
   const uint32_t* s_slc;
   const uint16_t* s_ord;
+  const uint32_t* longs;
   const int32_t* bnode;  // node of a ring row (degree requirements)
   int L, own, ownp, lo;
 
@@ -488,6 +542,7 @@ struct SmemRows {
     lo = h.lo;
     L = ownp + h.halo + 1;
     bnode = A.halo + (size_t)b * kRingHalo;
+    longs = A.longs + (size_t)b * kRingSlices;
     s_ent = smem;
     s_lam = reinterpret_cast<int*>(smem + (size_t)nent * (PACKED ? 4 : 8));  // two arrays of L
     int* ring = s_lam + 2 * L;
@@ -525,13 +580,15 @@ struct SmemRows {
     for (int sl = warp; sl < end; sl += NW) {
       const uint32_t od = s_slc[sl];
       const int row = s_ord[sl * 32 + lane];
-      if (row == 0xFFFF) continue;
+      const bool has = row != 0xFFFF;
+      if (MODE != 0 && !has) continue;  // with b_v = 2 the warp stays together (long rows)
       const int vl = sl < sown ? sl * 32 + lane : ownp + row - own;  // its local index
-      const int lv = in[vl], at = (int)(od >> 8) + lane * 2, depth = (int)(od & 255u);
+      const int lv = has ? in[vl] : 0, at = (int)(od >> kDepthBits) + lane * 2, depth = (int)(od & kDepthMask);
       int zb, zc, bv = 2;
       long long neg = 0;
       if constexpr (MODE == 0) {
-        row_top3<PACKED, BOUND>(s_ent, at, depth, A.F, lv, in, zb, zc, neg);
+        row_top3<PACKED, BOUND>(s_ent, at, depth, A.F, lv, in, longs + sl, zb, zc, neg);
+        if (!has) continue;
       } else {
         bv = __ldg(A.bint + (row < own ? lo + row : bnode[row - own]));
         row_pair_deg<PACKED, BOUND, MODE == 1 ? 5 : (MODE == 2 ? 8 : 0)>(s_ent, at, depth, A.F, lv, in, bv, zb, zc, neg);
@@ -576,7 +633,9 @@ __host__ __device__ __forceinline__ bool reg_packs(const RingStats& st, int nw) 
 // tile, costs below 2^19 - 1) with two CTAs per SM, 14 with one.  The two
 // lambda arrays lie a constant apart, so that a gather is one load with an
 // immediate offset (the two parities are compiled separately).
-template <int MODE, int R, int NW>
+// LONG: the warp takes what long rows have past kRingTail entries (b_v = 2); a form
+// of its own, since it spills a few registers.
+template <int MODE, int R, int NW, bool LONG>
 struct RegRows {
   static constexpr bool PACKED = R > 1;
   static constexpr int AB = reg_address_bits(NW);
@@ -585,7 +644,7 @@ struct RegRows {
   unsigned char* sm;
   int* s_ring;
   const int2* s_tail;
-  const uint32_t* s_dep;  // per slice: where its entries past D begin << 8 | depth
+  const uint32_t* s_dep;  // per slice: where its entries past D begin << kDepthBits | depth
   int F;
   uint16_t vl[R];         // local index, 0xFFFF for a padding row
   uint32_t ea[R][D];                  // address, or the packed entry
@@ -601,12 +660,12 @@ struct RegRows {
     const int lane = threadIdx.x & 31;
     int o = 0;
     if (depth > D) {
-      for (int q = lane; q < sl; q += 32) o += max(0, (int)(slc[q] & 255u) - D) * 32;
+      for (int q = lane; q < sl; q += 32) o += max(0, (int)(slc[q] & kDepthMask) - D) * 32;
       o = __reduce_add_sync(0xffffffffu, o);
       for (int k = D; k < depth; k += 2)
         *reinterpret_cast<int4*>(tl + o + (k - D) * 32 + lane * 2) = *reinterpret_cast<const int4*>(ent + at + k * 32);
     }
-    if (lane == 0) dep[sl] = (uint32_t)o << 8 | (uint32_t)depth;
+    if (lane == 0) dep[sl] = (uint32_t)o << kDepthBits | (uint32_t)depth;
   }
 
   __device__ __forceinline__ void init(const RingArgs& A, const RingHdr& h, int b, unsigned char* smem) {
@@ -637,8 +696,8 @@ struct RegRows {
       int at = 0, depth = 0;
       if (warp < NW && sl < nsl) {
         const uint32_t od = slc[sl];
-        depth = (int)(od & 255u);
-        at = (int)(od >> 8) + lane * 2;
+        depth = (int)(od & kDepthMask);
+        at = (int)(od >> kDepthBits) + lane * 2;
         const int row = A.order[(size_t)b * kRingSlots + sl * 32 + lane];
         if (row != 0xFFFF) vl[r] = (uint16_t)(row < h.own ? sl * 32 + lane : ownp + row - h.own);
         if (MODE > 0 && row != 0xFFFF)
@@ -678,12 +737,12 @@ struct RegRows {
 
   // the row's order pair from its first N entries and the tail
   template <int PAR, int N>
-  __device__ __forceinline__ void pair_of(int r, int l, int depth, uint32_t dt, int& zb, int& zc) const {
+  __device__ __forceinline__ void pair_of(const RingArgs& A, int r, int l, int depth, uint32_t dt, int& zb, int& zc) const {
     const int lane = threadIdx.x & 31;
     int z[N];
 #pragma unroll
     for (int k = 0; k < N; ++k) z[k] = z_of<PAR>(ea[r][k], PACKED ? 0 : ec[PACKED ? 0 : r][PACKED ? 0 : k], l);
-    const int4* tl = reinterpret_cast<const int4*>(s_tail + (dt >> 8) + lane * 2);
+    const int4* tl = reinterpret_cast<const int4*>(s_tail + (dt >> kDepthBits) + lane * 2);
     if constexpr (MODE == 0) {
       int a;
       top3_of4(z[0], z[1], z[2], z[3], a, zb, zc);
@@ -694,10 +753,17 @@ struct RegRows {
         top3_join(a1, b1, c1, a, zb, zc);
       }
       if constexpr (N == D) {
-        for (int k = D; k < depth; k += 2) {
+        const int stop = LONG && depth > kRingLong ? kRingTail : depth;
+        for (int k = D; k < stop; k += 2) {
           const int4 q = tl[(k - D) * 16];
           top3_insert_minmax(q.y - l - lam(PAR)[q.x], a, zb, zc);
           top3_insert_minmax(q.w - l - lam(PAR)[q.z], a, zb, zc);
+        }
+        if (LONG && depth > kRingLong) {
+          const int4* row0 = reinterpret_cast<const int4*>(s_tail + (dt >> kDepthBits));
+          long long none = 0;
+          long_rows<false>(A.longs[(size_t)(A.first_tile + blockIdx.x) * kRingSlices + (threadIdx.x >> 5) + r * NW], depth,
+                           l, [&](int k, int row) { return row0[(k - D) * 16 + row]; }, lam(PAR), a, zb, zc, none);
         }
       }
     } else {
@@ -737,14 +803,14 @@ struct RegRows {
       const int sl = warp + r * NW;
       if (sl >= end) break;
       const uint32_t dt = s_dep[sl];
-      const int depth = (int)(dt & 255u), v = vl[r];
+      const int depth = (int)(dt & kDepthMask), v = vl[r];
       const int l = v != 0xFFFF ? lam(PAR)[v] : 0;
       // no branch between a row's gathers: all are in flight together
       int zb, zc;
       if (depth <= 12)
-        pair_of<PAR, 12>(r, l, depth, dt, zb, zc);
+        pair_of<PAR, 12>(A, r, l, depth, dt, zb, zc);
       else
-        pair_of<PAR, D>(r, l, depth, dt, zb, zc);
+        pair_of<PAR, D>(A, r, l, depth, dt, zb, zc);
       const int nl = o.step(zb, zc, l, A.shift);
       if (v != 0xFFFF) {
         lam(PAR ^ 1)[v] = nl;
@@ -948,18 +1014,19 @@ gdp_ring_smem_kernel(const __grid_constant__ RingArgs A) {
     ring_run<SmemRows<MODE, BOUND, true, T / 32 - 1>, T>(A, h, smem, trace);
 }
 
-template <int MODE, int R, int T>
+template <int MODE, int R, int T, bool LONG = false>
 __global__ void __launch_bounds__(T, 1024 / T)
 gdp_ring_reg_kernel(const __grid_constant__ RingArgs A) {
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr int NW = T / 32 - 1;
   const RingStats st = *A.stats;
-  if (st.bad || st.bytes_reg > A.smem || st.slices > R * NW || (R > 1 && !reg_packs(st, NW))) {
+  if (st.bad || st.bytes_reg > A.smem || st.slices > R * NW || (R > 1 && !reg_packs(st, NW)) ||
+      (MODE == 0 && T == 1024 && LONG != (st.longs != 0))) {
     if (threadIdx.x == 0) atomicOr(A.status, kGdpNoFit);
     return;
   }
   const RingHdr h = A.hdr[A.first_tile + blockIdx.x];
-  ring_run<RegRows<MODE, R, NW>, T>(A, h, smem);
+  ring_run<RegRows<MODE, R, NW, LONG>, T>(A, h, smem);
 }
 
 // ---- host side -------------------------------------------------------------------------
@@ -982,24 +1049,27 @@ static cudaError_t grow(T** p, int64_t* cap, int64_t need) {
 }
 
 void ring_free(RingPlan& p) {
-  void* ptrs[] = {p.hdr, p.halo, p.order, p.slc, p.ent, p.pos, p.rec, p.words};
+  void* ptrs[] = {p.hdr, p.halo, p.order, p.slc, p.longs, p.ent, p.pos, p.rec, p.words};
   for (void* q : ptrs)
     if (q) dev_free(q);
   p = RingPlan();
 }
 
 cudaError_t ring_build(const GdpPlan& g, const int32_t* seg_off, const RingTile* list, int32_t tiles, int32_t K,
-                       int32_t F, int64_t entries_per_tile, int32_t nseg, RingPlan& p, cudaStream_t st) {
-  // room for a tile's sliced entries: its own and its inner rings', at most what
-  // the 4-byte form could hold in shared memory
-  const int64_t want = K > 1 ? entries_per_tile * 2 + 16384 : entries_per_tile * 3 / 2 + 4096;
-  const int64_t ecap = (want < 49152 ? want : 49152) / 64 * 64;
+                       int32_t F, int64_t entries_per_tile, int32_t maxdeg, int32_t nseg, RingPlan& p,
+                       cudaStream_t st) {
+  // room for a tile's sliced entries: its own and its inner rings'
+  const int64_t want = entries_per_tile < 0 ? kMaxEntries
+                       : K > 1              ? entries_per_tile * 2 + 16384
+                                            : entries_per_tile * 3 / 2 + 4096;
+  const int64_t ecap = (want < kMaxEntries ? want : kMaxEntries) / 64 * 64;
   p.version = -1;
   RCK(grow(&p.hdr, &p.hdr_cap, tiles));
   RCK(grow(&p.halo, &p.halo_cap, (int64_t)tiles * kRingHalo));
   RCK(grow(&p.pos, &p.pos_cap, g.n));
   RCK(grow(&p.order, &p.order_cap, (int64_t)tiles * kRingSlots));
   RCK(grow(&p.slc, &p.slc_cap, (int64_t)tiles * kRingSlices));
+  RCK(grow(&p.longs, &p.longs_cap, (int64_t)tiles * kRingSlices));
   RCK(grow(&p.ent, &p.ent_cap, (int64_t)tiles * ecap));
   if (p.seg_cap < nseg) {
     if (p.rec) dev_free(p.rec);
@@ -1011,8 +1081,8 @@ cudaError_t ring_build(const GdpPlan& g, const int32_t* seg_off, const RingTile*
   RCK(cudaMemsetAsync(&p.rec->stats, 0, sizeof(RingStats), st));
   constexpr size_t smem = 4 * (kHash + 2 * kRingHalo) + 2 * (kHash + kRingHalo + 2 * kRingLocals + kRingSlots);
   RCK(cudaFuncSetAttribute(ring_plan_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  ring_plan_kernel<<<tiles, kPlanThreads, smem, st>>>(g.irp, g.iec, list, seg_off, tiles, K, F, (int32_t)ecap, p.hdr,
-                                                      p.halo, p.order, p.slc, p.ent, p.pos, &p.rec->stats);
+  ring_plan_kernel<<<tiles, kPlanThreads, smem, st>>>(g.irp, g.iec, list, seg_off, tiles, K, F, (int32_t)ecap, maxdeg, p.hdr,
+                                                      p.halo, p.order, p.slc, p.longs, p.ent, p.pos, &p.rec->stats);
   count_launch();
   RCK(cudaGetLastError());
   p.ecap = (int32_t)ecap;
@@ -1039,8 +1109,9 @@ static const void* ring_kernel_of(bool bound) {
 }
 
 template <int R>
-static const void* ring_reg_kernel_of(int mode) {
-  return mode == 0   ? (const void*)gdp_ring_reg_kernel<0, R, 1024>
+static const void* ring_reg_kernel_of(int mode, bool longs) {
+  return mode == 0   ? (longs ? (const void*)gdp_ring_reg_kernel<0, R, 1024, true>
+                              : (const void*)gdp_ring_reg_kernel<0, R, 1024>)
          : mode == 1 ? (const void*)gdp_ring_reg_kernel<1, R, 1024>
                      : (const void*)gdp_ring_reg_kernel<2, R, 1024>;
 }
@@ -1064,13 +1135,13 @@ int32_t ring_smem(bool half, bool traced) {
 cudaError_t launch_gdp_ring(const GdpPlan& g, RingPlan& p, int32_t first_tile, int32_t tiles, const int32_t* lam_in,
                             int32_t* lam_out, int32_t shift, int32_t max_sweeps, long long* trace_b2,
                             unsigned long long* trace_ch, int64_t trace_cap, long long budget, const int32_t* bint,
-                            int32_t bmax, RingForm form, cudaStream_t st) {
+                            int32_t bmax, RingForm form, bool longs, cudaStream_t st) {
   const bool bound = trace_cap > 0, half = form == kRingHalf || form == kRingPair, reg = form > 0;
   const int mode = !bint ? 0 : (bmax < 5 ? 1 : (bmax < 8 ? 2 : 3));
   if (reg && (bound || mode > (form == kRingPair ? 0 : 2))) return cudaErrorInvalidValue;
   const int T = reg ? (half ? 512 : 1024) : (half || mode >= 2 ? 512 : 1024);
-  const void* kern = form == kRingReg1   ? ring_reg_kernel_of<1>(mode)
-                     : form == kRingReg2 ? ring_reg_kernel_of<2>(mode)
+  const void* kern = form == kRingReg1   ? ring_reg_kernel_of<1>(mode, longs)
+                     : form == kRingReg2 ? ring_reg_kernel_of<2>(mode, longs)
                      : form == kRingPair ? (const void*)gdp_ring_reg_kernel<0, 2, 512>
                      : half && mode == 0 ? ring_kernel_of<0, 512>(bound)
                      : mode == 0       ? ring_kernel_of<0, 1024>(bound)
@@ -1084,6 +1155,7 @@ cudaError_t launch_gdp_ring(const GdpPlan& g, RingPlan& p, int32_t first_tile, i
   a.halo = p.halo;
   a.order = p.order;
   a.slc = p.slc;
+  a.longs = p.longs;
   a.ent = p.ent;
   a.stats = &p.rec->stats;
   a.seg = p.rec->seg;
