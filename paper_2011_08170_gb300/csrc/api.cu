@@ -678,11 +678,12 @@ static f2m_status ring_phase(f2m_ctx* c, int64_t max_sweeps, int64_t* sweeps, lo
         CK(c, cudaMemsetAsync(tb, 0, sizeof(long long) * tcap, c->st));
         CK(c, cudaMemsetAsync(tc, 0, sizeof(unsigned long long) * tcap, c->st));
       }
+      const RingForm form = reg ? (RingForm)c->ring_rows : (half ? kRingHalf : kRingSmem);
       CK(c, cudaEventRecord(c->ev0, c->st));
       const cudaError_t e =
           launch_gdp_ring(c->plan, c->ring, 0, tiles, c->d_lam[c->cur], c->d_lam[c->cur ^ 1], c->p.damping_shift,
                           (int32_t)limit, tb, tc, replay ? 0 : tcap, c->p.barrier_budget_cycles, c->d_b_int, c->b_max,
-                          reg ? (RingForm)c->ring_rows : (half ? kRingHalf : kRingSmem), c->ring_longs, c->st);
+                          form, c->ring_longs, c->st);
       if (e == cudaErrorCooperativeLaunchTooLarge) {  // not on this device now
         cudaGetLastError();
         *ran = false;
@@ -706,7 +707,7 @@ static f2m_status ring_phase(f2m_ctx* c, int64_t max_sweeps, int64_t* sweeps, lo
         if ((status & kGdpNoFit) && fits && (fits != had || other)) continue;
       }
       if (status & kGdpNoFit) break;
-      const bool packed = reg ? c->ring_rows > 1 : rs.bytes8 > ring_smem(half, tcap > 0);
+      const bool packed = reg ? form == kRingReg2 : rs.bytes8 > ring_smem(half, tcap > 0);
       c->gdp_kernel = c->ring.K == 1 ? F2M_GDP_KERNEL_TILED
                                      : (packed ? F2M_GDP_KERNEL_TWO_SWEEP_PACKED : F2M_GDP_KERNEL_TWO_SWEEP);
       if (replay) break;
