@@ -360,6 +360,12 @@ cudaError_t ring_build(const GdpPlan& g, const int32_t* seg_off, const RingTile*
 int32_t ring_smem(bool half, bool traced);  // dynamic shared memory of a CTA
 // per phase: cleared segment records and status
 cudaError_t ring_start(RingPlan& p, int32_t n, int32_t nseg, cudaStream_t st);
+// whether tiles of n nodes and nnz entries in all might fit some form
+inline bool ring_can_fit(int64_t n, int64_t nnz, int64_t tiles, int64_t smem, bool half) {
+  const int64_t own = (n + tiles - 1) / tiles;
+  if (own + 34 > kRingLocals) return false;
+  return (!half && own <= 62 * 32) || 4 * (nnz / tiles) + 10 * own <= smem;
+}
 // Where the rows' entries are kept: registers (1 or 2 rows a thread, up to 1,984
 // rows a tile), registers with two CTAs per SM (up to 960 rows a tile, b_v = 2),
 // shared memory, or shared memory with two CTAs per SM.

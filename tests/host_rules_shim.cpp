@@ -36,3 +36,7 @@ extern "C" int shim_grow(long long had, long long need, long long room, int bloc
 }
 
 extern "C" long long shim_price_list_room(unsigned long long listed) { return f2m::price_list_room(listed); }
+
+extern "C" int shim_ring_can_fit(long long n, long long nnz, long long tiles, long long smem, int half) {
+  return f2m::ring_can_fit(n, nnz, tiles, smem, half != 0);
+}

@@ -54,3 +54,13 @@ def test_the_form_reported_is_the_one_that_ran(lib, n):
     slices = own / 32 + (rings - 1) * ((14 * math.sqrt(own) + 30) / 32 + 1)
     assert slices > 30  # the guess: two rows a thread, packed
     assert _kernel(_ctx(n, 10)) == PACKED
+
+
+def test_a_first_phase_does_not_try_what_cannot_fit(lib):
+    ctx = _ctx(900_000, 8)
+    used = []
+    for _ in range(2):
+        before = f2m.f2m_kernel_launches()
+        f2m.f2m_gdp(ctx, 5)
+        used.append(f2m.f2m_kernel_launches() - before)
+    assert used[0] == used[1]

@@ -1,6 +1,6 @@
 """Decisions that the library makes on the host, without a GPU: which arrays a kernel
-may write to, what a work array says of itself after an allocation failed, and how
-many block pairs a culled scan lists."""
+may write to, what a work array says of itself after an allocation failed, how many
+block pairs a culled scan lists, and which graphs are not tried on tiles."""
 import ctypes as C
 import os
 import shutil
@@ -73,3 +73,17 @@ def test_a_list_past_the_handed_out_numbers_is_refused(rules, listed):
     # scan and its list never met, and past 2^32 a 32-bit count wrapped
     rules.shim_price_list_room.argtypes, rules.shim_price_list_room.restype = [C.c_ulonglong], C.c_longlong
     assert rules.shim_price_list_room(listed) == 0
+
+
+SMEM = 232_448 - 128  # a CTA's shared memory
+
+
+@pytest.mark.parametrize("n,degree,half,want", [
+    (1000, 12, False, True), (200_000, 14, False, True), (301_568, 40, False, True),  # 1,984 rows a tile: registers
+    (301_569, 60, False, False), (550_000, 12, False, True), (600_000, 13, False, False), (700_000, 7, False, True),
+    (1_300_000, 3, False, False), (2_000_000, 12, False, False), (1 << 24, 3, False, False),
+    (200_000, 12, True, True), (301_568, 60, True, False)])
+def test_what_no_tile_can_hold_is_not_tried(rules, n, degree, half, want):
+    rules.shim_ring_can_fit.argtypes = [C.c_longlong] * 4 + [C.c_int]
+    tiles = 304 if half else 152
+    assert bool(rules.shim_ring_can_fit(n, n * degree, tiles, SMEM // 2 if half else SMEM, half)) == want
