@@ -195,7 +195,7 @@ typedef struct {
 #define F2M_GDP_KERNEL_TWO_SWEEP 2     /* on-chip tiles, two or more sweeps per exchange */
 #define F2M_GDP_KERNEL_TWO_SWEEP_PACKED 3  /* the same with 4-byte entries (larger tiles) */
 #define F2M_GDP_KERNEL_CLASSES 4       /* class-by-class sweeps */
-#define F2M_GDP_KERNEL_BATCH 5         /* batched, union CSR streamed */
+#define F2M_GDP_KERNEL_BATCH 5         /* batched, union CSR streamed (by some instances at least) */
 #define F2M_GDP_KERNEL_BATCH_CLUSTERS 6  /* batched, one thread-block cluster per instance */
 #define F2M_GDP_KERNEL_CUTS 7          /* node and subtour-cut duals, streaming */
 #define F2M_GDP_KERNEL_BATCH_TILES 8   /* batched, on-chip tiles, whole instances in waves */

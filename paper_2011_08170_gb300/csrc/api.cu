@@ -681,7 +681,7 @@ static f2m_status ring_phase(f2m_ctx* c, int64_t max_sweeps, int64_t* sweeps, lo
     // in shared memory: traces, and the counting selection of large b_v
     const bool reg = c->ring_reg && tcap == 0 && !(c->d_b && c->b_max >= 8);
     for (;;) {
-      CK(c, ring_start(c->ring, c->n, 1, c->st));
+      CK(c, ring_start(c->ring, c->n, tiles, 1, c->st));
       if (tcap > 0 && !replay) {
         CK(c, cudaMemsetAsync(tb, 0, sizeof(long long) * tcap, c->st));
         CK(c, cudaMemsetAsync(tc, 0, sizeof(unsigned long long) * tcap, c->st));

@@ -81,8 +81,9 @@ struct f2m_batch {
   std::vector<int32_t> res_fb, res_r0;  // fractional bits; first entry in the union's offsets
   std::vector<uint8_t> res_done;
   // tiles (gdp_ring.cu): those of a phase's active instances, wave by wave
-  bool ring_off = false;            // they don't fit: the streaming kernels
-  bool used_ring = false;           // the last phase ran on tiles
+  bool ring_off = false;            // not on this device: the streaming kernels
+  std::vector<uint8_t> ring_level;  // per instance: 0 any tiles, 1 only of kBatchTileRows rows, 2 none that fit
+  bool used_ring = false, used_stream = false;  // in a solve: some phase of some instance
   RingTile* d_rlist = nullptr;
   int64_t rlist_cap = 0;
   RingSeg* h_rseg = nullptr;        // pinned
@@ -642,30 +643,36 @@ static f2m_status batch_cluster_phase(f2m_batch* b, const std::vector<uint8_t>& 
 
 // A GDP phase on tiles of at most `rows` nodes and K rings: the tiles of an
 // instance stay on chip for the phase, two tiles per SM; whole instances go
-// together in waves of as many tiles as the GPU holds.  *ran false where some
-// tile does not fit.
-static f2m_status batch_ring_phase(f2m_batch* b, const std::vector<uint8_t>& active, int32_t rows, int32_t K,
-                                   std::vector<int64_t>& sweeps_out, double* ms, bool* ran) {
+// together in waves of as many tiles as the GPU holds.  Of the instances in `todo`
+// those that ran are cleared; one with a tile that does not fit keeps its lambda,
+// and its ring_level becomes `level` + 1.
+static f2m_status batch_ring_phase(f2m_batch* b, std::vector<uint8_t>& todo, int32_t rows, int32_t K, uint8_t level,
+                                   std::vector<int64_t>& sweeps_out, double* ms) {
   f2m_ctx* c = b->u;
-  *ran = false;
   const int32_t room = 2 * c->num_sms;
   std::vector<RingTile> list;
   std::vector<int32_t> waves{0};  // first tile of each wave
+  std::vector<int32_t> taken;     // the instances
   for (int32_t s = 0; s < b->count; ++s) {
-    if (!active[s]) continue;
+    if (!todo[s] || b->ring_level[s] > level) continue;
     const int32_t t = (b->n[s] + rows - 1) / rows;
-    if (t > room) return F2M_OK;
+    if (t > room) {
+      b->ring_level[s] = (uint8_t)(level + 1);
+      continue;
+    }
+    taken.push_back(s);
     if ((int32_t)list.size() + t - waves.back() > room) waves.push_back((int32_t)list.size());
     for (int32_t j = 0; j < t; ++j) list.push_back(RingTile{s, j, t});
   }
+  if (list.empty()) return F2M_OK;
   waves.push_back((int32_t)list.size());
   const int32_t tiles = (int32_t)list.size();
   CK(c, dgrow(&b->d_rlist, &b->rlist_cap, tiles, tiles + tiles / 8 + 64));
   if (!b->h_rseg) CK(c, pin_alloc((void**)&b->h_rseg, sizeof(RingSeg) * b->count));
   CK(c, cudaMemcpyAsync(b->d_rlist, list.data(), sizeof(RingTile) * tiles, cudaMemcpyHostToDevice, c->st));
-  CK(c, ring_build(c->plan, c->d_seg_off, b->d_rlist, tiles, K, c->p.frac_bits, rows * c->nnz / c->n, kBatchRowEntries, b->count, c->ring,
-                   c->st));
-  CK(c, ring_start(c->ring, c->n, b->count, c->st));
+  CK(c, ring_start(c->ring, c->n, tiles, b->count, c->st));
+  CK(c, ring_build(c->plan, c->d_seg_off, b->d_rlist, tiles, K, c->p.frac_bits, rows * c->nnz / c->n, kBatchRowEntries,
+                   b->count, c->ring, c->st, ring_pair_limit()));
   // the instances left alone keep their lambda
   const int32_t* in = c->d_lam[c->cur];
   int32_t* out = c->d_lam[c->cur ^ 1];
@@ -678,6 +685,7 @@ static f2m_status batch_ring_phase(f2m_batch* b, const std::vector<uint8_t>& act
     if (e == cudaErrorCooperativeLaunchTooLarge) {
       cudaGetLastError();
       CK(c, cudaStreamSynchronize(c->st));
+      b->ring_off = true;
       return F2M_OK;
     }
     CK(c, e);
@@ -687,14 +695,17 @@ static f2m_status batch_ring_phase(f2m_batch* b, const std::vector<uint8_t>& act
   CK(c, cudaMemcpyAsync(&status, &c->ring.rec->status, sizeof(status), cudaMemcpyDeviceToHost, c->st));
   CK(c, cudaMemcpyAsync(b->h_rseg, c->ring.rec->seg, sizeof(RingSeg) * b->count, cudaMemcpyDeviceToHost, c->st));
   CK(c, cudaStreamSynchronize(c->st));
-  if (status & kGdpNoFit) return F2M_OK;
-  *ran = true;
   float t_ms = 0.f;
   cudaEventElapsedTime(&t_ms, c->ev0, c->ev1);
   if (ms) *ms += t_ms;
   if (status & kGdpTimeout) return fail(c, F2M_ERR_TIMEOUT, "a wait for another tile exceeded its budget");
-  for (int32_t s = 0; s < b->count; ++s) {
-    if (!active[s]) continue;
+  for (int32_t s : taken) {
+    if (b->h_rseg[s].unfit) {
+      b->ring_level[s] = (uint8_t)(level + 1);
+      continue;
+    }
+    todo[s] = 0;
+    b->used_ring = true;
     sweeps_out[s] += b->h_rseg[s].sweeps;
     if (b->h_rseg[s].overflow) return fail(c, F2M_ERR_OVERFLOW, "|lambda| reached 2^29 in some instance");
   }
@@ -702,8 +713,8 @@ static f2m_status batch_ring_phase(f2m_batch* b, const std::vector<uint8_t>& act
   return F2M_OK;
 }
 
-static f2m_status batch_gdp_phase(f2m_batch* b, const std::vector<uint8_t>& active,
-                                  std::vector<int64_t>& sweeps_out, double* ms) {
+static f2m_status batch_gdp_phase(f2m_batch* b, std::vector<uint8_t> active, std::vector<int64_t>& sweeps_out,
+                                  double* ms) {
   f2m_ctx* c = b->u;
   c->lam_version += 1;
   GdpPlan& P = c->plan;
@@ -725,7 +736,6 @@ static f2m_status batch_gdp_phase(f2m_batch* b, const std::vector<uint8_t>& acti
       return batch_cluster_phase(b, active, sweeps_out, ms);
     }
   }
-  b->used_ring = false;
   if (c->p.batch_shape < 0 && !b->ring_off && c->p.max_iters > 0 && c->p.max_iters <= kRingSweeps) {
     // tiles of 960 rows, one sweep an exchange, in full waves (256 instances of
     // 1,000-20,000 points, all phases: 5.5 ms; tiles of 800 rows 5.8, 640 rows 6.0;
@@ -736,11 +746,12 @@ static f2m_status batch_gdp_phase(f2m_batch* b, const std::vector<uint8_t>& acti
     for (int32_t s = 0; s < b->count; ++s) nodes += active[s] ? b->n[s] : 0;
     const int32_t fine = (int32_t)std::max<int64_t>(96, (nodes / (2 * c->num_sms) + 31) / 32 * 32);
     f2m_status s = F2M_OK;
-    if (fine <= 320) s = batch_ring_phase(b, active, fine, fine <= 128 ? 3 : 2, sweeps_out, ms, &b->used_ring);
-    if (s == F2M_OK && !b->used_ring) s = batch_ring_phase(b, active, kBatchTileRows, 1, sweeps_out, ms, &b->used_ring);
-    if (s != F2M_OK || b->used_ring) return s;
-    b->ring_off = true;
+    if (fine <= 320) s = batch_ring_phase(b, active, fine, fine <= 128 ? 3 : 2, 0, sweeps_out, ms);
+    if (s == F2M_OK && !b->ring_off) s = batch_ring_phase(b, active, kBatchTileRows, 1, 1, sweeps_out, ms);
+    if (s != F2M_OK) return s;
+    if (std::find(active.begin(), active.end(), 1) == active.end()) return F2M_OK;
   }
+  b->used_stream = true;  // the instances left over: with rows, edges or sizes that no tile takes
   if (b->tiles_version != P.version) {
     f2m_status s = F2M_OK;
     if (c->p.batch_shape >= 0) {
@@ -930,6 +941,8 @@ extern "C" f2m_status f2m_solve_batch(f2m_batch* b, f2m_info* info_out, f2m_info
   f2m_info tot;
   std::memset(&tot, 0, sizeof(tot));
   c->fin_stats = FinisherStats();
+  b->used_ring = b->used_stream = false;
+  b->ring_level.resize(K, 0);
   f2m_status status = F2M_OK;
   auto any_in = [&](int st) {
     for (int s : state)
@@ -1080,8 +1093,9 @@ extern "C" f2m_status f2m_solve_batch(f2m_batch* b, f2m_info* info_out, f2m_info
   tot.nnz = b->res_used;
   tot.batch_shape = b->shape;
   tot.batch_graph = b->gexec != nullptr ? 1 : 0;
-  tot.gdp_kernel = b->used_ring ? F2M_GDP_KERNEL_BATCH_TILES
-                                : (b->used_clusters ? F2M_GDP_KERNEL_BATCH_CLUSTERS : F2M_GDP_KERNEL_BATCH);
+  tot.gdp_kernel = b->used_ring && !b->used_stream
+                       ? F2M_GDP_KERNEL_BATCH_TILES
+                       : (b->used_clusters ? F2M_GDP_KERNEL_BATCH_CLUSTERS : F2M_GDP_KERNEL_BATCH);
   tot.certified = 2;
   for (int32_t s = 0; s < K; ++s) {
     tot.certified = std::min(tot.certified, certified[s]);

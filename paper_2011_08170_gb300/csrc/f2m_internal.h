@@ -307,6 +307,10 @@ struct RingSeg {          // per instance, zeroed per phase
   unsigned int ovf[kRingRing];
   long long sweeps;       // the result
   int32_t fixed_point, overflow;
+  int32_t unfit;          // (batches) one of its tiles is past the form's limits: none of them runs
+};
+struct RingLimit {        // of a form, per tile (batches; smem 0: none)
+  int32_t smem, slices, locals, cost;
 };
 struct RingRecord {       // what the host reads after a phase, in one copy
   RingStats stats;        // zeroed per plan
@@ -356,10 +360,13 @@ void ring_free(RingPlan& p);
 // maxdeg: the longest row a tile takes, at most kRingDepth; entries_per_tile: their
 // mean (a tile's room is what near-even tiles need), -1: the most a tile can hold
 cudaError_t ring_build(const GdpPlan& g, const int32_t* seg_off, const RingTile* list, int32_t tiles, int32_t K,
-                       int32_t F, int64_t entries_per_tile, int32_t maxdeg, int32_t nseg, RingPlan& p, cudaStream_t st);
+                       int32_t F, int64_t entries_per_tile, int32_t maxdeg, int32_t nseg, RingPlan& p, cudaStream_t st,
+                       const RingLimit& limit = RingLimit{});
+RingLimit ring_pair_limit();  // of kRingPair
 int32_t ring_smem(bool half, bool traced);  // dynamic shared memory of a CTA
-// per phase: cleared segment records and status
-cudaError_t ring_start(RingPlan& p, int32_t n, int32_t nseg, cudaStream_t st);
+// per phase: cleared segment records and status; with limits before ring_build, which
+// flags the instances past them
+cudaError_t ring_start(RingPlan& p, int32_t n, int32_t tiles, int32_t nseg, cudaStream_t st);
 // whether tiles of n nodes and nnz entries in all might fit some form
 inline bool ring_can_fit(int64_t n, int64_t nnz, int64_t tiles, int64_t smem, bool half) {
   const int64_t own = (n + tiles - 1) / tiles;

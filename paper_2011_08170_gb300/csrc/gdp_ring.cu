@@ -100,7 +100,7 @@ ring_plan_kernel(const int32_t* __restrict__ irp, const int2* __restrict__ iec, 
                  const int32_t* __restrict__ seg_off, int32_t tiles, int32_t K, int32_t F, int32_t ecap, int32_t maxdeg,
                  RingHdr* __restrict__ hdr, int32_t* __restrict__ halo, uint16_t* __restrict__ order,
                  uint32_t* __restrict__ slc, uint32_t* __restrict__ longs, int2* __restrict__ ent,
-                 int32_t* __restrict__ pos, RingStats* stats) {
+                 int32_t* __restrict__ pos, RingStats* stats, RingSeg* seg, RingLimit limit) {
   extern __shared__ __align__(16) unsigned char smem[];
   int* keys = reinterpret_cast<int*>(smem);                         // [kHash] outside nodes
   int* ring = keys + kHash;                                         // [kRingHalo] in ring order
@@ -321,7 +321,11 @@ ring_plan_kernel(const int32_t* __restrict__ irp, const int2* __restrict__ iec, 
     if (s_long) stats->longs = 1;
     atomicMax(&stats->locals, ownp + HH + 2);
     atomicMax(&stats->maxcost, s_maxcost);
-    atomicMax(&stats->bytes_reg, 2 * kRingLamBytes + 4 * (HH + nsl) + 8 * s_tail + 64);
+    const int bytes_reg = 2 * kRingLamBytes + 4 * (HH + nsl) + 8 * s_tail + 64;
+    atomicMax(&stats->bytes_reg, bytes_reg);
+    if (limit.smem && (bad || bytes_reg > limit.smem || nsl > limit.slices || ownp + HH + 2 > limit.locals ||
+                       s_maxcost >= limit.cost))
+      seg[tl.seg].unfit = 1;
     if (bad) atomicOr(&stats->bad, bad);
   }
 }
@@ -991,7 +995,8 @@ __device__ __forceinline__ void ring_run(const RingArgs& A, const RingHdr& h, un
 
 }  // namespace
 
-// Every tile reads the same statistics, so all take the same form.
+// Every tile reads the same statistics, so all take the same form (two CTAs per SM,
+// a batch: an instance's tiles read its own flag).
 template <int MODE, bool BOUND, int T>
 __global__ void __launch_bounds__(T, T == 512 && MODE < 2 ? 2 : 1)
 gdp_ring_smem_kernel(const __grid_constant__ RingArgs A) {
@@ -1019,13 +1024,17 @@ __global__ void __launch_bounds__(T, 1024 / T)
 gdp_ring_reg_kernel(const __grid_constant__ RingArgs A) {
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr int NW = T / 32 - 1;
-  const RingStats st = *A.stats;
-  if (st.bad || st.bytes_reg > A.smem || st.slices > R * NW || (R > 1 && !reg_packs(st, NW)) ||
-      (MODE == 0 && T == 1024 && LONG != (st.longs != 0))) {
-    if (threadIdx.x == 0) atomicOr(A.status, kGdpNoFit);
-    return;
-  }
   const RingHdr h = A.hdr[A.first_tile + blockIdx.x];
+  if constexpr (T == 512) {
+    if (A.seg[h.seg].unfit) return;
+  } else {
+    const RingStats st = *A.stats;
+    if (st.bad || st.bytes_reg > A.smem || st.slices > R * NW || (R > 1 && !reg_packs(st, NW)) ||
+        (MODE == 0 && LONG != (st.longs != 0))) {
+      if (threadIdx.x == 0) atomicOr(A.status, kGdpNoFit);
+      return;
+    }
+  }
   ring_run<RegRows<MODE, R, NW, LONG>, T>(A, h, smem);
 }
 
@@ -1055,9 +1064,19 @@ void ring_free(RingPlan& p) {
   p = RingPlan();
 }
 
+static cudaError_t ring_records(RingPlan& p, int32_t nseg) {
+  if (p.seg_cap >= nseg) return cudaSuccess;
+  if (p.rec) dev_free(p.rec);
+  p.rec = nullptr;
+  p.seg_cap = 0;
+  RCK(dev_malloc((void**)&p.rec, sizeof(RingRecord) + sizeof(RingSeg) * (size_t)nseg));
+  p.seg_cap = nseg;
+  return cudaSuccess;
+}
+
 cudaError_t ring_build(const GdpPlan& g, const int32_t* seg_off, const RingTile* list, int32_t tiles, int32_t K,
                        int32_t F, int64_t entries_per_tile, int32_t maxdeg, int32_t nseg, RingPlan& p,
-                       cudaStream_t st) {
+                       cudaStream_t st, const RingLimit& limit) {
   // room for a tile's sliced entries: its own and its inner rings'
   const int64_t want = entries_per_tile < 0 ? kMaxEntries
                        : K > 1              ? entries_per_tile * 2 + 16384
@@ -1071,18 +1090,12 @@ cudaError_t ring_build(const GdpPlan& g, const int32_t* seg_off, const RingTile*
   RCK(grow(&p.slc, &p.slc_cap, (int64_t)tiles * kRingSlices));
   RCK(grow(&p.longs, &p.longs_cap, (int64_t)tiles * kRingSlices));
   RCK(grow(&p.ent, &p.ent_cap, (int64_t)tiles * ecap));
-  if (p.seg_cap < nseg) {
-    if (p.rec) dev_free(p.rec);
-    p.rec = nullptr;
-    p.seg_cap = 0;
-    RCK(dev_malloc((void**)&p.rec, sizeof(RingRecord) + sizeof(RingSeg) * (size_t)nseg));
-    p.seg_cap = nseg;
-  }
+  RCK(ring_records(p, nseg));
   RCK(cudaMemsetAsync(&p.rec->stats, 0, sizeof(RingStats), st));
   constexpr size_t smem = 4 * (kHash + 2 * kRingHalo) + 2 * (kHash + kRingHalo + 2 * kRingLocals + kRingSlots);
   RCK(cudaFuncSetAttribute(ring_plan_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   ring_plan_kernel<<<tiles, kPlanThreads, smem, st>>>(g.irp, g.iec, list, seg_off, tiles, K, F, (int32_t)ecap, maxdeg, p.hdr,
-                                                      p.halo, p.order, p.slc, p.longs, p.ent, p.pos, &p.rec->stats);
+                                                      p.halo, p.order, p.slc, p.longs, p.ent, p.pos, &p.rec->stats, p.rec->seg, limit);
   count_launch();
   RCK(cudaGetLastError());
   p.ecap = (int32_t)ecap;
@@ -1093,9 +1106,9 @@ cudaError_t ring_build(const GdpPlan& g, const int32_t* seg_off, const RingTile*
   return cudaSuccess;
 }
 
-cudaError_t ring_start(RingPlan& p, int32_t n, int32_t nseg, cudaStream_t st) {
-  if (p.seg_cap < nseg) return cudaErrorInvalidValue;
-  const int64_t m = (int64_t)n + 32LL * p.tiles;  // a tile's own slots are whole slices
+cudaError_t ring_start(RingPlan& p, int32_t n, int32_t tiles, int32_t nseg, cudaStream_t st) {
+  RCK(ring_records(p, nseg));
+  const int64_t m = (int64_t)n + 32LL * tiles;  // a tile's own slots are whole slices
   RCK(grow(&p.words, &p.words_cap, 2 * m));
   p.words_n = m;
   RCK(cudaMemsetAsync(p.words, 0, sizeof(unsigned) * 2 * m, st));
@@ -1120,6 +1133,11 @@ int ring_reg_rows(const RingStats& st) {
   if (st.bad || st.bytes_reg > ring_smem(false, false)) return 0;
   if (st.slices <= 31) return 1;
   return st.slices <= 62 && reg_packs(st, 31) ? 2 : 0;
+}
+
+RingLimit ring_pair_limit() {
+  constexpr int bits = reg_address_bits(15);
+  return RingLimit{ring_smem(true, false), 2 * 15, 1 << (bits - 2), reg_pad_cost(bits)};
 }
 
 int32_t ring_smem(bool half, bool traced) {

@@ -1,0 +1,86 @@
+"""Batches in which only some instances fit the tiles: the streaming kernels' results,
+whatever the reason (edges past the packed entries, a row past a tile's, more tiles
+than the GPU holds), in one wave and in several, over several phases; and the others
+stay on the tiles.
+
+That shows in the GDP time: 600 instances of 960 points are two waves on tiles and
+stream at over twice that; one more instance that streams alone adds the sweeps of a
+few tiles' rows.  The line is at three quarters of all streaming."""
+import numpy as np
+import pytest
+
+import instances as I
+import paper_2011_08170_gb300 as f2m
+from paper_2011_08170_gb300 import build as B
+
+pytestmark = pytest.mark.gpu
+TILES, STREAM = f2m.F2M_GDP_KERNEL_BATCH_TILES, f2m.F2M_GDP_KERNEL_BATCH
+
+
+@pytest.fixture(scope="module")
+def lib():
+    B.build()
+    return f2m.load()
+
+
+def _knn(xy, k):
+    return (xy,) + f2m.f2m_knn_csr(xy, k)
+
+
+def _far(n=12):  # edges across the square
+    rng = np.random.default_rng(n)
+    return _knn(np.unique(rng.choice([0, (1 << 20) - 1, 5, 9], size=(8 * n, 2)), axis=0)[:n].astype(np.int32), 7)
+
+
+def _star(n=900, length=255):
+    xy, rp, col = _knn(I.uniform_points(n, 7), 6)
+    keep = [c for c in np.arange(1, n) if c not in set(col[:rp[1]].tolist())][:length - int(rp[1])]
+    key = np.unique(np.concatenate([np.repeat(np.arange(n), np.diff(rp)) * n + col, np.array(keep), np.array(keep) * n]))
+    rp = np.zeros(n + 1, np.int32)
+    rp[1:] = np.cumsum(np.bincount(key // n, minlength=n))
+    assert rp[1] == length
+    return xy, rp, (key % n).astype(np.int32)
+
+
+def _solve(insts, **kw):
+    b = f2m.f2m_create_batch(insts, f2m.f2m_default_params(**kw))
+    res = []
+    for _ in range(2):  # the second solve starts from the first's lambda and graph
+        infos, tot = f2m.f2m_solve_batch(b, raise_on_error=False)
+        for i, f in enumerate(infos):
+            r = [f.iterations, f.phases, f.pricing_rounds, f.bound2, f.frac_bits, f.certified, f.status]
+            if f.certified:
+                r += [f2m.f2m_batch_get_lambda(b, i)[0].tobytes()] + [a.tobytes() for a in f2m.f2m_batch_get_x(b, i)]
+            res.append(r)
+    return tot, res
+
+
+def _some(sizes, k=8):
+    return [_knn(I.uniform_points(n, 40 + i) if i % 2 else I.mixture_points(n, 40 + i), min(k, n - 1))
+            for i, n in enumerate(sizes)]
+
+
+@pytest.mark.parametrize("make", [
+    lambda: _some((40, 300, 1200)) + [_far()],
+    lambda: [_far()] + _some((2500, 961, 960, 17)) + [_star()],
+    lambda: _some((20_000,) * 15) + [_far(), _star()] + _some((5000, 400)),
+    lambda: _some((300_000, 1500, 700), 6)])
+def test_mixed_batches_equal_streaming(lib, make):
+    insts = make()
+    tot, got = _solve(insts)
+    assert tot.gdp_kernel == STREAM
+    tot, want = _solve(insts, batch_shape=5)
+    assert got == want
+
+
+def test_the_others_stay_on_tiles(lib):
+    base = _some((960,) * 12)
+    insts = [base[i % 12] for i in range(600)]
+    ms = {}
+    for name, batch, kw in (("tiles", insts, {}), ("mixed", insts + [_far()], {}), ("stream", insts, dict(batch_shape=5))):
+        for _ in range(3):
+            b = f2m.f2m_create_batch(batch, f2m.f2m_default_params(pricing=0, finisher=0, **kw))
+            _, tot = f2m.f2m_solve_batch(b, raise_on_error=False)
+            ms[name] = min(ms.get(name, 1e9), tot.ms_gdp)
+            assert tot.gdp_kernel == (TILES if name == "tiles" else STREAM)
+    assert ms["mixed"] < 0.75 * ms["stream"], ms
