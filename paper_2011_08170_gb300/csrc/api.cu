@@ -689,7 +689,7 @@ static f2m_status ring_phase(f2m_ctx* c, int64_t max_sweeps, int64_t* sweeps, lo
       const RingForm form = reg ? (RingForm)c->ring_rows : (half ? kRingHalf : kRingSmem);
       CK(c, cudaEventRecord(c->ev0, c->st));
       const cudaError_t e =
-          launch_gdp_ring(c->plan, c->ring, 0, tiles, c->d_lam[c->cur], c->d_lam[c->cur ^ 1], c->p.damping_shift,
+          launch_gdp_ring(c->plan, c->ring, tiles, c->d_lam[c->cur], c->d_lam[c->cur ^ 1], c->p.damping_shift,
                           (int32_t)limit, tb, tc, replay ? 0 : tcap, c->p.barrier_budget_cycles, c->d_b_int, c->b_max,
                           form, c->ring_longs, c->st);
       if (e == cudaErrorCooperativeLaunchTooLarge) {  // not on this device now

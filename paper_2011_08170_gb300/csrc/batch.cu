@@ -671,17 +671,22 @@ static f2m_status batch_ring_phase(f2m_batch* b, std::vector<uint8_t>& todo, int
   if (!b->h_rseg) CK(c, pin_alloc((void**)&b->h_rseg, sizeof(RingSeg) * b->count));
   CK(c, cudaMemcpyAsync(b->d_rlist, list.data(), sizeof(RingTile) * tiles, cudaMemcpyHostToDevice, c->st));
   CK(c, ring_start(c->ring, c->n, tiles, b->count, c->st));
-  CK(c, ring_build(c->plan, c->d_seg_off, b->d_rlist, tiles, K, c->p.frac_bits, rows * c->nnz / c->n, kBatchRowEntries,
-                   b->count, c->ring, c->st, ring_pair_limit()));
   // the instances left alone keep their lambda
   const int32_t* in = c->d_lam[c->cur];
   int32_t* out = c->d_lam[c->cur ^ 1];
   CK(c, cudaMemcpyAsync(out, in, sizeof(int32_t) * c->n, cudaMemcpyDeviceToDevice, c->st));
   CK(c, cudaEventRecord(c->ev0, c->st));
+  // a wave's tiles are built when it is next, in the arrays of the one before: their
+  // scratch (150 to 400 KB a tile) does not grow with the batch
+  int32_t most = 0;
+  for (size_t w = 0; w + 1 < waves.size(); ++w) most = std::max(most, waves[w + 1] - waves[w]);
   for (size_t w = 0; w + 1 < waves.size(); ++w) {
-    const cudaError_t e = launch_gdp_ring(c->plan, c->ring, waves[w], waves[w + 1] - waves[w], in, out,
-                                          c->p.damping_shift, (int32_t)c->p.max_iters, nullptr, nullptr, 0,
-                                          c->p.barrier_budget_cycles, nullptr, 2, kRingPair, false, c->st);
+    const int32_t cnt = waves[w + 1] - waves[w];
+    CK(c, ring_build(c->plan, c->d_seg_off, b->d_rlist + waves[w], cnt, K, c->p.frac_bits, rows * c->nnz / c->n,
+                     kBatchRowEntries, b->count, c->ring, c->st, ring_pair_limit(), waves[w], most));
+    const cudaError_t e = launch_gdp_ring(c->plan, c->ring, cnt, in, out, c->p.damping_shift, (int32_t)c->p.max_iters,
+                                          nullptr, nullptr, 0, c->p.barrier_budget_cycles, nullptr, 2, kRingPair, false,
+                                          c->st);
     if (e == cudaErrorCooperativeLaunchTooLarge) {
       cudaGetLastError();
       CK(c, cudaStreamSynchronize(c->st));

@@ -337,7 +337,7 @@ struct RingArgs {
   unsigned long long* trace_ch;
   long long trace_cap, budget;
   int32_t max_sweeps;      // at most kRingSweeps
-  int32_t first_tile, K, F, shift, ecap, smem;
+  int32_t K, F, shift, ecap, smem;
 };
 struct RingPlan {
   int64_t version = -1;    // GdpPlan::version it was built from
@@ -357,11 +357,13 @@ struct RingPlan {
 void ring_free(RingPlan& p);
 // the tiles of K rings over the internal CSR: `tiles` equal shares of the one
 // segment's nodes (list NULL), or those of the device list; seg_off on the device;
+// first: of the phase's tiles, where these are some of them (their arrays have room
+// for `room` tiles, and `first` sets their words apart from the others')
 // maxdeg: the longest row a tile takes, at most kRingDepth; entries_per_tile: their
 // mean (a tile's room is what near-even tiles need), -1: the most a tile can hold
 cudaError_t ring_build(const GdpPlan& g, const int32_t* seg_off, const RingTile* list, int32_t tiles, int32_t K,
                        int32_t F, int64_t entries_per_tile, int32_t maxdeg, int32_t nseg, RingPlan& p, cudaStream_t st,
-                       const RingLimit& limit = RingLimit{});
+                       const RingLimit& limit = RingLimit{}, int32_t first = 0, int32_t room = 0);
 RingLimit ring_pair_limit();  // of kRingPair
 int32_t ring_smem(bool half, bool traced);  // dynamic shared memory of a CTA
 // per phase: cleared segment records and status; with limits before ring_build, which
@@ -379,8 +381,8 @@ inline bool ring_can_fit(int64_t n, int64_t nnz, int64_t tiles, int64_t smem, bo
 enum RingForm { kRingHalf = -1, kRingSmem = 0, kRingReg1 = 1, kRingReg2 = 2, kRingPair = 3 };
 int ring_reg_rows(const RingStats& st);  // rows a thread of the register form (0: does not fit)
 // (longs: the register form for graphs with rows past kRingLong entries, b_v = 2)
-// one cooperative launch over tiles [first_tile, first_tile + tiles): whole instances
-cudaError_t launch_gdp_ring(const GdpPlan& g, RingPlan& p, int32_t first_tile, int32_t tiles, const int32_t* lam_in,
+// one cooperative launch over the plan's tiles: whole instances
+cudaError_t launch_gdp_ring(const GdpPlan& g, RingPlan& p, int32_t tiles, const int32_t* lam_in,
                             int32_t* lam_out, int32_t shift, int32_t max_sweeps, long long* trace_b2,
                             unsigned long long* trace_ch, int64_t trace_cap, long long budget, const int32_t* bint,
                             int32_t bmax, RingForm form, bool longs, cudaStream_t st);

@@ -100,7 +100,8 @@ ring_plan_kernel(const int32_t* __restrict__ irp, const int2* __restrict__ iec, 
                  const int32_t* __restrict__ seg_off, int32_t tiles, int32_t K, int32_t F, int32_t ecap, int32_t maxdeg,
                  RingHdr* __restrict__ hdr, int32_t* __restrict__ halo, uint16_t* __restrict__ order,
                  uint32_t* __restrict__ slc, uint32_t* __restrict__ longs, int2* __restrict__ ent,
-                 int32_t* __restrict__ pos, RingStats* stats, RingSeg* seg, RingLimit limit) {
+                 int32_t* __restrict__ pos, RingStats* stats, RingSeg* seg, RingLimit limit,
+                 int32_t first) {
   extern __shared__ __align__(16) unsigned char smem[];
   int* keys = reinterpret_cast<int*>(smem);                         // [kHash] outside nodes
   int* ring = keys + kHash;                                         // [kRingHalo] in ring order
@@ -136,7 +137,7 @@ ring_plan_kernel(const int32_t* __restrict__ irp, const int2* __restrict__ iec, 
   h.seg = tl.seg;
   h.count = tl.count;
   h.first = tl.j == 0;
-  h.word0 = lo + 32 * b;
+  h.word0 = lo + 32 * (first + b);
   int bad = room < 32 ? kRingBadSize : 0;
   auto insert = [&](int c) {
     if (c >= lo && c < hi) return;
@@ -766,7 +767,7 @@ struct RegRows {
         if (LONG && depth > kRingLong) {
           const int4* row0 = reinterpret_cast<const int4*>(s_tail + (dt >> kDepthBits));
           long long none = 0;
-          long_rows<false>(A.longs[(size_t)(A.first_tile + blockIdx.x) * kRingSlices + (threadIdx.x >> 5) + r * NW], depth,
+          long_rows<false>(A.longs[(size_t)blockIdx.x * kRingSlices + (threadIdx.x >> 5) + r * NW], depth,
                            l, [&](int k, int row) { return row0[(k - D) * 16 + row]; }, lam(PAR), a, zb, zc, none);
         }
       }
@@ -926,7 +927,7 @@ __device__ __forceinline__ void ring_run(const RingArgs& A, const RingHdr& h, un
                                          RingTrace* trace = nullptr) {
   constexpr int NW = T / 32 - 1;  // warps with rows
   __shared__ RingShared S;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, b = A.first_tile + blockIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, b = blockIdx.x;
   const int ownp = (h.own + 31) & ~31;
   const uint16_t* order = A.order + (size_t)b * kRingSlots;
   const int32_t* halo = A.halo + (size_t)b * kRingHalo;
@@ -1007,7 +1008,7 @@ gdp_ring_smem_kernel(const __grid_constant__ RingArgs A) {
     if (threadIdx.x == 0) atomicOr(A.status, kGdpNoFit);
     return;
   }
-  const RingHdr h = A.hdr[A.first_tile + blockIdx.x];
+  const RingHdr h = A.hdr[blockIdx.x];
   RingTrace* trace = nullptr;
   if constexpr (BOUND) {
     __shared__ RingTrace s_trace;
@@ -1024,7 +1025,7 @@ __global__ void __launch_bounds__(T, 1024 / T)
 gdp_ring_reg_kernel(const __grid_constant__ RingArgs A) {
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr int NW = T / 32 - 1;
-  const RingHdr h = A.hdr[A.first_tile + blockIdx.x];
+  const RingHdr h = A.hdr[blockIdx.x];
   if constexpr (T == 512) {
     if (A.seg[h.seg].unfit) return;
   } else {
@@ -1076,26 +1077,27 @@ static cudaError_t ring_records(RingPlan& p, int32_t nseg) {
 
 cudaError_t ring_build(const GdpPlan& g, const int32_t* seg_off, const RingTile* list, int32_t tiles, int32_t K,
                        int32_t F, int64_t entries_per_tile, int32_t maxdeg, int32_t nseg, RingPlan& p,
-                       cudaStream_t st, const RingLimit& limit) {
+                       cudaStream_t st, const RingLimit& limit, int32_t first, int32_t room) {
   // room for a tile's sliced entries: its own and its inner rings'
   const int64_t want = entries_per_tile < 0 ? kMaxEntries
                        : K > 1              ? entries_per_tile * 2 + 16384
                                             : entries_per_tile * 3 / 2 + 4096;
   const int64_t ecap = (want < kMaxEntries ? want : kMaxEntries) / 64 * 64;
   p.version = -1;
-  RCK(grow(&p.hdr, &p.hdr_cap, tiles));
-  RCK(grow(&p.halo, &p.halo_cap, (int64_t)tiles * kRingHalo));
+  const int64_t m = room > tiles ? room : tiles;
+  RCK(grow(&p.hdr, &p.hdr_cap, m));
+  RCK(grow(&p.halo, &p.halo_cap, m * kRingHalo));
   RCK(grow(&p.pos, &p.pos_cap, g.n));
-  RCK(grow(&p.order, &p.order_cap, (int64_t)tiles * kRingSlots));
-  RCK(grow(&p.slc, &p.slc_cap, (int64_t)tiles * kRingSlices));
-  RCK(grow(&p.longs, &p.longs_cap, (int64_t)tiles * kRingSlices));
-  RCK(grow(&p.ent, &p.ent_cap, (int64_t)tiles * ecap));
+  RCK(grow(&p.order, &p.order_cap, m * kRingSlots));
+  RCK(grow(&p.slc, &p.slc_cap, m * kRingSlices));
+  RCK(grow(&p.longs, &p.longs_cap, m * kRingSlices));
+  RCK(grow(&p.ent, &p.ent_cap, m * ecap));
   RCK(ring_records(p, nseg));
   RCK(cudaMemsetAsync(&p.rec->stats, 0, sizeof(RingStats), st));
   constexpr size_t smem = 4 * (kHash + 2 * kRingHalo) + 2 * (kHash + kRingHalo + 2 * kRingLocals + kRingSlots);
   RCK(cudaFuncSetAttribute(ring_plan_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   ring_plan_kernel<<<tiles, kPlanThreads, smem, st>>>(g.irp, g.iec, list, seg_off, tiles, K, F, (int32_t)ecap, maxdeg, p.hdr,
-                                                      p.halo, p.order, p.slc, p.longs, p.ent, p.pos, &p.rec->stats, p.rec->seg, limit);
+                                                      p.halo, p.order, p.slc, p.longs, p.ent, p.pos, &p.rec->stats, p.rec->seg, limit, first);
   count_launch();
   RCK(cudaGetLastError());
   p.ecap = (int32_t)ecap;
@@ -1150,7 +1152,7 @@ int32_t ring_smem(bool half, bool traced) {
   return ((half ? sm / 2 - 1024 : optin) - 128 - (traced ? (int)sizeof(RingTrace) : 0)) & ~15;
 }
 
-cudaError_t launch_gdp_ring(const GdpPlan& g, RingPlan& p, int32_t first_tile, int32_t tiles, const int32_t* lam_in,
+cudaError_t launch_gdp_ring(const GdpPlan& g, RingPlan& p, int32_t tiles, const int32_t* lam_in,
                             int32_t* lam_out, int32_t shift, int32_t max_sweeps, long long* trace_b2,
                             unsigned long long* trace_ch, int64_t trace_cap, long long budget, const int32_t* bint,
                             int32_t bmax, RingForm form, bool longs, cudaStream_t st) {
@@ -1190,7 +1192,6 @@ cudaError_t launch_gdp_ring(const GdpPlan& g, RingPlan& p, int32_t first_tile, i
   a.trace_cap = trace_cap;
   a.max_sweeps = (int32_t)max_sweeps;
   a.budget = budget;
-  a.first_tile = first_tile;
   a.K = p.K;
   a.F = p.F;
   a.shift = shift;

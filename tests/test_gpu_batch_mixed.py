@@ -84,3 +84,19 @@ def test_the_others_stay_on_tiles(lib):
             ms[name] = min(ms.get(name, 1e9), tot.ms_gdp)
             assert tot.gdp_kernel == (TILES if name == "tiles" else STREAM)
     assert ms["mixed"] < 0.75 * ms["stream"], ms
+
+
+def test_scratch_does_not_grow_with_the_batch(lib):
+    # 6,000 tiles of 200 rows, twenty waves of them.  A wave's scratch is at most 304
+    # tiles of 430 KB, 0.13 GB; words, result arenas and the finisher's arrays of 1.2 M
+    # nodes and 14 M entries take 0.4 GB more.  All tiles' at once took 1.1 GB.
+    import torch
+    base = _some((200,) * 12)
+    insts = [base[i % 12] for i in range(6000)]
+    b = f2m.f2m_create_batch(insts, f2m.f2m_default_params(pricing=0, finisher=0, max_iters=8))
+    free = torch.cuda.mem_get_info()[0]
+    infos, tot = f2m.f2m_solve_batch(b, raise_on_error=False)
+    assert tot.gdp_kernel == TILES
+    assert free - torch.cuda.mem_get_info()[0] < 600 << 20
+    single = f2m.f2m_create(*base[5], f2m.f2m_default_params(pricing=0, finisher=0, max_iters=8))
+    assert infos[5999 // 12 * 12 - 7].iterations == f2m.f2m_solve(single, raise_on_error=False).iterations
