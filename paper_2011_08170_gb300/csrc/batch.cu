@@ -81,6 +81,7 @@ struct f2m_batch {
   std::vector<int32_t> res_fb, res_r0;  // fractional bits; first entry in the union's offsets
   std::vector<uint8_t> res_done;
   // tiles (gdp_ring.cu): those of a phase's active instances, wave by wave
+  bool ring_probed = false;         // the small instances' levels are known
   bool ring_off = false;            // not on this device: the streaming kernels
   std::vector<uint8_t> ring_level;  // per instance: 0 any tiles, 1 only of kBatchTileRows rows, 2 none that fit
   bool used_ring = false, used_stream = false;  // in a solve: some phase of some instance
@@ -314,6 +315,7 @@ extern "C" f2m_status f2m_create_batch_parts(int32_t count, const int32_t* n, co
 }
 
 constexpr int32_t kBatchRowEntries = 254;  // the longest row of a tile (the streaming kernels' smallest shape takes 256)
+constexpr int32_t kBatchSmall = 128;       // points below which an instance may be better streamed
 constexpr int32_t kBatchTileRows = 960;  // rows a tile: 15 warps of 2 slices
 
 // ---- GDP phase: tiles, kernel shape (autotuned), captured launch ----------------------
@@ -645,9 +647,9 @@ static f2m_status batch_cluster_phase(f2m_batch* b, const std::vector<uint8_t>& 
 // instance stay on chip for the phase, two tiles per SM; whole instances go
 // together in waves of as many tiles as the GPU holds.  Of the instances in `todo`
 // those that ran are cleared; one with a tile that does not fit keeps its lambda,
-// and its ring_level becomes `level` + 1.
+// and its ring_level becomes `level` + 1.  probe: just that, nothing runs.
 static f2m_status batch_ring_phase(f2m_batch* b, std::vector<uint8_t>& todo, int32_t rows, int32_t K, uint8_t level,
-                                   std::vector<int64_t>& sweeps_out, double* ms) {
+                                   std::vector<int64_t>& sweeps_out, double* ms, bool probe = false) {
   f2m_ctx* c = b->u;
   const int32_t room = 2 * c->num_sms;
   std::vector<RingTile> list;
@@ -684,6 +686,7 @@ static f2m_status batch_ring_phase(f2m_batch* b, std::vector<uint8_t>& todo, int
     const int32_t cnt = waves[w + 1] - waves[w];
     CK(c, ring_build(c->plan, c->d_seg_off, b->d_rlist + waves[w], cnt, K, c->p.frac_bits, rows * c->nnz / c->n,
                      kBatchRowEntries, b->count, c->ring, c->st, ring_pair_limit(), waves[w], most));
+    if (probe) continue;
     const cudaError_t e = launch_gdp_ring(c->plan, c->ring, cnt, in, out, c->p.damping_shift, (int32_t)c->p.max_iters,
                                           nullptr, nullptr, 0, c->p.barrier_budget_cycles, nullptr, 2, kRingPair, false,
                                           c->st);
@@ -709,12 +712,13 @@ static f2m_status batch_ring_phase(f2m_batch* b, std::vector<uint8_t>& todo, int
       b->ring_level[s] = (uint8_t)(level + 1);
       continue;
     }
+    if (probe) continue;
     todo[s] = 0;
     b->used_ring = true;
     sweeps_out[s] += b->h_rseg[s].sweeps;
     if (b->h_rseg[s].overflow) return fail(c, F2M_ERR_OVERFLOW, "|lambda| reached 2^29 in some instance");
   }
-  c->cur ^= 1;
+  if (!probe) c->cur ^= 1;
   return F2M_OK;
 }
 
@@ -751,12 +755,37 @@ static f2m_status batch_gdp_phase(f2m_batch* b, std::vector<uint8_t> active, std
     for (int32_t s = 0; s < b->count; ++s) nodes += active[s] ? b->n[s] : 0;
     const int32_t fine = (int32_t)std::max<int64_t>(96, (nodes / (2 * c->num_sms) + 31) / 32 * 32);
     f2m_status s = F2M_OK;
-    if (fine <= 320) s = batch_ring_phase(b, active, fine, fine <= 128 ? 3 : 2, 0, sweeps_out, ms);
-    if (s == F2M_OK && !b->ring_off) s = batch_ring_phase(b, active, kBatchTileRows, 1, 1, sweeps_out, ms);
+    // Small instances waste their tiles' rows (a wave of 304 takes 0.22 ms for 128
+    // sweeps however small they are), while streaming costs 0.9 ms and then 6 ns a
+    // node.  So instances of less than 128 points stream when they are more than four
+    // waves (10,000 of 64 points: 7.3 ms on tiles, 5.1 streaming; 20,000 of 100 points
+    // 16.6 and 12.1; but 5,000 of 200 points 4.7 and 6.9, 64 of 100 points 0.2 and
+    // 0.9), or when some instance has to stream in any case, which the first phase
+    // finds out for the small ones beforehand.
+    std::vector<uint8_t> todo = active;
+    int32_t small = 0;
+    for (int32_t i = 0; i < b->count; ++i) small += active[i] && b->n[i] < kBatchSmall;
+    if (small > 0) {
+      bool stream = small > 8 * c->num_sms;
+      if (!stream && !b->ring_probed) {
+        std::vector<uint8_t> few(b->count);
+        for (int32_t i = 0; i < b->count; ++i) few[i] = active[i] && b->n[i] < kBatchSmall;
+        s = batch_ring_phase(b, few, kBatchTileRows, 1, 1, sweeps_out, nullptr, true);
+        if (s != F2M_OK) return s;
+        b->ring_probed = true;
+      }
+      for (int32_t i = 0; i < b->count && !stream; ++i) stream = active[i] && b->ring_level[i] > 1;
+      for (int32_t i = 0; i < b->count && stream; ++i) todo[i] = todo[i] && b->n[i] >= kBatchSmall;
+    }
+    const std::vector<uint8_t> was = todo;
+    if (fine <= 320) s = batch_ring_phase(b, todo, fine, fine <= 128 ? 3 : 2, 0, sweeps_out, ms);
+    if (s == F2M_OK && !b->ring_off) s = batch_ring_phase(b, todo, kBatchTileRows, 1, 1, sweeps_out, ms);
     if (s != F2M_OK) return s;
+    for (int32_t i = 0; i < b->count; ++i)
+      if (was[i] && !todo[i]) active[i] = 0;
     if (std::find(active.begin(), active.end(), 1) == active.end()) return F2M_OK;
   }
-  b->used_stream = true;  // the instances left over: with rows, edges or sizes that no tile takes
+  b->used_stream = true;  // the instances left over: of rows, edges or sizes that no tile takes, or small
   if (b->tiles_version != P.version) {
     f2m_status s = F2M_OK;
     if (c->p.batch_shape >= 0) {

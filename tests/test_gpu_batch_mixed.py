@@ -100,3 +100,39 @@ def test_scratch_does_not_grow_with_the_batch(lib):
     assert free - torch.cuda.mem_get_info()[0] < 600 << 20
     single = f2m.f2m_create(*base[5], f2m.f2m_default_params(pricing=0, finisher=0, max_iters=8))
     assert infos[5999 // 12 * 12 - 7].iterations == f2m.f2m_solve(single, raise_on_error=False).iterations
+
+
+def _close(n, count, seed=0):  # points near each other: short edges
+    rng = np.random.default_rng(seed)
+    return [_knn(np.unique(rng.integers(0, 60_000, (2 * n, 2)), axis=0)[:n].astype(np.int32), 6) for _ in range(count)]
+
+
+@pytest.mark.parametrize("n,count,extra,want", [
+    (40, 300, 0, TILES), (127, 1216, 0, TILES), (127, 1217, 0, STREAM), (128, 1300, 0, TILES), (30, 3000, 2, STREAM),
+    (20, 5, 1, STREAM)])
+def test_small_instances(lib, n, count, extra, want):
+    # 1,216 is four waves of 304 tiles; `extra` larger ones keep their tiles
+    base = _close(n, min(count, 20))
+    insts = [base[i % len(base)] for i in range(count)] + _some((1500, 700)[:extra])
+    if extra == 1:
+        insts.append(_far())
+    tot, got = _solve(insts)
+    assert tot.gdp_kernel == want
+    assert got == _solve(insts, batch_shape=5)[1]
+
+
+def test_many_small_instances_cost_what_they_did(lib):
+    # 10,000 instances of 64 points, 33 waves of tiles, take half as long again on tiles
+    # as streamed; the line is at a fifth
+    base = _close(64, 20)
+    insts = [base[i % 20] for i in range(10_000)]
+
+    def ms(shape):
+        best = 1e9
+        for _ in range(3):
+            b = f2m.f2m_create_batch(insts, f2m.f2m_default_params(pricing=0, finisher=0, batch_shape=shape))
+            best = min(best, f2m.f2m_solve_batch(b, raise_on_error=False)[1].ms_gdp)
+        return best
+
+    default, best = ms(-1), min(ms(shape) for shape in range(12))
+    assert default < 1.2 * best, (default, best)
