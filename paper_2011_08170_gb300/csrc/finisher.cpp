@@ -272,15 +272,22 @@ FinisherWork* finisher_work_take(int32_t n) {
 
 void finisher_work_free(FinisherWork* w) {
   const size_t bytes = work_bytes(w);
+  if (bytes > kWorkCacheMax) {
+    delete w;
+    return;
+  }
+  std::vector<FinisherWork*> old;  // the longest unused make room
   {
     std::lock_guard<std::mutex> lk(g_work_mu);
-    if (g_work_bytes + bytes <= kWorkCacheMax && g_work_free.size() < 64) {
-      g_work_bytes += bytes;
-      g_work_free.push_back(w);
-      return;
-    }
+    size_t k = 0;
+    for (; k < g_work_free.size() && (g_work_bytes + bytes > kWorkCacheMax || g_work_free.size() - k >= 64); ++k)
+      g_work_bytes -= work_bytes(g_work_free[k]);
+    old.assign(g_work_free.begin(), g_work_free.begin() + k);
+    g_work_free.erase(g_work_free.begin(), g_work_free.begin() + k);
+    g_work_bytes += bytes;
+    g_work_free.push_back(w);
   }
-  delete w;
+  for (FinisherWork* o : old) delete o;
 }
 
 void host_copy(const std::vector<HostCopy>& parts) {

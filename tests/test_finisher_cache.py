@@ -61,3 +61,16 @@ def test_copies_without_threads(tmp_path):
                     "-o", exe], check=True, capture_output=True)
     r = subprocess.run([exe], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0 and r.stdout == "copied\n", (r.returncode, r.stderr)
+
+
+def test_what_is_freed_last_is_kept(cache):
+    # a block near the bound (2.9 M nodes, 255 MB) makes room for others
+    cache.shim_free(cache.shim_take(2_900_000))
+    sizes = [400_000, 300_000, 50_000]
+    for n in sizes:
+        cache.shim_free(cache.shim_take(n))
+    assert [cache.shim_nodes(cache.shim_take(n - 1)) for n in sizes] == sizes
+    many = [cache.shim_take(20_000 + 100 * i) for i in range(70)]  # more than 64: the first six go
+    for w in many:
+        cache.shim_free(w)
+    assert cache.shim_nodes(cache.shim_take(20_000)) == 20_600
