@@ -66,7 +66,7 @@ def test_copies_without_threads(tmp_path):
 def test_what_is_freed_last_is_kept(cache):
     # a block near the bound (2.9 M nodes, 255 MB) makes room for others
     cache.shim_free(cache.shim_take(2_900_000))
-    sizes = [400_000, 300_000, 50_000]
+    sizes = [400_000, 150_000, 50_000]
     for n in sizes:
         cache.shim_free(cache.shim_take(n))
     assert [cache.shim_nodes(cache.shim_take(n - 1)) for n in sizes] == sizes
