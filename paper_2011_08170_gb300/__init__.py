@@ -349,8 +349,9 @@ def f2m_price(ctx: Ctx, cap: int | None = None):
     if cap is not None and c > cap:
         return c, None
     if c > room:
-        out = np.zeros((c, 2), np.int32)
+        out = np.empty((c, 2), np.int32)
         _check(ctx, L.f2m_price(ctx.handle, C.byref(cnt), out.ctypes.data, c))
+        return c, out
     return c, out[:c].copy()
 
 
