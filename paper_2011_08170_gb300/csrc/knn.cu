@@ -17,8 +17,10 @@
 // 2k + 4 points, and where it was too small the k-th distance found says what the
 // next one has to cover; (ii) rows are taken from the point outwards, and with a
 // full list only the cells within its last distance are read; (iii) an entry is
-// one word, d^2 above the index, kept sorted by min and max without branches (128
-// bits where 41 + the index bits pass 64).  Rings of cells of 2 points each, with
+// one word, d^2 above the index, kept sorted by min and max without branches (where 41
+// + the index bits pass 64, points too far for the rest are left out, and where a
+// point has fewer than k others nearer, all queries run again with 128 bits: 8.4 M
+// uniform points, k = 8, 36 ms with 128 bits, below 3 without).  Rings of cells of 2 points each, with
 // 64-bit compares of pairs, took 152 us at 100,000 uniform points, k = 10, and 520
 // us at 200,000 clustered ones, k = 16: now 46 and 246,
 // the latter with the features of the points.  Not faster: offsets
@@ -134,12 +136,13 @@ __device__ __forceinline__ void write_features(const long long (&d2)[kFeatures],
   *scale = sh;
 }
 
-// FEAT: the features of each point (k = 16) instead of its list
-template <int K, typename Key, bool FEAT>
+// FEAT: the features of each point (k = 16) instead of its list.  CUT: entries hold d^2
+// below 2^(64 - ibits); *far is set where a list has none for its place k.
+template <int K, typename Key, bool FEAT, bool CUT>
 __global__ void __launch_bounds__(128)
 knn_query_kernel(const int4* __restrict__ pts, const int32_t* __restrict__ start, int32_t n, int32_t k, KnnGrid g,
                  int ibits, int32_t* __restrict__ nbr, long long* __restrict__ d2out, float* __restrict__ feat,
-                 float* __restrict__ scale) {
+                 float* __restrict__ scale, int32_t* __restrict__ far) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n) return;
   const int4 me = pts[t];
@@ -187,7 +190,9 @@ knn_query_kernel(const int4* __restrict__ pts, const int32_t* __restrict__ start
         for (int a = start[(gy << g.gbits) + ga]; a < b; ++a) {
           const int4 q = pts[a];
           const int dx = q.x - x, dy = q.y - y;
-          Key key = ((Key)((unsigned long long)((long long)dx * dx + (long long)dy * dy)) << ibits) | (Key)(unsigned)q.z;
+          const unsigned long long dd = (unsigned long long)((long long)dx * dx + (long long)dy * dy);
+          if (CUT && dd >> (64 - ibits)) continue;
+          Key key = ((Key)dd << ibits) | (Key)(unsigned)q.z;
           if (a != t && key < best[K - 1]) {
 #pragma unroll
             for (int p = 0; p < K; ++p) {
@@ -212,6 +217,7 @@ knn_query_kernel(const int4* __restrict__ pts, const int32_t* __restrict__ start
 #pragma unroll
     for (int p = 0; p < K - 1; ++p) kth = p == k - 1 ? best[p] : kth;
     if (kth == none) {
+      if (CUT && (unsigned long long)(bnd * bnd) >> (64 - ibits)) break;  // the others are too far
       r = 2 * r + 1;
       continue;
     }
@@ -219,6 +225,12 @@ knn_query_kernel(const int4* __restrict__ pts, const int32_t* __restrict__ start
     if (d2 < bnd * bnd) break;
     // a square of this half side covers the k-th distance (checked again after it)
     r = max(r + 1, (int)(sqrtf((float)d2) * 1.000001f / (float)(1 << g.shift)) + 1);
+  }
+  if (CUT) {
+    Key kth = best[K - 1];
+#pragma unroll
+    for (int p = 0; p < K - 1; ++p) kth = p == k - 1 ? best[p] : kth;
+    if (kth == none) *far = 1;
   }
   if (FEAT) {
     long long d2[kFeatures];
@@ -342,10 +354,11 @@ KnnGrid knn_grid(int32_t n) {
   return KnnGrid{20 - g, g};
 }
 
-template <int K, typename Key, bool FEAT = false>
+template <int K, typename Key, bool FEAT = false, bool CUT = false>
 void knn_query(const int4* pts, const int32_t* start, int32_t n, int32_t k, KnnGrid g, int ibits, int32_t* nbr,
-               long long* d2, float* feat, float* scale, cudaStream_t st) {
-  knn_query_kernel<K, Key, FEAT><<<blocks_for(n, 128), 128, 0, st>>>(pts, start, n, k, g, ibits, nbr, d2, feat, scale);
+               long long* d2, float* feat, float* scale, int32_t* far, cudaStream_t st) {
+  knn_query_kernel<K, Key, FEAT, CUT><<<blocks_for(n, 128), 128, 0, st>>>(pts, start, n, k, g, ibits, nbr, d2, feat,
+                                                                         scale, far);
   count_launch();
 }
 
@@ -374,10 +387,24 @@ cudaError_t knn_enqueue(KnnScope& w, const int2* d_xy, int32_t n, int32_t k, int
   using u64 = unsigned long long;
   using u128 = unsigned __int128;
   const bool wide = ibits > 64 - 41;  // d^2 < 2^41
-#define F2M_KNN(...) knn_query<__VA_ARGS__>(pts, start, n, k, g, ibits, d_nbr, d_d2, feat, scale, st)
-  if (feat && wide) F2M_KNN(kFeatures, u128, true);
-  else if (feat) F2M_KNN(kFeatures, u64, true);
-  else if (wide) F2M_KNN(32, u128);
+  int32_t* far = nullptr;
+#define F2M_KNN(...) knn_query<__VA_ARGS__>(pts, start, n, k, g, ibits, d_nbr, d_d2, feat, scale, far, st)
+  if (wide) {
+    e = w.get(&far, 1);
+    if (e == cudaSuccess) e = cudaMemsetAsync(far, 0, sizeof(int32_t), st);
+    if (e != cudaSuccess) return e;
+    if (feat) F2M_KNN(kFeatures, u64, true, true);
+    else if (k <= 8) F2M_KNN(8, u64, false, true);
+    else if (k <= 16) F2M_KNN(16, u64, false, true);
+    else F2M_KNN(32, u64, false, true);
+    e = cudaGetLastError();
+    int32_t h = 0;
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&h, far, sizeof(h), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess || !h) return e;
+    if (feat) F2M_KNN(kFeatures, u128, true);
+    else F2M_KNN(32, u128);
+  } else if (feat) F2M_KNN(kFeatures, u64, true);
   else if (k <= 8) F2M_KNN(8, u64);
   else if (k <= 10) F2M_KNN(10, u64);
   else if (k <= 12) F2M_KNN(12, u64);
