@@ -83,7 +83,7 @@ typedef struct {
   int64_t barrier_budget_cycles;/* spin budget of one device-wide barrier wait; default 4e9 */
   int32_t finisher;             /* 1 = exact finisher when rule (7) gives an infeasible x (default) */
   uint32_t flags;               /* F2M_FLAG_* bits; default 0 */
-  int32_t gdp_lanes;            /* lanes per node in the tiled GDP kernel: 1 (one thread per node); 0 = auto */
+  int32_t gdp_lanes;            /* 0 or 1; no effect (the tiled GDP kernel takes one thread per node) */
   int32_t gdp_ctas_per_sm;      /* tiled GDP CTAs per SM: 1 (x1024 threads), 2 (x512, one sweep
                                    per exchange); 0 = auto */
   int32_t batch_shape;          /* batched GDP: -1 = on-chip tiles, or where they do not fit the

@@ -360,7 +360,7 @@ extern "C" void f2m_destroy(f2m_ctx* c) {
   dfree(c->d_mlmax); dfree(c->d_mframes); dfree(c->d_mcand); dfree(c->d_mncand);
   dfree(c->d_lam_ref); dfree(c->d_raised); dfree(c->d_pts_raised);
   dfree(c->d_boxes); dfree(c->d_smax); dfree(c->d_pctl); dfree(c->d_pseg); dfree(c->d_plist);
-  dfree(c->d_count); dfree(c->d_tile); dfree(c->d_deg); dfree(c->d_tmp_rp); dfree(c->d_new_rp);
+  dfree(c->d_count); dfree(c->d_deg); dfree(c->d_tmp_rp); dfree(c->d_new_rp);
   dfree(c->d_block_sums); dfree(c->d_tmp_col); dfree(c->d_out_a); dfree(c->d_out_b);
   dfree(c->d_check); dfree(c->d_scalar); dfree(c->d_bad); dfree(c->d_b); dfree(c->d_b_int);
   dfree(c->d_ring_seg);
@@ -915,7 +915,6 @@ static f2m_status price_mma(f2m_ctx* c, const int32_t* lam, int32_t fb, double* 
   // the tile-pair list depends only on the segments scanned: it stays on the
   // device from one scan to the next while they are the same
   if (!c->d_count) CK(c, dalloc(&c->d_count, 1));
-  if (!c->d_tile) CK(c, dalloc(&c->d_tile, 1));
   if (!c->d_pts4) CK(c, dalloc(&c->d_pts4, c->n));
   if (!c->d_pstat) CK(c, dalloc(&c->d_pstat, 1));
   if (!c->d_mncand) CK(c, dalloc(&c->d_mncand, 1));
@@ -964,7 +963,7 @@ static f2m_status price_mma(f2m_ctx* c, const int32_t* lam, int32_t fb, double* 
     CK(c, launch_pricing_mma_scan(c->d_pts4, c->d_xy, lam, c->d_rp, c->d_ec, fb, c->d_tiles, c->d_mtblk,
                                   (int32_t)c->ntiles, c->d_mranges, (int32_t)c->mblocks, c->d_mbox, c->d_mlmax,
                                   c->d_mframes, c->d_mcand, c->mcand_cap, c->d_mncand, c->d_pairs,
-                                  c->pairs_cap, c->d_count, c->d_tile, c->d_pstat, c->num_sms, c->st));
+                                  c->pairs_cap, c->d_count, c->d_pstat, c->num_sms, c->st));
     CK(c, cudaEventRecord(c->ev1, c->st));
     unsigned long long cnt = 0, ncand = 0;
     int32_t pstat = 0;

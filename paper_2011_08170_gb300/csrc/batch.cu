@@ -2,10 +2,11 @@
 //
 // The instances become one disjoint union of segments (instance s = nodes
 // [seg_off[s], seg_off[s+1]) of the union).  Every device step of a solve
-// covers all instances at once -- one persistent GDP launch per phase
-// (gdp_batch_kernel, converged instances frozen), one pricing scan over the
-// tile pairs of the instances that need one, one merge, one extraction, one
-// finisher call -- and the host keeps, per instance, the state of the solve
+// covers all instances at once -- one GDP phase (on tiles, in waves of whole
+// instances; those that no tile takes stream, gdp_batch_kernel, converged ones
+// frozen), one pricing scan over the tile pairs of the instances that need one,
+// one merge, one extraction, one finisher call -- and the host keeps, per
+// instance, the state of the solve
 // loop of f2m_solve.  Since no step mixes instances, each instance's lambda,
 // x and bound are those of its own solve (the finisher is told which
 // instances it may touch).

@@ -56,8 +56,7 @@ struct f2m_ctx {
   int64_t x2_cap = 0;
   int32_t* d_lam[2] = {nullptr, nullptr};
   int32_t* d_lam2 = nullptr;
-  int32_t* d_exl = nullptr;   // [n] the finisher's surpluses (its own: the plan's scratch
-                              // still feeds a two-sweep plan built later)
+  int32_t* d_exl = nullptr;   // [n] the finisher's surpluses
   int32_t* d_b = nullptr;  // degree requirements b_v, caller order (NULL: b_v = 2)
   int32_t* d_b_int = nullptr;  // the same in the renumbered (internal) order
   int32_t b_max = 2;       // the largest b_v
@@ -99,7 +98,6 @@ struct f2m_ctx {
   int64_t pairs_cap = 0;
   int64_t npairs = 0;   // pairs held in d_pairs after the last scan
   unsigned long long* d_count = nullptr;
-  unsigned int* d_tile = nullptr;
   int32_t* d_deg = nullptr;
   int32_t* d_tmp_rp = nullptr;
   int32_t* d_new_rp = nullptr;

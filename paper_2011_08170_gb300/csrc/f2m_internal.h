@@ -180,7 +180,7 @@ cudaError_t launch_pricing_mma_scan(const int4* pts4, const int2* xy, const int3
                                     int32_t ntiles, const int2* ranges, int32_t nblocks, int4* box, int32_t* lmax,
                                     int4* frames, int2* cand, int64_t cand_cap, unsigned long long* ncand,
                                     int2* pairs, int64_t cap, unsigned long long* count,
-                                    unsigned int* tile_counter, int32_t* status, int num_sms, cudaStream_t st);
+                                    int32_t* status, int num_sms, cudaStream_t st);
 // CSR union with pairs; sizes: see graph.cu.  Returns the new nnz through *new_nnz_dev.
 struct MergeBuffers {
   int32_t* deg;        // [n+1]
@@ -268,7 +268,7 @@ cudaError_t scatter_perm(const int32_t* src, const int32_t* perm, int32_t n, int
                          cudaStream_t st);
 void plan_free(GdpPlan& p);
 // ---- GDP on shared-memory tiles (gdp_ring.cu) --------------------------------------
-constexpr int kRingMax = 6;          // rings around a tile: sweeps per exchange
+constexpr int kRingMax = 4;          // rings around a tile: sweeps per exchange (ring_sweeps asks for no more)
 constexpr int kRingLocals = 8192;    // nodes a tile knows (own, rings, two padding slots)
 constexpr int kRingHalo = 4096;      // of them in rings
 constexpr int kRingDepth = 1536;     // entries of a row at most: 32 such rows are all that a tile can hold

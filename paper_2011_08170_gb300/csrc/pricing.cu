@@ -225,9 +225,8 @@ __device__ __noinline__ void pricing_confirm(int i, int j, const int2* __restric
   if ((long long)k < cap) pairs[k] = make_int2(i, j);
 }
 
-// The filter of one pair, from a_v, c_v, y_v of the j-point and the negated
-// a_u, c_u, y_u of the i-point; the hot loop evaluates the same operations two
-// pairs at a time
+// The fp32 filter of one pair (test 2), from a_v, c_v, y_v of the j-point and the
+// negated a_u, c_u, y_u of the i-point
 __device__ __forceinline__ float pricing_filter(float aj, float cj, float yj, float nai, float nci, float nyi) {
   const float u = __fadd_rn(aj, nci), w = __fadd_rn(cj, nai), dy = __fadd_rn(yj, nyi);
   return __fmaf_rn(dy, dy, __fmaf_rn(u, w, -1.0f));
@@ -657,7 +656,6 @@ struct MmaArgs {
   int2* pairs;
   long long cap;
   unsigned long long* count;
-  unsigned int* tile_counter;
   int32_t* status;         // bit 0: an mbarrier wait gave up
   int2* cand;              // candidate pairs {ii, jj} (positions), decided by pricing_mma_confirm_kernel
   unsigned long long* ncand;
@@ -1036,10 +1034,9 @@ cudaError_t launch_pricing_mma_scan(const int4* pts4, const int2* xy, const int3
                                     int32_t ntiles, const int2* ranges, int32_t nblocks, int4* box, int32_t* lmax,
                                     int4* frames, int2* cand, int64_t cand_cap, unsigned long long* ncand,
                                     int2* pairs, int64_t cap, unsigned long long* count,
-                                    unsigned int* tile_counter, int32_t* status, int num_sms, cudaStream_t st) {
+                                    int32_t* status, int num_sms, cudaStream_t st) {
   cudaError_t err = cudaMemsetAsync(count, 0, sizeof(unsigned long long), st);
   if (err == cudaSuccess) err = cudaMemsetAsync(ncand, 0, sizeof(unsigned long long), st);
-  if (err == cudaSuccess) err = cudaMemsetAsync(tile_counter, 0, sizeof(unsigned int), st);
   if (err == cudaSuccess) err = cudaMemsetAsync(status, 0, sizeof(int32_t), st);
   if (err != cudaSuccess) return err;
   if (ntiles == 0) return cudaSuccess;
@@ -1062,7 +1059,6 @@ cudaError_t launch_pricing_mma_scan(const int4* pts4, const int2* xy, const int3
   a.pairs = pairs;
   a.cap = cap;
   a.count = count;
-  a.tile_counter = tile_counter;
   a.status = status;
   a.cand = cand;
   a.ncand = ncand;
