@@ -1171,8 +1171,8 @@ f2m_status f2m::merge_internal(f2m_ctx* c, const int2* d_pairs, int64_t npairs, 
     CK(c, launch_merge_fill(c->d_rp, c->d_ec, d_pairs, npairs, n, mb, c->st));
   }
   CK(c, dgrow(&c->d_ec_alt, &c->ec_alt_cap, need, need + (need >> 3)));  // the merged rows go there
-  CK(c, dgrow(&c->d_x2, &c->x2_cap, need, need + (need >> 3)));
   if (fresh) {
+    CK(c, dgrow(&c->d_x2, &c->x2_cap, need, need + (need >> 3)));
     CK(c, plan_merge(c->d_xy, c->d_rp, c->d_ec, d_pairs, npairs, n, need, mb, c->d_ec_alt, c->plan, c->st));
     std::swap(c->d_ec, c->d_ec_alt);
     std::swap(c->ec_cap, c->ec_alt_cap);
@@ -1183,15 +1183,17 @@ f2m_status f2m::merge_internal(f2m_ctx* c, const int2* d_pairs, int64_t npairs, 
     return F2M_OK;
   }
   CK(c, launch_merge_finish(c->d_xy, c->d_rp, c->d_ec, n, mb, c->d_ec_alt, c->st));
-  std::swap(c->d_ec, c->d_ec_alt);
-  std::swap(c->ec_cap, c->ec_alt_cap);
-  CK(c, cudaMemcpyAsync(c->d_rp, c->d_new_rp, sizeof(int32_t) * (n + 1), cudaMemcpyDeviceToDevice, c->st));
   int32_t nnz_h = 0;
   CK(c, cudaMemcpyAsync(&nnz_h, c->d_new_rp + n, sizeof(int32_t), cudaMemcpyDeviceToHost, c->st));
   CheckCtl h{};
   CK(c, read_check(c, &h));
-  c->nnz = nnz_h;
+  // refused pairs leave the graph as it was, in both orders
   if (h.flags) return fail(c, F2M_ERR_INVALID_ARG, check_message(h.flags, h.first_bad));
+  CK(c, dgrow(&c->d_x2, &c->x2_cap, need, need + (need >> 3)));
+  std::swap(c->d_ec, c->d_ec_alt);
+  std::swap(c->ec_cap, c->ec_alt_cap);
+  CK(c, cudaMemcpyAsync(c->d_rp, c->d_new_rp, sizeof(int32_t) * (n + 1), cudaMemcpyDeviceToDevice, c->st));
+  c->nnz = nnz_h;
   // the internal CSR now (the finisher reads it); the GDP tiles only serve GDP
   // phases: built when the next one starts (a merge before the finisher and the
   // last scan needs none)
