@@ -1172,7 +1172,7 @@ f2m_status f2m::merge_internal(f2m_ctx* c, const int2* d_pairs, int64_t npairs, 
   }
   CK(c, dgrow(&c->d_ec_alt, &c->ec_alt_cap, need, need + (need >> 3)));  // the merged rows go there
   if (fresh) {
-    CK(c, dgrow(&c->d_x2, &c->x2_cap, need, need + (need >> 3)));
+    CK(c, dev_regrow(&c->d_x2, &c->x2_cap, need, need + (need >> 3)));
     CK(c, plan_merge(c->d_xy, c->d_rp, c->d_ec, d_pairs, npairs, n, need, mb, c->d_ec_alt, c->plan, c->st));
     std::swap(c->d_ec, c->d_ec_alt);
     std::swap(c->ec_cap, c->ec_alt_cap);
@@ -1189,7 +1189,8 @@ f2m_status f2m::merge_internal(f2m_ctx* c, const int2* d_pairs, int64_t npairs, 
   CK(c, read_check(c, &h));
   // refused pairs leave the graph as it was, in both orders
   if (h.flags) return fail(c, F2M_ERR_INVALID_ARG, check_message(h.flags, h.first_bad));
-  CK(c, dgrow(&c->d_x2, &c->x2_cap, need, need + (need >> 3)));
+  CK(c, dev_regrow(&c->d_x2, &c->x2_cap, need, need + (need >> 3)));
+  CK(c, plan_room(n, nnz_h, c->plan));
   std::swap(c->d_ec, c->d_ec_alt);
   std::swap(c->ec_cap, c->ec_alt_cap);
   CK(c, cudaMemcpyAsync(c->d_rp, c->d_new_rp, sizeof(int32_t) * (n + 1), cudaMemcpyDeviceToDevice, c->st));

@@ -61,6 +61,20 @@ enum CheckBits {
 cudaError_t dev_malloc(void** p, size_t bytes);
 void dev_free(void* p);
 void dev_free_synced(void* p);
+// Room for `need` items in *p, whose values are not kept: as it is, or a block of
+// `room`.  Where there is no memory the old block stays, so that calls after a
+// failed one find every array that the graph they see needs.
+template <typename T>
+cudaError_t dev_regrow(T** p, int64_t* cap, int64_t need, int64_t room) {
+  if (*p && *cap >= need) return cudaSuccess;
+  void* q = nullptr;
+  const cudaError_t e = dev_malloc(&q, sizeof(T) * (size_t)room);
+  if (e != cudaSuccess) return e;
+  if (*p) dev_free(*p);
+  *p = (T*)q;
+  *cap = room;
+  return cudaSuccess;
+}
 // whether a kernel on device `current` may write to memory of this kind on `device`
 // (another GPU's memory only by a copy)
 inline bool kernel_reaches(cudaMemoryType type, int device, int current) {
@@ -260,6 +274,8 @@ cudaError_t plan_renumber(const int2* xy, int32_t n, const std::vector<int32_t>&
 cudaError_t plan_merge(const int2* xy, const int32_t* rp, const int2* ec_in, const int2* pairs, int64_t npairs,
                        int32_t n, int64_t nnz, MergeBuffers& mb, int2* ec_out, GdpPlan& p, cudaStream_t st);
 // the CSR in the renumbered order
+// room for a graph of nnz entries (the arrays stay as they are where there is none)
+cudaError_t plan_room(int32_t n, int64_t nnz, GdpPlan& p);
 cudaError_t plan_build(const int32_t* rp, const int2* ec, int32_t n, int64_t nnz, GdpPlan& p, cudaStream_t st);
 // dst[i] = src[perm[i]]  /  dst[perm[i]] = src[i]
 cudaError_t gather_perm(const int32_t* src, const int32_t* perm, int32_t n, int32_t* dst,

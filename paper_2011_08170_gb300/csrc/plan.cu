@@ -89,14 +89,7 @@ __global__ void scatter_perm_kernel(const int32_t* __restrict__ src, const int32
 
 template <typename T>
 static cudaError_t grow(T** p, int64_t* cap, int64_t need) {
-  if (*p && *cap >= need) return cudaSuccess;
-  if (*p) dev_free(*p);
-  *p = nullptr;
-  *cap = 0;
-  const int64_t c = need + (need >> 3) + 64;
-  cudaError_t e = dev_malloc((void**)p, sizeof(T) * (size_t)c);
-  if (e == cudaSuccess) *cap = c;
-  return e;
+  return dev_regrow(p, cap, need, need + (need >> 3) + 64);
 }
 
 void plan_free(GdpPlan& p) {

@@ -35,6 +35,21 @@ extern "C" int shim_grow(long long had, long long need, long long room, int bloc
   return r;
 }
 
+// dev_regrow: bit 0 success, bit 1 a block is held, bit 2 the capacity covers `need`,
+// bit 3 the block is the old one
+extern "C" int shim_regrow(long long had, long long need, long long room, int blocks) {
+  int* p = nullptr;
+  int64_t cap = 0;
+  g_blocks = 1;
+  if (had) f2m::dev_regrow(&p, &cap, had, had);
+  const int* old = p;
+  g_blocks = blocks;
+  const bool ok = f2m::dev_regrow(&p, &cap, need, room) == cudaSuccess;
+  const int r = ok | (p != nullptr) << 1 | (cap >= need) << 2 | (had && p == old) << 3;
+  std::free(p);
+  return r;
+}
+
 extern "C" long long shim_price_list_room(unsigned long long listed) { return f2m::price_list_room(listed); }
 
 extern "C" int shim_ring_can_fit(long long n, long long nnz, long long tiles, long long smem, int half) {

@@ -52,6 +52,19 @@ def test_a_failed_allocation_claims_no_room(rules, had, need, room, blocks, want
     assert rules.shim_grow(had, need, room, blocks) == want
 
 
+OLD = 8
+
+
+@pytest.mark.parametrize("had,need,room,blocks,want", [
+    (0, 10, 15, 1, OK | HELD | COVERS), (20, 10, 15, 0, OK | HELD | COVERS | OLD), (5, 10, 15, 1, OK | HELD | COVERS),
+    (5, 10, 15, 0, HELD | OLD),  # no memory: the graph keeps its arrays
+    (0, 10, 15, 0, 0)])
+def test_a_failed_merge_leaves_the_graph_its_arrays(rules, had, need, room, blocks, want):
+    # given back first, the renumbered graph was gone and the next sweep read through null
+    rules.shim_regrow.argtypes = [C.c_longlong] * 3 + [C.c_int]
+    assert rules.shim_regrow(had, need, room, blocks) == want
+
+
 def test_no_capacity_is_noted_before_its_allocation():
     # the sources: a member's capacity is assigned from its size only after the block is there
     import re
