@@ -283,7 +283,7 @@ f2m_status f2m_price(f2m_ctx* ctx, int64_t* count, int32_t* pairs, int64_t cap);
 /* Adds undirected edges to the candidate graph (both directions, rows kept
  * sorted, pairs already present ignored) and their costs.
  *   pairs  [npairs][2] int32, host or device, u != v, both in [0, n).
- * Errors: INVALID_ARG, OOM, CUDA. */
+ * Errors: INVALID_ARG, OOM (the graph stays as it was), CUDA. */
 f2m_status f2m_add_edges(f2m_ctx* ctx, const int32_t* pairs, int64_t npairs);
 
 /* Primal from rule (7): x2_e = 2 if z_e < 0, 1 if z_e = 0, 0 if z_e > 0 (x in
